@@ -155,7 +155,7 @@ int alloc_plan(Plan* p) {
     GB_TRY(dalloc(&p->Yhat, (int64_t)p->l * p->D));
     GB_TRY(dalloc(&p->Cls, 2 * (int64_t)p->l * k2));
     GB_TRY(dalloc(&p->YPhi, (int64_t)p->l * k2));
-    GB_TRY(dalloc(&p->clsPart, 128 * (int64_t)p->l * p->D + 128 * (int64_t)p->l));
+    GB_TRY(dalloc(&p->clsPart, 128 * (int64_t)p->l * p->D + 129 * (int64_t)p->l));
   }
   GB_TRY(dalloc(&p->st, 1));
   GB_CUDA(cudaMallocHost(reinterpret_cast<void**>(&p->st_host), sizeof(DevState)));

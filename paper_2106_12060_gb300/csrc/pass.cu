@@ -391,15 +391,32 @@ __global__ void phi_convert_kernel(const double* __restrict__ a, Tacc* __restric
     b[i] = (Tacc)a[i];
 }
 
-// class-mean rows times Phi: Cls (l x NC) = means (l x d) Phi (d x 2k), FDA only
-__global__ void lda_cls_kernel(const double* __restrict__ means, const double* __restrict__ Phi, int l,
-                               int d, int k2, int stride, double* __restrict__ Cls) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= l * k2) return;
-  int cls = e / k2, c = e % k2;
-  double s = 0;
-  for (int j = 0; j < d; ++j) s += means[(int64_t)cls * d + j] * Phi[(int64_t)j * stride + c];
-  Cls[e] = s;
+// out (r x c) = T (r x d) Phi[:, 0:c], Phi row-major with row stride `stride`:
+// a class table (FDA: the class means, or Yhat) times the current Phi.  One
+// warp per entry, the lanes over the inner index with four partial sums in
+// flight, a fixed shuffle tree.  Latency bound (r c is a few hundred, d at
+// most 1024): one thread per entry walking all d terms is a chain of d
+// dependent FP64 adds behind d loads (l = 10, d = 784, 18 columns: 184 us a
+// launch, once per iteration); with a warp per entry 25 terms per lane remain.
+__global__ void __launch_bounds__(256) table_phi_kernel(const double* __restrict__ T, const double* __restrict__ Phi,
+                                                        int r, int d, int c, int stride, double* __restrict__ out,
+                                                        const int* done) {
+  if (done != nullptr && *done) return;
+  const int e = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (e >= r * c) return;
+  const int row = e / c, q = e - row * c;
+  const double* t = T + (int64_t)row * d;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  int j = lane;
+  for (; j + 96 < d; j += 128) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[u] += t[j + 32 * u] * Phi[(int64_t)(j + 32 * u) * stride + q];
+  }
+#pragma unroll
+  for (int u = 0; u < 3; ++u)
+    if (j + 32 * u < d) s[u] += t[j + 32 * u] * Phi[(int64_t)(j + 32 * u) * stride + q];
+  const double v = warp_sum((s[0] + s[1]) + (s[2] + s[3]));
+  if (lane == 0) out[e] = v;
 }
 
 template <typename Tacc>
@@ -528,9 +545,7 @@ int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* 
   Tacc* cls = nullptr;
   if (p.kind == kLDA) {
     int len = p.l * phi_cols;
-    lda_cls_kernel<<<ceil_div(len, 128), 128, 0, st>>>(p.means, p.v[0].Phi, p.l, p.v[0].d, phi_cols, 2 * p.k,
-                                                       p.Cls);
-    GB_CHECK_LAUNCH();
+    GB_TRY(table_phi(p.means, p.v[0].Phi, p.l, p.v[0].d, phi_cols, 2 * p.k, p.Cls, st, nullptr));
     if (std::is_same<Tacc, double>::value) {
       cls = reinterpret_cast<Tacc*>(p.Cls);
     } else {
@@ -557,6 +572,13 @@ int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* 
 }
 
 }  // namespace
+
+int table_phi(const double* T, const double* Phi, int r, int d, int c, int stride, double* out, cudaStream_t st,
+              const int* done) {
+  table_phi_kernel<<<ceil_div(r * c, 8), 256, 0, st>>>(T, Phi, r, d, c, stride, out, done);
+  GB_CHECK_LAUNCH();
+  return GBCCA_OK;
+}
 
 // low = accumulate in FP32 (BF16/FP32 data); otherwise FP64.  gram_only
 // skips Z^T W (the Rayleigh-Ritz refinement needs only W^T W).  phi_cols =
@@ -594,7 +616,10 @@ int fused_pass_cores(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi
 
 // ------------------------------------------------------------ FDA statistics
 // Per-class column sums in FP64: CTA = (row chunk, 256-column block); each
-// thread owns one column, so the accumulation order is fixed.
+// thread owns one column, so the accumulation order is fixed.  The loads of
+// kRowsInFlight rows are issued before their additions, so that the memory
+// latency is paid once per group instead of once per row.
+constexpr int kRowsInFlight = 8;
 template <typename Tin>
 __global__ void class_sums_kernel(const Tin* __restrict__ X, int64_t ld, int64_t n, int d,
                                   const int32_t* __restrict__ y, int l, int64_t rows_per_chunk,
@@ -603,27 +628,52 @@ __global__ void class_sums_kernel(const Tin* __restrict__ X, int64_t ld, int64_t
   const int c = blockIdx.y * 256 + threadIdx.x;
   for (int k = 0; k < l; ++k) acc[k * 256 + threadIdx.x] = 0;
   const int64_t r0 = blockIdx.x * rows_per_chunk, r1 = min(n, r0 + rows_per_chunk);
-  if (c < d)
-    for (int64_t i = r0; i < r1; ++i) {
-      const int yi = y[i];
-      if (yi >= 0 && yi < l) acc[yi * 256 + threadIdx.x] += to_f64(X[i * ld + c]);  // bad labels: see label_check
+  const bool counts = blockIdx.y == 0 && threadIdx.x < l;
+  int cn = 0;
+  for (int64_t i0 = r0; i0 < r1; i0 += kRowsInFlight) {
+    int yv[kRowsInFlight];
+    Tin x[kRowsInFlight];
+#pragma unroll
+    for (int u = 0; u < kRowsInFlight; ++u) {
+      yv[u] = i0 + u < r1 ? y[i0 + u] : -1;
+      x[u] = i0 + u < r1 && c < d ? X[(i0 + u) * ld + c] : Tin(0.0f);
     }
+#pragma unroll
+    for (int u = 0; u < kRowsInFlight; ++u) {
+      if (c < d && yv[u] >= 0 && yv[u] < l) acc[yv[u] * 256 + threadIdx.x] += to_f64(x[u]);  // bad labels: see label_check
+      if (counts) cn += yv[u] == (int)threadIdx.x ? 1 : 0;
+    }
+  }
   if (c < d)
     for (int k = 0; k < l; ++k) part[((int64_t)blockIdx.x * l + k) * d + c] = acc[k * 256 + threadIdx.x];
-  if (blockIdx.y == 0 && threadIdx.x < l) {
-    double cn = 0;
-    for (int64_t i = r0; i < r1; ++i) cn += (y[i] == (int)threadIdx.x) ? 1.0 : 0.0;
-    cnt_part[(int64_t)blockIdx.x * l + threadIdx.x] = cn;
-  }
+  if (counts) cnt_part[(int64_t)blockIdx.x * l + threadIdx.x] = (double)cn;
 }
 
-__global__ void class_finish_kernel(const double* __restrict__ part, const double* __restrict__ cnt_part,
-                                    int chunks, int l, int d, double* __restrict__ counts,
+// sums[e] = sum over chunks of part[c][e], e < len, in chunk order, eight
+// loads in flight.
+__global__ void class_total_kernel(const double* __restrict__ part, int chunks, int len, double* __restrict__ sums) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= len) return;
+  double s = 0;
+  for (int c0 = 0; c0 < chunks; c0 += 8) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = c0 + u < chunks ? part[(int64_t)(c0 + u) * len + e] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
+  sums[e] = s;
+}
+
+// Class means (in: `means` holds the class sums, l x d) and Yhat.  A thread
+// per column over the l classes only; the sums over the row chunks are formed
+// by class_total_kernel, one thread per (class, column) (both in one thread
+// per column was a chain of l x 128 loads: 584 us for l = 10, d = 784).
+__global__ void class_finish_kernel(const double* __restrict__ cnt, int l, int d, double* __restrict__ counts,
                                     double* __restrict__ means, double* __restrict__ Yhat, int* flag) {
   __shared__ double cn[kMaxClasses];
   if (threadIdx.x < l) {
-    double s = 0;
-    for (int c = 0; c < chunks; ++c) s += cnt_part[(int64_t)c * l + threadIdx.x];
+    const double s = cnt[threadIdx.x];
     cn[threadIdx.x] = s;
     if (blockIdx.x == 0) {
       counts[threadIdx.x] = s;
@@ -635,14 +685,13 @@ __global__ void class_finish_kernel(const double* __restrict__ part, const doubl
   for (int k = 0; k < l; ++k) ntot += cn[k];
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d; j += gridDim.x * blockDim.x) {
     double tot = 0;
+    for (int k = 0; k < l; ++k) tot += means[k * d + j];
+    const double m = tot / ntot;
     for (int k = 0; k < l; ++k) {
-      double s = 0;
-      for (int c = 0; c < chunks; ++c) s += part[((int64_t)c * l + k) * d + j];
-      means[k * d + j] = cn[k] > 0 ? s / cn[k] : 0.0;
-      tot += s;
+      const double mk = cn[k] > 0 ? means[k * d + j] / cn[k] : 0.0;
+      means[k * d + j] = mk;
+      Yhat[k * d + j] = sqrt(cn[k]) * (mk - m);
     }
-    double m = tot / ntot;
-    for (int k = 0; k < l; ++k) Yhat[k * d + j] = sqrt(cn[k]) * (means[k * d + j] - m);
   }
 }
 
@@ -682,8 +731,13 @@ int lda_class_stats(Plan& p, cudaStream_t st) {
     }
   }
   GB_CHECK_LAUNCH();
-  class_finish_kernel<<<ceil_div(p.D, 256), 256, 0, st>>>(part, cnt, chunks, p.l, p.D, p.counts, p.means,
-                                                          p.Yhat, p.flag);
+  class_total_kernel<<<ceil_div(p.l * p.D, 128), 128, 0, st>>>(part, chunks, p.l * p.D, p.means);
+  GB_CHECK_LAUNCH();
+  // the class counts, behind their partials
+  double* total = cnt + (int64_t)chunks * p.l;
+  class_total_kernel<<<1, 64, 0, st>>>(cnt, chunks, p.l, total);
+  GB_CHECK_LAUNCH();
+  class_finish_kernel<<<ceil_div(p.D, 64), 64, 0, st>>>(total, p.l, p.D, p.counts, p.means, p.Yhat, p.flag);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }

@@ -241,6 +241,9 @@ int fused_pass(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols 
 int fused_pass_cores(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols,
                const int* done);
 int exact_gram(Plan& p, int view, double* out, cudaStream_t st);
+// out (r x c) = T (r x d) Phi[:, 0:c] (row stride `stride`)
+int table_phi(const double* T, const double* Phi, int r, int d, int c, int stride, double* out, cudaStream_t st,
+              const int* done);
 int lda_class_stats(Plan& p, cudaStream_t st);
 
 // pass_tc.cu

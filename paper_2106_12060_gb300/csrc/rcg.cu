@@ -1751,18 +1751,6 @@ __global__ void copy_sigma_kernel(const DevState* st, double* out, int k) {
   if (threadIdx.x < k) out[threadIdx.x] = st->sigma[threadIdx.x];
 }
 
-// FDA: Yhat Phi (l x 2k)
-__global__ void yphi_kernel(const DevState* st, const double* Yhat, const double* Phi, int l, int d, int k2,
-                            double* YPhi, int check_done) {
-  if (check_done && st->done) return;
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= l * k2) return;
-  int c = e / k2, q = e % k2;
-  double s = 0;
-  for (int j = 0; j < d; ++j) s += Yhat[(int64_t)c * d + j] * Phi[(int64_t)j * k2 + q];
-  YPhi[e] = s;
-}
-
 // ============================================================== driver
 namespace {
 
@@ -1786,12 +1774,10 @@ int phigram(Plan& p, cudaStream_t st, const int* done, double* out = nullptr) {
                    p.nviews > 1 ? p.v[1].Phi : nullptr, k2, k2, k2, p.phipart, st, done, out);
 }
 
-int yphi(Plan& p, cudaStream_t st, int check_done) {
+// FDA: Yhat Phi (l x 2k)
+int yphi(Plan& p, cudaStream_t st, const int* done) {
   if (p.kind != kLDA) return GBCCA_OK;
-  int len = p.l * 2 * p.k;
-  yphi_kernel<<<ceil_div(len, 128), 128, 0, st>>>(p.st, p.Yhat, p.v[0].Phi, p.l, p.D, 2 * p.k, p.YPhi, check_done);
-  GB_CHECK_LAUNCH();
-  return GBCCA_OK;
+  return table_phi(p.Yhat, p.v[0].Phi, p.l, p.D, 2 * p.k, 2 * p.k, p.YPhi, st, done);
 }
 
 int thin_blocks(const Plan& p) {
@@ -1808,17 +1794,18 @@ int iteration_post(Plan& p, bool low, cudaStream_t st) {
   const int k = p.k, kk = k * k;
   const int* done = &p.st->done;
   if (p.pass_forked) {
-    // the Phi Gram (Phi is final once the pass has rounded it) on the side
-    // branch, beside the reduction and the Gram of the pass on `st`
+    // the Phi Gram and Yhat Phi (Phi is final once the pass has rounded it)
+    // on the side branch, beside the reduction and the Gram of the pass on `st`
     GB_CUDA(cudaStreamWaitEvent(p.side_stream, p.pass_fork, 0));
     GB_TRY(phigram(p, p.side_stream, done, p.phired));
+    GB_TRY(yphi(p, p.side_stream, done));
     GB_CUDA(cudaEventRecord(p.pass_join, p.side_stream));
     GB_CUDA(cudaStreamWaitEvent(st, p.pass_join, 0));
     p.pass_forked = false;
   } else {
     GB_TRY(phigram(p, st, done, p.phired));
+    GB_TRY(yphi(p, st, done));
   }
-  GB_TRY(yphi(p, st, 1));
   const bool ritz = p.opt.rtol > 0;
   if (ritz) {
     // convergence check on the Rayleigh-Ritz values of span([U, eta]) at this
@@ -2136,7 +2123,7 @@ int rcg_finish(Plan& p, double* out0, double* out1, double* vals, gbcca_info* in
     GB_TRY(fused_pass(p, low, false, st, 0, nullptr));
   }
   GB_TRY(phigram(p, st, nullptr));
-  GB_TRY(yphi(p, st, 0));
+  GB_TRY(yphi(p, st, nullptr));
   {
     RRArgs a{};
     a.st = p.st;
