@@ -54,6 +54,7 @@ void free_plan(Plan* p) {
                   (void*)p->ws, (void*)p->flag, (void*)p->tc_img, (void*)p->tc_part, (void*)p->mt_part, (void*)p->dfx, (void*)p->ls_f, (void*)p->ls_L})
     dfree(q);
   for (int v = 0; v < 2; ++v) dfree(p->ts_copy[v]);
+  dfree(p->means_df);
   if (p->st_host != nullptr) cudaFreeHost(p->st_host);
   if (p->flag_host != nullptr) cudaFreeHost(p->flag_host);
   for (int i = 0; i < p->nev; ++i) cudaEventDestroy(p->ev[i]);

@@ -174,6 +174,7 @@ struct Plan {
   __nv_bfloat16* ts_copy[2] = {nullptr, nullptr};
   int64_t ts_ld[2] = {0, 0};
   bool ts_ready = false;
+  float* means_df = nullptr;  // FDA: the class means as float pairs (l x d padded to 4: hi, then lo)
   cudaEvent_t kev0 = nullptr;  // when set: recorded around the data kernel of the next pass
   cudaEvent_t kev1 = nullptr;  // resident 2-CTA clusters of the tensor-core pass (0: not yet queried)
 };

@@ -44,3 +44,69 @@ def test_class_tables_and_fda_pass_f64(gb, n, d, l, k):
     gamma = 4 * (n + 2 * d + l + 4) * eps
     assert bound_ratio(np64(G), (X - M[y]).T @ W, (np.abs(X) + aM[y]).T @ aW, gamma) <= 1.0
     assert bound_ratio(np64(Gram), W.T @ W, aW.T @ aW, gamma) <= 1.0
+
+
+def _layouts(a, tdt):
+    """The same matrix contiguous, with rows padded to 16 bytes, with an odd
+    row stride, and starting one element past an aligned address."""
+    import torch
+    t = torch.from_numpy(a).to(tdt).cuda()
+    n, d = t.shape
+    out = [t]
+    for ld, off in (((d + 7) // 8 * 8, 0), (d + 1 + d % 2, 0), ((d + 7) // 8 * 8, 1)):
+        buf = torch.full((n * ld + off,), float("nan"), dtype=tdt, device="cuda")
+        v = buf[off:].view(n, ld)[:, :d]
+        v.copy_(t)
+        out.append(v)
+    return out
+
+
+@pytest.mark.parametrize("n,d", [(5, 1), (33, 3), (700, 31), (1500, 301), (2100, 516)])
+def test_f32_copy_layouts_cca(gb, n, d):
+    """The BF16 hi/lo copy of FP32 views (16-byte and element-wise loads, a
+    ragged last chunk): the pass over it is bitwise the same for every layout
+    of the same values, and within 2^-16 (the representation of data and Phi)
+    plus FP32 accumulation of the exact products."""
+    import torch
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((n, d)).astype(np.float32)
+    k = 1
+    P = rng.standard_normal((d, 2 * k))
+    got = []
+    for x in _layouts(X, torch.float32):
+        plan = gb.cca_plan(n, d, d, k, "f32", gb.default_options(warm_start=0))
+        gb.cca_precondition(plan, x, x, 1e-1, 1e-1)
+        Phi = torch.from_numpy(P).cuda()
+        Gx, Gy, _ = gb.fused_pass(plan, Phi, Phi)
+        got.append((np64(Gx), np64(Gy)))
+    for g in got[1:]:
+        assert np.array_equal(g[0], got[0][0]) and np.array_equal(g[1], got[0][1])
+    X64 = X.astype(np.float64)
+    W = np.hstack([X64 @ P, X64 @ P])
+    aW = np.hstack([np.abs(X64) @ np.abs(P)] * 2)
+    gamma = 4 * 2.0 ** -16 + 2 * (n + d + 8) * 2.0 ** -23
+    assert bound_ratio(got[0][0], X64.T @ W, np.abs(X64).T @ aW, gamma) <= 1.0
+
+
+@pytest.mark.parametrize("n,d,l", [(60, 3, 2), (900, 33, 5), (1400, 301, 10)])
+def test_f32_copy_layouts_fda(gb, n, d, l):
+    """The copy of the class-centred rows: bitwise the same pass for every
+    layout, and within the same bound of the exact centred products."""
+    import torch
+    P = lda_problem(n, d, l, dtype="f32", seed=d)
+    y = P["y"]
+    k = 1
+    Phi = np.random.default_rng(d + 1).standard_normal((d, 2 * k))
+    got = []
+    for x in _layouts(P["X"], torch.float32):
+        plan = gb.lda_plan(n, d, l, k, "f32", gb.default_options(max_iter=1))
+        gb.lda_solve(plan, x, torch.from_numpy(y).cuda(), 1e-1)
+        got.append(np64(gb.fused_pass(plan, torch.from_numpy(Phi).cuda())[0]))
+    for g in got[1:]:
+        assert np.array_equal(g, got[0])
+    X = P["X64"]
+    M = np.stack([X[y == c].mean(0) for c in range(l)])
+    Xc = X - M[y]
+    W, aW = Xc @ Phi, np.abs(Xc) @ np.abs(Phi)
+    gamma = 4 * 2.0 ** -16 + 2 * (n + d + 8) * 2.0 ** -23
+    assert bound_ratio(got[0], Xc.T @ W, np.abs(Xc).T @ aW, gamma) <= 1.0
