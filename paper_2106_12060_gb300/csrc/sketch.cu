@@ -94,14 +94,21 @@ __global__ void cs_count_kernel(const int32_t* __restrict__ h, int64_t n, int64_
   }
 }
 
-// per bucket: exclusive prefix over chunks (in place) and the bucket total
+// per bucket: exclusive prefix over chunks (in place) and the bucket total;
+// eight loads in flight (one at a time behind its own store took 48 us for
+// 152 chunks of 2336 buckets)
 __global__ void cs_colscan_kernel(int32_t* __restrict__ tab, int nch, int64_t s, int32_t* __restrict__ total) {
   for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < s; b += (int64_t)gridDim.x * blockDim.x) {
     int32_t acc = 0;
-    for (int c = 0; c < nch; ++c) {
-      int32_t t = tab[(int64_t)c * s + b];
-      tab[(int64_t)c * s + b] = acc;
-      acc += t;
+    for (int c0 = 0; c0 < nch; c0 += 8) {
+      int32_t t[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) t[u] = c0 + u < nch ? tab[(int64_t)(c0 + u) * s + b] : 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (c0 + u < nch) tab[(int64_t)(c0 + u) * s + b] = acc;
+        acc += t[u];
+      }
     }
     total[b] = acc;
   }
@@ -134,29 +141,47 @@ __global__ void cs_scan_kernel(const int32_t* __restrict__ total, int64_t s, int
 
 // in-order placement: one warp walks its chunk 32 rows at a time; rows of
 // the same bucket inside a group of 32 are ranked by lane (= row) order.
-__global__ void cs_place_kernel(const int32_t* __restrict__ h, int64_t n, int64_t rpc, int64_t s,
-                                int32_t* __restrict__ tab, const int32_t* __restrict__ off,
-                                int32_t* __restrict__ perm) {
+// The chunk's next free place of every bucket is a shared-memory counter
+// where s counters fit (kSmem), since a step depends on the counters of the
+// step before it (through global memory: 44 us for 1974 rows a chunk); the
+// buckets of the next kPlaceAhead groups are loaded ahead of that chain.
+constexpr int kPlaceAhead = 8;
+constexpr int64_t kPlaceSmem = 48 * 1024;  // counters in shared memory up to s = 12288
+template <bool kSmem>
+__global__ void __launch_bounds__(32) cs_place_kernel(const int32_t* __restrict__ h, int64_t n, int64_t rpc, int64_t s,
+                                                      int32_t* __restrict__ tab, const int32_t* __restrict__ off,
+                                                      int32_t* __restrict__ perm) {
+  extern __shared__ int32_t cnt_s[];
   const int lane = threadIdx.x;
   const int64_t r0 = blockIdx.x * rpc, r1 = min(n, r0 + rpc);
   int32_t* cur = tab + (int64_t)blockIdx.x * s;
-  for (int64_t i0 = r0; i0 < r1; i0 += 32) {
-    const int64_t i = i0 + lane;
-    int32_t b = -1;
-    if (i < r1) {
-      b = h[i];
-      if (b < 0 || b >= s) b = -1;  // reported by cs_count_kernel
-    }
-    const unsigned peers = __match_any_sync(0xffffffffu, b);
-    const bool act = b >= 0;
-    const bool last = act && (peers >> lane) == 1u;  // highest lane of its group
-    if (act) {
-      const int rank = __popc(peers & ((1u << lane) - 1u));
-      perm[off[b] + cur[b] + rank] = (int32_t)i;
-    }
+  if (kSmem) {
+    for (int b = lane; b < (int)s; b += 32) cnt_s[b] = off[b] + cur[b];
     __syncwarp();
-    if (last) cur[b] += __popc(peers);
-    __syncwarp();
+  }
+  for (int64_t g0 = r0; g0 < r1; g0 += 32 * kPlaceAhead) {
+    int32_t bv[kPlaceAhead];
+#pragma unroll
+    for (int u = 0; u < kPlaceAhead; ++u) {
+      const int64_t i = g0 + 32 * u + lane;
+      bv[u] = i < r1 ? h[i] : -1;
+      if (bv[u] < 0 || bv[u] >= s) bv[u] = -1;  // reported by cs_count_kernel
+    }
+#pragma unroll
+    for (int u = 0; u < kPlaceAhead; ++u) {
+      const int64_t i = g0 + 32 * u + lane;
+      const int32_t b = bv[u];
+      const unsigned peers = __match_any_sync(0xffffffffu, b);
+      const bool act = b >= 0;
+      const bool last = act && (peers >> lane) == 1u;  // highest lane of its group
+      if (act) {
+        const int rank = __popc(peers & ((1u << lane) - 1u));
+        perm[(kSmem ? cnt_s[b] : off[b] + cur[b]) + rank] = (int32_t)i;
+      }
+      __syncwarp();
+      if (last) (kSmem ? cnt_s[b] : cur[b]) += __popc(peers);
+      __syncwarp();
+    }
   }
 }
 
@@ -170,66 +195,123 @@ int countsketch_prepare(Plan& p, cudaStream_t st) {
   GB_CHECK_LAUNCH();
   cs_scan_kernel<<<1, 1024, 0, st>>>(total, p.s, p.cs_off);
   GB_CHECK_LAUNCH();
-  cs_place_kernel<<<p.cs_nch, 32, 0, st>>>(p.h, p.n, rpc, p.s, p.cs_tab, p.cs_off, p.perm);
+  const size_t csm = sizeof(int32_t) * (size_t)p.s;
+  if ((int64_t)csm <= kPlaceSmem)
+    cs_place_kernel<true><<<p.cs_nch, 32, csm, st>>>(p.h, p.n, rpc, p.s, p.cs_tab, p.cs_off, p.perm);
+  else
+    cs_place_kernel<false><<<p.cs_nch, 32, 0, st>>>(p.h, p.n, rpc, p.s, p.cs_tab, p.cs_off, p.perm);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }
 
-// one warp per bucket; each lane owns columns lane, lane + 32, ...
-template <typename Tin>
+// FP32 -> FP64 by moving the bits (a hardware conversion runs at the FP64
+// rate); zeros included, subnormals and non-finite values by the conversion.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u || m == 0u)  // normal, or zero
+    return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 3) + 0x38000000u)), (int)(u << 29));
+  return (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(__nv_bfloat16 x) { return widen(__bfloat162float(x)); }
+
+// kV consecutive values of a row: one 16- or 8-byte load
+template <typename Tin, int kV> struct alignas(sizeof(Tin) * kV) RowVec { Tin v[kV]; };
+
+// One warp per (bucket, 32 kV columns): lane l owns kV consecutive columns and
+// adds the bucket's rows in row order, so the sums do not depend on the grid.
+// The order and signs of a bucket's rows are read 32 at a time and handed out
+// by shuffles, kCsRows rows' values in flight per lane.  Bound by the FP64
+// rate: one addition per element (two with class means), the sign applied to
+// the bits.  A warp per bucket over all columns, one row at a time behind its
+// index, with a conversion and a multiply-add per element took 1310 us for
+// 300000 x 384 FP32.  kV = 1 serves rows that are not aligned for the wide load.
+constexpr int kCsRows = 4;
+template <typename Tin, int kV, bool kCentre>
 __global__ void __launch_bounds__(256)
-cs_sum_kernel(const Tin* __restrict__ Z, int64_t ld, int d, int64_t s, const int32_t* __restrict__ off,
+cs_sum_kernel(const Tin* __restrict__ Z, int64_t ld, int d, int64_t s, int ncol, const int32_t* __restrict__ off,
               const int32_t* __restrict__ perm, const int8_t* __restrict__ g, const int32_t* __restrict__ labels,
               const double* __restrict__ means, double* __restrict__ SZ) {
   const int lane = threadIdx.x & 31;
-  const int64_t b = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int64_t b = w / ncol;
   if (b >= s) return;
-  double acc[kMaxD / 32];
+  const int c = ((int)(w - b * ncol) * 32 + lane) * kV;
+  const int nv = min(kV, d - c);  // columns of this lane (none: nv <= 0)
+  double acc[kV];
 #pragma unroll
-  for (int q = 0; q < kMaxD / 32; ++q) acc[q] = 0.0;
-  const int nq = (d + 31) / 32;
-  for (int32_t pos = off[b]; pos < off[b + 1]; ++pos) {
-    const int32_t i = perm[pos];
-    const double sg = (double)g[i];
-    const Tin* row = Z + (int64_t)i * ld;
-    const double* mrow = labels != nullptr ? means + (int64_t)labels[i] * d : nullptr;
+  for (int q = 0; q < kV; ++q) acc[q] = 0.0;
+  const int32_t p1 = off[b + 1];
+  for (int32_t pos = off[b]; pos < p1; pos += 32) {
+    const int cnt = min(32, p1 - pos);
+    const int32_t ri = lane < cnt ? perm[pos + lane] : 0;
+    const int rs = lane < cnt ? (int)g[ri] : 0;
+    const int rl = kCentre && lane < cnt ? labels[ri] : 0;
+    for (int r0 = 0; r0 < cnt; r0 += kCsRows) {
+      RowVec<Tin, kV> z[kCsRows];
+      double m[kCsRows][kCentre ? kV : 1];
+      int sg[kCsRows];
 #pragma unroll
-    for (int q = 0; q < kMaxD / 32; ++q) {
-      int c = lane + 32 * q;
-      if (q < nq && c < d) {
-        double x = to_f64(row[c]);
-        if (mrow != nullptr) x -= mrow[c];
-        acc[q] += sg * x;
+      for (int u = 0; u < kCsRows; ++u) {
+        const int r = min(r0 + u, cnt - 1);
+        const int64_t i = __shfl_sync(0xffffffffu, ri, r);
+        sg[u] = __shfl_sync(0xffffffffu, rs, r);
+        const Tin* row = Z + i * ld + c;
+        if (nv == kV) {
+          z[u] = *reinterpret_cast<const RowVec<Tin, kV>*>(row);
+        } else {
+#pragma unroll
+          for (int q = 0; q < kV; ++q) z[u].v[q] = q < nv ? row[q] : Tin(0.0f);
+        }
+        if (kCentre) {
+          const double* mrow = means + (int64_t)__shfl_sync(0xffffffffu, rl, r) * d + c;
+#pragma unroll
+          for (int q = 0; q < kV; ++q) m[u][q] = q < nv ? mrow[q] : 0.0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kCsRows; ++u) {
+        if (r0 + u < cnt) {
+#pragma unroll
+          for (int q = 0; q < kV; ++q) {
+            double x = widen(z[u].v[q]);
+            if (kCentre) x -= m[u][q];
+            acc[q] += sg[u] == 1 ? x : (sg[u] == -1 ? -x : (double)sg[u] * x);
+          }
+        }
       }
     }
   }
 #pragma unroll
-  for (int q = 0; q < kMaxD / 32; ++q) {
-    int c = lane + 32 * q;
-    if (q < nq && c < d) SZ[b * d + c] = acc[q];
-  }
+  for (int q = 0; q < kV; ++q)
+    if (q < nv) SZ[b * d + c + q] = acc[q];
+}
+
+template <typename Tin, int kV>
+int cs_sum_run(Plan& p, View& v, bool center, cudaStream_t st) {
+  const int ncol = ceil_div(v.d, 32 * kV);
+  const int grid = ceil_div(p.s * ncol, 8);
+  auto kern = center ? cs_sum_kernel<Tin, kV, true> : cs_sum_kernel<Tin, kV, false>;
+  kern<<<grid, 256, 0, st>>>(static_cast<const Tin*>(v.Z), v.ld, v.d, p.s, ncol, p.cs_off, p.perm, p.g,
+                             center ? p.labels : nullptr, center ? p.means : nullptr, v.SZ);
+  GB_CHECK_LAUNCH();
+  return GBCCA_OK;
+}
+
+// kV columns per lane where every row starts on a kV-element boundary
+template <typename Tin, int kV>
+int cs_sum_any(Plan& p, View& v, bool center, cudaStream_t st) {
+  const bool vec = v.ld % kV == 0 && reinterpret_cast<uintptr_t>(v.Z) % (sizeof(Tin) * kV) == 0;
+  return vec ? cs_sum_run<Tin, kV>(p, v, center, st) : cs_sum_run<Tin, 1>(p, v, center, st);
 }
 
 int countsketch_apply(Plan& p, int view, bool center, cudaStream_t st) {
   View& v = p.v[view];
-  const int32_t* lab = center ? p.labels : nullptr;
-  const double* mean = center ? p.means : nullptr;
-  int grid = ceil_div(p.s, 8);
   switch (p.dtype) {
-    case GBCCA_FP64:
-      cs_sum_kernel<double><<<grid, 256, 0, st>>>((const double*)v.Z, v.ld, v.d, p.s, p.cs_off, p.perm, p.g, lab,
-                                                  mean, v.SZ);
-      break;
-    case GBCCA_FP32:
-      cs_sum_kernel<float><<<grid, 256, 0, st>>>((const float*)v.Z, v.ld, v.d, p.s, p.cs_off, p.perm, p.g, lab, mean,
-                                                 v.SZ);
-      break;
-    default:
-      cs_sum_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)v.Z, v.ld, v.d, p.s, p.cs_off, p.perm,
-                                                         p.g, lab, mean, v.SZ);
+    case GBCCA_FP64: return cs_sum_any<double, 2>(p, v, center, st);
+    case GBCCA_FP32: return cs_sum_any<float, 4>(p, v, center, st);
+    default: return cs_sum_any<__nv_bfloat16, 4>(p, v, center, st);
   }
-  GB_CHECK_LAUNCH();
-  return GBCCA_OK;
 }
 
 // ---------------------------------------------------------------- SRHT

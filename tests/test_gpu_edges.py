@@ -110,3 +110,30 @@ def test_f32_copy_layouts_fda(gb, n, d, l):
     W, aW = Xc @ Phi, np.abs(Xc) @ np.abs(Phi)
     gamma = 4 * 2.0 ** -16 + 2 * (n + d + 8) * 2.0 ** -23
     assert bound_ratio(got[0], Xc.T @ W, np.abs(Xc).T @ aW, gamma) <= 1.0
+
+
+@pytest.mark.parametrize("dt", ["bf16", "f32", "f64"])
+@pytest.mark.parametrize("n,d,s", [(3, 1, 2), (257, 33, 40), (2003, 131, 131), (40000, 260, 13000)])
+def test_countsketch_sum_layouts(gb, dt, n, d, s):
+    """Sums of buckets of every size (empty ones; more than 32 rows), columns
+    that do not fill a lane's vector, more buckets than the shared-memory
+    counters hold, and every row alignment, against exact row-order FP64
+    sums: bitwise equal, since the order of a bucket's rows is fixed."""
+    import torch
+    tdt = {"bf16": torch.bfloat16, "f32": torch.float32, "f64": torch.float64}[dt]
+    rng = np.random.default_rng(n + d)
+    X = rng.standard_normal((n, d)) * 10.0 ** rng.integers(-3, 4, (n, 1))
+    X[rng.random((n, d)) < 0.05] = 0.0
+    X = torch.from_numpy(X).to(tdt).double().numpy()
+    h = rng.integers(0, s, n).astype(np.int32)
+    if n > 1000:
+        h[:100] = 1
+        h[h == 0] = 2  # an empty bucket
+    g = np.where(rng.random(n) < 0.5, -1, 1).astype(np.int8)
+    ref = np.zeros((s, d))
+    for i in range(n):
+        ref[h[i]] += g[i] * X[i]
+    for x in _layouts(X, tdt):
+        plan = gb.cca_plan(n, d, d, 1, dt, gb.default_options(s=s, warm_start=0))
+        gb.cca_precondition(plan, x, x, 1e3, 1e3, torch.from_numpy(h).cuda(), torch.from_numpy(g).cuda())
+        assert np.array_equal(np64(gb.query(plan, gb.Q_SKETCH_X)).reshape(s, d), ref)
