@@ -48,7 +48,7 @@ void free_plan(Plan* p) {
       dfree(q);
   }
   for (void* q : {(void*)p->h, (void*)p->g, (void*)p->cs_tab, (void*)p->cs_off, (void*)p->perm, p->srht_T,
-                  (void*)p->G, (void*)p->Gt, (void*)p->Gram, p->Wbuf, p->partG, p->partGram, p->partCls, (void*)p->counts,
+                  (void*)p->G, (void*)p->tc_gpart, (void*)p->Gram, p->Wbuf, p->partG, p->partGram, p->partCls, (void*)p->counts,
                   (void*)p->means, (void*)p->Yhat, (void*)p->Cls, (void*)p->YPhi, (void*)p->clsPart, (void*)p->st,
                   (void*)p->phigram, (void*)p->phipart, (void*)p->phired, (void*)p->cross, (void*)p->crosspart, (void*)p->history, (void*)p->ritz_hist,
                   (void*)p->ws, (void*)p->flag, (void*)p->tc_img, (void*)p->tc_part, (void*)p->mt_part, (void*)p->dfx, (void*)p->ls_f, (void*)p->ls_L})
@@ -187,8 +187,8 @@ int alloc_plan(Plan* p) {
     const int64_t img = (2 * k <= 24 ? 1 : 2) * (tc_cca ? 2 * (dmax > 512 ? 2 : 1) : 2) * 49152;
     GB_TRY(dalloc(&p->tc_img, img));
     GB_CUDA(cudaMemset(p->tc_img, 0, img));
-    GB_TRY(dalloc(&p->Gt, (int64_t)p->D * p->NC));
-    GB_TRY(dalloc(&p->tc_part, (int64_t)p->sm_count * p->D * (k4 + 8)));
+    GB_TRY(dalloc(&p->tc_gpart, tc_gpart_len(*p)));
+    GB_TRY(dalloc(&p->tc_part, tc_part_len(*p)));
   }
   GB_TRY(hilo_alloc(*p));
   GB_CUDA(cudaStreamCreateWithFlags(&p->side_stream, cudaStreamNonBlocking));
@@ -517,11 +517,6 @@ int lda_solve(gbcca_plan_t plan, const void* X, int64_t ldx, const int32_t* labe
   return rcg_run(*p, mu, tol, W, nullptr, rho, info, st);
 }
 
-__global__ void scatter_rows_kernel(const double* G, int NC, int row0, int d, double* out) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < d * NC) out[e] = G[(int64_t)row0 * NC + e];
-}
-
 int gbcca_fused_pass(gbcca_plan_t plan, const double* Phi_x, const double* Phi_y, double* Gx, double* Gy,
                      double* Gram, void* stream) {
   Plan* p = as_plan(plan);
@@ -535,19 +530,8 @@ int gbcca_fused_pass(gbcca_plan_t plan, const double* Phi_x, const double* Phi_y
     return GBCCA_ERR_STATE;
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const int k2 = 2 * p->k;
-  GB_CUDA(cudaMemcpyAsync(p->v[0].Phi, Phi_x, sizeof(double) * p->v[0].d * k2, cudaMemcpyDeviceToDevice, st));
-  if (p->kind == kCCA)
-    GB_CUDA(cudaMemcpyAsync(p->v[1].Phi, Phi_y, sizeof(double) * p->v[1].d * k2, cudaMemcpyDeviceToDevice, st));
-  GB_TRY(fused_pass(*p, p->dtype != GBCCA_FP64, false, st, 0, nullptr));
-  scatter_rows_kernel<<<ceil_div(p->v[0].d * p->NC, 256), 256, 0, st>>>(p->G, p->NC, 0, p->v[0].d, Gx);
-  GB_CHECK_LAUNCH();
-  if (p->kind == kCCA) {
-    scatter_rows_kernel<<<ceil_div(p->v[1].d * p->NC, 256), 256, 0, st>>>(p->G, p->NC, p->v[0].d, p->v[1].d, Gy);
-    GB_CHECK_LAUNCH();
-  }
-  GB_CUDA(cudaMemcpyAsync(Gram, p->Gram, sizeof(double) * p->NC * p->NC, cudaMemcpyDeviceToDevice, st));
-  return GBCCA_OK;
+  const PassIO io{{Phi_x, Phi_y}, {Gx, Gy}, Gram};
+  return fused_pass(*p, p->dtype != GBCCA_FP64, false, st, 0, nullptr, &io);
 }
 
 int64_t gbcca_query_size(gbcca_plan_t plan, int32_t what) {

@@ -104,6 +104,7 @@ int enqueue_iteration(Batch& b, const std::vector<char>& active, cudaStream_t st
       Plan& p = *b.plans[i];
       GB_CUDA(cudaStreamWaitEvent(b.side[i], b.fork_b, 0));
       GB_TRY(tc_batch_post(b.tc[b.tc_table[i]], b.tc_index[i], p, b.side[i], &p.st->done));
+      p.phired_ready = true;
       GB_TRY(iteration_post(p, p.dtype != GBCCA_FP64, b.side[i]));
       GB_CUDA(cudaEventRecord(b.join_b[i], b.side[i]));
     }
@@ -457,29 +458,26 @@ int gbcca_batch_fused_pass(gbcca_batch_t h, const double* const* Phi_x, const do
     return GBCCA_ERR_UNSUPPORTED;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // every plan's images, one batched launch per table, every plan's sums:
+  // three kinds of launch for all plans instead of a chain of copies and
+  // small kernels per plan
+  for (int i = 0; i < n; ++i) GB_CUDA(cudaMemsetAsync(&b->plans[i]->st->done, 0, sizeof(int), st));
+  std::vector<PassIO> io[2];
   for (int i = 0; i < n; ++i) {
-    Plan& p = *b->plans[i];
-    const int k2 = 2 * p.k;
-    GB_CUDA(cudaMemsetAsync(&p.st->done, 0, sizeof(int), st));
-    GB_CUDA(cudaMemcpyAsync(p.v[0].Phi, Phi_x[i], sizeof(double) * p.v[0].d * k2, cudaMemcpyDeviceToDevice, st));
-    GB_CUDA(cudaMemcpyAsync(p.v[1].Phi, Phi_y[i], sizeof(double) * p.v[1].d * k2, cudaMemcpyDeviceToDevice, st));
-    GB_TRY(tc_batch_pre(b->tc[b->tc_table[i]], p, st));
+    const Plan& p = *b->plans[i];
+    io[b->tc_table[i]].push_back(
+        PassIO{{Phi_x[i], Phi_y[i]}, {G[i], G[i] + (int64_t)p.v[0].d * 4 * p.k}, Gram[i]});
   }
   for (int t = 0; t < 2; ++t) {
     if (b->tc[t] == nullptr) continue;
     const int m = (int)b->tc_plans[t].size();
+    GB_TRY(tc_batch_pre_all(b->tc[t], b->tc_plans[t].data(), m, io[t].data(), st));
     std::unique_ptr<bool[]> a(new bool[std::max(m, 1)]);
     for (int i = 0; i < m; ++i) a[i] = true;
     GB_TRY(tc_batch_schedule(b->tc[t], a.get(),
                              b->opt.clusters > 0 ? b->opt.clusters : tc_batch_max_clusters(b->tc[t]), st));
     GB_TRY(tc_batch_launch(b->tc[t], st, nullptr, nullptr));
-  }
-  for (int i = 0; i < n; ++i) {
-    Plan& p = *b->plans[i];
-    GB_TRY(tc_batch_post(b->tc[b->tc_table[i]], b->tc_index[i], p, st, nullptr));
-    const int k4 = 4 * p.k;
-    GB_CUDA(cudaMemcpyAsync(G[i], p.G, sizeof(double) * p.D * k4, cudaMemcpyDeviceToDevice, st));
-    GB_CUDA(cudaMemcpyAsync(Gram[i], p.Gram, sizeof(double) * k4 * k4, cudaMemcpyDeviceToDevice, st));
+    GB_TRY(tc_batch_post_all(b->tc[t], b->tc_plans[t].data(), m, io[t].data(), st));
   }
   int err[2] = {0, 0};
   for (int t = 0; t < 2; ++t)

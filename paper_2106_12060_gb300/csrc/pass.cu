@@ -347,7 +347,8 @@ pass_g_async_kernel(PassViews pv, int64_t n, int NC, int D, const float* __restr
 
 __global__ void pass_reduce_kernel(const double* __restrict__ partG, int chunks, int64_t nG,
                                    const double* __restrict__ partGram, int ctas, int64_t nGram,
-                                   double* __restrict__ G, double* __restrict__ Gram, const int* done) {
+                                   double* __restrict__ G0, double* __restrict__ G1, int64_t n0,
+                                   double* __restrict__ Gram, const int* done) {
   if (done != nullptr && *done) return;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nG + nGram;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -355,7 +356,8 @@ __global__ void pass_reduce_kernel(const double* __restrict__ partG, int chunks,
     if (e < nG) {
       if (partG != nullptr) {
         for (int c = 0; c < chunks; ++c) s += (double)partG[(int64_t)c * nG + e];
-        G[e] = s;
+        if (e < n0) G0[e] = s;  // view 0's rows, then view 1's
+        else G1[e - n0] = s;
       }
     } else {
       int64_t f = e - nG;
@@ -518,7 +520,7 @@ int dispatch_g(Plan& p, const PassViews& pv, const Tacc* W, cudaStream_t st) {
 }
 
 template <typename Tin, typename Tacc>
-int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* done) {
+int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* done, const PassIO* io) {
   PassViews pv{};
   pv.nviews = p.nviews;
   pv.k2 = phi_cols;
@@ -533,11 +535,12 @@ int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* 
     pv.dofs[v] = dofs;
     pv.ocol[v] = v * phi_cols;
     dofs += p.v[v].d;
+    const double* Phi = io != nullptr ? io->Phi[v] : p.v[v].Phi;
     if (std::is_same<Tacc, double>::value) {
-      pv.Phi[v] = p.v[v].Phi;
+      pv.Phi[v] = Phi;
     } else {
       int64_t len = (int64_t)p.v[v].d * 2 * p.k;
-      phi_convert_kernel<float><<<ceil_div(len, 256), 256, 0, st>>>(p.v[v].Phi, p.v[v].Phi32, len);
+      phi_convert_kernel<float><<<ceil_div(len, 256), 256, 0, st>>>(Phi, p.v[v].Phi32, len);
       GB_CHECK_LAUNCH();
       pv.Phi[v] = p.v[v].Phi32;
     }
@@ -545,7 +548,7 @@ int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* 
   Tacc* cls = nullptr;
   if (p.kind == kLDA) {
     int len = p.l * phi_cols;
-    GB_TRY(table_phi(p.means, p.v[0].Phi, p.l, p.v[0].d, phi_cols, 2 * p.k, p.Cls, st, nullptr));
+    GB_TRY(table_phi(p.means, io != nullptr ? io->Phi[0] : p.v[0].Phi, p.l, p.v[0].d, phi_cols, 2 * p.k, p.Cls, st, nullptr));
     if (std::is_same<Tacc, double>::value) {
       cls = reinterpret_cast<Tacc*>(p.Cls);
     } else {
@@ -558,14 +561,18 @@ int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* 
   GB_TRY((dispatch_w<Tin, Tacc>(p, pv, NC, W, st, cls)));
   if (!gram_only) GB_TRY((dispatch_g<Tin, Tacc>(p, pv, W, st)));
   int64_t nG = gram_only ? 0 : (int64_t)p.D * NC;
+  const int64_t n0 = (int64_t)p.v[0].d * NC;
+  double* G0 = io != nullptr ? io->G[0] : p.G;
+  double* G1 = io != nullptr ? io->G[1] : p.G + n0;
   int64_t nGram = (int64_t)NC * NC;
   pass_reduce_kernel<<<ceil_div(nG + nGram, 256), 256, 0, st>>>(
       gram_only ? nullptr : reinterpret_cast<const double*>(p.partG), p.chunksB, nG,
-      reinterpret_cast<const double*>(p.partGram), p.ctasA, nGram, p.G, p.Gram, done);
+      reinterpret_cast<const double*>(p.partGram), p.ctasA, nGram, G0, G1, n0,
+      io != nullptr ? io->Gram : p.Gram, done);
   GB_CHECK_LAUNCH();
   if (p.kind == kLDA && !gram_only) {
     lda_correct_kernel<<<ceil_div((int64_t)p.D * NC, 256), 256, 0, st>>>(
-        reinterpret_cast<const double*>(p.partCls), p.ctasA, p.l, NC, p.D, p.means, p.G, done);
+        reinterpret_cast<const double*>(p.partCls), p.ctasA, p.l, NC, p.D, p.means, G0, done);
     GB_CHECK_LAUNCH();
   }
   return GBCCA_OK;
@@ -584,32 +591,39 @@ int table_phi(const double* T, const double* Phi, int r, int d, int c, int strid
 // skips Z^T W (the Rayleigh-Ritz refinement needs only W^T W).  phi_cols =
 // columns of Phi used per view (0 = all 2k).  `done` (device, may be null)
 // turns the launches into no-ops once the solver has stopped.
-int fused_pass(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols, const int* done) {
+// io (may be null): a stand-alone pass over the caller's arrays.
+int fused_pass(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols, const int* done, const PassIO* io) {
   if (phi_cols <= 0) phi_cols = 2 * p.k;
+  p.phired_ready = false;
   if (low && !gram_only && phi_cols == 2 * p.k && p.opt.tensor_cores) {
-    if (p.tc_img != nullptr && tc_pass_eligible(p)) return tc_pass(p, st, done);
+    if (p.tc_img != nullptr && tc_pass_eligible(p)) {
+      GB_TRY(tc_pass(p, st, done, io));
+      p.phired_ready = true;
+      return GBCCA_OK;
+    }
   }
   if (p.kev0 != nullptr) GB_CUDA(record_timing_event(p.kev0, st));
-  const int rc = fused_pass_cores(p, low, gram_only, st, phi_cols, done);
+  const int rc = fused_pass_cores(p, low, gram_only, st, phi_cols, done, io);
   if (rc == GBCCA_OK && p.kev1 != nullptr) GB_CUDA(record_timing_event(p.kev1, st));
   return rc;
 }
 
 // CUDA-core passes (FP64 / FP32 data, LDA, and the BF16 plans the
 // tensor-core pass does not serve)
-int fused_pass_cores(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols, const int* done) {
+int fused_pass_cores(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols, const int* done,
+                     const PassIO* io) {
   if (p.kind == kLDA && p.l * phi_cols > 256 * kCI) {
     set_last_error("too many classes x columns for the FDA pass");
     return GBCCA_ERR_UNSUPPORTED;
   }
   switch (p.dtype) {
-    case GBCCA_FP64: return run_pass<double, double>(p, gram_only, st, phi_cols, done);
+    case GBCCA_FP64: return run_pass<double, double>(p, gram_only, st, phi_cols, done, io);
     case GBCCA_FP32:
-      return low ? run_pass<float, float>(p, gram_only, st, phi_cols, done)
-                 : run_pass<float, double>(p, gram_only, st, phi_cols, done);
+      return low ? run_pass<float, float>(p, gram_only, st, phi_cols, done, io)
+                 : run_pass<float, double>(p, gram_only, st, phi_cols, done, io);
     case GBCCA_BF16:
-      return low ? run_pass<__nv_bfloat16, float>(p, gram_only, st, phi_cols, done)
-                 : run_pass<__nv_bfloat16, double>(p, gram_only, st, phi_cols, done);
+      return low ? run_pass<__nv_bfloat16, float>(p, gram_only, st, phi_cols, done, io)
+                 : run_pass<__nv_bfloat16, double>(p, gram_only, st, phi_cols, done, io);
   }
   return GBCCA_ERR_INVALID_ARG;
 }

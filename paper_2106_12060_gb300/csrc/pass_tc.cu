@@ -129,14 +129,20 @@ struct Lay {
   static_assert(kSmemBytes <= kMaxSmem, "shared memory");
 };
 
+// Rows of a view in a partial slab: padded so that a block of kPostRows rows
+// belongs to one view and starts on a 16-byte boundary.  The padding is never
+// written and its sums are never used.
+constexpr int kPostRows = 8;
+__host__ __device__ __forceinline__ int pad_rows(int d) { return (d + kPostRows - 1) / kPostRows * kPostRows; }
+
 // One instance of a batched pass (device memory; the tensor maps are read by
 // the TMA unit from there; CUtensorMap carries its own 128-byte alignment).
 struct Inst {
   CUtensorMap map[2];      // views X, Y (BF16 data, or the interleaved hi/lo copy)
   const uint8_t* phi_img;  // [view][K-box][2 kH1][128 B], pre-swizzled
-  float* partG;            // [slab][D][4k] partials of this instance
+  float* partG;            // partial slabs of this instance
   const int* done;         // the instance's convergence flag: skip it when set
-  int64_t slab;            // floats per partial slab (D * 4k)
+  int64_t slab;            // floats per partial slab (see tc_slab)
   int64_t img_view;        // bytes between the two views' Phi images
   int d[2];
   int pairs[2];
@@ -162,8 +168,8 @@ struct Args {
   int k2;        // columns of Phi per view (2k)
   int ntiles;
   const uint8_t* phi_img;  // [view][K-box][2 kH1][128 B], pre-swizzled
-  float* partG;            // [cluster][D][4k] (one view: [cluster][d][2k])
-  int64_t slab;            // floats between the clusters' partial slabs (a multiple of 4)
+  float* partG;            // [cluster][column][padded rows of the views]
+  int64_t slab;            // floats between the clusters' partial slabs
   int* err;
   const int* done;
   int64_t img_view;        // bytes between the two views' Phi images
@@ -700,7 +706,9 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
         // the slab is column-major (D rows, kNvs k2 columns): the 32 lanes
         // of a warp hold 32 consecutive rows, so every store of a column is
         // one 128-byte line
-        const int D = sv.d0 + sv.d1;
+        // (each view's rows padded to kPostRows)
+        const int o0 = pad_rows(sv.d0);
+        const int D = o0 + pad_rows(sv.d1);
         const int dv = view == 0 ? sv.d0 : sv.d1;
         for (int p = 0; p < npairs; ++p) {
           float g[L::kN2];
@@ -709,7 +717,7 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
           tmem_ld_wait();
           const int col = 128 * (sv.pb + p) + rg;
           if (col < dv) {
-            float* o = sv.out + view * sv.d0 + col;
+            float* o = sv.out + view * o0 + col;
 #pragma unroll
             for (int c = 0; c < (kSolo ? L::kHalf : L::kNW); ++c) {
               const int vv = c / L::kHalf, cc = c - vv * L::kHalf;
@@ -741,130 +749,207 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
   }
 }
 
-// Phi image: per view, K-boxes of 64 columns; B rows 0..23 hold the bf16 hi
-// parts of the 2k columns [U | eta], rows 24..47 their lo parts (x - hi);
-// 128B-swizzled.  Phi is then rounded in place to hi + lo so that the point
-// the pass evaluates is exactly the point the solver holds.  One thread per
-// element of Phi (both views in one launch); the padding of the image is
-// zero from its allocation and never written.
-// Columns col0 .. col0 + ng - 1 of Phi (row stride k2) form the image (a
-// column group: plans with 2k > 24 run the pass once per group).
-__global__ void phi_image_kernel(double* __restrict__ Phix, double* __restrict__ Phiy, int dx, int dy, int k2,
-                                 int col0, int ng, int h1, uint8_t* __restrict__ img, int64_t img_view,
-                                 const int* done) {
-  if (done != nullptr && *done) return;
+// Phi image: per view, K-boxes of 64 columns; B rows 0..h-1 hold the bf16 hi
+// parts of the 2k columns [U | eta] (of a column group of them), rows h ..
+// their lo parts (x - hi); 128B-swizzled.  The point the pass evaluates, hi +
+// lo, is written to Phi, so that it is exactly the point the solver holds
+// (src may be Phi itself).  One thread per element of Phi (every view and
+// group in one launch); the padding of the image is zero from its allocation
+// and never written.
+struct ImageArgs {
+  const double* src[2];  // d x k2 row-major
+  double* Phi[2];
+  int d[2];
+  int k2;
+  int ng0;               // columns of group 0 (the rest are group 1's)
+  int h[2];              // image rows per half of each group
+  uint8_t* img[2];       // per group
+  int64_t img_view;
+  const int* done;
+};
+constexpr int kManyPlans = 16;  // plans of one launch of the per-plan kernels
+template <int N> struct Images { ImageArgs a[N]; };
+
+template <int N>
+__global__ void __launch_bounds__(256) phi_image_kernel(const __grid_constant__ Images<N> many) {
+  const ImageArgs& m = many.a[blockIdx.z];
+  if (m.done != nullptr && *m.done) return;
   const int v = blockIdx.y;
-  const int d = v == 0 ? dx : dy;
-  double* Phi = v == 0 ? Phix : Phiy;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;  // (data column j, group column c)
-  if (e >= d * ng) return;
-  const int j = e / ng, c = e - j * ng;
-  double* px = Phi + (int64_t)j * k2 + col0 + c;
-  const double x = *px;
+  const int d = v == 0 ? m.d[0] : m.d[1];
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;  // (data column j, Phi column q)
+  if (e >= d * m.k2) return;
+  const int j = e / m.k2, q = e - j * m.k2;
+  const int g = q < m.ng0 ? 0 : 1, c = q - (g == 0 ? 0 : m.ng0);
+  const double x = (v == 0 ? m.src[0] : m.src[1])[e];
+  const int h1 = g == 0 ? m.h[0] : m.h[1];
   const __nv_bfloat16 hi = __double2bfloat16(x);
   const __nv_bfloat16 lo = __double2bfloat16(x - (double)__bfloat162float(hi));
-  uint8_t* base = img + (int64_t)v * img_view + (int64_t)(j >> 6) * (2 * h1 * 128);
+  uint8_t* base = (g == 0 ? m.img[0] : m.img[1]) + (int64_t)v * m.img_view + (int64_t)(j >> 6) * (2 * h1 * 128);
   *reinterpret_cast<__nv_bfloat16*>(base + swz(c, j & 63)) = hi;
   *reinterpret_cast<__nv_bfloat16*>(base + swz(h1 + c, j & 63)) = lo;
-  *px = (double)__bfloat162float(hi) + (double)__bfloat162float(lo);
+  (v == 0 ? m.Phi[0] : m.Phi[1])[e] = (double)__bfloat162float(hi) + (double)__bfloat162float(lo);
 }
 
-// G (D x 4k, FP64) = sum over clusters of the FP32 partials, in cluster
-// order.  A CTA covers 256 consecutive entries: 64 float4 groups x 4 quarters
-// of the partials; each quarter is summed with Neumaier-compensated FP32
-// arithmetic (8 loads in flight), then the four (sum, compensation) pairs are
-// combined in fixed order.  Error ~2 ulp of the sum, far below the partials'
-// own rounding.
-// `stride` is the distance of the partial slabs (floats, a multiple of 4, at
-// least len); entries len .. stride - 1 of a slab are padding.  A slab is
-// column-major with D = len / (nvs ng) rows: its columns are, for CCA
-// (nvs = 2), the view-x then the view-y products of group columns 0 .. ng - 1
-// (one view: nvs = 1), and entry (row, vv ng + c) goes to G column
-// vv k2 + col0 + c of the row-major G (rows of nvs k2).  A plan with one
-// column group passes ng = k2, col0 = 0.
-// Gt (optional) receives the same values column-major (nvs k2 rows of D):
-// the slabs' order, so these stores are coalesced and the Gram kernel reads
-// them so.
-__global__ void __launch_bounds__(256) tc_reduce_kernel(const float* __restrict__ part, int nparts, int64_t len,
-                                                        int64_t stride, double* __restrict__ G, const int* done,
-                                                        const int* nparts_dev, int ng, int col0, int k2, int nvs,
-                                                        double* __restrict__ Gt) {
-  if (done != nullptr && *done) return;
-  if (nparts_dev != nullptr) nparts = *nparts_dev;  // batched pass: the schedule's slab count
-  __shared__ float4 red_s[4][64], red_c[4][64];
-  const int g = threadIdx.x & 63, qtr = threadIdx.x >> 6;
-  const int64_t e4 = (int64_t)blockIdx.x * 64 + g;  // float4 group
-  const bool in = 4 * e4 < len;
-  const int per = (nparts + 3) / 4;
-  const int p0 = qtr * per, p1 = min(nparts, p0 + per);
-  float s[4] = {0.f, 0.f, 0.f, 0.f}, cp[4] = {0.f, 0.f, 0.f, 0.f};
-  if (in) {
-    const float4* src = reinterpret_cast<const float4*>(part) + e4;
-    const int64_t stride4 = stride / 4;
-    for (int b0 = p0; b0 < p1; b0 += 8) {
-      float4 v[8];
+// After the data kernel: G = the sum of the clusters' partial slabs, and the
+// partial sums of the Grams that need it, Phi_v^T [G_v | Phi_v], of every
+// block of kPostRows rows of a view.
+//
+// The slabs (12.5 MB for 1024 x 40 columns and 76 clusters) sit in L2 when
+// the data kernel ends, so this is a matter of loads in flight and of FP64
+// rate (about two multiply-adds per clock and SM: 1.2M of them for the two
+// Grams, 2 us over 128 SMs), and of launches: one pass over the slabs, with
+// the Grams formed from the block's rows while they are in shared memory,
+// replaces a reduction, a Gram kernel that read G back (27 us together for
+// 1024 x 40, 19 now, cold) and the Gram of Phi (two launches).  A slab is column-major with the views' rows
+// padded to kPostRows; a CTA reads kPostRows rows of every column as two
+// float4 per (column, slab), the slabs strided over the S threads that share
+// an item (S = kPostThreads / items, so narrow plans split their slabs wider),
+// kPostLoads loads in flight each.  Sums are Neumaier-compensated FP32 per
+// thread, then the S pairs are added in double-float, in fixed order: the
+// error is ~2^-45 of the largest partial, far below the partials' own
+// rounding, and does not depend on scheduling.
+constexpr int kPostThreads = 512;
+constexpr int kPostLoads = 8;
+struct PostArgs {
+  const float* part[2];      // per column group
+  int64_t slab[2];
+  const int* nparts_dev[2];  // batched pass: the schedule's slab counts
+  int nparts;
+  int ng0;                   // columns of group 0 (per view)
+  int d[2], nv, k2;
+  const double* Phi[2];
+  double* G[2];              // row-major, nv k2 columns
+  double* gpart;             // [block][k2 x (nv k2 + k2)]
+  double* Gram;              // nv k2 x nv k2
+  double* phired;            // [view][k2 x k2], or null
+  const int* done;
+};
+template <int N> struct Posts { PostArgs a[N]; };
+
+__device__ __forceinline__ void df_pair_add(float& S, float& C, float s2, float c2) {
+  const float t = S + s2;
+  const float bp = t - S;
+  const float err = (S - (t - bp)) + (s2 - bp);
+  S = t;
+  C += err + c2;
+}
+
+template <int N>
+__global__ void __launch_bounds__(kPostThreads) tc_post_kernel(const __grid_constant__ Posts<N> many) {
+  const PostArgs& m = many.a[blockIdx.y];
+  if (m.done != nullptr && *m.done) return;
+  const int d0p = pad_rows(m.d[0]);
+  const int r0 = blockIdx.x * kPostRows;  // first padded row of the block
+  const int D = d0p + (m.nv > 1 ? pad_rows(m.d[1]) : 0);
+  if (r0 >= D) return;
+  const int v = r0 < d0p ? 0 : 1;
+  const int row0 = v == 0 ? r0 : r0 - d0p;                              // row within the view
+  const int nr = min(kPostRows, (v == 0 ? m.d[0] : m.d[1]) - row0);
+  const int NC = m.nv * m.k2, items = 2 * NC;
+  __shared__ float4 red_s[kPostThreads], red_c[kPostThreads];
+  __shared__ double Gs[kPostRows][4 * kMaxK], Ps[kPostRows][2 * kMaxK];
+  const int t = threadIdx.x;
+  const int S = kPostThreads / items;  // items <= 160
+  const int it = t % items, sl = t / items;
+  for (int e = t; e < kPostRows * m.k2; e += kPostThreads) {
+    const int r = e / m.k2, c = e - r * m.k2;
+    Ps[r][c] = r < nr ? (v == 0 ? m.Phi[0] : m.Phi[1])[(int64_t)(row0 + r) * m.k2 + c] : 0.0;
+  }
+  if (sl < S) {
+    const int c = it >> 1;  // column of G: view-x products, then view-y products
+    const int vv = c / m.k2, q = c - vv * m.k2;
+    const int g = q < m.ng0 ? 0 : 1;
+    const int ng = g == 0 ? m.ng0 : m.k2 - m.ng0;
+    const int sc = vv * ng + (g == 0 ? q : q - m.ng0);  // its column in the slab
+    const int* np = g == 0 ? m.nparts_dev[0] : m.nparts_dev[1];
+    const int nparts = np != nullptr ? *np : m.nparts;
+    const int64_t stride = (g == 0 ? m.slab[0] : m.slab[1]) / 4;
+    const float4* src = reinterpret_cast<const float4*>((g == 0 ? m.part[0] : m.part[1]) + (int64_t)sc * D + r0) + (it & 1);
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, cp[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int b0 = sl; b0 < nparts; b0 += S * kPostLoads) {
+      float4 x4[kPostLoads];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = (b0 + u < p1) ? src[(int64_t)(b0 + u) * stride4] : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < kPostLoads; ++u)
+        x4[u] = b0 + u * S < nparts ? src[(int64_t)(b0 + u * S) * stride] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+      for (int u = 0; u < kPostLoads; ++u) {
+        const float x[4] = {x4[u].x, x4[u].y, x4[u].z, x4[u].w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float t = s[i] + x[i];
-          cp[i] += (fabsf(s[i]) >= fabsf(x[i])) ? ((s[i] - t) + x[i]) : ((x[i] - t) + s[i]);
-          s[i] = t;
+          const float tt = s[i] + x[i];
+          cp[i] += (fabsf(s[i]) >= fabsf(x[i])) ? ((s[i] - tt) + x[i]) : ((x[i] - tt) + s[i]);
+          s[i] = tt;
         }
       }
     }
+    red_s[sl * items + it] = make_float4(s[0], s[1], s[2], s[3]);
+    red_c[sl * items + it] = make_float4(cp[0], cp[1], cp[2], cp[3]);
   }
-  red_s[qtr][g] = make_float4(s[0], s[1], s[2], s[3]);
-  red_c[qtr][g] = make_float4(cp[0], cp[1], cp[2], cp[3]);
   __syncthreads();
-  if (qtr == 0 && in) {
-    double out[4];
-    for (int i = 0; i < 4; ++i) out[i] = 0.0;
-    for (int q = 0; q < 4; ++q) {
-      const float4 a = red_s[q][g], c = red_c[q][g];
-      out[0] += (double)a.x + (double)c.x;
-      out[1] += (double)a.y + (double)c.y;
-      out[2] += (double)a.z + (double)c.z;
-      out[3] += (double)a.w + (double)c.w;
+  double* G = v == 0 ? m.G[0] : m.G[1];
+  const float* rs = reinterpret_cast<const float*>(red_s);
+  const float* rc = reinterpret_cast<const float*>(red_c);
+  for (int e = t; e < kPostRows * NC; e += kPostThreads) {
+    const int r = e / NC, c = e - r * NC;
+    const int o = 4 * (2 * c + (r >> 2)) + (r & 3);
+    float sum = 0.f, comp = 0.f;
+    for (int q = 0; q < S; ++q) df_pair_add(sum, comp, rs[4 * q * items + o], rc[4 * q * items + o]);
+    const double gv = (double)sum + (double)comp;
+    Gs[r][c] = gv;
+    if (r < nr) G[(int64_t)(row0 + r) * NC + c] = gv;
+  }
+  __syncthreads();
+  const int W = NC + m.k2;
+  double* out = m.gpart + (int64_t)blockIdx.x * m.k2 * W;
+  for (int e = t; e < m.k2 * W; e += kPostThreads) {
+    const int i = e / W, b = e - i * W;
+    double sum = 0.0;
+    if (b < NC) {
+      for (int r = 0; r < nr; ++r) sum += Ps[r][i] * Gs[r][b];
+    } else {
+      for (int r = 0; r < nr; ++r) sum += Ps[r][i] * Ps[r][b - NC];
     }
-    const int64_t D = len / (nvs * ng);
-    for (int i = 0; i < 4; ++i) {
-      const int64_t idx = 4 * e4 + i;
-      if (idx >= len) continue;
-      const int col = (int)(idx / D);
-      const int64_t row = idx - (int64_t)col * D;
-      const int vv = col / ng, c = col - vv * ng;
-      G[row * nvs * k2 + vv * k2 + col0 + c] = out[i];
-      if (Gt != nullptr) Gt[(int64_t)(vv * k2 + col0 + c) * D + row] = out[i];
-    }
+    out[e] = sum;
   }
 }
 
-// W^T W = Phi_bd^T G (4k x 4k), Phi_bd = blkdiag(Phi_x, Phi_y), in FP64: one
-// warp per entry, lanes over rows, fixed shuffle tree, G read column-major
-// (Gt: NC rows of D = dx + dy).  One view (nv = 1, FDA): Phi^T G (2k x 2k).
-__global__ void tc_gram_kernel(const double* __restrict__ Phix, const double* __restrict__ Phiy, int dx, int dy,
-                               int k2, int nv, const double* __restrict__ Gt, double* __restrict__ Gram,
-                               const int* done) {
-  if (done != nullptr && *done) return;
-  const int k4 = nv * k2;
-  const int e = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (e >= k4 * k4) return;
-  const int a = e / k4, b = e - a * k4;
-  const int v = a < k2 ? 0 : 1;
-  const int ca = a - v * k2;
-  const double* Phi = v == 0 ? Phix : Phiy;
-  const int d = v == 0 ? dx : dy;
-  const int off = v == 0 ? 0 : dx;
-  double s = 0;
-  const double* gb = Gt + (int64_t)b * (dx + dy) + off;
-  for (int j = lane; j < d; j += 32) s += Phi[(int64_t)j * k2 + ca] * gb[j];
+// Gram = Phi_bd^T G and the views' Phi^T Phi from the blocks' partials: a CTA
+// takes 32 consecutive entries (the lanes) and splits the blocks over its
+// eight warps, eight loads in flight; the warps' sums are added in order.
+template <int N>
+__global__ void __launch_bounds__(256) gram_sum_kernel(const __grid_constant__ Posts<N> many) {
+  const PostArgs& m = many.a[blockIdx.y];
+  if (m.done != nullptr && *m.done) return;
+  __shared__ double red[8][32];
+  const int NC = m.nv * m.k2, W = NC + m.k2, per_view = m.k2 * W;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if ((int)blockIdx.x * 32 >= m.nv * per_view) return;
+  const int e = blockIdx.x * 32 + lane;
+  const int v = e < per_view ? 0 : 1, f = e - v * per_view;
+  const int nb0 = pad_rows(m.d[0]) / kPostRows;
+  const int first = v == 0 ? 0 : nb0, nb = v == 0 ? nb0 : pad_rows(m.d[1]) / kPostRows;
+  double s = 0.0;
+  if (e < m.nv * per_view) {
+    const int per = (nb + 7) / 8, b1 = min(nb, (w + 1) * per);
+    const double* src = m.gpart + (int64_t)first * per_view + f;
+    for (int b0 = w * per; b0 < b1; b0 += 8) {
+      double x[8];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) Gram[e] = s;
+      for (int u = 0; u < 8; ++u) x[u] = b0 + u < b1 ? src[(int64_t)(b0 + u) * per_view] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += x[u];
+    }
+  }
+  red[w][lane] = s;
+  __syncthreads();
+  if (w != 0 || e >= m.nv * per_view) return;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) s += red[q][lane];
+  const int i = f / W, b = f - i * W;
+  if (b < NC)
+    m.Gram[(v * m.k2 + i) * NC + b] = s;
+  else if (m.phired != nullptr)
+    m.phired[((int64_t)v * m.k2 + i) * m.k2 + (b - NC)] = s;
 }
 
 }  // namespace tc
@@ -923,9 +1008,10 @@ bool tc_quad(const Plan& p) { return p.kind == kCCA && std::max(p.v[0].d, p.v[1]
 static int64_t tc_img_view(const Plan& p) { return (tc_quad(p) || tc_solo(p) ? 2 : 1) * (int64_t)tc::kPhiView; }
 static int tc_nviews(const Plan& p) { return tc_solo(p) ? 1 : 2; }
 static uint8_t* tc_group_img(const Plan& p, int g) { return p.tc_img + (int64_t)g * tc_nviews(p) * tc_img_view(p); }
-// floats of one cluster's partial slab of a group of ng columns: D x 2 ng
-// (one view: d x ng, rounded up to a multiple of 4)
-static int64_t tc_slab(const Plan& p, int ng) { return ((int64_t)p.D * tc_nviews(p) * ng + 3) / 4 * 4; }
+// floats of one cluster's partial slab of a group of ng columns: 2 ng columns
+// (one view: ng) of the views' padded rows
+static int tc_rows(const Plan& p) { return tc::pad_rows(p.v[0].d) + (tc_nviews(p) > 1 ? tc::pad_rows(p.v[1].d) : 0); }
+static int64_t tc_slab(const Plan& p, int ng) { return (int64_t)tc_rows(p) * tc_nviews(p) * ng; }
 // partial slabs of group g: clusters (at most half the SMs) x one slab each
 static float* tc_group_part(const Plan& p, int g) {
   int col0 = 0, ng0 = 0;
@@ -933,23 +1019,93 @@ static float* tc_group_part(const Plan& p, int g) {
   return p.tc_part + (int64_t)g * (p.sm_count / 2) * tc_slab(p, ng0);
 }
 
-// The Phi images of a plan (both views, every column group), group g with
-// h1 rows per half (h1 = 0: each group's own); also rounds Phi to the bf16
-// hi + lo point the pass evaluates.
-int tc_phi_image(Plan& p, int h1, cudaStream_t st, const int* done) {
+// Doubles of the partial Grams and floats of the partial slabs that a
+// tensor-core plan needs (all its column groups).
+int64_t tc_gpart_len(const Plan& p) {
   const int k2 = 2 * p.k;
+  return (int64_t)(tc_rows(p) / tc::kPostRows) * k2 * (tc_nviews(p) * k2 + k2);
+}
+int64_t tc_part_len(const Plan& p) { return (int64_t)(p.sm_count / 2) * tc_slab(p, 2 * p.k); }
+
+// Arguments of the Phi images of a plan (both views, every column group),
+// group g with h1 rows per half (h1 = 0: each group's own); Phi is read from
+// the caller's blocks when `io` is given, else from the plan's own.
+static tc::ImageArgs tc_image_args(const Plan& p, int h1, const int* done, const PassIO* io) {
+  tc::ImageArgs a{};
   const int nv = tc_nviews(p);
-  const int d1 = nv > 1 ? p.v[1].d : 0;
-  double* Phi1 = nv > 1 ? p.v[1].Phi : p.v[0].Phi;
-  const int dmax = std::max(p.v[0].d, d1);
+  for (int v = 0; v < nv; ++v) {
+    a.src[v] = io != nullptr ? io->Phi[v] : p.v[v].Phi;
+    a.Phi[v] = p.v[v].Phi;
+    a.d[v] = p.v[v].d;
+  }
+  a.k2 = 2 * p.k;
   for (int g = 0; g < tc_groups(p); ++g) {
     int col0 = 0, ng = 0;
     tc_group(p, g, &col0, &ng);
-    const int hg = h1 > 0 ? h1 : tc_group_h1(p, ng);
-    tc::phi_image_kernel<<<dim3(ceil_div(dmax * ng, 256), nv), 256, 0, st>>>(
-        p.v[0].Phi, Phi1, p.v[0].d, d1, k2, col0, ng, hg, tc_group_img(p, g), tc_img_view(p), done);
-    GB_CHECK_LAUNCH();
+    if (g == 0) a.ng0 = ng;
+    a.h[g] = h1 > 0 ? h1 : tc_group_h1(p, ng);
+    a.img[g] = tc_group_img(p, g);
   }
+  a.img_view = tc_img_view(p);
+  a.done = done;
+  return a;
+}
+static int tc_image_blocks(const Plan& p) {
+  const int dmax = std::max(p.v[0].d, tc_nviews(p) > 1 ? p.v[1].d : 0);
+  return ceil_div(dmax * 2 * p.k, 256);
+}
+
+// The Phi images of a plan; also rounds Phi to the bf16 hi + lo point the
+// pass evaluates.
+int tc_phi_image(Plan& p, int h1, cudaStream_t st, const int* done, const PassIO* io) {
+  tc::Images<1> m{};
+  m.a[0] = tc_image_args(p, h1, done, io);
+  tc::phi_image_kernel<1><<<dim3(tc_image_blocks(p), tc_nviews(p), 1), 256, 0, st>>>(m);
+  GB_CHECK_LAUNCH();
+  return GBCCA_OK;
+}
+
+static tc::PostArgs tc_post_args(const Plan& p, int nparts, const int* nparts_dev, const int* done, const PassIO* io) {
+  tc::PostArgs a{};
+  const int nv = tc_nviews(p), k2 = 2 * p.k;
+  for (int g = 0; g < tc_groups(p); ++g) {
+    int col0 = 0, ng = 0;
+    tc_group(p, g, &col0, &ng);
+    if (g == 0) a.ng0 = ng;
+    a.part[g] = tc_group_part(p, g);
+    a.slab[g] = tc_slab(p, ng);
+    a.nparts_dev[g] = nparts_dev != nullptr ? nparts_dev + g : nullptr;
+  }
+  a.nparts = nparts;
+  a.nv = nv;
+  a.k2 = k2;
+  for (int v = 0; v < nv; ++v) {
+    a.d[v] = p.v[v].d;
+    a.Phi[v] = p.v[v].Phi;
+    a.G[v] = io != nullptr ? io->G[v] : p.G + (v == 0 ? 0 : (int64_t)p.v[0].d * nv * k2);
+  }
+  a.gpart = p.tc_gpart;
+  a.Gram = io != nullptr ? io->Gram : p.Gram;
+  a.phired = p.phired;
+  a.done = done;
+  return a;
+}
+
+// Sum of the partial slabs into G, then W^T W = Phi_bd^T G and the Grams of
+// Phi, for `n` plans (n <= N).
+template <int N>
+static int tc_post_launch(const tc::Posts<N>& m, Plan* const* plans, int n, cudaStream_t st) {
+  int blocks = 1, entries = 1;
+  for (int i = 0; i < n; ++i) {
+    const Plan& p = *plans[i];
+    const int k2 = 2 * p.k, nv = tc_nviews(p);
+    blocks = std::max(blocks, tc_rows(p) / tc::kPostRows);
+    entries = std::max(entries, nv * k2 * (nv * k2 + k2));
+  }
+  tc::tc_post_kernel<N><<<dim3(blocks, n), tc::kPostThreads, 0, st>>>(m);
+  GB_CHECK_LAUNCH();
+  tc::gram_sum_kernel<N><<<dim3(ceil_div(entries, 32), n), 256, 0, st>>>(m);
+  GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }
 
@@ -966,7 +1122,7 @@ static void tc_sources(const Plan& p, const void* src[2], int64_t ld[2], int64_t
   }
 }
 
-int tc_pass(Plan& p, cudaStream_t st, const int* done) {
+int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io) {
   // FP32 data: the row-interleaved hi/lo copy (2n rows) made when the data
   // was bound; BF16 data: the caller's matrices
   const bool fp32 = p.dtype == GBCCA_FP32;
@@ -982,8 +1138,7 @@ int tc_pass(Plan& p, cudaStream_t st, const int* done) {
     p.tc_map_for[0] = src[0];
     p.tc_map_for[1] = src[1];
   }
-  const int k2 = 2 * p.k, k4 = nv * k2;
-  GB_TRY(tc_phi_image(p, 0, st, done));
+  GB_TRY(tc_phi_image(p, 0, st, done, io));
   const CUtensorMap* mx = reinterpret_cast<const CUtensorMap*>(p.tc_map[0]);
   const CUtensorMap* my = reinterpret_cast<const CUtensorMap*>(p.tc_map[1]);
   const int groups = tc_groups(p);
@@ -1047,19 +1202,10 @@ int tc_pass(Plan& p, cudaStream_t st, const int* done) {
     GB_CUDA(cudaEventRecord(p.pass_fork, st));
     p.pass_forked = true;
   }
-  for (int g = 0; g < groups; ++g) {
-    int col0 = 0, ng = 0;
-    tc_group(p, g, &col0, &ng);
-    // partial slabs, one per cluster
-    const int64_t len = (int64_t)p.D * nv * ng;
-    tc::tc_reduce_kernel<<<ceil_div(len, 256), 256, 0, st>>>(tc_group_part(p, g), ncl, len, tc_slab(p, ng), p.G,
-                                                             done, nullptr, ng, col0, k2, nv, p.Gt);
-    GB_CHECK_LAUNCH();
-  }
-  tc::tc_gram_kernel<<<ceil_div(k4 * k4 * 32, 256), 256, 0, st>>>(
-      p.v[0].Phi, nv > 1 ? p.v[1].Phi : p.v[0].Phi, p.v[0].d, nv > 1 ? p.v[1].d : 0, k2, nv, p.Gt, p.Gram, done);
-  GB_CHECK_LAUNCH();
-  return GBCCA_OK;
+  tc::Posts<1> m{};
+  m.a[0] = tc_post_args(p, ncl, nullptr, done, io);
+  Plan* one = &p;
+  return tc_post_launch<1>(m, &one, 1, st);
 }
 
 
@@ -1181,7 +1327,7 @@ TcBatch* tc_batch_create(Plan* const* plans, int n, cudaStream_t st, int* rc) {
       I.done = &p.st->done;
       I.k2 = ng;
       I.pair_sum = p.dtype == GBCCA_FP32 ? 1 : 0;
-      I.slab = (int64_t)p.D * 2 * ng;
+      I.slab = tc_slab(p, ng);
     }
   }
   cudaError_t e = cudaMemcpyAsync(b->inst_d, b->inst_h, sizeof(tc::Inst) * n1, cudaMemcpyHostToDevice, st);
@@ -1267,7 +1413,26 @@ int tc_batch_schedule(TcBatch* b, const bool* plan_active, int clusters, cudaStr
 
 // The Phi images of a batch member (h1 of the batch); nothing once the plan
 // has finished.
-int tc_batch_pre(const TcBatch* b, Plan& p, cudaStream_t st) { return tc_phi_image(p, b->h1, st, &p.st->done); }
+int tc_batch_pre(const TcBatch* b, Plan& p, cudaStream_t st) {
+  return tc_phi_image(p, b->h1, st, &p.st->done, nullptr);
+}
+
+// The same for all n plans of the table, a few plans per launch, from the
+// callers' blocks.
+int tc_batch_pre_all(const TcBatch* b, Plan* const* plans, int n, const PassIO* io, cudaStream_t st) {
+  for (int i0 = 0; i0 < n; i0 += tc::kManyPlans) {
+    const int m = std::min(tc::kManyPlans, n - i0);
+    tc::Images<tc::kManyPlans> a{};
+    int blocks = 1;
+    for (int i = 0; i < m; ++i) {
+      a.a[i] = tc_image_args(*plans[i0 + i], b->h1, nullptr, &io[i0 + i]);
+      blocks = std::max(blocks, tc_image_blocks(*plans[i0 + i]));
+    }
+    tc::phi_image_kernel<tc::kManyPlans><<<dim3(blocks, 2, m), 256, 0, st>>>(a);
+    GB_CHECK_LAUNCH();
+  }
+  return GBCCA_OK;
+}
 
 // One launch over every scheduled tile of the batch.
 int tc_batch_launch(TcBatch* b, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1) {
@@ -1303,21 +1468,24 @@ int tc_batch_launch(TcBatch* b, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1)
   return GBCCA_OK;
 }
 
-// Sum of plan i's slabs (every column group) into its G, then its Gram.
+// Sum of plan i's slabs (every column group) into its G, then its Grams.
 int tc_batch_post(const TcBatch* b, int i, Plan& p, cudaStream_t st, const int* done) {
-  const int k2 = 2 * p.k, k4 = 4 * p.k;
-  const int groups = b->count[i];
-  for (int g = 0; g < groups; ++g) {
-    int col0 = 0, ng = 0;
-    tc_group(p, g, &col0, &ng);
-    const int64_t len = (int64_t)p.D * 2 * ng;
-    tc::tc_reduce_kernel<<<ceil_div(len, 256), 256, 0, st>>>(tc_group_part(p, g), 1, len, len, p.G, done,
-                                                             b->nparts_d + b->first[i] + g, ng, col0, k2, 2, p.Gt);
-    GB_CHECK_LAUNCH();
+  tc::Posts<1> m{};
+  m.a[0] = tc_post_args(p, 1, b->nparts_d + b->first[i], done, nullptr);
+  Plan* one = &p;
+  return tc_post_launch<1>(m, &one, 1, st);
+}
+
+// The same for all n plans of the table, a few plans per launch, into the
+// callers' buffers.
+int tc_batch_post_all(const TcBatch* b, Plan* const* plans, int n, const PassIO* io, cudaStream_t st) {
+  for (int i0 = 0; i0 < n; i0 += tc::kManyPlans) {
+    const int c = std::min(tc::kManyPlans, n - i0);
+    tc::Posts<tc::kManyPlans> m{};
+    for (int i = 0; i < c; ++i)
+      m.a[i] = tc_post_args(*plans[i0 + i], 1, b->nparts_d + b->first[i0 + i], nullptr, &io[i0 + i]);
+    GB_TRY(tc_post_launch<tc::kManyPlans>(m, plans + i0, c, st));
   }
-  tc::tc_gram_kernel<<<ceil_div(k4 * k4 * 32, 256), 256, 0, st>>>(p.v[0].Phi, p.v[1].Phi, p.v[0].d, p.v[1].d, k2,
-                                                                  2, p.Gt, p.Gram, done);
-  GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }
 

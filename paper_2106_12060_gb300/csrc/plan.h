@@ -101,7 +101,7 @@ struct Plan {
 
   // pass buffers
   double* G = nullptr;        // D x NC
-  double* Gt = nullptr;       // NC x D: G column-major (tensor-core pass plans), for the Gram
+  double* tc_gpart = nullptr; // partial Grams of the tensor-core pass's row blocks
   double* Gram = nullptr;     // NC x NC
   void* Wbuf = nullptr;       // n x NC (pass intermediate)
   void* partG = nullptr;      // chunksB x D x NC
@@ -163,6 +163,7 @@ struct Plan {
   // pass_fork after its data kernels (pass_forked)
   cudaEvent_t pass_fork = nullptr, pass_join = nullptr;
   bool fork_after_pass = false, pass_forked = false;
+  bool phired_ready = false;  // the pass has also formed the Grams of Phi (tensor-core pass)
   cudaGraphExec_t batch_exec = nullptr;
   const void* batch_key_ptr[3] = {nullptr, nullptr, nullptr};
   int batch_key_n = 0;
@@ -177,6 +178,14 @@ struct Plan {
   float* means_df = nullptr;  // FDA: the class means as float pairs (l x d padded to 4: hi, then lo)
   cudaEvent_t kev0 = nullptr;  // when set: recorded around the data kernel of the next pass
   cudaEvent_t kev1 = nullptr;  // resident 2-CTA clusters of the tensor-core pass (0: not yet queried)
+};
+
+// Blocks of a stand-alone pass: Phi read from, and G (per view) and the Gram
+// written to, the caller's arrays instead of the plan's.
+struct PassIO {
+  const double* Phi[2];
+  double* G[2];
+  double* Gram;
 };
 
 // sketch.cu
@@ -238,9 +247,9 @@ int mat_thin(const T* A, int ra, int ca, bool transA, bool tri, const double* B,
 
 // pass.cu
 int fused_pass(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols = 0,
-               const int* done = nullptr);
+               const int* done = nullptr, const PassIO* io = nullptr);
 int fused_pass_cores(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols,
-               const int* done);
+               const int* done, const PassIO* io);
 int exact_gram(Plan& p, int view, double* out, cudaStream_t st);
 // out (r x c) = T (r x d) Phi[:, 0:c] (row stride `stride`)
 int table_phi(const double* T, const double* Phi, int r, int d, int c, int stride, double* out, cudaStream_t st,
@@ -249,8 +258,10 @@ int lda_class_stats(Plan& p, cudaStream_t st);
 
 // pass_tc.cu
 bool tc_pass_eligible(const Plan& p);
-int tc_pass(Plan& p, cudaStream_t st, const int* done);
-int tc_phi_image(Plan& p, int h1, cudaStream_t st, const int* done);
+int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io);
+int tc_phi_image(Plan& p, int h1, cudaStream_t st, const int* done, const PassIO* io);
+int64_t tc_gpart_len(const Plan& p);
+int64_t tc_part_len(const Plan& p);
 int tc_groups(const Plan& p);
 bool tc_quad(const Plan& p);
 // batched tensor-core pass over several eligible plans (one persistent launch)
@@ -261,6 +272,8 @@ int tc_batch_schedule(TcBatch* b, const bool* active, int clusters, cudaStream_t
 int tc_batch_pre(const TcBatch* b, Plan& p, cudaStream_t st);
 int tc_batch_launch(TcBatch* b, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1);
 int tc_batch_post(const TcBatch* b, int i, Plan& p, cudaStream_t st, const int* done);
+int tc_batch_pre_all(const TcBatch* b, Plan* const* plans, int n, const PassIO* io, cudaStream_t st);
+int tc_batch_post_all(const TcBatch* b, Plan* const* plans, int n, const PassIO* io, cudaStream_t st);
 int tc_batch_h1(const TcBatch* b);
 int* tc_batch_err(TcBatch* b);
 int tc_batch_max_clusters(const TcBatch* b);

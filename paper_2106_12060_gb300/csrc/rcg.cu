@@ -1793,19 +1793,21 @@ int thin_blocks(const Plan& p) {
 int iteration_post(Plan& p, bool low, cudaStream_t st) {
   const int k = p.k, kk = k * k;
   const int* done = &p.st->done;
-  if (p.pass_forked) {
-    // the Phi Gram and Yhat Phi (Phi is final once the pass has rounded it)
-    // on the side branch, beside the reduction and the Gram of the pass on `st`
+  // the Grams of Phi: formed by the tensor-core pass beside its own, else here
+  const bool need_phi = !p.phired_ready, need_y = p.kind == kLDA;
+  if (p.pass_forked && (need_phi || need_y)) {
+    // what needs only Phi (final once the pass has rounded it) on the side
+    // branch, beside the reduction and the Gram of the pass on `st`
     GB_CUDA(cudaStreamWaitEvent(p.side_stream, p.pass_fork, 0));
-    GB_TRY(phigram(p, p.side_stream, done, p.phired));
+    if (need_phi) GB_TRY(phigram(p, p.side_stream, done, p.phired));
     GB_TRY(yphi(p, p.side_stream, done));
     GB_CUDA(cudaEventRecord(p.pass_join, p.side_stream));
     GB_CUDA(cudaStreamWaitEvent(st, p.pass_join, 0));
-    p.pass_forked = false;
   } else {
-    GB_TRY(phigram(p, st, done, p.phired));
+    if (need_phi) GB_TRY(phigram(p, st, done, p.phired));
     GB_TRY(yphi(p, st, done));
   }
+  p.pass_forked = false;
   const bool ritz = p.opt.rtol > 0;
   if (ritz) {
     // convergence check on the Rayleigh-Ritz values of span([U, eta]) at this
@@ -1958,7 +1960,7 @@ int iteration(Plan& p, bool low, cudaStream_t st, cudaEvent_t e0 = nullptr, cuda
   p.kev0 = e0;
   p.kev1 = e1;
   p.pass_forked = false;
-  p.fork_after_pass = true;
+  p.fork_after_pass = p.kind == kLDA;  // Yhat Phi beside the pass reduction
   const int prc = fused_pass(p, low, false, st, 0, &p.st->done);
   p.fork_after_pass = false;
   p.kev0 = p.kev1 = nullptr;
@@ -2122,7 +2124,7 @@ int rcg_finish(Plan& p, double* out0, double* out1, double* vals, gbcca_info* in
   } else {
     GB_TRY(fused_pass(p, low, false, st, 0, nullptr));
   }
-  GB_TRY(phigram(p, st, nullptr));
+  if (!p.phired_ready) GB_TRY(phigram(p, st, nullptr));
   GB_TRY(yphi(p, st, nullptr));
   {
     RRArgs a{};
@@ -2137,8 +2139,8 @@ int rcg_finish(Plan& p, double* out0, double* out1, double* vals, gbcca_info* in
       a.offx = 0;
       a.offy = 2 * k;
     }
-    a.phipart = p.phipart;
-    a.nblk = thin_blocks(p);
+    a.phipart = p.phired_ready ? p.phired : p.phipart;
+    a.nblk = p.phired_ready ? 1 : thin_blocks(p);
     a.k = k;
     a.kind = p.kind;
     a.l = p.l;

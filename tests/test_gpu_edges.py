@@ -137,3 +137,33 @@ def test_countsketch_sum_layouts(gb, dt, n, d, s):
         plan = gb.cca_plan(n, d, d, 1, dt, gb.default_options(s=s, warm_start=0))
         gb.cca_precondition(plan, x, x, 1e3, 1e3, torch.from_numpy(h).cuda(), torch.from_numpy(g).cuda())
         assert np.array_equal(np64(gb.query(plan, gb.Q_SKETCH_X)).reshape(s, d), ref)
+
+
+@pytest.mark.parametrize("dt", ["bf16", "f32"])
+@pytest.mark.parametrize("n,dx,dy,k", [(9, 1, 2, 1), (64, 8, 7, 3), (513, 9, 130, 9), (1300, 121, 17, 12),
+                                       (1290, 129, 520, 13), (2050, 1024, 41, 20)])
+def test_tc_pass_sums(gb, dt, n, dx, dy, k):
+    """Views whose rows do not fill a block of the slab sums, every split of
+    the slabs over the threads, one and two column groups: G and the Gram
+    against the exact products at the rounded Phi, within 2^-16 of W (its
+    hi + lo operand) and FP32 accumulation."""
+    import torch
+    rng = np.random.default_rng(n + k)
+    tdt = {"bf16": torch.bfloat16, "f32": torch.float32}[dt]
+    data = []
+    for d in (dx, dy):
+        t = torch.zeros(n, (d + 7) // 8 * 8, dtype=tdt, device="cuda")[:, :d]
+        t.copy_(torch.from_numpy(rng.standard_normal((n, d))))
+        data.append(t)
+    P = [rng.standard_normal((d, 2 * k)) for d in (dx, dy)]
+    plan = gb.cca_plan(n, dx, dy, k, dt, gb.default_options(warm_start=0))
+    gb.cca_precondition(plan, *data, 1.0, 1.0)
+    Gx, Gy, Gram = (np64(t) for t in gb.fused_pass(plan, *(torch.from_numpy(p).cuda() for p in P)))
+    Z = [np64(t) for t in data]
+    W = np.hstack([z @ p for z, p in zip(Z, P)])
+    aW = np.hstack([np.abs(z) @ np.abs(p) for z, p in zip(Z, P)])
+    gamma = 6 * 2.0 ** -16 + 2 * (n + dx + dy + 8) * 2.0 ** -23
+    for G, z in ((Gx, Z[0]), (Gy, Z[1])):
+        assert bound_ratio(G, z.T @ W, np.abs(z).T @ aW, gamma) <= 1.0
+    ref = np.vstack([np.abs(p).T @ (np.abs(z).T @ aW) for p, z in zip(P, Z)])
+    assert bound_ratio(Gram, W.T @ W, ref, gamma) <= 1.0
