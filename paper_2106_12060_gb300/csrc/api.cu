@@ -42,7 +42,7 @@ void free_plan(Plan* p) {
   if (p == nullptr) return;
   for (int v = 0; v < 2; ++v) {
     View& w = p->v[v];
-    for (void* q : {(void*)w.SZ, (void*)w.R, (void*)w.Rinv, (void*)w.Rinv32, (void*)w.Minv_hi, (void*)w.Minv_lo, (void*)w.SZh, (void*)w.SZl, (void*)w.RRh, (void*)w.RRl, (void*)w.Phi, (void*)w.Phi32,
+    for (void* q : {(void*)w.SZ, (void*)w.R, (void*)w.Rinv, (void*)w.Minv_hi, (void*)w.Minv_lo, (void*)w.SZh, (void*)w.SZl, (void*)w.RRh, (void*)w.RRl, (void*)w.Phi, (void*)w.Phi32,
                     (void*)w.Meta, (void*)w.gold, (void*)w.Mgold, (void*)w.LL, (void*)w.RR, (void*)w.tmp,
                     (void*)w.warm, (void*)w.wsU, (void*)w.wsT})
       dfree(q);
@@ -51,7 +51,7 @@ void free_plan(Plan* p) {
                   (void*)p->G, (void*)p->tc_gpart, (void*)p->Gram, p->Wbuf, p->partG, p->partGram, p->partCls, (void*)p->counts,
                   (void*)p->means, (void*)p->Yhat, (void*)p->Cls, (void*)p->YPhi, (void*)p->clsPart, (void*)p->st,
                   (void*)p->phigram, (void*)p->phipart, (void*)p->phired, (void*)p->cross, (void*)p->crosspart, (void*)p->history, (void*)p->ritz_hist,
-                  (void*)p->ws, (void*)p->flag, (void*)p->tc_img, (void*)p->tc_part, (void*)p->mt_part, (void*)p->dfx, (void*)p->ls_f, (void*)p->ls_L})
+                  (void*)p->ws, (void*)p->flag, (void*)p->tc_img, (void*)p->tc_part, (void*)p->dfx, (void*)p->ls_f, (void*)p->ls_L})
     dfree(q);
   for (int v = 0; v < 2; ++v) dfree(p->ts_copy[v]);
   dfree(p->means_df);
@@ -80,7 +80,6 @@ int alloc_plan(Plan* p) {
     GB_TRY(dalloc(&w.SZ, p->s * d));
     GB_TRY(dalloc(&w.R, (int64_t)d * d));
     GB_TRY(dalloc(&w.Rinv, (int64_t)d * d));
-    GB_TRY(dalloc(&w.Rinv32, (int64_t)d * d));
     if (p->dtype != GBCCA_FP64) {
       GB_TRY(dalloc(&w.Minv_hi, (int64_t)d * d));
       GB_TRY(dalloc(&w.Minv_lo, (int64_t)d * d));
@@ -172,7 +171,6 @@ int alloc_plan(Plan* p) {
   GB_TRY(dalloc(&p->ritz_hist, (int64_t)p->ritz_len * k));
   p->ws_len = 8 * (int64_t)dmax * dmax + 3 * (int64_t)dmax * std::max(std::max(p->l, k2), 1) + 4096;
   GB_TRY(dalloc(&p->ws, p->ws_len));
-  GB_TRY(dalloc(&p->mt_part, (int64_t)ceil_div(dmax, 64) * dmax * 40));
   GB_TRY(dalloc(&p->dfx, 2 * (int64_t)dmax * k2));
   GB_TRY(dalloc(&p->ls_f, 64));
   GB_TRY(dalloc(&p->ls_L, 64 * 2 * (int64_t)kMaxK * kMaxK));
@@ -297,11 +295,10 @@ int read_flag(Plan& p, cudaStream_t st) {
 
 // Sketch every view, factor the sketch preconditioner and compute the warm
 // start; then install the metric factor the options ask for.
-// Derived forms of R^{-1} used by the iterations: the FP32 copy and, for
-// FP32/BF16 plans, the double-float M^{-1}.
+// Derived form of R^{-1} used by the iterations: for FP32/BF16 plans, the
+// double-float M^{-1}.
 int finish_factor(Plan& p, int v, cudaStream_t st) {
   View& w = p.v[v];
-  GB_TRY(to_f32(w.Rinv, w.Rinv32, (int64_t)w.d * w.d, st));
   if (w.Minv_hi != nullptr) GB_TRY(minv_df_build(w.Rinv, w.d, w.Minv_hi, w.Minv_lo, p.ws, p.ws_len, st));
   return GBCCA_OK;
 }

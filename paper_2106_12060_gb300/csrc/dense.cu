@@ -747,102 +747,86 @@ int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t 
   return GBCCA_OK;
 }
 
-__global__ void to_f32_kernel(const double* __restrict__ a, float* __restrict__ b, int64_t len) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-    b[i] = (float)a[i];
-}
-
-int to_f32(const double* a, float* b, int64_t len, cudaStream_t st) {
-  to_f32_kernel<<<std::min(ceil_div(len, 256), 4096), 256, 0, st>>>(a, b, len);
-  GB_CHECK_LAUNCH();
-  return GBCCA_OK;
-}
-
 // ------------------------------------------------------ factor x thin block
-// C (m x c) = op(A) B with A ra x ca row-major (op = identity or transpose),
-// B (rows = columns of op(A)) and C FP64 with row strides ldb, ldc.  T = double
-// (FP64 path) or float (the FP32 copy of R^{-1} used with BF16/FP32 data).
-// With tri set, A is upper triangular and its zero tiles are skipped.
-// Grid = (16-row blocks) x (64-wide slices of the inner dimension); each CTA
-// writes a partial product and a second kernel adds the slices in order.
-constexpr int kMR = 16, kMK = 64, kMC = 40;
+// C (m x c) = op(A) B for up to two problems in one launch, FP64: A ra x ca
+// row-major (op = identity or transpose), B and C with row strides ldb, ldc.
+// With tri set, A is upper triangular and the inner range is cut to where
+// op(A) is non-zero.  A CTA owns a few rows of C and at most 64 columns; its
+// threads are outputs x 64-wide slices of the inner dimension, each slice one
+// chain in the order of its terms, and the slices are added in order through
+// shared memory (no scratch, no second launch).  Bound by the FP64 rate (a
+// warp-wide multiply-add takes 64 cycles whatever its lanes hold, four warps
+// saturate an SM), so lanes hold outputs only; a tile version that computed
+// 40 columns whatever the shape took 23 + 3 us per product of a 50 x 50 factor
+// with 10 columns, eight of them an iteration for two views.
+constexpr int kSlice = 64;
 
-template <typename T>
-__global__ void __launch_bounds__(128)
-mat_thin_kernel(const T* __restrict__ A, int ra, int ca, int transA, int tri, const double* __restrict__ B,
-                int64_t ldb, double* __restrict__ part, int c) {
-  __shared__ T As[kMK][kMR + 1];   // As[l][r] = op(A)[i0 + r][l0 + l]
-  __shared__ T Bs[kMK][kMC];
-  const int tr = threadIdx.x & 15, tg = threadIdx.x >> 4;  // row, column group (8 groups)
-  const int m = transA ? ca : ra;   // rows of op(A)
-  const int K = transA ? ra : ca;   // columns of op(A)
-  const int i0 = blockIdx.x * kMR, l0 = blockIdx.y * kMK;
-  double* out = part + ((int64_t)blockIdx.y * m) * c;
-  // op(A)[i][l] is nonzero only for l >= i (A upper) or l <= i (A^T lower)
-  const bool zero = (tri && !transA && l0 + kMK - 1 < i0) || (tri && transA && l0 > i0 + kMR - 1);
-  T acc[kMC / 8] = {};
-  if (!zero) {
-    if (transA) {
-      for (int e = threadIdx.x; e < kMK * kMR; e += 128) {
-        int l = e / kMR, r = e % kMR;
-        As[l][r] = (l0 + l < K && i0 + r < m) ? A[(int64_t)(l0 + l) * ca + i0 + r] : T(0);
-      }
-    } else {
-      for (int e = threadIdx.x; e < kMK * kMR; e += 128) {
-        int r = e / kMK, l = e % kMK;
-        As[l][r] = (l0 + l < K && i0 + r < m) ? A[(int64_t)(i0 + r) * ca + l0 + l] : T(0);
-      }
-    }
-    for (int e = threadIdx.x; e < kMK * kMC; e += 128) {
-      int l = e / kMC, cc = e % kMC;
-      Bs[l][cc] = (l0 + l < K && cc < c) ? (T)B[(int64_t)(l0 + l) * ldb + cc] : T(0);
-    }
-    __syncthreads();
-#pragma unroll 16
-    for (int l = 0; l < kMK; ++l) {
-      const T a = As[l][tr];
+// (rows per CTA: as many as its 256 threads hold outputs x slices of, at most 8)
+static int thin_rows(int c, int K) { return std::max(1, std::min(8, 256 / (c * ceil_div(K, kSlice)))); }
+
+__global__ void __launch_bounds__(256) mat_thin_kernel(ThinMul p0, ThinMul p1, int rows0, int rows1, int transA, int tri,
+                                                       int c, int c0, const int* done) {
+  if (done != nullptr && *done) return;
+  extern __shared__ double red[];  // [slice][rows x c]
+  const bool b1 = blockIdx.y != 0;
+  const double* A = b1 ? p1.A : p0.A;
+  const double* B = (b1 ? p1.B : p0.B) + c0;
+  const int ra = b1 ? p1.ra : p0.ra, ca = b1 ? p1.ca : p0.ca, rows = b1 ? rows1 : rows0;
+  const int64_t ldb = b1 ? p1.ldb : p0.ldb;
+  const int m = transA ? ca : ra, K = transA ? ra : ca;
+  const int i0 = blockIdx.x * rows;
+  if (i0 >= m) return;  // uniform over the CTA
+  const int nout = rows * c, ns = (K + kSlice - 1) / kSlice;
+  for (int f = threadIdx.x; f < nout * ns; f += 256) {
+    const int sl = f / nout, e = f - sl * nout, r = e / c, col = e - r * c, i = i0 + r;
+    // op(A)[i][l] is non-zero for l >= i (A upper) or l <= i (its transpose)
+    const int lo = max(sl * kSlice, tri && !transA ? i : 0);
+    const int hi = min(min(K, (sl + 1) * kSlice), tri && transA ? i + 1 : K);
+    double s = 0.0;
+    if (i < m) {
+      const double* Ai = transA ? A + i : A + (int64_t)i * ca;
+      const int64_t sa = transA ? ca : 1;
+      for (int l = lo; l < hi; l += 8) {
+        double x[8], y[8];
 #pragma unroll
-      for (int q = 0; q < kMC / 8; ++q) acc[q] += a * Bs[l][tg + 8 * q];
+        for (int u = 0; u < 8; ++u) {
+          const int q = min(l + u, hi - 1);
+          x[u] = Ai[q * sa];
+          y[u] = B[q * ldb + col];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (l + u < hi) s += x[u] * y[u];
+      }
     }
+    red[f] = s;
   }
-  const int i = i0 + tr;
-  if (i < m) {
-#pragma unroll
-    for (int q = 0; q < kMC / 8; ++q) {
-      const int cc = tg + 8 * q;
-      if (cc < c) out[(int64_t)i * c + cc] = (double)acc[q];
-    }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nout; e += 256) {
+    const int r = e / c, col = e - r * c;
+    if (i0 + r >= m) continue;
+    double s = 0.0;
+    for (int q = 0; q < ns; ++q) s += red[q * nout + e];
+    (b1 ? p1.C : p0.C)[(int64_t)(i0 + r) * (b1 ? p1.ldc : p0.ldc) + c0 + col] = s;
   }
 }
 
-__global__ void mat_thin_sum_kernel(const double* __restrict__ part, int nslices, int m, int c,
-                                    double* __restrict__ C, int64_t ldc) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= m * c) return;
-  double s = 0;
-  for (int q = 0; q < nslices; ++q) s += part[(int64_t)q * m * c + e];
-  C[(int64_t)(e / c) * ldc + e % c] = s;
-}
-
-template <typename T>
-int mat_thin(const T* A, int ra, int ca, bool transA, bool tri, const double* B, int64_t ldb, double* C,
-             int64_t ldc, int c, double* part, cudaStream_t st) {
-  const int m = transA ? ca : ra;
-  const int K = transA ? ra : ca;
-  const int ns = ceil_div(K, kMK);
-  for (int c0 = 0; c0 < c; c0 += kMC) {
-    const int cw = std::min(kMC, c - c0);
-    mat_thin_kernel<T><<<dim3(ceil_div(m, kMR), ns), 128, 0, st>>>(A, ra, ca, transA ? 1 : 0, tri ? 1 : 0, B + c0,
-                                                                   ldb, part, cw);
-    GB_CHECK_LAUNCH();
-    mat_thin_sum_kernel<<<ceil_div(m * cw, 256), 256, 0, st>>>(part, ns, m, cw, C + c0, ldc);
+int mat_thin(const ThinMul* p, int nprob, bool transA, bool tri, int c, cudaStream_t st, const int* done) {
+  for (int c0 = 0; c0 < c; c0 += 64) {
+    const int cw = std::min(64, c - c0);
+    int blocks = 1, rows[2] = {1, 1};
+    size_t smem = 0;
+    for (int b = 0; b < nprob; ++b) {
+      const int m = transA ? p[b].ca : p[b].ra, K = transA ? p[b].ra : p[b].ca;
+      rows[b] = thin_rows(cw, K);
+      blocks = std::max(blocks, ceil_div(m, rows[b]));
+      smem = std::max(smem, sizeof(double) * rows[b] * cw * ceil_div(K, kSlice));
+    }
+    mat_thin_kernel<<<dim3(blocks, nprob), 256, smem, st>>>(p[0], p[nprob > 1 ? 1 : 0], rows[0], rows[1],
+                                                            transA ? 1 : 0, tri ? 1 : 0, cw, c0, done);
     GB_CHECK_LAUNCH();
   }
   return GBCCA_OK;
 }
-template int mat_thin<double>(const double*, int, int, bool, bool, const double*, int64_t, double*, int64_t, int,
-                              double*, cudaStream_t);
-template int mat_thin<float>(const float*, int, int, bool, bool, const double*, int64_t, double*, int64_t, int,
-                             double*, cudaStream_t);
 
 }  // namespace gbcca

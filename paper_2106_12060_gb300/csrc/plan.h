@@ -55,7 +55,6 @@ struct View {
   float* SZl = nullptr;
   double* R = nullptr;      // d x d upper triangular, R^T R = M
   double* Rinv = nullptr;   // d x d, R^{-1}
-  float* Rinv32 = nullptr;  // FP32 copy for the low-precision path
   float* Minv_hi = nullptr; // M^{-1} = R^{-1} R^{-T} as a float pair (low-precision plans)
   float* Minv_lo = nullptr;
   float* RRh = nullptr;     // d x 2k: RR[:, 0:2k] as a float pair (input of the M^{-1} product)
@@ -131,7 +130,6 @@ struct Plan {
   double* history = nullptr;    // 3 (max_iter + 1)
   double* ritz_hist = nullptr;  // Ritz values at every check: (max_iter / check_every + 2) x k
   int ritz_len = 0;             // rows of ritz_hist
-  double* mt_part = nullptr;    // slice partials of mat_thin
   float* dfx = nullptr;         // 2 x dmax x 2k floats: split blocks for double-float products
   double* ls_f = nullptr;       // line-search trial values (kNTrials)
   double* ls_L = nullptr;       // line-search trial factors (kNTrials x 2 x kMaxK^2)
@@ -237,13 +235,18 @@ int split_df(const double* A, int r, int c, bool trans, float* hi, float* lo, cu
 int minv_df_build(const double* Rinv, int d, float* hi, float* lo, double* ws, int64_t ws_len, cudaStream_t st);
 // Rinv = R^{-1} (upper triangular, d x d); ws holds at least d * d doubles.
 int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t ws_len, cudaStream_t st);
-int to_f32(const double* a, float* b, int64_t len, cudaStream_t st);
-// C (m x c, ldc) = op(A) B (rows of B = columns of op(A), ldb); A is
-// ra x ca row-major; tri = 1 skips the zero half of an upper-triangular A.
-// `part` is scratch of ceil(K / 64) * m * min(c, 40) doubles.
-template <typename T>
-int mat_thin(const T* A, int ra, int ca, bool transA, bool tri, const double* B, int64_t ldb, double* C,
-             int64_t ldc, int c, double* part, cudaStream_t st);
+// C (m x c, ldc) = op(A) B (rows of B = columns of op(A), ldb), A ra x ca
+// row-major, for one or two problems in one launch; tri: A upper triangular,
+// its zero half skipped.
+struct ThinMul {
+  const double* A;
+  int ra, ca;
+  const double* B;
+  int64_t ldb;
+  double* C;
+  int64_t ldc;
+};
+int mat_thin(const ThinMul* p, int nprob, bool transA, bool tri, int c, cudaStream_t st, const int* done = nullptr);
 
 // pass.cu
 int fused_pass(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi_cols = 0,

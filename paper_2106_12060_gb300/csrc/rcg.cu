@@ -1754,18 +1754,18 @@ __global__ void copy_sigma_kernel(const DevState* st, double* out, int k) {
 // ============================================================== driver
 namespace {
 
-int minv(Plan& p, int v, cudaStream_t st) {
-  View& w = p.v[v];
-  const int k = p.k, k2 = 2 * k, k4 = 4 * k;
-  // tmp = R^{-T} RR[:, 0:2k]; LL[:, 0:2k] = R^{-1} tmp
-  if (p.dtype == GBCCA_FP64) {
-    GB_TRY(mat_thin<double>(w.Rinv, w.d, w.d, true, true, w.RR, k4, w.tmp, k2, k2, p.mt_part, st));
-    GB_TRY(mat_thin<double>(w.Rinv, w.d, w.d, false, true, w.tmp, k2, w.LL, k4, k2, p.mt_part, st));
-  } else {
-    GB_TRY(mat_thin<float>(w.Rinv32, w.d, w.d, true, true, w.RR, k4, w.tmp, k2, k2, p.mt_part, st));
-    GB_TRY(mat_thin<float>(w.Rinv32, w.d, w.d, false, true, w.tmp, k2, w.LL, k4, k2, p.mt_part, st));
+// FP64 plans: LL[:, 0:2k] = R^{-1} (R^{-T} RR[:, 0:2k]), every view in one
+// launch per factor
+int minv(Plan& p, cudaStream_t st, const int* done) {
+  const int k2 = 2 * p.k, k4 = 4 * p.k;
+  ThinMul t[2], u[2];
+  for (int v = 0; v < p.nviews; ++v) {
+    View& w = p.v[v];
+    t[v] = ThinMul{w.Rinv, w.d, w.d, w.RR, k4, w.tmp, k2};
+    u[v] = ThinMul{w.Rinv, w.d, w.d, w.tmp, k2, w.LL, k4};
   }
-  return GBCCA_OK;
+  GB_TRY(mat_thin(t, p.nviews, true, true, k2, st, done));
+  return mat_thin(u, p.nviews, false, true, k2, st, done);
 }
 
 int phigram(Plan& p, cudaStream_t st, const int* done, double* out = nullptr) {
@@ -1901,7 +1901,7 @@ int iteration_post(Plan& p, bool low, cudaStream_t st) {
     m.done = done;
     GB_TRY(dfmv(m, p.nviews, st));
   } else {
-    for (int v = 0; v < p.nviews; ++v) GB_TRY(minv(p, v, st));
+    GB_TRY(minv(p, st, done));
   }
   GB_TRY(thin_gram(p, p.v[0].LL, p.nviews > 1 ? p.v[1].LL : nullptr, 4 * k, p.v[0].RR,
                    p.nviews > 1 ? p.v[1].RR : nullptr, 4 * k, 4 * k, 4 * k, p.crosspart, st, done, p.cross));
@@ -2435,15 +2435,18 @@ int warm_start(Plan& p, cudaStream_t st) {
     };
     auto rx = [&](bool tr, const double* B, double* C, int cc) {
       if (low && cc == c) return dmv(tr ? RxT : Rx, dx, dx, B, C);
-      return mat_thin<double>(x.Rinv, dx, dx, tr, true, B, cc, C, cc, cc, p.mt_part, st);
+      const ThinMul t{x.Rinv, dx, dx, B, cc, C, cc};
+      return mat_thin(&t, 1, tr, true, cc, st);
     };
     auto ry = [&](bool tr, const double* B, double* C, int cc) {
       if (low && cc == c) return dmv(tr ? RyT : Ry, dy, dy, B, C);
-      return mat_thin<double>(y.Rinv, dy, dy, tr, true, B, cc, C, cc, cc, p.mt_part, st);
+      const ThinMul t{y.Rinv, dy, dy, B, cc, C, cc};
+      return mat_thin(&t, 1, tr, true, cc, st);
     };
     auto cxy = [&](bool tr, const double* B, double* C) {
       if (low) return tr ? dmv(CfT, dy, dx, B, C) : dmv(Cf, dx, dy, B, C);
-      return mat_thin<double>(Cxy, dx, dy, tr, false, B, c, C, c, c, p.mt_part, st);
+      const ThinMul t{Cxy, dx, dy, B, c, C, c};
+      return mat_thin(&t, 1, tr, false, c, st);
     };
     rand_block_kernel<<<ceil_div(dy * c, 256), 256, 0, st>>>(Vb, dy, c, p.opt.seed);
     GB_CHECK_LAUNCH();
@@ -2507,7 +2510,8 @@ int warm_start(Plan& p, cudaStream_t st) {
   (void)YhT;
   transpose_kernel<<<ceil_div(l * d, 256), 256, 0, st>>>(p.Yhat, l, d, YT);
   GB_CHECK_LAUNCH();
-  GB_TRY(mat_thin<double>(x.Rinv, d, d, true, true, YT, l, Gt, l, l, p.mt_part, st));
+  const ThinMul t1{x.Rinv, d, d, YT, l, Gt, l};
+  GB_TRY(mat_thin(&t1, 1, true, true, l, st));
   {
     ThinArgs a{};
     a.A[0] = Gt;
@@ -2531,7 +2535,8 @@ int warm_start(Plan& p, cudaStream_t st) {
     double* Wwh = p.ws + 2 * (int64_t)d * l;  // d x k
     thin_apply_kernel<<<ceil_div(d, 128), 128, 0, st>>>(Gt, d, l, rot, k, Wwh);
     GB_CHECK_LAUNCH();
-    GB_TRY(mat_thin<double>(x.Rinv, d, d, false, true, Wwh, k, x.warm, k, k, p.mt_part, st));
+    const ThinMul t2{x.Rinv, d, d, Wwh, k, x.warm, k};
+    GB_TRY(mat_thin(&t2, 1, false, true, k, st));
   }
   return GBCCA_OK;
 }

@@ -167,3 +167,24 @@ def test_tc_pass_sums(gb, dt, n, dx, dy, k):
         assert bound_ratio(G, z.T @ W, np.abs(z).T @ aW, gamma) <= 1.0
     ref = np.vstack([np.abs(p).T @ (np.abs(z).T @ aW) for p, z in zip(P, Z)])
     assert bound_ratio(Gram, W.T @ W, ref, gamma) <= 1.0
+
+
+@pytest.mark.parametrize("d,k", [(1, 1), (7, 3), (33, 10), (130, 20)])
+def test_thin_products_f64(gb, d, k):
+    """The FP64 products with R^{-1} (inner ranges cut at the diagonal): the
+    warm start maps an orthonormal block back through R^{-1}, so R times it
+    has orthonormal columns, to FP64 rounding times the condition of R."""
+    import torch
+    from synth import countsketch_draws
+    n, s, lam = 8 * d + 40, 3 * d + 10, 1e-1
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((n, d))
+    Y = 0.5 * X + rng.standard_normal((n, d))
+    h, g = countsketch_draws(n, s, seed=3)
+    plan = gb.cca_plan(n, d, d, k, "f64", gb.default_options(s=s, max_iter=1, gtol=0.0))
+    gb.cca_precondition(plan, torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), lam, lam,
+                        torch.from_numpy(h).cuda(), torch.from_numpy(g).cuda())
+    for q, w in ((gb.Q_R_X, gb.Q_WARM_U), (gb.Q_R_Y, gb.Q_WARM_V)):
+        R = np64(gb.query(plan, q)).reshape(d, d)
+        A = R @ np64(gb.query(plan, w)).reshape(d, k)
+        assert np.max(np.abs(A.T @ A - np.eye(k))) < 1e-10
