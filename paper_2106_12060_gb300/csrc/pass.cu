@@ -1,5 +1,5 @@
-// The per-iteration data pass on CUDA cores (any storage type) and the LDA
-// class statistics.
+// The per-iteration data pass on CUDA cores (FP32 accumulation; the FP64 one
+// is pass64.cu) and the LDA class statistics.
 //
 // One Riemannian-CG iteration needs, for Phi_x = [U, eta_U], Phi_y = [V, eta_V]
 // (Sec. 4.2 gradient, Table 1 retraction and projection, Cor. 4.6 cost):
@@ -11,7 +11,7 @@
 // the class-mean rows and accumulates per-class column sums of P); kernel B
 // accumulates Z^T W over row chunks x column blocks; a fixed-order reduction
 // sums the per-CTA partials in FP64, so results are bitwise reproducible.
-#include "plan.h"
+#include "pass64.h"
 
 namespace gbcca {
 
@@ -345,26 +345,30 @@ pass_g_async_kernel(PassViews pv, int64_t n, int NC, int D, const float* __restr
   }
 }
 
-__global__ void pass_reduce_kernel(const double* __restrict__ partG, int chunks, int64_t nG,
-                                   const double* __restrict__ partGram, int ctas, int64_t nGram,
-                                   double* __restrict__ G0, double* __restrict__ G1, int64_t n0,
-                                   double* __restrict__ Gram, const int* done) {
-  if (done != nullptr && *done) return;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nG + nGram;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    double s = 0;
-    if (e < nG) {
-      if (partG != nullptr) {
-        for (int c = 0; c < chunks; ++c) s += (double)partG[(int64_t)c * nG + e];
-        if (e < n0) G0[e] = s;  // view 0's rows, then view 1's
-        else G1[e - n0] = s;
-      }
-    } else {
-      int64_t f = e - nG;
-      for (int c = 0; c < ctas; ++c) s += (double)partGram[(int64_t)c * nGram + f];
-      Gram[f] = s;
-    }
+// Sums of the partials, in order, sixteen loads in flight per thread (one at a
+// time it was a chain of loads: 12 us for 1800 + 400 entries of 63 and 32
+// partials).
+__device__ __forceinline__ double sum_strided(const double* __restrict__ src, int64_t stride, int n) {
+  double s = 0.0;
+  for (int b0 = 0; b0 < n; b0 += 16) {
+    double x[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) x[u] = b0 + u < n ? src[(int64_t)(b0 + u) * stride] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) s += x[u];
   }
+  return s;
+}
+
+__global__ void __launch_bounds__(64) pass_reduce_kernel(const double* __restrict__ partG, int chunks, int64_t nG,
+                                                         const double* __restrict__ partGram, int ctas, int64_t nGram,
+                                                         double* __restrict__ G0, double* __restrict__ G1, int64_t n0,
+                                                         double* __restrict__ Gram, const int* done) {
+  if (done != nullptr && *done) return;
+  const int64_t e = blockIdx.x * (int64_t)64 + threadIdx.x;
+  if (e < n0 && e < nG) G0[e] = sum_strided(partG + e, nG, chunks);  // view 0's rows, then view 1's
+  else if (e < nG) G1[e - n0] = sum_strided(partG + e, nG, chunks);
+  else if (e < nG + nGram) Gram[e - nG] = sum_strided(partGram + (e - nG), nGram, ctas);
 }
 
 // FDA: Xhat^T P = X^T P - sum_k m_k (sum_{i in k} P_i)^T.
@@ -373,9 +377,7 @@ __global__ void lda_correct_kernel(const double* __restrict__ partCls, int ctas,
   __shared__ double sP[kMaxClasses * 48];
   if (done != nullptr && *done) return;
   for (int e = threadIdx.x; e < l * NC; e += blockDim.x) {
-    double s = 0;
-    for (int c = 0; c < ctas; ++c) s += (double)partCls[(int64_t)c * l * NC + e];
-    sP[e] = s;
+    sP[e] = sum_strided(partCls + e, (int64_t)l * NC, ctas);
   }
   __syncthreads();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * NC; e += gridDim.x * blockDim.x) {
@@ -519,8 +521,27 @@ int dispatch_g(Plan& p, const PassViews& pv, const Tacc* W, cudaStream_t st) {
   }
 }
 
-template <typename Tin, typename Tacc>
-int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* done, const PassIO* io) {
+// Partial Grams of G (chunks) and of W^T W (ctas) summed into place.
+int reduce_parts(Plan& p, const double* partG, int NC, int ctas, cudaStream_t st, const int* done, const PassIO* io) {
+  const int64_t nG = partG == nullptr ? 0 : (int64_t)p.D * NC, nGram = (int64_t)NC * NC;
+  const int64_t n0 = (int64_t)p.v[0].d * NC;
+  double* G0 = io != nullptr ? io->G[0] : p.G;
+  double* G1 = io != nullptr ? io->G[1] : p.G + n0;
+  pass_reduce_kernel<<<ceil_div(nG + nGram, 64), 64, 0, st>>>(partG, p.chunksB, nG,
+                                                               reinterpret_cast<const double*>(p.partGram), ctas, nGram,
+                                                               G0, G1, n0, io != nullptr ? io->Gram : p.Gram, done);
+  GB_CHECK_LAUNCH();
+  if (p.kind == kLDA && partG != nullptr) {
+    lda_correct_kernel<<<ceil_div((int64_t)p.D * NC, 256), 256, 0, st>>>(
+        reinterpret_cast<const double*>(p.partCls), ctas, p.l, NC, p.D, p.means, G0, done);
+    GB_CHECK_LAUNCH();
+  }
+  return GBCCA_OK;
+}
+
+// FP32 accumulation
+template <typename Tin>
+int run_pass32(Plan& p, cudaStream_t st, int phi_cols, const int* done, const PassIO* io) {
   PassViews pv{};
   pv.nviews = p.nviews;
   pv.k2 = phi_cols;
@@ -535,47 +556,54 @@ int run_pass(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* 
     pv.dofs[v] = dofs;
     pv.ocol[v] = v * phi_cols;
     dofs += p.v[v].d;
-    const double* Phi = io != nullptr ? io->Phi[v] : p.v[v].Phi;
-    if (std::is_same<Tacc, double>::value) {
-      pv.Phi[v] = Phi;
-    } else {
-      int64_t len = (int64_t)p.v[v].d * 2 * p.k;
-      phi_convert_kernel<float><<<ceil_div(len, 256), 256, 0, st>>>(Phi, p.v[v].Phi32, len);
-      GB_CHECK_LAUNCH();
-      pv.Phi[v] = p.v[v].Phi32;
-    }
+    const int64_t len = (int64_t)p.v[v].d * 2 * p.k;
+    phi_convert_kernel<float><<<ceil_div(len, 256), 256, 0, st>>>(io != nullptr ? io->Phi[v] : p.v[v].Phi,
+                                                                  p.v[v].Phi32, len);
+    GB_CHECK_LAUNCH();
+    pv.Phi[v] = p.v[v].Phi32;
   }
-  Tacc* cls = nullptr;
+  float* cls = nullptr;
   if (p.kind == kLDA) {
-    int len = p.l * phi_cols;
-    GB_TRY(table_phi(p.means, io != nullptr ? io->Phi[0] : p.v[0].Phi, p.l, p.v[0].d, phi_cols, 2 * p.k, p.Cls, st, nullptr));
-    if (std::is_same<Tacc, double>::value) {
-      cls = reinterpret_cast<Tacc*>(p.Cls);
-    } else {
-      cls = reinterpret_cast<Tacc*>(p.Cls + p.l * 2 * p.k);  // FP32 copy stored after the FP64 one
-      cast_cls_kernel<Tacc><<<ceil_div(len, 128), 128, 0, st>>>(p.Cls, cls, len);
-      GB_CHECK_LAUNCH();
-    }
-  }
-  Tacc* W = gram_only ? nullptr : reinterpret_cast<Tacc*>(p.Wbuf);
-  GB_TRY((dispatch_w<Tin, Tacc>(p, pv, NC, W, st, cls)));
-  if (!gram_only) GB_TRY((dispatch_g<Tin, Tacc>(p, pv, W, st)));
-  int64_t nG = gram_only ? 0 : (int64_t)p.D * NC;
-  const int64_t n0 = (int64_t)p.v[0].d * NC;
-  double* G0 = io != nullptr ? io->G[0] : p.G;
-  double* G1 = io != nullptr ? io->G[1] : p.G + n0;
-  int64_t nGram = (int64_t)NC * NC;
-  pass_reduce_kernel<<<ceil_div(nG + nGram, 256), 256, 0, st>>>(
-      gram_only ? nullptr : reinterpret_cast<const double*>(p.partG), p.chunksB, nG,
-      reinterpret_cast<const double*>(p.partGram), p.ctasA, nGram, G0, G1, n0,
-      io != nullptr ? io->Gram : p.Gram, done);
-  GB_CHECK_LAUNCH();
-  if (p.kind == kLDA && !gram_only) {
-    lda_correct_kernel<<<ceil_div((int64_t)p.D * NC, 256), 256, 0, st>>>(
-        reinterpret_cast<const double*>(p.partCls), p.ctasA, p.l, NC, p.D, p.means, G0, done);
+    const int len = p.l * phi_cols;
+    GB_TRY(table_phi(p.means, io != nullptr ? io->Phi[0] : p.v[0].Phi, p.l, p.v[0].d, phi_cols, 2 * p.k, p.Cls, st,
+                     nullptr));
+    cls = reinterpret_cast<float*>(p.Cls + p.l * 2 * p.k);  // FP32 copy stored after the FP64 one
+    cast_cls_kernel<float><<<ceil_div(len, 128), 128, 0, st>>>(p.Cls, cls, len);
     GB_CHECK_LAUNCH();
   }
-  return GBCCA_OK;
+  float* W = reinterpret_cast<float*>(p.Wbuf);
+  GB_TRY((dispatch_w<Tin, float>(p, pv, NC, W, st, cls)));
+  GB_TRY((dispatch_g<Tin, float>(p, pv, W, st)));
+  return reduce_parts(p, reinterpret_cast<const double*>(p.partG), NC, p.ctasA, st, done, io);
+}
+
+// FP64 arithmetic (any storage type; Z^T W with FP64 data only)
+int run_pass64(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int* done, const PassIO* io) {
+  Pass64 a{};
+  a.nviews = p.nviews;
+  a.kc = phi_cols;
+  a.phistride = 2 * p.k;
+  a.n = p.n;
+  a.NC = p.nviews * phi_cols;
+  a.done = done;
+  for (int v = 0; v < p.nviews; ++v) {
+    a.Z[v] = p.v[v].Z;
+    a.ld[v] = p.v[v].ld;
+    a.d[v] = p.v[v].d;
+    a.Phi[v] = io != nullptr ? io->Phi[v] : p.v[v].Phi;
+  }
+  if (p.kind == kLDA) {
+    GB_TRY(table_phi(p.means, a.Phi[0], p.l, p.v[0].d, phi_cols, 2 * p.k, p.Cls, st, nullptr));
+    a.labels = p.labels;
+    a.Cls = p.Cls;
+    a.l = p.l;
+    a.partCls = gram_only ? nullptr : reinterpret_cast<double*>(p.partCls);
+  }
+  a.W = reinterpret_cast<double*>(p.Wbuf);
+  a.partGram = reinterpret_cast<double*>(p.partGram);
+  double* partG = gram_only ? nullptr : reinterpret_cast<double*>(p.partG);
+  GB_TRY(pass64(a, p.dtype, p.ctasA, p.chunksB, p.D, partG, st));
+  return reduce_parts(p, partG, a.NC, p.ctasA, st, done, io);
 }
 
 }  // namespace
@@ -616,16 +644,9 @@ int fused_pass_cores(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi
     set_last_error("too many classes x columns for the FDA pass");
     return GBCCA_ERR_UNSUPPORTED;
   }
-  switch (p.dtype) {
-    case GBCCA_FP64: return run_pass<double, double>(p, gram_only, st, phi_cols, done, io);
-    case GBCCA_FP32:
-      return low ? run_pass<float, float>(p, gram_only, st, phi_cols, done, io)
-                 : run_pass<float, double>(p, gram_only, st, phi_cols, done, io);
-    case GBCCA_BF16:
-      return low ? run_pass<__nv_bfloat16, float>(p, gram_only, st, phi_cols, done, io)
-                 : run_pass<__nv_bfloat16, double>(p, gram_only, st, phi_cols, done, io);
-  }
-  return GBCCA_ERR_INVALID_ARG;
+  if (!low || p.dtype == GBCCA_FP64) return run_pass64(p, gram_only, st, phi_cols, done, io);
+  return p.dtype == GBCCA_FP32 ? run_pass32<float>(p, st, phi_cols, done, io)
+                               : run_pass32<__nv_bfloat16>(p, st, phi_cols, done, io);
 }
 
 // ------------------------------------------------------------ FDA statistics

@@ -204,17 +204,6 @@ int countsketch_prepare(Plan& p, cudaStream_t st) {
   return GBCCA_OK;
 }
 
-// FP32 -> FP64 by moving the bits (a hardware conversion runs at the FP64
-// rate); zeros included, subnormals and non-finite values by the conversion.
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
-  if (m - 0x00800000u < 0x7f000000u || m == 0u)  // normal, or zero
-    return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 3) + 0x38000000u)), (int)(u << 29));
-  return (double)x;
-}
-__device__ __forceinline__ double widen(double x) { return x; }
-__device__ __forceinline__ double widen(__nv_bfloat16 x) { return widen(__bfloat162float(x)); }
-
 // kV consecutive values of a row: one 16- or 8-byte load
 template <typename Tin, int kV> struct alignas(sizeof(Tin) * kV) RowVec { Tin v[kV]; };
 

@@ -169,6 +169,28 @@ def test_tc_pass_sums(gb, dt, n, dx, dy, k):
     assert bound_ratio(Gram, W.T @ W, ref, gamma) <= 1.0
 
 
+@pytest.mark.parametrize("n,dx,dy,k", [(2, 1, 1, 1), (15, 9, 3, 2), (70, 65, 33, 9), (1000, 128, 31, 11),
+                                       (5000, 260, 64, 20)])
+def test_pass_f64_edges(gb, n, dx, dy, k):
+    """The FP64 pass at row counts around its tiles and chunks, inner
+    dimensions around its steps and every column count class: chains of dx +
+    dy + n terms in FP64, entrywise."""
+    import torch
+    rng = np.random.default_rng(n + k)
+    X, Y = rng.standard_normal((n, dx)), rng.standard_normal((n, dy))
+    P = [rng.standard_normal((d, 2 * k)) for d in (dx, dy)]
+    plan = gb.cca_plan(n, dx, dy, k, "f64", gb.default_options(warm_start=0))
+    gb.cca_precondition(plan, torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), 1.0, 1.0)
+    Gx, Gy, Gram = (np64(t) for t in gb.fused_pass(plan, *(torch.from_numpy(p).cuda() for p in P)))
+    W = np.hstack([X @ P[0], Y @ P[1]])
+    aW = np.hstack([np.abs(X) @ np.abs(P[0]), np.abs(Y) @ np.abs(P[1])])
+    gamma = 4 * (n + dx + dy + 8) * 2.0 ** -53
+    assert bound_ratio(Gx, X.T @ W, np.abs(X).T @ aW, gamma) <= 1.0
+    assert bound_ratio(Gy, Y.T @ W, np.abs(Y).T @ aW, gamma) <= 1.0
+    assert bound_ratio(Gram, W.T @ W, aW.T @ aW, gamma) <= 1.0
+    assert np.array_equal(Gram, Gram.T)
+
+
 @pytest.mark.parametrize("d,k", [(1, 1), (7, 3), (33, 10), (130, 20)])
 def test_thin_products_f64(gb, d, k):
     """The FP64 products with R^{-1} (inner ranges cut at the diagonal): the
