@@ -653,7 +653,8 @@ int fused_pass_cores(Plan& p, bool low, bool gram_only, cudaStream_t st, int phi
 // Per-class column sums in FP64: CTA = (row chunk, 256-column block); each
 // thread owns one column, so the accumulation order is fixed.  The loads of
 // kRowsInFlight rows are issued before their additions, so that the memory
-// latency is paid once per group instead of once per row.
+// latency is paid once per group instead of once per row.  Bound by the FP64
+// rate: one addition per element, the conversion done on the bits.
 constexpr int kRowsInFlight = 8;
 template <typename Tin>
 __global__ void class_sums_kernel(const Tin* __restrict__ X, int64_t ld, int64_t n, int d,
@@ -675,7 +676,7 @@ __global__ void class_sums_kernel(const Tin* __restrict__ X, int64_t ld, int64_t
     }
 #pragma unroll
     for (int u = 0; u < kRowsInFlight; ++u) {
-      if (c < d && yv[u] >= 0 && yv[u] < l) acc[yv[u] * 256 + threadIdx.x] += to_f64(x[u]);  // bad labels: see label_check
+      if (c < d && yv[u] >= 0 && yv[u] < l) acc[yv[u] * 256 + threadIdx.x] += widen(x[u]);  // bad labels: see label_check
       if (counts) cn += yv[u] == (int)threadIdx.x ? 1 : 0;
     }
   }

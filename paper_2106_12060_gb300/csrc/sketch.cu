@@ -204,6 +204,10 @@ int countsketch_prepare(Plan& p, cudaStream_t st) {
   return GBCCA_OK;
 }
 
+// x times a sign outside +-1 (a caller's own draws); out of line, so that the
+// usual signs cost no FP64 instruction
+static __device__ __noinline__ double scale_by(double x, int sg) { return (double)sg * x; }
+
 // kV consecutive values of a row: one 16- or 8-byte load
 template <typename Tin, int kV> struct alignas(sizeof(Tin) * kV) RowVec { Tin v[kV]; };
 
@@ -265,7 +269,11 @@ cs_sum_kernel(const Tin* __restrict__ Z, int64_t ld, int d, int64_t s, int ncol,
           for (int q = 0; q < kV; ++q) {
             double x = widen(z[u].v[q]);
             if (kCentre) x -= m[u][q];
-            acc[q] += sg[u] == 1 ? x : (sg[u] == -1 ? -x : (double)sg[u] * x);
+            if (sg[u] == 1 || sg[u] == -1)  // uniform over the warp
+              x = __hiloint2double(__double2hiint(x) ^ (sg[u] & 0x80000000), __double2loint(x));
+            else
+              x = scale_by(x, sg[u]);
+            acc[q] += x;
           }
         }
       }
