@@ -22,6 +22,7 @@
 // Each kernel returns at once when the device flag `done` is set, so the host
 // enqueues iterations in batches and reads the flag between batches.
 #include "plan.h"
+#include "small_dense.cuh"
 
 namespace gbcca {
 
@@ -517,6 +518,7 @@ struct LSArgs {
   double* ls_f;           // kNTrials trial values
   double* ls_L;           // kNTrials x 2 x kMaxK^2 trial factors
   int polar;              // 1: polar retraction (factors Gram(t)^{-1/2})
+  int fp64;               // FP64 plan
 };
 
 // Work area of one line-search trial (doubles): Gram_x, Gram_y, Cross, two
@@ -702,8 +704,8 @@ __device__ double ls_eval_polar(const LSArgs& a, const double* coef, double t, d
 }
 
 // Every trial step of the sequential Armijo rule is evaluated at once, one
-// CTA (one warp) per trial, so the FP64 work of the k x k Cholesky factors
-// is spread over kNTrials SMs instead of queueing on one SM's FP64 pipe:
+// CTA per trial, so the FP64 work of the k x k factors is spread over
+// kNTrials SMs instead of queueing on one SM's FP64 pipe:
 //   trial 0: t = 0 (the Armijo reference, at the point of this pass),
 //   trials 1 .. kMaxExpand + 1: t0 2^0 .. t0 2^kMaxExpand (t0 and its expansions),
 //   trials kMaxExpand + 2 ..: t0 2^-1 .. t0 2^-(kMaxLS - 1) (backtracking).
@@ -711,175 +713,284 @@ __device__ double ls_eval_polar(const LSArgs& a, const double* coef, double t, d
 // to finish applies the sequential rule (first accepted backtracking step; or
 // t0 and then doublings while f decreases and Armijo holds) to the stored
 // values, so the accepted step is exactly the one of the sequential search.
+//
+// QR retraction of FP32/BF16 plans: the Grams are formed at t straight from the pass Grams (their
+// lower triangles only), each view's four warps invert their Cholesky factor
+// (group_chol_inverse), and
+//   CCA  f = -sum_i mu_i sum_{a <= i} Lx^{-1}_ia (Cross(t) Ly^{-T})_ai,
+//   FDA  f = -1/2 sum_i mu_i |(Yhat W(t)) L^{-T}|_i^2,
+// one product per entry.  Bound by the latency of those dependent steps: with
+// a Cholesky by one warp and the triangular inverse a column per lane a
+// launch took 32 us at k = 10 (20 us of it in the factors, 5 us in the
+// decision, whose comparisons one lane made in turn).
 __device__ __forceinline__ double ls_trial_t(int i, double t0) {
   if (i == 0) return 0.0;
-  if (i <= kMaxExpand + 1) return ldexp(t0, i - 1);
-  return ldexp(t0, -(i - kMaxExpand - 1));
+  // t0 times an exact power of two
+  const int e = i <= kMaxExpand + 1 ? i - 1 : -(i - kMaxExpand - 1);
+  return t0 * __hiloint2double((1023 + e) << 20, 0);
 }
 
-__global__ void linesearch_kernel(LSArgs a) {
+// Coefficient matrices of a trial (kk each): Gram_v(t) = A + t B + t^2 C at 3 v
+// .. 3 v + 2, Cross(t) (FDA: S_B(t)) = X0 + t X1 + t^2 X2 at 6 .. 8.
+__device__ void ls_coefficients(const LSArgs& a, double* coef) {
+  DevState* st = a.st;
+  const int k = a.k, kk = k * k, k2 = 2 * k, NC = a.NC, tid = threadIdx.x;
+  for (int e = tid; e < kk; e += blockDim.x) {
+    const int r = e / k, c = e % k;
+    auto G = [&](int bi, int bj) { return a.Gram[(bi * k + r) * NC + bj * k + c]; };
+    for (int v = 0; v < a.nviews; ++v) {
+      const double* pg = a.phipart + v * 4 * kk;  // 2k x 2k
+      auto P = [&](int bi, int bj) { return pg[(bi * k + r) * k2 + bj * k + c]; };
+      const double lam = st->lam[v];
+      const int b0 = 2 * v;  // pass blocks of this view: [P_U, P_eta] or [Q_V, Q_eta]
+      coef[(3 * v + 0) * kk + e] = G(b0, b0) + lam * P(0, 0);
+      coef[(3 * v + 1) * kk + e] = G(b0, b0 + 1) + G(b0 + 1, b0) + lam * (P(0, 1) + P(1, 0));
+      coef[(3 * v + 2) * kk + e] = G(b0 + 1, b0 + 1) + lam * P(1, 1);
+    }
+    if (a.kind == kCCA) {
+      coef[6 * kk + e] = G(0, 2);
+      coef[7 * kk + e] = G(0, 3) + G(1, 2);
+      coef[8 * kk + e] = G(1, 3);
+    } else {
+      // S_B(t) = (Yhat W + t Yhat eta)^T (Yhat W + t Yhat eta)
+      double s0 = 0, s1 = 0, s2 = 0;
+      for (int cl = 0; cl < a.l; ++cl) {
+        const double wi = a.YPhi[cl * k2 + r], wj = a.YPhi[cl * k2 + c];
+        const double ei = a.YPhi[cl * k2 + k + r], ej = a.YPhi[cl * k2 + k + c];
+        s0 += wi * wj;
+        s1 += wi * ej + ei * wj;
+        s2 += ei * ej;
+      }
+      coef[6 * kk + e] = s0;
+      coef[7 * kk + e] = s1;
+      coef[8 * kk + e] = s2;
+    }
+  }
+  __syncthreads();
+}
+
+// Trials from the coefficient matrices: the polar retraction, and the QR
+// retraction of FP64 plans (one warp per factor; the iterations of an FP64
+// plan amplify a change of rounding here, so the order of its sums stays).
+__device__ double ls_trial_coef(const LSArgs& a, double* lsm, double t, const double* mu, double* Lout) {
+  const int k = a.k, kk = k * k, tid = threadIdx.x;
+  double* coef = lsm;           // 9 kk
+  double* w = coef + 9 * kk;    // ls_work_doubles(k)
+  ls_coefficients(a, coef);
+  const double* Li = w + 3 * kk;  // view 1 (FDA: the only view)
+  const double* Lt = w + 4 * kk;
+  double f = 0.0;
+  if (a.polar) {
+    f = ls_eval_polar(a, coef, t, w, mu);
+    for (int e = tid; e < kk; e += blockDim.x) {  // symmetric factors
+      Lout[e] = a.kind == kCCA ? Lt[e] : Li[e];
+      Lout[kMaxK * kMaxK + e] = Li[e];
+    }
+    return f;
+  }
+  if (a.kind == kCCA) {
+    f = ls_eval_cca_cta(a, coef, t, w, mu);
+  } else {
+    if (tid < 32) f = ls_eval(a, coef, t, w, mu);
+    __syncthreads();
+    Lt = Li;
+  }
+  for (int e = tid; e < kk; e += blockDim.x) {
+    const int r = e / k, c = e - r * k;
+    Lout[e] = Lt[c * k + r];
+    if (a.kind == kCCA) Lout[kMaxK * kMaxK + e] = Li[c * k + r];
+  }
+  return f;
+}
+
+// QR retraction in Cholesky form: f(t) and L_v(t)^{-T}.
+__device__ double ls_trial_qr(const LSArgs& a, double* lsm, double t, const double* mu, double* Lout) {
+  const int k = a.k, kk = k * k, k2 = 2 * k, NC = a.NC, tid = threadIdx.x;
+  double* Cm = lsm;                                   // CCA: Cross(t), kk; FDA: Yhat W(t), l x k
+  double* A = Cm + max(kk, a.l * k);                  // per view kk
+  double* Li = A + 2 * kk;                            // per view kk
+  double* rs = Li + 2 * kk;                           // per view kMaxK
+  __shared__ int s_ok[2];
+  __shared__ double s_part[8];
+  const int v = tid >> 7, g = tid & 127;  // threads 0 .. 127: view 0, the rest view 1
+  const bool cca = a.kind == kCCA;
+  if (v < a.nviews) {
+    const double lam = a.st->lam[v];
+    const double* pg = a.phipart + v * 4 * kk;
+    const int b0 = 2 * v;  // pass blocks of this view: [P_U, P_eta] or [Q_V, Q_eta]
+    for (int e = g; e < k * (k + 1) / 2; e += 128) {
+      int r = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+      while ((r + 1) * (r + 2) / 2 <= e) ++r;
+      while (r * (r + 1) / 2 > e) --r;
+      const int c = e - r * (r + 1) / 2;
+      auto G = [&](int bi, int bj) { return a.Gram[(bi * k + r) * NC + bj * k + c]; };
+      auto P = [&](int bi, int bj) { return pg[(bi * k + r) * k2 + bj * k + c]; };
+      const double c0 = G(b0, b0) + lam * P(0, 0);
+      const double c1 = G(b0, b0 + 1) + G(b0 + 1, b0) + lam * (P(0, 1) + P(1, 0));
+      const double c2 = G(b0 + 1, b0 + 1) + lam * P(1, 1);
+      A[v * kk + r * k + c] = c0 + t * (c1 + t * c2);
+    }
+  }
+  if (cca) {
+    for (int e = tid; e < kk; e += blockDim.x) {
+      const int r = e / k, c = e - r * k;
+      auto G = [&](int bi, int bj) { return a.Gram[(bi * k + r) * NC + bj * k + c]; };
+      Cm[e] = G(0, 2) + t * ((G(0, 3) + G(1, 2)) + t * G(1, 3));
+    }
+  } else {
+    for (int e = tid; e < a.l * k; e += blockDim.x) {
+      const int cl = e / k, c = e - cl * k;
+      Cm[e] = a.YPhi[cl * k2 + c] + t * a.YPhi[cl * k2 + k + c];
+    }
+  }
+  if (v < a.nviews) {
+    const bool ok = group_chol_inverse<128>(A + v * kk, Li + v * kk, rs + v * kMaxK, k, g, 1 + v);
+    if (g == 0) s_ok[v] = ok;
+  }
+  __syncthreads();
+  double part = 0.0;
+  if (cca) {
+    // entries (i, c), c <= i: mu_i Lx^{-1}_ic (Cross Ly^{-T})_ci
+    const double *Lx = Li, *Ly = Li + kk;
+    for (int e = tid; e < k * (k + 1) / 2; e += blockDim.x) {
+      int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+      while ((i + 1) * (i + 2) / 2 <= e) ++i;
+      while (i * (i + 1) / 2 > e) --i;
+      const int c = e - i * (i + 1) / 2;
+      double z = 0.0;
+      for (int b = 0; b <= i; ++b) z += Cm[c * k + b] * Ly[i * k + b];
+      part += mu[i] * Lx[i * k + c] * z;
+    }
+  } else {
+    for (int e = tid; e < a.l * k; e += blockDim.x) {
+      const int cl = e / k, i = e - cl * k;
+      double z = 0.0;
+      for (int b = 0; b <= i; ++b) z += Cm[cl * k + b] * Li[i * k + b];
+      part += 0.5 * mu[i] * (z * z);
+    }
+  }
+  part = warp_sum(part);
+  if ((tid & 31) == 0) s_part[tid >> 5] = part;
+  for (int e = tid; e < kk; e += blockDim.x) {
+    const int r = e / k, c = e - r * k;
+    Lout[e] = Li[c * k + r];
+    if (cca) Lout[kMaxK * kMaxK + e] = Li[kk + c * k + r];
+  }
+  __syncthreads();
+  double f = 0.0;
+  if (tid == 0) {
+    for (int q = 0; q < 8; ++q) f -= s_part[q];
+    if (!s_ok[0] || (cca && !s_ok[1]) || !(f == f)) f = INFINITY;
+  }
+  return f;  // (thread 0)
+}
+
+inline size_t ls_smem(int k, int l) {
+  const size_t kk = (size_t)k * k;
+  const size_t qr = std::max<size_t>(kk, (size_t)l * k) + 4 * kk + 2 * kMaxK;
+  return sizeof(double) * std::max(qr, 9 * kk + (size_t)ls_work_doubles(k));
+}
+
+__global__ void __launch_bounds__(256) linesearch_kernel(LSArgs a) {
   DevState* st = a.st;
   if (st->done) return;
   extern __shared__ double lsm[];
   const int k = a.k, kk = k * k, k2 = 2 * k;
   const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
   const bool zero_step = st->force_zero_step != 0;
-  double* coef = lsm;                       // 9 kk
-  double* phig = coef + 9 * kk;             // 2 views x 4 kk
-  double* w = phig + 8 * kk;                // ls_work_doubles(k)
+  const double t0 = st->t0, df = st->df;
   __shared__ double mu_s[kMaxK];
-  __shared__ int last;
+  __shared__ int last, s_acc;
   if (!zero_step || i == 0) {
-    // the whole CTA loads (several loads in flight per thread); warp 0 then
-    // evaluates the trial
     if (tid < k) mu_s[tid] = st->mu[tid];
-    for (int e = tid; e < a.nviews * 4 * kk; e += blockDim.x) phig[e] = a.phipart[e];
     __syncthreads();
-    // coefficient matrices: Gram_v(t) = A + t B + t^2 C, Cross(t) = X0 + t X1 + t^2 X2
-    const int NC = a.NC;
-    for (int e = tid; e < kk; e += blockDim.x) {
-      const int r = e / k, c = e % k;
-      auto G = [&](int bi, int bj) { return a.Gram[(bi * k + r) * NC + bj * k + c]; };
-      for (int v = 0; v < a.nviews; ++v) {
-        const double* pg = phig + v * 4 * kk;  // 2k x 2k
-        auto P = [&](int bi, int bj) { return pg[(bi * k + r) * k2 + bj * k + c]; };
-        const double lam = st->lam[v];
-        const int b0 = 2 * v;  // pass blocks of this view: [P_U, P_eta] or [Q_V, Q_eta]
-        coef[(3 * v + 0) * kk + e] = G(b0, b0) + lam * P(0, 0);
-        coef[(3 * v + 1) * kk + e] = G(b0, b0 + 1) + G(b0 + 1, b0) + lam * (P(0, 1) + P(1, 0));
-        coef[(3 * v + 2) * kk + e] = G(b0 + 1, b0 + 1) + lam * P(1, 1);
-      }
-      if (a.kind == kCCA) {
-        coef[6 * kk + e] = G(0, 2);
-        coef[7 * kk + e] = G(0, 3) + G(1, 2);
-        coef[8 * kk + e] = G(1, 3);
-      } else {
-        // S_B(t) = (Yhat W + t Yhat eta)^T (Yhat W + t Yhat eta)
-        double s0 = 0, s1 = 0, s2 = 0;
-        for (int cl = 0; cl < a.l; ++cl) {
-          const double wi = a.YPhi[cl * k2 + r], wj = a.YPhi[cl * k2 + c];
-          const double ei = a.YPhi[cl * k2 + k + r], ej = a.YPhi[cl * k2 + k + c];
-          s0 += wi * wj;
-          s1 += wi * ej + ei * wj;
-          s2 += ei * ej;
-        }
-        coef[6 * kk + e] = s0;
-        coef[7 * kk + e] = s1;
-        coef[8 * kk + e] = s2;
-      }
-    }
-    __syncthreads();
-    const double t = ls_trial_t(i, st->t0);
+    const double t = ls_trial_t(i, t0);
     // factors L_v(t)^{-T} of this trial (row-major), kept for the decision
     double* Lout = a.ls_L + (int64_t)i * 2 * kMaxK * kMaxK;
-    if (a.polar) {
-      const double f = ls_eval_polar(a, coef, t, w, mu_s);
-      const double* Fy = w + 3 * kk;
-      const double* Fx = a.kind == kCCA ? w + 4 * kk : Fy;
-      for (int e = tid; e < kk; e += blockDim.x) {
-        Lout[e] = Fx[e];
-        Lout[kMaxK * kMaxK + e] = Fy[e];
-      }
-      if (tid == 0) a.ls_f[i] = f;
-    } else if (a.kind == kCCA) {
-      const double f = ls_eval_cca_cta(a, coef, t, w, mu_s);
-      const double* Li = w + 3 * kk;
-      const double* Lt = w + 4 * kk;
-      for (int e = tid; e < kk; e += blockDim.x) {
-        const int r = e / k, c = e % k;
-        Lout[e] = Lt[c * k + r];
-        Lout[kMaxK * kMaxK + e] = Li[c * k + r];
-      }
-      if (tid == 0) a.ls_f[i] = f;
-    } else if (tid < 32) {
-      const double f = ls_eval(a, coef, t, w, mu_s);
-      const double* Li = w + 3 * kk;
-      for (int e = lane; e < kk; e += 32) {
-        const int r = e / k, c = e % k;
-        Lout[e] = Li[c * k + r];
-      }
-      if (lane == 0) a.ls_f[i] = f;
-    }
+    const double f = a.polar || a.fp64 ? ls_trial_coef(a, lsm, t, mu_s, Lout) : ls_trial_qr(a, lsm, t, mu_s, Lout);
+    if (tid == 0) a.ls_f[i] = f;
   }
-  // the last CTA to finish decides (warp 0 of it)
+  // the last CTA to finish decides
   __threadfence();
   __syncthreads();
   if (tid == 0) last = atomicAdd(&st->ls_count, 1) == (int)gridDim.x - 1;
   __syncthreads();
-  if (!last || tid >= 32) return;
+  if (!last) return;
   __threadfence();
-  if (lane == 0) st->ls_count = 0;
-  // every trial value at once from L2 (two per lane; the other CTAs' stores
-  // are visible there after their fences and atomics), then the sequential
-  // rule on warp shuffles: all lanes take the same decisions
-  static_assert(kNTrials <= 64, "two trial values per lane");
-  const double fva = lane < (int)gridDim.x ? __ldcg(&a.ls_f[lane]) : 0.0;
-  const double fvb = lane + 32 < (int)gridDim.x ? __ldcg(&a.ls_f[lane + 32]) : 0.0;
-  auto fv = [&](int e) {
-    const double x = __shfl_sync(0xffffffffu, fva, e & 31);
-    const double y = __shfl_sync(0xffffffffu, fvb, e & 31);
-    return e < 32 ? x : y;
-  };
-  const double t0 = st->t0, df = st->df;
-  const double f0 = fv(0);
-  int acc = -1, trials = 1;
-  if (zero_step) {
-    acc = 0;
-  } else if (fv(1) <= f0 + kC1 * t0 * df) {
-    acc = 1;
-    trials = 2;
-    for (int e = 2; e <= kMaxExpand + 1; ++e) {
-      const double te = ls_trial_t(e, t0);
-      ++trials;
-      const double fe = fv(e);
-      if (fe < fv(acc) && fe <= f0 + kC1 * te * df)
+  if (tid < 32) {
+    // every trial value at once from L2 (two per lane; the other CTAs' stores
+    // are visible there after their fences and atomics); each lane tests its
+    // own trials, and the sequential rule is read off the ballots
+    static_assert(kNTrials <= 64, "two trial values per lane");
+    const int n = (int)gridDim.x;
+    const double fa = lane < n ? __ldcg(&a.ls_f[lane]) : INFINITY;
+    const double fb = lane + 32 < n ? __ldcg(&a.ls_f[lane + 32]) : INFINITY;
+    const double f0 = __shfl_sync(0xffffffffu, fa, 0);
+    const double prev = __shfl_up_sync(0xffffffffu, fa, 1);  // trial e - 1
+    const bool ok_a = fa <= f0 + kC1 * ls_trial_t(lane, t0) * df,
+               ok_b = fb <= f0 + kC1 * ls_trial_t(lane + 32, t0) * df;
+    const unsigned long long ok = (unsigned long long)__ballot_sync(0xffffffffu, ok_a && lane < n) |
+                                  ((unsigned long long)__ballot_sync(0xffffffffu, ok_b && lane + 32 < n) << 32);
+    const unsigned dec = __ballot_sync(0xffffffffu, fa < prev);
+    int acc = -1, trials = 1;
+    if (zero_step) {
+      acc = 0;
+    } else if (ok >> 1 & 1) {
+      acc = 1;  // then doublings while f decreases and Armijo holds
+      trials = 2;
+      for (int e = 2; e <= kMaxExpand + 1; ++e) {
+        ++trials;
+        if (!((ok >> e & 1) && (dec >> e & 1))) break;
         acc = e;
-      else
-        break;
+      }
+    } else {
+      const unsigned long long back = ok >> (kMaxExpand + 2) << (kMaxExpand + 2);
+      acc = back != 0 ? __ffsll((long long)back) - 1 : -1;
+      trials = 2 + (acc >= 0 ? acc : n - 1) - (kMaxExpand + 1);
     }
-  } else {
-    trials = 2;
-    for (int e = kMaxExpand + 2; e < (int)gridDim.x; ++e) {
-      ++trials;
-      if (fv(e) <= f0 + kC1 * ls_trial_t(e, t0) * df) {
-        acc = e;
-        break;
+    if (lane == 0) {
+      st->ls_count = 0;
+      s_acc = acc;
+      if (acc < 0) {
+        st->stalled = 1;
+        st->done = 1;
+        st->ls_trials = trials;
+      } else {
+        const double t = ls_trial_t(acc, t0);
+        st->t = t;
+        st->ls_trials = trials;
+        if (!zero_step) {
+          st->t_prev = t;
+          st->df_prev = df;
+          st->iter += 1;
+        }
       }
     }
-  }
-  if (acc < 0) {
-    if (lane == 0) {
-      st->stalled = 1;
-      st->done = 1;
-      st->ls_trials = trials;
+    if (acc >= 0) {
+      const double f_acc = __shfl_sync(0xffffffffu, acc < 32 ? fa : fb, acc & 31);
+      if (lane == 0) st->f = f_acc;
     }
-    return;
   }
+  __syncthreads();
+  const int acc = s_acc;
+  if (acc < 0) return;
   const double t = ls_trial_t(acc, t0);
-  const volatile double* L = a.ls_L + (int64_t)acc * 2 * kMaxK * kMaxK;
-  for (int e = lane; e < kk; e += 32) {
-    st->Linv[0][e] = L[e];
-    if (a.kind == kCCA) st->Linv[1][e] = L[kMaxK * kMaxK + e];
+  const double* L = a.ls_L + (int64_t)acc * 2 * kMaxK * kMaxK;
+  double* Ls = lsm;  // kk
+  for (int e = tid; e < kk; e += blockDim.x) {
+    const double x = __ldcg(L + e);
+    Ls[e] = x;
+    st->Linv[0][e] = x;
+    if (a.kind == kCCA) st->Linv[1][e] = __ldcg(L + kMaxK * kMaxK + e);
   }
-  __syncwarp();
   if (a.kind == kLDA) {
     // YW+ = (Yhat W + t Yhat eta) L^{-T}
-    for (int e = lane; e < a.l * k; e += 32) {
-      const int cl = e / k, c = e % k;
+    __syncthreads();
+    for (int e = tid; e < a.l * k; e += blockDim.x) {
+      const int cl = e / k, c = e - cl * k;
       double s = 0;
-      for (int q = 0; q < k; ++q) s += (a.YPhi[cl * k2 + q] + t * a.YPhi[cl * k2 + k + q]) * st->Linv[0][q * k + c];
+      for (int q = 0; q < k; ++q) s += (a.YPhi[cl * k2 + q] + t * a.YPhi[cl * k2 + k + q]) * Ls[q * k + c];
       st->YW[e] = s;
-    }
-  }
-  const double f_acc = fv(acc);  // (all lanes: a shuffle)
-  if (lane == 0) {
-    st->t = t;
-    st->f = f_acc;
-    st->ls_trials = trials;
-    if (!zero_step) {
-      st->t_prev = t;
-      st->df_prev = st->df;
-      st->iter += 1;
     }
   }
 }
@@ -999,6 +1110,138 @@ __device__ void blk_sum(double (&v)[NV], double* red) {
   __syncthreads();
 }
 
+// What the last CTA of a direction kernel does with the views' sums (called by
+// all its threads; `first` and `it` were read before any CTA could finish).
+// kIeee: divisions and square roots rounded to nearest (FP64 plans); else
+// reciprocals by rcp_nr / rsqrt_nr.
+template <bool kIeee>
+__device__ void direction_tail(const DirArgs& a, int first, int it) {
+  DevState* st = a.st;
+  // The last CTA: beta, slope and first trial step on one thread, gradient
+  // norm and the stopping tests on a thread of another warp.
+  const int tid = threadIdx.x;
+  if (tid != 0 && tid != 32) return;
+  __threadfence();
+  // every view's sums at once, from L2 (the other CTA's stores are visible
+  // there after its fence and our atomic), beside the state's scalars
+  double da[2][6];
+#pragma unroll
+  for (int w = 0; w < 2; ++w)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) da[w][q] = w < a.nviews ? __ldcg(&st->dacc[w][q]) : 0.0;
+  const double t_prev = st->t_prev, df_prev = st->df_prev, f_cur = st->f, t_cur = st->t;
+  const double gtol = st->gtol, gn0_old = st->gn0;
+  auto sum = [&](int q) { return a.nviews > 1 ? da[0][q] + da[1][q] : da[0][q]; };  // in view order
+  const double gg = sum(0);
+  if (tid == 0) {
+    const double g_Tg = sum(1), Te_g = sum(2), Te_Tg = sum(3), dfg = sum(4), dfTe = sum(5);
+    double beta = 0;
+    if (!first) {
+      const double num = gg - g_Tg, den = Te_g - Te_Tg;
+      beta = den != 0.0 ? fmax(0.0, kIeee ? num / den : num * rcp_nr(den)) : 0.0;
+    }
+    double df = -dfg + beta * dfTe;
+    if (df >= 0) {
+      beta = 0;
+      df = -gg;
+    }
+    if (kIeee || !(gg > 0.0)) st->t0 = first ? 1.0 / sqrt(fmax(gg, 0.0)) : t_prev * df_prev / df;
+    else st->t0 = first ? rsqrt_nr(gg) : t_prev * df_prev * rcp_nr(df);
+    st->beta = beta;
+    st->df = df;
+    st->dcount = 0;
+    st->force_zero_step = 0;
+    st->qsyl_valid = 1;
+  } else {
+    const double gn = !kIeee && gg > 0.0 ? gg * rsqrt_nr(gg) : sqrt(fmax(gg, 0.0));
+    const double gn0 = first ? gn : gn0_old;
+    if (first) st->gn0 = gn;
+    st->gn = gn;
+    if (a.history != nullptr && it <= a.max_iter) {
+      a.history[3 * it + 0] = f_cur;
+      a.history[3 * it + 1] = gn;
+      a.history[3 * it + 2] = first ? 0.0 : t_cur;
+    }
+    st->first = 0;
+    if (!(gn > gtol * gn0)) {
+      st->done = 1;
+      st->status = GBCCA_OK;
+    } else if (it >= a.max_iter) {
+      st->done = 1;
+      st->status = GBCCA_ERR_MAXITER;
+    }
+  }
+}
+
+// Shared memory of the direction kernel (doubles): this view's cross Gram,
+// S, sym(X00), A S, reduction scratch, and the FP32 working area of the
+// eigendecomposition and the rotated blocks.
+inline size_t direction_smem(int k) {
+  const size_t kk = (size_t)k * k;
+  return sizeof(double) * (16 * kk + 3 * kk + kk + 3 * kk + 64) + sizeof(float) * (11 * kk + kMaxK);
+}
+
+// S_r = Q ((Q^T RHS_r Q) ./ (lam_i + lam_j)) Q^T for the three symmetric
+// right-hand sides RHS_r (k x k each, in T2), all in R; the result, symmetric
+// by construction (i <= j computed, mirrored), goes to `out(e, value)` for
+// every entry e of the three blocks.  T, T2: 3 kk scratch.  Two products of
+// the four need every entry, two only the upper triangle.
+template <typename R, typename F>
+__device__ __forceinline__ void sylvester_apply(const R* Q, const R* lam, R* T, R* T2, int k, F out) {
+  const int kk = k * k, nf = 3 * kk, kt = k * (k + 1) / 2, nu = 3 * kt;
+  auto full = [&](int e, int& r, int& i, int& j) {
+    r = e / kk;
+    const int f = e - r * kk;
+    i = f / k;
+    j = f - i * k;
+  };
+  auto upper = [&](int e, int& r, int& i, int& j) {  // e = r kt + j (j + 1) / 2 + i, i <= j
+    r = e / kt;
+    const int f = e - r * kt;
+    j = (int)((sqrtf(8.f * (float)f + 1.f) - 1.f) * 0.5f);
+    if ((j + 1) * (j + 2) / 2 <= f) ++j;
+    if (j * (j + 1) / 2 > f) --j;
+    i = f - j * (j + 1) / 2;
+  };
+  for (int e = threadIdx.x; e < nf; e += blockDim.x) {  // T = Q^T RHS
+    int r, i, j;
+    full(e, r, i, j);
+    R sum = 0;
+#pragma unroll 5
+    for (int q = 0; q < k; ++q) sum += Q[q * k + i] * T2[r * kk + q * k + j];
+    T[e] = sum;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nu; e += blockDim.x) {  // T2 = (T Q) ./ (lam_i + lam_j)
+    int r, i, j;
+    upper(e, r, i, j);
+    R sum = 0;
+#pragma unroll 5
+    for (int q = 0; q < k; ++q) sum += T[r * kk + i * k + q] * Q[q * k + j];
+    sum /= lam[i] + lam[j];
+    T2[r * kk + i * k + j] = sum;
+    T2[r * kk + j * k + i] = sum;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nf; e += blockDim.x) {  // T = Q T2
+    int r, i, j;
+    full(e, r, i, j);
+    R sum = 0;
+#pragma unroll 5
+    for (int q = 0; q < k; ++q) sum += Q[i * k + q] * T2[r * kk + q * k + j];
+    T[e] = sum;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nu; e += blockDim.x) {  // S = T Q^T
+    int r, i, j;
+    upper(e, r, i, j);
+    R sum = 0;
+#pragma unroll 5
+    for (int q = 0; q < k; ++q) sum += T[r * kk + i * k + q] * Q[j * k + q];
+    out(r, i, j, sum);
+  }
+}
+
 // Per factor: X = [Wn, xi, eta, g]^T [BU, egrad, M eta, M g] (4k x 4k blocks
 // X[a][b]).  The projection of Table 1 needs S with A S + S A = C + C^T for
 // A = sym(X[0][0]) = U^T B M^{-1} B U and C = X[a][0]^T (a = 1: gradient,
@@ -1006,17 +1249,185 @@ __device__ void blk_sum(double (&v)[NV], double* red) {
 // S = Q ((Q^T (C + C^T) Q) ./ (lam_i + lam_j)) Q^T.  Inner products in g of
 // u = L_a - Wn Su with M w = R_b - BU Sw expand into
 //   tr X[a][b] - tr(X[a][0] Sw) - tr(Su^T X[0][b]) + tr(Su^T X[0][0] Sw).
-template <typename R>
-__global__ void direction_kernel(DirArgs a) {
+//
+// FP32/BF16 plans (FP64 plans: direction64_kernel): the eigendecomposition and
+// the rotated products run in FP32 (A rotated into the previous iteration's
+// eigenbasis first, from scratch every 32 iterations so that the basis does
+// not drift from orthogonality), and one FP64 residual corrects S:
+// E = RHS - (A S + S A), S += the FP32 solve of E.
+//
+// Bound by dependent small steps on one SM.  With an in-place Jacobi by one
+// warp (53 us of it), divisions and square roots on one thread (11 us) and
+// every product over all entries a launch took 64 us at k = 10.
+__global__ void __launch_bounds__(256) direction_kernel(DirArgs a) {
   DevState* st = a.st;
   if (st->done) return;
   extern __shared__ double dsm[];
   const int k = a.k, kk = k * k, k4 = 4 * k;
-  double* X = dsm;                 // 16 kk per view (FP64 cross Gram)
-  double* Y = X + 2 * 16 * kk;     // 2 kk: X00 Sg, X00 So (FP64), then 3 kk: S (FP64)
+  const int tid = threadIdx.x;
+  double* X = dsm;            // 16 kk (cross Gram of this view)
+  double* Sd = X + 16 * kk;   // 3 kk: S_g, S_e, S_o
+  double* A64 = Sd + 3 * kk;  // kk
+  double* M = A64 + kk;       // 3 kk: A S
+  double* red = M + 3 * kk;   // 64
+  double* work = red + 64;    // 11 kk + kMaxK floats
+  // one CTA per view; the last CTA to finish combines the views' sums
+  const int v = blockIdx.x;
+  const double* Q0g = st->Qsyl[v];
+  // (read here: the last CTA's two threads below write the state separately)
+  const int first = st->first, it = st->iter;
+  const bool warm = st->qsyl_valid != 0 && (it & 31) != 0;
+  float* fA = reinterpret_cast<float*>(work);
+  float* fA2 = fA + kk;
+  float* fQ = fA2 + kk;
+  float* fQ2 = fQ + kk;
+  float* Q0 = fQ2 + kk;
+  float* fl = Q0 + kk;       // kMaxK eigenvalues
+  float* T = fl + kMaxK;     // 3 kk
+  float* T2 = T + 3 * kk;    // 3 kk
+  for (int e = tid; e < kk; e += blockDim.x) Q0[e] = warm ? (float)Q0g[e] : 0.f;
+  sum_blocks(a.crosspart + (int64_t)v * a.nblk * 16 * kk, a.nblk, 16 * kk, X);
+  auto XB = [&](int ab, int bb, int i, int j) { return X[(ab * k + i) * k4 + bb * k + j]; };
+  for (int e = tid; e < kk; e += blockDim.x) {
+    const int i = e / k, j = e - i * k;
+    const double x = 0.5 * (XB(0, 0, i, j) + XB(0, 0, j, i));
+    A64[e] = x;
+    T2[e] = (float)x;
+  }
+  __syncthreads();
+  if (warm) {
+    for (int e = tid; e < kk; e += blockDim.x) {  // T = A Q0
+      const int i = e / k, j = e - i * k;
+      float sum = 0;
+#pragma unroll 5
+      for (int q = 0; q < k; ++q) sum += T2[i * k + q] * Q0[q * k + j];
+      T[e] = sum;
+    }
+    __syncthreads();
+    for (int e = tid; e < kk; e += blockDim.x) {  // A' = Q0^T T
+      const int i = e / k, j = e - i * k;
+      float sum = 0;
+#pragma unroll 5
+      for (int q = 0; q < k; ++q) sum += Q0[q * k + i] * T[q * k + j];
+      fA[e] = sum;
+    }
+  } else {
+    for (int e = tid; e < kk; e += blockDim.x) fA[e] = T2[e];
+  }
+  blk_jacobi_f32(fA, fA2, fQ, fQ2, k);  // A' = J diag(lam) J^T, J in fQ (synchronizes first)
+  if (warm) {
+    for (int e = tid; e < kk; e += blockDim.x) {  // Q = Q0 J
+      const int i = e / k, j = e - i * k;
+      float sum = 0;
+#pragma unroll 5
+      for (int q = 0; q < k; ++q) sum += Q0[i * k + q] * fQ[q * k + j];
+      fQ2[e] = sum;
+    }
+  } else {
+    for (int e = tid; e < kk; e += blockDim.x) fQ2[e] = fQ[e];
+  }
+  float* Q = fQ2;
+  if (tid < k) fl[tid] = fA[tid * k + tid];
+  // right-hand sides C_r + C_r^T, C_r = X[r+1][0]^T
+  for (int e = tid; e < 3 * kk; e += blockDim.x) {
+    const int r = e / kk, f = e - r * kk, i = f / k, j = f - i * k;
+    T2[e] = (float)(XB(r + 1, 0, i, j) + XB(r + 1, 0, j, i));
+  }
+  __syncthreads();
+  for (int e = tid; e < kk; e += blockDim.x) st->Qsyl[v][e] = (double)Q[e];
+  for (int pass = 0; pass < 2; ++pass) {
+    sylvester_apply<float>(Q, fl, T, T2, k, [&](int r, int i, int j, float x) {
+      const int e = r * kk + i * k + j;
+      const double s = (pass == 0 ? 0.0 : Sd[e]) + (double)x;
+      Sd[e] = s;
+      Sd[r * kk + j * k + i] = s;
+    });
+    __syncthreads();
+    if (pass == 1) break;
+    // residual in FP64: M = A S, E = RHS - (M + M^T) (S symmetric)
+    for (int e = tid; e < 3 * kk; e += blockDim.x) {
+      const int r = e / kk, f = e - r * kk, i = f / k, j = f - i * k;
+      double sum = 0;
+#pragma unroll 5
+      for (int q = 0; q < k; ++q) sum += A64[i * k + q] * Sd[r * kk + q * k + j];
+      M[e] = sum;
+    }
+    __syncthreads();
+    for (int e = tid; e < 3 * kk; e += blockDim.x) {
+      const int r = e / kk, f = e - r * kk, i = f / k, j = f - i * k;
+      T2[e] = (float)((XB(r + 1, 0, i, j) + XB(r + 1, 0, j, i)) - (M[e] + M[r * kk + j * k + i]));
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < 3 * kk; e += blockDim.x) st->S[v][e / kk][e % kk] = Sd[e];
+  double acc[6] = {0, 0, 0, 0, 0, 0};  // gg, g_Tg, Te_g, Te_Tg, dfg, dfTe
+  // Items (w, i, j): w = 0 the terms with S_g on the right, w = 1 those with
+  // S_o; Y_ij = (X00 S_w)_ij, and with S symmetric
+  //   tr X[a][b] - tr(X[a][0] S_w) - tr(S_u X[0][b]) + tr(S_u X00 S_w)
+  //   = tr X[a][b] + sum_ij S_u (Y - X[0][b]) - X[a][0] S_w.
+  for (int e = tid; e < 2 * kk; e += blockDim.x) {
+    const int w = e / kk, f = e - w * kk, i = f / k, j = f - i * k;
+    const double* Sw = Sd + (w == 0 ? 0 : 2 * kk);
+    const double sg = Sd[f], se = Sd[kk + f], sw = Sw[f];
+    const double x0b = XB(0, w == 0 ? 1 : 3, i, j);
+    double y = 0;
+#pragma unroll 5
+    for (int q = 0; q < k; ++q) y += XB(0, 0, i, q) * Sw[q * k + j];
+    const double p = y - x0b, x10 = XB(1, 0, i, j), x20 = XB(2, 0, i, j);
+    const double g0 = sg * p - x10 * sw, e0 = se * p - x20 * sw;
+    if (w == 0) {
+      acc[0] += g0;
+      acc[2] += e0;
+      acc[4] -= sg * x0b;
+      acc[5] -= se * x0b;
+    } else {
+      acc[1] += g0;
+      acc[3] += e0;
+    }
+  }
+  if (tid >= 256 - k) {  // the traces (by threads with fewer items)
+    const int i = 255 - tid;
+    const double x11 = XB(1, 1, i, i), x21 = XB(2, 1, i, i);
+    acc[0] += x11;
+    acc[1] += XB(1, 3, i, i);
+    acc[2] += x21;
+    acc[3] += XB(2, 3, i, i);
+    acc[4] += x11;
+    acc[5] += x21;
+  }
+  blk_sum<6>(acc, red);
+  __shared__ int last;
+  if (tid == 0) {
+    for (int q = 0; q < 6; ++q) st->dacc[v][q] = acc[q];
+    __threadfence();
+    last = atomicAdd(&st->dcount, 1) == a.nviews - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  direction_tail<false>(a, first, it);
+}
+
+inline size_t direction64_smem(int k) {
+  const size_t kk = (size_t)k * k;
+  return sizeof(double) * (16 * kk + 5 * kk + 100 + 64 + 11 * kk + kMaxK);
+}
+
+// The same for FP64 plans, in FP64 throughout (A warm-started from the previous
+// eigenbasis).  Their iterations amplify a change of rounding here by about
+// 1e7 over 40 iterations, so the order of every sum is part of the result.
+// 66 us at k = 5, 50 of it in the Jacobi rotations' divisions and square roots.
+__global__ void __launch_bounds__(256) direction64_kernel(DirArgs a) {
+  using R = double;
+  DevState* st = a.st;
+  if (st->done) return;
+  extern __shared__ double dsm[];
+  const int k = a.k, kk = k * k, k4 = 4 * k;
+  const int first = st->first, it = st->iter;
+  double* X = dsm;                 // 16 kk (this view's cross Gram)
+  double* Y = X + 16 * kk;     // 2 kk: X00 Sg, X00 So (FP64), then 3 kk: S (FP64)
   double* rot = Y + 5 * kk;        // 100
-  double* red = rot + 100;         // 6 x 256
-  R* A = reinterpret_cast<R*>(red + 6 * 256);  // kk
+  double* red = rot + 100;         // 64
+  R* A = red + 64;                 // kk
   R* Q = A + kk;                   // kk
   R* lam = Q + kk;                 // kMaxK
   R* T = lam + kMaxK;              // 3 kk
@@ -1024,10 +1435,10 @@ __global__ void direction_kernel(DirArgs a) {
   R* S = T2 + 3 * kk;              // 3 kk (this view's S_g, S_e, S_o)
   // one CTA per view; the last CTA to finish combines the views' sums
   const int v = blockIdx.x;
-  sum_blocks(a.crosspart + (int64_t)v * a.nblk * 16 * kk, a.nblk, 16 * kk, X + v * 16 * kk);
+  sum_blocks(a.crosspart + (int64_t)v * a.nblk * 16 * kk, a.nblk, 16 * kk, X);
   double acc[6] = {0, 0, 0, 0, 0, 0};  // gg, g_Tg, Te_g, Te_Tg, dfg, dfTe
   {
-    const double* Xv = X + v * 16 * kk;
+    const double* Xv = X;
     auto XB = [&](int ab, int bb, int i, int j) { return Xv[(ab * k + i) * k4 + bb * k + j]; };
     // warm start: rotate A into the previous iteration's eigenbasis Q0 (A
     // changes little between iterations, so few Jacobi sweeps remain)
@@ -1075,18 +1486,14 @@ __global__ void direction_kernel(DirArgs a) {
     __syncthreads();
     // Sylvester solves for the three right-hand sides (C_r + C_r^T,
     // C_r = X[r+1][0]^T) with A = Q diag(lam) Q^T: S_r = Q ((Q^T RHS Q) ./
-    // (lam_i + lam_j)) Q^T in R arithmetic.  With R = float one FP64
-    // residual correction follows: E = RHS - (A S + S A) in FP64, S += the
-    // R-arithmetic solve of A dS + dS A = E.
+    // (lam_i + lam_j)) Q^T.
     double* Sd = Y + 2 * kk;  // 3 kk doubles
-    double* A64 = Y;          // sym(X00) in FP64 for the residual (Y is free until the end)
     for (int e = threadIdx.x; e < 3 * kk; e += blockDim.x) {
       int r = e / kk, f = e % kk, i = f / k, j = f % k;
       T2[e] = R(XB(r + 1, 0, i, j) + XB(r + 1, 0, j, i));
-      if (r == 0) A64[f] = 0.5 * (XB(0, 0, i, j) + XB(0, 0, j, i));
     }
     __syncthreads();
-    for (int pass = 0; pass < (sizeof(R) == 8 ? 1 : 2); ++pass) {
+    {
       // T = Q^T RHS ; T2 = (T Q) ./ (lam_i + lam_j) ; T = Q T2 ; S = T Q^T
       for (int e = threadIdx.x; e < 3 * kk; e += blockDim.x) {
         int r = e / kk, f = e % kk, i = f / k, j = f % k;
@@ -1113,24 +1520,11 @@ __global__ void direction_kernel(DirArgs a) {
         int r = e / kk, f = e % kk, i = f / k, j = f % k;
         R sum = 0;
         for (int q = 0; q < k; ++q) sum += T[r * kk + i * k + q] * Q[j * k + q];
-        Sd[e] = (pass == 0 ? 0.0 : Sd[e]) + (double)sum;
+        Sd[e] = sum;
       }
       __syncthreads();
-      if (sizeof(R) == 8) break;
-      if (pass == 0) {
-        // residual in FP64: E = RHS - (A S + S A), A = sym(X00)
-        for (int e = threadIdx.x; e < 3 * kk; e += blockDim.x) {
-          int r = e / kk, f = e % kk, i = f / k, j = f % k;
-          const double* Sr = Sd + r * kk;
-          double sum = XB(r + 1, 0, i, j) + XB(r + 1, 0, j, i);
-          for (int q = 0; q < k; ++q) sum -= A64[i * k + q] * Sr[q * k + j] + Sr[i * k + q] * A64[q * k + j];
-          T2[e] = R(sum);
-        }
-        __syncthreads();
-      }
     }
     for (int e = threadIdx.x; e < 3 * kk; e += blockDim.x) {
-      S[e] = R(Sd[e]);
       st->S[v][e / kk][e % kk] = Sd[e];
     }
     __syncthreads();
@@ -1172,65 +1566,7 @@ __global__ void direction_kernel(DirArgs a) {
   }
   __syncthreads();
   if (!last) return;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    // every view's sums at once, from L2 (the other CTA's stores are visible
-    // there after its fence and our atomic)
-    double da[2][6];
-#pragma unroll
-    for (int w = 0; w < 2; ++w)
-#pragma unroll
-      for (int q = 0; q < 6; ++q) da[w][q] = w < a.nviews ? __ldcg(&st->dacc[w][q]) : 0.0;
-    for (int q = 0; q < 6; ++q) {
-      acc[q] = 0;
-      for (int w = 0; w < a.nviews; ++w) acc[q] += da[w][q];  // view order: deterministic
-    }
-    st->dcount = 0;
-  }
-  const double gg = acc[0], g_Tg = acc[1], Te_g = acc[2], Te_Tg = acc[3], dfg = acc[4], dfTe = acc[5];
-  if (threadIdx.x == 0) {
-    // the state's scalars in one batch of loads (each would otherwise wait
-    // for the stores before it)
-    const int first = st->first, it = st->iter;
-    const double t_prev = st->t_prev, df_prev = st->df_prev, f_cur = st->f, t_cur = st->t;
-    const double gtol = st->gtol, gn0_old = st->gn0;
-    double beta = 0;
-    if (!first) {
-      double num = gg - g_Tg, den = Te_g - Te_Tg;
-      beta = den != 0.0 ? fmax(0.0, num / den) : 0.0;
-    }
-    double df = -dfg + beta * dfTe;
-    if (df >= 0) {
-      beta = 0;
-      df = -gg;
-    }
-    double gn = sqrt(fmax(gg, 0.0));
-    const double gn0 = first ? gn : gn0_old;
-    if (first) {
-      st->gn0 = gn;
-      st->t0 = 1.0 / gn;
-    } else {
-      st->t0 = t_prev * df_prev / df;
-    }
-    st->beta = beta;
-    st->df = df;
-    st->gn = gn;
-    if (a.history != nullptr && it <= a.max_iter) {
-      a.history[3 * it + 0] = f_cur;
-      a.history[3 * it + 1] = gn;
-      a.history[3 * it + 2] = first ? 0.0 : t_cur;
-    }
-    st->first = 0;
-    st->force_zero_step = 0;
-    st->qsyl_valid = 1;
-    if (!(gn > gtol * gn0)) {
-      st->done = 1;
-      st->status = GBCCA_OK;
-    } else if (it >= a.max_iter) {
-      st->done = 1;
-      st->status = GBCCA_ERR_MAXITER;
-    }
-  }
+  direction_tail<true>(a, first, it);
 }
 
 // ========================================================== new direction
@@ -1791,7 +2127,7 @@ int thin_blocks(const Plan& p) {
 // Everything of one iteration after its data pass (the pass outputs G and
 // Gram are in place).
 int iteration_post(Plan& p, bool low, cudaStream_t st) {
-  const int k = p.k, kk = k * k;
+  const int k = p.k;
   const int* done = &p.st->done;
   // the Grams of Phi: formed by the tensor-core pass beside its own, else here
   const bool need_phi = !p.phired_ready, need_y = p.kind == kLDA;
@@ -1856,7 +2192,8 @@ int iteration_post(Plan& p, bool low, cudaStream_t st) {
     a.ls_f = p.ls_f;
     a.ls_L = p.ls_L;
     a.polar = p.opt.retraction == 1 ? 1 : 0;
-    size_t smem = sizeof(double) * (9 * kk + 8 * kk + ls_work_doubles(k));
+    a.fp64 = low ? 0 : 1;
+    const size_t smem = ls_smem(k, p.l);
     GB_CUDA(cudaFuncSetAttribute(linesearch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     linesearch_kernel<<<kNTrials, 256, smem, st>>>(a);
     GB_CHECK_LAUNCH();
@@ -1914,15 +2251,10 @@ int iteration_post(Plan& p, bool low, cudaStream_t st) {
     a.nviews = p.nviews;
     a.history = p.history;
     a.max_iter = p.opt.max_iter;
-    size_t smem = sizeof(double) * (2 * 16 * kk + 5 * kk + 100 + 6 * 256 + 11 * kk + kMaxK);
-    if (low) {
-      GB_CUDA(cudaFuncSetAttribute(direction_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      direction_kernel<float><<<p.nviews, 256, smem, st>>>(a);
-    } else {
-      GB_CUDA(cudaFuncSetAttribute(direction_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)smem));
-      direction_kernel<double><<<p.nviews, 256, smem, st>>>(a);
-    }
+    const size_t smem = low ? direction_smem(k) : direction64_smem(k);
+    auto kern = low ? direction_kernel : direction64_kernel;
+    GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<p.nviews, 256, smem, st>>>(a);
     GB_CHECK_LAUNCH();
   }
   {

@@ -1,0 +1,188 @@
+// Small dense factorizations inside one CTA (matrices of at most 40 columns in
+// shared memory).  What bounds them on this GPU is the latency of dependent
+// FP64 instructions and their issue rate (a warp-wide FP64 instruction holds
+// its scheduler for tens of cycles), so every step uses as few dependent FP64
+// instructions and barriers as possible, all four schedulers, and FP32 where
+// the result is corrected afterwards.
+#pragma once
+#include "common.cuh"
+
+namespace gbcca {
+
+// 1 / x in FP64: the FP32 reciprocal corrected by one third-order step,
+// y (1 + e + e^2) with e = 1 - x y, |e| < 2^-22: three dependent
+// multiply-adds instead of a division.  Outside the float range: 1 / x.
+__device__ __forceinline__ double rcp_nr(double x) {
+  const float xf = (float)x;
+  if (!(fabsf(xf) > 1e-37f && fabsf(xf) < 1e37f)) return 1.0 / x;
+  const double y = (double)__frcp_rn(xf);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// Barrier over the G threads of a group (id 0: the whole CTA).
+template <int G>
+__device__ __forceinline__ void group_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(G) : "memory");
+}
+
+// L^{-1} of the Cholesky factor A = L L^T of an n x n symmetric positive
+// definite matrix (row-major, lower triangle read and destroyed) by G threads
+// with barrier `id`; g is the thread's index in the group.  Li (n x n,
+// row-major) receives L^{-1}, its upper triangle zero; rs is scratch of n.
+// Returns false, in every thread of the group, if a pivot is not positive
+// (the result is then void).  n <= 20 with G = 128, n <= 40 with G = 256.
+//
+// LDL^T with the inverse carried along: at step j the entry (i, c) of row
+// i > j, c in 0 .. i, is the trailing matrix for c > j and the unit inverse
+// for c <= j, and both are updated by -a_ij (row j entry) / d_j, so a step is
+// one reciprocal, one multiply and one multiply-add per entry behind a single
+// barrier, over all entries at once; the square roots follow at the end, all
+// at once.  (A Cholesky by one warp followed by the inverse, a column per
+// lane, was a chain of several hundred FP64 instructions.)
+template <int G>
+__device__ bool group_chol_inverse(double* A, double* Li, double* rs, int n, int g, int id) {
+  constexpr int kItems = G == 128 ? 2 : 4;  // entries (i, c), c <= i, per thread
+  int ri[kItems], ci[kItems];
+#pragma unroll
+  for (int u = 0; u < kItems; ++u) {
+    const int e = g + G * u;
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    while ((i + 1) * (i + 2) / 2 <= e) ++i;
+    while (i * (i + 1) / 2 > e) --i;
+    ri[u] = i;
+    ci[u] = e - i * (i + 1) / 2;
+    if (i < n) {
+      Li[i * n + ci[u]] = i == ci[u] ? 1.0 : 0.0;
+      if (i != ci[u]) Li[ci[u] * n + i] = 0.0;
+    }
+  }
+  bool ok = true;
+  for (int j = 0; j < n; ++j) {
+    group_sync<G>(id);
+    double d = A[j * n + j];
+    if (!(d > 0.0)) {
+      ok = false;
+      d = 1.0;
+    }
+    if (j == n - 1) break;
+    const double r = rcp_nr(d);
+#pragma unroll
+    for (int u = 0; u < kItems; ++u) {
+      const int i = ri[u], c = ci[u];
+      if (i > j && i < n) {
+        const double a = A[i * n + j];
+        if (c > j)
+          A[i * n + c] -= a * (A[c * n + j] * r);
+        else
+          Li[i * n + c] -= a * (Li[j * n + c] * r);
+      }
+    }
+  }
+  if (g < n) {
+    const double d = A[g * n + g];
+    rs[g] = d > 0.0 ? rsqrt_nr(d) : 1.0;
+  }
+  group_sync<G>(id);
+#pragma unroll
+  for (int u = 0; u < kItems; ++u)
+    if (ri[u] < n) Li[ri[u] * n + ci[u]] *= rs[ri[u]];
+  group_sync<G>(id);
+  return ok;
+}
+
+// Symmetric eigendecomposition in FP32 by parallel (round-robin ordered)
+// two-sided Jacobi, n <= 20, by all 256 threads of the CTA: on return the
+// diagonal of *A holds the eigenvalues (unsorted) and the columns of *Q the
+// eigenvectors.  A2 and Q2 are second buffers; the pointers come back swapped
+// as the last round left them.  Every warp forms all rotations of a round in
+// its own lanes, a thread updates one or two entries of A (four old entries,
+// two rotations) and of Q from one buffer into the other, so a round costs
+// one barrier.  A sweep in which no pair exceeded 1e-6 of its diagonal ends
+// it.  (One warp updating rows, then columns, in place took 53 us for n = 10.)
+__device__ __forceinline__ void jacobi_role(int i, int r, int m, int np, int& pair, int& partner) {
+  auto mod = [&](int x) { return x >= m - 1 ? x - (m - 1) : x; };
+  if (i == 0) {
+    pair = 0;
+    partner = 1 + mod(m - 2 + r);
+    return;
+  }
+  int t = i - 1 - r;
+  if (t < 0) t += m - 1;
+  if (t <= np - 2) {
+    pair = t + 1;
+    partner = 1 + mod(m - 2 - pair + r);
+  } else {
+    pair = m - 2 - t;
+    partner = pair == 0 ? 0 : 1 + mod(pair - 1 + r);
+  }
+}
+
+__device__ __forceinline__ void blk_jacobi_f32(float*& A, float*& A2, float*& Q, float*& Q2, int n) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int m = n + (n & 1), np = m / 2;
+  int ei[2], ej[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int e = tid + 256 * u;
+    ei[u] = e / n;
+    ej[u] = e - ei[u] * n;
+    if (ei[u] < n) Q[e] = ei[u] == ej[u] ? 1.f : 0.f;
+  }
+  __syncthreads();
+  for (int sweep = 0; sweep < 12; ++sweep) {
+    bool big = false;
+    for (int r = 0; r < m - 1; ++r) {
+      float c = 1.f, s = 0.f;
+      if (lane < np) {
+        const int x = lane - 1 + r, y = m - 2 - lane + r;
+        const int a = lane == 0 ? 0 : 1 + (x >= m - 1 ? x - (m - 1) : x);
+        const int b = 1 + (y >= m - 1 ? y - (m - 1) : y);
+        const int p = min(a, b), q = max(a, b);
+        if (q < n) {
+          const float apq = A[p * n + q], app = A[p * n + p], aqq = A[q * n + q];
+          const float w = fabsf(app * aqq);
+          if (apq * apq > 1e-16f * w) {
+            big = apq * apq > 1e-12f * w || big;
+            const float tau = (aqq - app) / (2.f * apq);
+            const float t = __fdividef(tau >= 0.f ? 1.f : -1.f, fabsf(tau) + sqrtf(1.f + tau * tau));
+            c = rsqrtf(1.f + t * t);
+            s = t * c;
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const bool in = ei[u] < n;
+        if (u == 1 && n * n <= 256) break;  // uniform
+        const int i = in ? ei[u] : 0, j = in ? ej[u] : 0;
+        int pi, qi, pj, qj;
+        jacobi_role(i, r, m, np, pi, qi);
+        jacobi_role(j, r, m, np, pj, qj);
+        const float c_i = __shfl_sync(0xffffffffu, c, pi), c_j = __shfl_sync(0xffffffffu, c, pj);
+        float s_i = __shfl_sync(0xffffffffu, s, pi), s_j = __shfl_sync(0xffffffffu, s, pj);
+        if (i < qi) s_i = -s_i;
+        if (j < qj) s_j = -s_j;
+        if (qi >= n) qi = i;  // a bye (its rotation is the identity)
+        if (qj >= n) qj = j;
+        if (in) {
+          const float x0 = c_i * A[i * n + j] + s_i * A[qi * n + j];
+          const float x1 = c_i * A[i * n + qj] + s_i * A[qi * n + qj];
+          A2[i * n + j] = c_j * x0 + s_j * x1;
+          Q2[i * n + j] = c_j * Q[i * n + j] + s_j * Q[i * n + qj];
+        }
+      }
+      __syncthreads();
+      float* t = A;
+      A = A2;
+      A2 = t;
+      t = Q;
+      Q = Q2;
+      Q2 = t;
+    }
+    // every warp formed the same rotations: the verdict is uniform
+    if (!__any_sync(0xffffffffu, big)) break;
+  }
+}
+
+}  // namespace gbcca

@@ -210,3 +210,93 @@ def test_thin_products_f64(gb, d, k):
         R = np64(gb.query(plan, q)).reshape(d, d)
         A = R @ np64(gb.query(plan, w)).reshape(d, k)
         assert np.max(np.abs(A.T @ A - np.eye(k))) < 1e-10
+
+
+@pytest.mark.parametrize("retraction", [0, 1])
+@pytest.mark.parametrize("kind,d,k", [("cca", 1, 1), ("cca", 9, 2), ("cca", 40, 11), ("cca", 60, 17), ("cca", 64, 20),
+                                      ("lda", 6, 1), ("lda", 30, 5), ("lda", 80, 20)])
+def test_small_geometry_trajectory_f64(gb, kind, d, k, retraction):
+    """Line search and direction (factors, Jacobi sweeps and Sylvester
+    solves for odd and even k up to the largest): ten iterations of an FP64
+    solve from a random start follow the oracle's Riemannian CG with the
+    library's own R.  Both compute in FP64, so f agrees to rounding grown by
+    the iterations (1e-9 relative), the accepted steps and the gradient norm
+    to 1e-6."""
+    import torch
+    from oracle import lda as OL
+    from oracle.cca import sigmas
+    from oracle.problems import CCAProblem, FDAProblem
+    from oracle.rcg import rcg
+    n, iters, lam = 20 * d + 60, 10, 1e-1
+    rng = np.random.default_rng(10 * d + k)
+    mu = np.linspace(2.0, 1.0, k) if k > 1 else np.ones(1)
+    opt = gb.default_options(warm_start=0, max_iter=iters, gtol=0.0, retraction=retraction)
+    if kind == "cca":
+        X, Y = rng.standard_normal((n, d)), rng.standard_normal((n, d + 1))
+        Y[:, :d] += X * np.linspace(1.5, 0.2, d)
+        starts = [rng.standard_normal((d, k)), rng.standard_normal((d + 1, k))]
+        plan = gb.cca_plan(n, d, d + 1, k, "f64", opt)
+        gb.cca_precondition(plan, torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), lam, lam)
+        gb.cca_solve(plan, mu=list(mu), U=torch.from_numpy(starts[0].copy()).cuda(),
+                     V=torch.from_numpy(starts[1].copy()).cuda())
+        prob = CCAProblem(*sigmas(X, Y, lam, lam), mu)
+        dims = (d, d + 1)
+    else:
+        P = lda_problem(n, d, k + 1, dtype="f64", seed=d, var_range=(0.1, 1.0))
+        starts = [rng.standard_normal((d, k))]
+        plan = gb.lda_plan(n, d, k + 1, k, "f64", opt)
+        gb.lda_solve(plan, to_dev(P["X"], "f64"), torch.from_numpy(P["y"]).cuda(), lam, mu=list(mu),
+                     W=torch.from_numpy(starts[0].copy()).cuda())
+        _, _, _, Yhat, Xhat = OL.class_stats(P["X64"], P["y"], k + 1)
+        prob = FDAProblem(Yhat.T @ Yhat, Xhat.T @ Xhat + lam * np.eye(d), mu)
+        dims = (d,)
+    hist = np64(gb.query(plan, gb.Q_HISTORY)).reshape(-1, 3)
+    Ms = []
+    for q, m in zip((gb.Q_R_X, gb.Q_R_Y), dims):
+        R = np64(gb.query(plan, q)).reshape(m, m)
+        Ms.append(R.T @ R)
+    ho = np.array(rcg(prob, Ms, starts, max_iter=iters, gtol=0.0,
+                      retraction="polar" if retraction else "qr")["history"])
+    m = len(ho)
+    if k == d:  # U spans everything: f is constant and the steps are rounding
+        m = 1
+    assert m > 1 or k == d
+    assert np.max(np.abs(hist[:m, 0] - ho[:, 0][:m]) / np.abs(ho[:m, 0])) < 1e-9
+    if m > 1:
+        assert np.max(np.abs(hist[1:m, 2] - ho[1:m, 2]) / np.abs(ho[1:m, 2])) < 1e-6
+        assert np.max(np.abs(hist[:m, 1] - ho[:m, 1]) / np.abs(ho[:m, 1])) < 1e-6
+
+
+@pytest.mark.parametrize("retraction", [0, 1])
+@pytest.mark.parametrize("d,k", [(9, 1), (12, 2), (40, 11), (60, 17), (64, 20)])
+def test_small_geometry_f32(gb, d, k, retraction):
+    """Line search and direction of FP32 plans for odd and even k: the first
+    iterations follow the oracle's Riemannian CG.  The pass is good to some
+    2^-16 of the sums of |terms|, so f is held to 1e-3; a wrong factor,
+    direction or coefficient changes it by far more."""
+    import torch
+    from oracle.cca import sigmas
+    from oracle.problems import CCAProblem
+    from oracle.rcg import rcg
+    n, iters, lam = 20 * d + 60, 4, 1e-1
+    rng = np.random.default_rng(10 * d + k)
+    mu = np.linspace(2.0, 1.0, k) if k > 1 else np.ones(1)
+    X, Y = rng.standard_normal((n, d)), rng.standard_normal((n, d + 1))
+    Y[:, :d] += X * np.linspace(1.5, 0.2, d)
+    X, Y = X.astype(np.float32), Y.astype(np.float32)
+    starts = [rng.standard_normal((d, k)), rng.standard_normal((d + 1, k))]
+    plan = gb.cca_plan(n, d, d + 1, k, "f32", gb.default_options(warm_start=0, max_iter=iters, gtol=0.0, refine=0,
+                                                                 retraction=retraction))
+    gb.cca_precondition(plan, torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), lam, lam)
+    gb.cca_solve(plan, mu=list(mu), U=torch.from_numpy(starts[0].copy()).cuda(),
+                 V=torch.from_numpy(starts[1].copy()).cuda())
+    hist = np64(gb.query(plan, gb.Q_HISTORY)).reshape(-1, 3)
+    Ms = []
+    for q, m in zip((gb.Q_R_X, gb.Q_R_Y), (d, d + 1)):
+        R = np64(gb.query(plan, q)).reshape(m, m)
+        Ms.append(R.T @ R)
+    prob = CCAProblem(*sigmas(X.astype(np.float64), Y.astype(np.float64), lam, lam), mu)
+    ho = np.array(rcg(prob, Ms, starts, max_iter=iters, gtol=0.0, retraction="polar" if retraction else "qr")["history"])
+    m = min(len(ho), len(hist))
+    assert m > 1
+    assert np.max(np.abs(hist[:m, 0] - ho[:m, 0]) / np.abs(ho[:m, 0])) < 1e-3
