@@ -171,7 +171,7 @@ int alloc_plan(Plan* p) {
   GB_TRY(dalloc(&p->ritz_hist, (int64_t)p->ritz_len * k));
   p->ws_len = 8 * (int64_t)dmax * dmax + 3 * (int64_t)dmax * std::max(std::max(p->l, k2), 1) + 4096;
   GB_TRY(dalloc(&p->ws, p->ws_len));
-  GB_TRY(dalloc(&p->dfx, 2 * (int64_t)dmax * k2));
+  GB_TRY(dalloc(&p->dfx, 4 * (int64_t)dmax * k2));
   GB_TRY(dalloc(&p->ls_f, 64));
   GB_TRY(dalloc(&p->ls_L, 64 * 2 * (int64_t)kMaxK * kMaxK));
   GB_TRY(dalloc(&p->flag, 1));

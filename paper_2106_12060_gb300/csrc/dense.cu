@@ -262,27 +262,38 @@ __device__ __forceinline__ void df_add(float& S, float& Cc, float s2, float c2) 
   Cc += err + c2;
 }
 
-constexpr int kMvRows = 4;            // output rows per CTA
+constexpr int kMvRows = 8;             // output rows per CTA
 constexpr int kMvThreads = 256;
-constexpr int kMvStageBytes = 98304;  // shared memory of one staged K chunk (A rows + X rows)
+constexpr int kMvStageBytes = 118784;  // shared memory of one staged K chunk (A rows + X rows)
 
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
-               "l"(gmem)
-               : "memory");
+// n floats (4, 2 or 1) from global to shared memory, asynchronously
+__device__ __forceinline__ void cp_async_f(float* smem, const float* gmem, int n) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
+  if (n == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem) : "memory");
+  else if (n == 2) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gmem) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// the widest of those that keeps every row start of two matrices aligned
+static int copy_width(const float* a, const float* b, int cols, int ld) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b);
+  if ((cols | ld) % 4 == 0 && at % 16 == 0) return 4;
+  return (cols | ld) % 2 == 0 && at % 8 == 0 ? 2 : 1;
+}
+__host__ __device__ __forceinline__ int mv_cols(int c) { return (c + 3) / 4 * 4; }
 
 // Y_b (m x c) = A_b X_b for problem b = blockIdx.y, A_b (m x K, row-major)
-// and X_b (K x c, row stride ldx) as double-float pairs hi + lo.  A CTA owns
-// kMvRows rows of Y.  The K range is walked in chunks: the chunk's rows of A
-// and of X are copied into shared memory as (hi, lo) pairs by asynchronous
-// copies (all of them in flight at once), then thread t computes output
-// e = t mod (kMvRows c) over the inner indices q = t / (kMvRows c) + j KS of
-// the chunk (KS = the threads per output), in two double-float chains.  The
-// KS partial pairs of an output are added in fixed order through shared
-// memory at the end: no scratch in global memory, no atomics, and the result
-// does not depend on scheduling.
+// and X_b (K x c, row stride ldx) as double-float pairs hi + lo; optionally
+// Y_b as a pair too (Yh, Yl, row stride c).  A CTA owns kMvRows rows of Y.  The
+// K range is walked in chunks staged in shared memory by the widest
+// asynchronous copies the alignment allows, in two halves, so that the first
+// is worked on while the second arrives.  A thread owns 2 rows x 4 columns of
+// an interleaved slice of K (KS slices): eight double-float multiply-adds (12
+// FP32 instructions each) for six shared-memory loads.  The KS partial pairs
+// of an output are added in fixed order through shared memory at the end: no
+// scratch in global memory, no atomics, and the result does not depend on
+// scheduling.  Bound by FP32 issue (512 x 512 x 20, two views: 3 us of
+// arithmetic); one output per thread behind 4-byte copies of all of X per
+// four rows took 13 to 19 us a launch.
 __global__ void __launch_bounds__(kMvThreads) dfmv_kernel(DfmvArgs a) {
   if (a.done != nullptr && *a.done) return;
   // the problem's fields by selection (a dynamic index into the parameter
@@ -293,72 +304,106 @@ __global__ void __launch_bounds__(kMvThreads) dfmv_kernel(DfmvArgs a) {
     const float *hi, *lo, *Xh, *Xl;
     double* Y;
     int m, K, ldx, ldy;
-  } P{GB_SEL(hi), GB_SEL(lo), GB_SEL(Xh), GB_SEL(Xl), GB_SEL(Y), GB_SEL(m), GB_SEL(K), GB_SEL(ldx), GB_SEL(ldy)};
+    float *Yh, *Yl;
+    int wa, wx;
+  } P{GB_SEL(hi), GB_SEL(lo), GB_SEL(Xh), GB_SEL(Xl), GB_SEL(Y), GB_SEL(m), GB_SEL(K), GB_SEL(ldx), GB_SEL(ldy),
+      GB_SEL(Yh), GB_SEL(Yl), GB_SEL(wa), GB_SEL(wx)};
 #undef GB_SEL
   const int r0 = blockIdx.x * kMvRows;
   if (r0 >= P.m) return;  // uniform over the CTA
-  extern __shared__ float2 mv[];
-  const int c = a.c, Kc = a.kc;
-  float2* As = mv;                 // [kMvRows][Kc]
-  float2* Xs = mv + kMvRows * Kc;  // [Kc][c]
+  extern __shared__ __align__(16) float mvs[];
+  const int c = a.c, cp = mv_cols(c), Kc = a.kc, lda = Kc + 4;
+  float* Ah = mvs;                 // [kMvRows][lda]
+  float* Al = Ah + kMvRows * lda;
+  float* Xh = Al + kMvRows * lda;  // [Kc][cp]
+  float* Xl = Xh + Kc * cp;
   const int t = threadIdx.x;
-  const int nout = kMvRows * c;
-  const int KS = max(1, kMvThreads / nout);
-  const bool active = t < nout * KS;
-  const int e = t % nout, ks = t / nout;
-  const int rr = e / c, col = e - rr * c;
-  float S0 = 0.f, C0 = 0.f, S1 = 0.f, C1 = 0.f;
+  const int CG = cp / 4, per = 4 * CG;  // threads of a slice: 4 row pairs x CG column groups
+  const int KS = kMvThreads / per;
+  const int ks = t / per, w = t - ks * per, rg = w / CG, cg = w - rg * CG;
+  const bool active = ks < KS;
+  const int wa = P.wa, wx = P.wx;
+  // pad columns of X hold zeros (they are never copied)
+  if (cp != c)
+    for (int i = t; i < Kc * (cp - c); i += kMvThreads) {
+      const int q = i / (cp - c), cc = c + i - q * (cp - c);
+      Xh[q * cp + cc] = 0.f;
+      Xl[q * cp + cc] = 0.f;
+    }
+  float S[2][4] = {}, Cc[2][4] = {};
   for (int k0 = 0; k0 < P.K; k0 += Kc) {
-    const int kn = min(Kc, P.K - k0);
+    const int kn = min(Kc, P.K - k0), half = min(kn, (kn + 7) / 8 * 4);
     __syncthreads();  // the previous chunk has been consumed
-    for (int i = t; i < kMvRows * kn; i += kMvThreads) {
-      const int r2 = i / kn, q = i - r2 * kn;
-      float2* d = As + r2 * Kc + q;
-      if (r0 + r2 < P.m) {
-        const int64_t o = (int64_t)(r0 + r2) * P.K + k0 + q;
-        cp_async4(&d->x, P.hi + o);
-        cp_async4(&d->y, P.lo + o);
-      } else {
-        *d = make_float2(0.f, 0.f);
+    for (int h = 0; h < 2; ++h) {
+      const int q0 = h == 0 ? 0 : half, qn = (h == 0 ? half : kn) - q0;
+      const int na = qn / wa;  // (half and K are multiples of wa)
+      for (int i = t; i < kMvRows * na; i += kMvThreads) {
+        const int r = i / na, q = q0 + (i - r * na) * wa;
+        const int64_t o = (int64_t)min(r0 + r, P.m - 1) * P.K + k0 + q;
+        cp_async_f(Ah + r * lda + q, P.hi + o, wa);
+        cp_async_f(Al + r * lda + q, P.lo + o, wa);
       }
-    }
-    for (int i = t; i < kn * c; i += kMvThreads) {
-      const int q = i / c, cc = i - q * c;
-      const int64_t o = (int64_t)(k0 + q) * P.ldx + cc;
-      cp_async4(&Xs[i].x, P.Xh + o);
-      cp_async4(&Xs[i].y, P.Xl + o);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    if (active) {
-      const float2* ar = As + rr * Kc;
-      int q = ks;
-      for (; q + KS < kn; q += 2 * KS) {
-        const float2 a0 = ar[q], x0 = Xs[q * c + col];
-        const float2 a1 = ar[q + KS], x1 = Xs[(q + KS) * c + col];
-        df_acc(S0, C0, a0.x, a0.y, x0.x, x0.y);
-        df_acc(S1, C1, a1.x, a1.y, x1.x, x1.y);
+      const int nx = c / wx;
+      for (int i = t; i < qn * nx; i += kMvThreads) {
+        const int q = q0 + i / nx, cc = (i % nx) * wx;
+        const int64_t o = (int64_t)(k0 + q) * P.ldx + cc;
+        cp_async_f(Xh + q * cp + cc, P.Xh + o, wx);
+        cp_async_f(Xl + q * cp + cc, P.Xl + o, wx);
       }
-      if (q < kn) {
-        const float2 a0 = ar[q], x0 = Xs[q * c + col];
-        df_acc(S0, C0, a0.x, a0.y, x0.x, x0.y);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int h = 0; h < 2; ++h) {
+      if (h == 0) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      if (active) {
+        const float *ah = Ah + 2 * rg * lda, *al = Al + 2 * rg * lda;
+        const int q1 = h == 0 ? half : kn;
+#pragma unroll 2
+        for (int q = (h == 0 ? 0 : half) + ks; q < q1; q += KS) {
+          const float4 xh = *reinterpret_cast<const float4*>(Xh + q * cp + 4 * cg);
+          const float4 xl = *reinterpret_cast<const float4*>(Xl + q * cp + 4 * cg);
+          const float xhv[4] = {xh.x, xh.y, xh.z, xh.w}, xlv[4] = {xl.x, xl.y, xl.z, xl.w};
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const float vh = ah[u * lda + q], vl = al[u * lda + q];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) df_acc(S[u][j], Cc[u][j], vh, vl, xhv[j], xlv[j]);
+          }
+        }
       }
     }
   }
-  df_add(S0, C0, S1, C1);
   __syncthreads();
-  float2* red = mv;  // [KS][nout]
-  if (active) red[ks * nout + e] = make_float2(S0, C0);
+  float2* red = reinterpret_cast<float2*>(mvs);  // [KS][kMvRows][cp]
+  const int nout = kMvRows * cp;
+  if (active) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) red[ks * nout + (2 * rg + u) * cp + 4 * cg + j] = make_float2(S[u][j], Cc[u][j]);
+  }
   __syncthreads();
-  if (t < nout && r0 + rr < P.m) {
-    float s = 0.f, cc = 0.f;
-    for (int k2 = 0; k2 < KS; ++k2) df_add(s, cc, red[k2 * nout + t].x, red[k2 * nout + t].y);
-    P.Y[(int64_t)(r0 + rr) * P.ldy + col] = (double)s + (double)cc;
+  for (int e = t; e < kMvRows * c; e += kMvThreads) {
+    const int r = e / c, col = e - r * c;
+    if (r0 + r >= P.m) continue;
+    float sum = 0.f, cc = 0.f;
+    for (int q = 0; q < KS; ++q) {
+      const float2 v = red[q * nout + r * cp + col];
+      df_add(sum, cc, v.x, v.y);
+    }
+    const double y = (double)sum + (double)cc;
+    P.Y[(int64_t)(r0 + r) * P.ldy + col] = y;
+    if (P.Yh != nullptr) {
+      const float h = (float)y;
+      P.Yh[(int64_t)(r0 + r) * c + col] = h;
+      P.Yl[(int64_t)(r0 + r) * c + col] = (float)(y - (double)h);
+    }
   }
 }
 
 int dfmv(const DfmvArgs& a, int nprob, cudaStream_t st) {
-  if (a.c < 1 || kMvRows * a.c > kMvThreads || nprob < 1 || nprob > 2) {
+  if (a.c < 1 || a.c > 64 || nprob < 1 || nprob > 2) {
     set_last_error("dfmv: unsupported column count");
     return GBCCA_ERR_INVALID_ARG;
   }
@@ -371,11 +416,17 @@ int dfmv(const DfmvArgs& a, int nprob, cudaStream_t st) {
     mmax = std::max(mmax, a.p[b].m);
     kmax = std::max(kmax, a.p[b].K);
   }
-  // K chunk: the chunk's rows of A and of X (float pairs) fill at most
-  // kMvStageBytes of shared memory; the final reduction reuses the space
+  // K chunk: as few equal chunks (multiples of 32) as the staged rows of A
+  // and X allow; the final reduction (at most 16 KB) reuses the space
   DfmvArgs g = a;
-  g.kc = std::max(1, std::min(kmax, kMvStageBytes / (8 * (kMvRows + a.c))));
-  const size_t smem = std::max<size_t>(8 * (size_t)g.kc * (kMvRows + a.c), 8 * (size_t)kMvThreads);
+  for (int b = 0; b < nprob; ++b) {
+    g.p[b].wa = copy_width(a.p[b].hi, a.p[b].lo, a.p[b].K, 0);
+    g.p[b].wx = copy_width(a.p[b].Xh, a.p[b].Xl, a.c, a.p[b].ldx);
+  }
+  const int per_q = 8 * (kMvRows + mv_cols(a.c));
+  const int chunks = ceil_div((int64_t)kmax * per_q, kMvStageBytes);
+  g.kc = (ceil_div(kmax, chunks) + 31) / 32 * 32;
+  const size_t smem = std::max<size_t>((size_t)per_q * g.kc + 8 * kMvRows * 4, 8 * 8 * (size_t)kMvThreads);
   GB_CUDA(cudaFuncSetAttribute(dfmv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dfmv_kernel<<<dim3(ceil_div(mmax, kMvRows), nprob), kMvThreads, smem, st>>>(g);
   GB_CHECK_LAUNCH();

@@ -130,7 +130,7 @@ struct Plan {
   double* history = nullptr;    // 3 (max_iter + 1)
   double* ritz_hist = nullptr;  // Ritz values at every check: (max_iter / check_every + 2) x k
   int ritz_len = 0;             // rows of ritz_hist
-  float* dfx = nullptr;         // 2 x dmax x 2k floats: split blocks for double-float products
+  float* dfx = nullptr;         // 4 x dmax x 2k floats: the warm start's blocks as float pairs
   double* ls_f = nullptr;       // line-search trial values (kNTrials)
   double* ls_L = nullptr;       // line-search trial factors (kNTrials x 2 x kMaxK^2)
   double* ws = nullptr;         // FP64 scratch for dense routines
@@ -219,6 +219,9 @@ struct DfmvProblem {
   double* Y;         // m x c (row stride ldy doubles)
   int m, K;
   int ldx, ldy;
+  float* Yh;         // optional: Y as a float pair too (row stride c)
+  float* Yl;
+  int wa, wx;        // floats per copy of A and X rows (set by dfmv)
 };
 struct DfmvArgs {
   DfmvProblem p[2];

@@ -2233,7 +2233,8 @@ int iteration_post(Plan& p, bool low, cudaStream_t st) {
     DfmvArgs m{};
     for (int v = 0; v < p.nviews; ++v)
       m.p[v] = DfmvProblem{p.v[v].Minv_hi, p.v[v].Minv_lo, p.v[v].RRh, p.v[v].RRl, p.v[v].LL,
-                           p.v[v].d,       p.v[v].d,       2 * k,       4 * k};
+                           p.v[v].d,       p.v[v].d,       2 * k,       4 * k,       nullptr,      nullptr,
+                           0,              0};
     m.c = 2 * k;
     m.done = done;
     GB_TRY(dfmv(m, p.nviews, st));
@@ -2580,9 +2581,50 @@ __global__ void rand_block_kernel(double* B, int d, int c, uint64_t seed) {
   B[e] = (double)(r >> 11) * (1.0 / 9007199254740992.0) - 0.5;
 }
 
-// small Gram (c x c) of a d x c block: reduce partials, Cholesky (ridge for
+// small Gram G (c x c, c <= 40) of a d x c block: the lower triangle of the
+// partials' sum, a ridge for safety, and R^{-1} = L^{-T} of G = L L^T in out.
+__global__ void __launch_bounds__(256) small_chol_kernel(const double* part, int nblk, int c, double* out, int* flag) {
+  extern __shared__ double ssm[];
+  double* G = ssm;
+  double* Li = G + c * c;
+  double* rs = Li + c * c;
+  __shared__ double s_tr;
+  for (int e = threadIdx.x; e < c * (c + 1) / 2; e += blockDim.x) {
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    while ((i + 1) * (i + 2) / 2 <= e) ++i;
+    while (i * (i + 1) / 2 > e) --i;
+    const int f = i * c + (e - i * (i + 1) / 2);
+    double s = 0;
+    for (int b0 = 0; b0 < nblk; b0 += 8) {
+      double x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = b0 + u < nblk ? part[(int64_t)(b0 + u) * c * c + f] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += x[u];
+    }
+    G[f] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double tr = 0;
+    for (int i = threadIdx.x; i < c; i += 32) tr += G[i * c + i];
+    tr = warp_sum(tr);
+    if (threadIdx.x == 0) s_tr = tr;
+  }
+  __syncthreads();
+  if (threadIdx.x < c) G[threadIdx.x * c + threadIdx.x] += 1e-14 * s_tr / c;
+  const bool ok = group_chol_inverse<256>(G, Li, rs, c, threadIdx.x, 0);
+  if (!ok && threadIdx.x == 0) atomicExch(flag, kFlagNotSpd);
+  for (int e = threadIdx.x; e < c * c; e += blockDim.x) {
+    const int i = e / c, j = e - i * c;
+    out[e] = Li[j * c + i];
+  }
+}
+
+// The same for FP64 plans, whose iterations amplify a change of rounding in
+// their starting point: reduce partials, Cholesky (ridge for
 // safety) -> upper R in out (R^T R = G), and its inverse in out + c*c.
-__global__ void small_chol_kernel(const double* part, int nblk, int c, double* out, int* flag) {
+__global__ void small_chol64_kernel(const double* part, int nblk, int c, double* out, int* flag) {
   extern __shared__ double ssm[];
   double* G = ssm;
   double* Li = G + c * c;
@@ -2617,9 +2659,10 @@ __global__ void small_chol_kernel(const double* part, int nblk, int c, double* o
 // B (d x c) <- B Rinv (c x c upper): a CTA stages kApplyRows rows of B in
 // shared memory and each thread forms one entry (at most c multiply-adds),
 // so the FP64 work spreads over many SMs instead of one chain per row.
+// Optionally the result as a float pair (Bh, Bl) as well.
 constexpr int kApplyRows = 8;
 __global__ void __launch_bounds__(kApplyRows * 2 * kMaxK) apply_small_kernel(double* B, int d, int c,
-                                                                            const double* Rinv) {
+                                                                            const double* Rinv, float* Bh, float* Bl) {
   __shared__ double rows[kApplyRows * 2 * kMaxK];
   const int j0 = blockIdx.x * kApplyRows;
   const int nr = min(kApplyRows, d - j0);
@@ -2630,7 +2673,13 @@ __global__ void __launch_bounds__(kApplyRows * 2 * kMaxK) apply_small_kernel(dou
   const int r = e / c, q = e - r * c;
   double s = 0;
   for (int t = 0; t <= q; ++t) s += rows[r * c + t] * Rinv[t * c + q];
-  B[(int64_t)(j0 + r) * c + q] = s;
+  const int64_t o = (int64_t)(j0 + r) * c + q;
+  B[o] = s;
+  if (Bh != nullptr) {
+    const float h = (float)s;
+    Bh[o] = h;
+    Bl[o] = (float)(s - (double)h);
+  }
 }
 
 // Rayleigh-Ritz of the power iteration: Bsmall = U^T (C V) (c x c), take the
@@ -2690,7 +2739,8 @@ __global__ void fda_warm_kernel(const double* part, int nblk, int l, int k, doub
 
 namespace {
 
-int orth(Plan& p, double* B, int d, int c, double* part, double* small, cudaStream_t st) {
+int orth(Plan& p, double* B, int d, int c, double* part, double* small, cudaStream_t st, float* Bh = nullptr,
+         float* Bl = nullptr) {
   // Gram of B (d x c) via a one-view thin Gram
   ThinArgs a{};
   a.A[0] = B;
@@ -2707,9 +2757,10 @@ int orth(Plan& p, double* B, int d, int c, double* part, double* small, cudaStre
   GB_CUDA(cudaFuncSetAttribute(thin_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   thin_gram_kernel<<<dim3(a.nblk, 1), 256, smem, st>>>(a);
   GB_CHECK_LAUNCH();
-  small_chol_kernel<<<1, 256, sizeof(double) * (2 * c * c + c), st>>>(part, a.nblk, c, small, p.flag);
+  auto chol = p.dtype == GBCCA_FP64 ? small_chol64_kernel : small_chol_kernel;
+  chol<<<1, 256, sizeof(double) * (2 * c * c + c), st>>>(part, a.nblk, c, small, p.flag);
   GB_CHECK_LAUNCH();
-  apply_small_kernel<<<ceil_div(d, kApplyRows), kApplyRows * 2 * kMaxK, 0, st>>>(B, d, c, small);
+  apply_small_kernel<<<ceil_div(d, kApplyRows), kApplyRows * 2 * kMaxK, 0, st>>>(B, d, c, small, Bh, Bl);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }
@@ -2734,70 +2785,79 @@ int warm_start(Plan& p, cudaStream_t st) {
     double* Ub = x.wsU;  // dx x c
     double* part = p.crosspart;
     double* small = p.phigram;
-    // Products of the power iteration.  FP64 plans: FP64 triangular / dense
-    // products.  FP32/BF16 plans: the same products with double-float copies
-    // of R_x^{-1}, R_y^{-1}, Cxy and their transposes (~2^-44 relative, at
-    // FP32 instruction rates); FP32 copies of R^{-1} (kappa ~ 1e4) give a
-    // visibly worse start point and more solver iterations.
-    const bool low = p.dtype != GBCCA_FP64 && (c & 1) == 0;
-    float* F = reinterpret_cast<float*>(p.ws);
+    // Products of the power iteration with C = R_x^{-T} Cxy R_y^{-1}.  FP64
+    // plans: FP64 triangular / dense products one after another.  FP32/BF16
+    // plans: C is formed once in double-float (~2^-44 relative, at FP32
+    // instruction rates), in place of three products per half step; FP32
+    // copies of R^{-1} (kappa ~ 1e4) give a visibly worse start point and
+    // more solver iterations.
+    const bool low = p.dtype != GBCCA_FP64;
+    const int64_t N = (std::max((int64_t)dx * dx, std::max((int64_t)dy * dy, (int64_t)dx * dy)) + 1) / 2 * 2;
+    float* w0 = reinterpret_cast<float*>(p.ws);          // pairs of at most N entries each
+    float* w1 = reinterpret_cast<float*>(p.ws + N);
     const int64_t nx = (int64_t)dx * dx, ny = (int64_t)dy * dy, nc = (int64_t)dx * dy;
-    float* Rx[2] = {F, F + nx};              // R_x^{-1} hi, lo
-    float* RxT[2] = {F + 2 * nx, F + 3 * nx};
-    float* Ry[2] = {F + 4 * nx, F + 4 * nx + ny};
-    float* RyT[2] = {F + 4 * nx + 2 * ny, F + 4 * nx + 3 * ny};
-    float* Cf[2] = {F + 4 * nx + 4 * ny, F + 4 * nx + 4 * ny + nc};
-    float* CfT[2] = {F + 4 * nx + 4 * ny + 2 * nc, F + 4 * nx + 4 * ny + 3 * nc};
+    float* Cf[2] = {w0, w0 + nc};
+    float* CfT[2] = {w1, w1 + nc};
+    float* Vp[2] = {p.dfx, p.dfx + (int64_t)dy * c};
+    float* Up[2] = {p.dfx + 2 * (int64_t)dy * c, p.dfx + 2 * (int64_t)dy * c + (int64_t)dx * c};
     if (low) {
-      GB_TRY(split_df(x.Rinv, dx, dx, false, Rx[0], Rx[1], st));
-      GB_TRY(split_df(x.Rinv, dx, dx, true, RxT[0], RxT[1], st));
-      GB_TRY(split_df(y.Rinv, dy, dy, false, Ry[0], Ry[1], st));
-      GB_TRY(split_df(y.Rinv, dy, dy, true, RyT[0], RyT[1], st));
+      double* P = p.ws + 2 * N;
+      double* part64 = p.ws + 3 * N;
+      const int64_t plen = p.ws_len - nc - 3 * N;
+      GB_TRY(split_df(x.Rinv, dx, dx, false, w0, w0 + nx, st));
+      GB_TRY(split_df(Cxy, dx, dy, false, w1, w1 + nc, st));
+      GB_TRY(gram_df_split(w0, w0 + nx, dx, w1, w1 + nc, dy, dx, dx, dy, P, 0.0, part64, plen, st));   // R_x^{-T} Cxy
+      GB_TRY(split_df(P, dx, dy, true, w0, w0 + nc, st));
+      GB_TRY(split_df(y.Rinv, dy, dy, false, w1, w1 + ny, st));
+      GB_TRY(gram_df_split(w0, w0 + nc, dx, w1, w1 + ny, dy, dy, dx, dy, Cxy, 0.0, part64, plen, st));  // ... R_y^{-1}
       GB_TRY(split_df(Cxy, dx, dy, false, Cf[0], Cf[1], st));
       GB_TRY(split_df(Cxy, dx, dy, true, CfT[0], CfT[1], st));
     }
-    auto dmv = [&](float* const* A, int m, int K, const double* B, double* C) {
-      float* bh = p.dfx;
-      float* bl = p.dfx + (int64_t)K * c;
-      GB_TRY(split_rows(B, K, c, c, bh, bl, st));
+    auto dmv = [&](float* const* A, int m, int K, float* const* B, double* Y, float* const* Yp) {
       DfmvArgs g{};
-      g.p[0] = DfmvProblem{A[0], A[1], bh, bl, C, m, K, c, c};
+      g.p[0] = DfmvProblem{A[0], A[1], B[0], B[1], Y, m, K, c, c, Yp != nullptr ? Yp[0] : nullptr,
+                           Yp != nullptr ? Yp[1] : nullptr, 0, 0};
       g.c = c;
       return dfmv(g, 1, st);
     };
     auto rx = [&](bool tr, const double* B, double* C, int cc) {
-      if (low && cc == c) return dmv(tr ? RxT : Rx, dx, dx, B, C);
       const ThinMul t{x.Rinv, dx, dx, B, cc, C, cc};
       return mat_thin(&t, 1, tr, true, cc, st);
     };
     auto ry = [&](bool tr, const double* B, double* C, int cc) {
-      if (low && cc == c) return dmv(tr ? RyT : Ry, dy, dy, B, C);
       const ThinMul t{y.Rinv, dy, dy, B, cc, C, cc};
       return mat_thin(&t, 1, tr, true, cc, st);
     };
     auto cxy = [&](bool tr, const double* B, double* C) {
-      if (low) return tr ? dmv(CfT, dy, dx, B, C) : dmv(Cf, dx, dy, B, C);
       const ThinMul t{Cxy, dx, dy, B, c, C, c};
       return mat_thin(&t, 1, tr, false, c, st);
     };
     rand_block_kernel<<<ceil_div(dy * c, 256), 256, 0, st>>>(Vb, dy, c, p.opt.seed);
     GB_CHECK_LAUNCH();
-    GB_TRY(orth(p, Vb, dy, c, part, small, st));
+    GB_TRY(orth(p, Vb, dy, c, part, small, st, low ? Vp[0] : nullptr, low ? Vp[1] : nullptr));
     const int iters = p.opt.warm_iters > 0 ? p.opt.warm_iters : 12;
     for (int it = 0; it <= iters; ++it) {
-      // U = orth(R_x^{-T} Cxy R_y^{-1} V)
-      GB_TRY(ry(false, Vb, y.wsT, c));
-      GB_TRY(cxy(false, y.wsT, x.wsT));
-      GB_TRY(rx(true, x.wsT, Ub, c));
+      // U = C V
+      if (low) {
+        GB_TRY(dmv(Cf, dx, dy, Vp, Ub, Up));
+      } else {
+        GB_TRY(ry(false, Vb, y.wsT, c));
+        GB_TRY(cxy(false, y.wsT, x.wsT));
+        GB_TRY(rx(true, x.wsT, Ub, c));
+      }
       if (it == iters) break;  // Ub = C V (unnormalized) for the Rayleigh-Ritz step
-      // V = orth(C^T U) with C = R_x^{-T} Cxy R_y^{-1}: U = C V needs no
-      // orthonormalization of its own (span(C^T C V) is the same either way,
-      // and one step changes the conditioning of the block only by the
-      // spread of the top 2k singular values)
-      GB_TRY(rx(false, Ub, x.wsT, c));
-      GB_TRY(cxy(true, x.wsT, y.wsT));
-      GB_TRY(ry(true, y.wsT, Vb, c));
-      GB_TRY(orth(p, Vb, dy, c, part, small, st));
+      // V = orth(C^T U): U = C V needs no orthonormalization of its own
+      // (span(C^T C V) is the same either way, and one step changes the
+      // conditioning of the block only by the spread of the top 2k singular
+      // values)
+      if (low) {
+        GB_TRY(dmv(CfT, dy, dx, Up, Vb, nullptr));
+      } else {
+        GB_TRY(rx(false, Ub, x.wsT, c));
+        GB_TRY(cxy(true, x.wsT, y.wsT));
+        GB_TRY(ry(true, y.wsT, Vb, c));
+      }
+      GB_TRY(orth(p, Vb, dy, c, part, small, st, low ? Vp[0] : nullptr, low ? Vp[1] : nullptr));
     }
     // Ub = C V: take U0 = orth(Ub) and Bm = U0^T (C V)
     GB_CUDA(cudaMemcpyAsync(x.wsT, Ub, sizeof(double) * dx * c, cudaMemcpyDeviceToDevice, st));
@@ -2836,10 +2896,8 @@ int warm_start(Plan& p, cudaStream_t st) {
   // FDA
   View& x = p.v[0];
   const int d = x.d, l = p.l;
-  double* YhT = x.wsT;              // d x l  (wsT has d x 2k >= ... use ws instead when l > 2k)
   double* Gt = p.ws;                // d x l: R^{-T} Yhat^T
   double* YT = p.ws + (int64_t)d * l;
-  (void)YhT;
   transpose_kernel<<<ceil_div(l * d, 256), 256, 0, st>>>(p.Yhat, l, d, YT);
   GB_CHECK_LAUNCH();
   const ThinMul t1{x.Rinv, d, d, YT, l, Gt, l};

@@ -300,3 +300,30 @@ def test_small_geometry_f32(gb, d, k, retraction):
     m = min(len(ho), len(hist))
     assert m > 1
     assert np.max(np.abs(hist[:m, 0] - ho[:m, 0]) / np.abs(ho[:m, 0])) < 1e-3
+
+
+@pytest.mark.parametrize("d,k", [(1, 1), (5, 2), (31, 3), (33, 9), (49, 11), (130, 20)])
+def test_warm_start_blocks_f32(gb, d, k):
+    """The warm start of FP32 plans (products in double-float form over odd
+    and even column counts, orthonormalization, small singular value
+    decomposition): U and V orthonormal in the sketched metric, and U^T S_xy V
+    diagonal with descending entries, since it ends with a Rayleigh-Ritz step.
+    The products carry 2^-44 per term, so 1e-10 leaves the condition of R."""
+    import torch
+    from synth import countsketch_draws
+    n, s, lam = 8 * d + 40, 3 * d + 10, 1e-1
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((n, d)).astype(np.float32)
+    Y = (0.5 * X + rng.standard_normal((n, d))).astype(np.float32)
+    h, g = countsketch_draws(n, s, seed=3)
+    plan = gb.cca_plan(n, d, d, k, "f32", gb.default_options(s=s))
+    gb.cca_precondition(plan, torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), lam, lam,
+                        torch.from_numpy(h).cuda(), torch.from_numpy(g).cuda())
+    S = [np64(gb.query(plan, q)).reshape(s, d) for q in (gb.Q_SKETCH_X, gb.Q_SKETCH_Y)]
+    B = [np64(gb.query(plan, q)).reshape(d, k) for q in (gb.Q_WARM_U, gb.Q_WARM_V)]
+    for Z, b in zip(S, B):
+        assert np.max(np.abs(b.T @ (Z.T @ (Z @ b)) + lam * b.T @ b - np.eye(k))) < 1e-10
+    C = (S[0] @ B[0]).T @ (S[1] @ B[1])
+    sig = np.diag(C)
+    assert np.max(np.abs(C - np.diag(sig))) < 1e-10
+    assert np.all(sig > 0) and np.all(np.diff(sig) <= 0)
