@@ -289,6 +289,13 @@ __device__ void warp_jacobi(R* A, R* Q, R* lam, int n, int max_sweeps = 20, R to
   __syncwarp();
 }
 
+// blk_eig with the FP64 Jacobi above for what its refinement leaves coupled;
+// W: 3 n^2 doubles.
+__device__ void sym_eig(const double* T, double* Q, double* lam, int n, double* W) {
+  __shared__ double s_rot[100];
+  blk_eig(T, Q, lam, n, W, [&](double* A, double* J, double* l, int m) { blk_jacobi<double>(A, J, l, m, s_rot); });
+}
+
 // In-place Cholesky A = L L^T (lower; upper part zeroed).  Returns false
 // (uniformly in the block) if a pivot is not positive.
 __device__ bool blk_chol(double* A, int n) {
@@ -1314,7 +1321,7 @@ __global__ void __launch_bounds__(256) direction_kernel(DirArgs a) {
   } else {
     for (int e = tid; e < kk; e += blockDim.x) fA[e] = T2[e];
   }
-  blk_jacobi_f32(fA, fA2, fQ, fQ2, k);  // A' = J diag(lam) J^T, J in fQ (synchronizes first)
+  blk_jacobi_f32<2>(fA, fA2, fQ, fQ2, k);  // A' = J diag(lam) J^T, J in fQ (synchronizes first)
   if (warm) {
     for (int e = tid; e < kk; e += blockDim.x) {  // Q = Q0 J
       const int i = e / k, j = e - i * k;
@@ -1639,22 +1646,22 @@ struct RRArgs {
 // correlations; when that Gram is numerically rank deficient (eta ~ 0 or
 // nearly dependent on U: a pivot below 1e-12 of the largest diagonal) the
 // kernel falls back to m = k.
-__global__ void rr_kernel(RRArgs a) {
+__global__ void __launch_bounds__(256) rr_kernel(RRArgs a) {
   extern __shared__ double rsm[];
   DevState* st = a.st;
   // uniform over the CTA: a check runs at iterations every, 2 every, ... only
   if (a.check && (st->done || st->force_zero_step || st->iter == 0 || st->iter % a.every != 0)) return;
   const int k = a.k, k2 = 2 * k, mm0 = a.m0 * a.m0;
-  double* Gx = rsm;
+  double* Gx = rsm;        // Gx, Gy, T2: the eigendecomposition's scratch once the factors are inverted
   double* Gy = Gx + mm0;
-  double* C = Gy + mm0;
+  double* T2 = Gy + mm0;
+  double* C = T2 + mm0;
   double* Lxi = C + mm0;
   double* Lyi = Lxi + mm0;
   double* T1 = Lyi + mm0;
-  double* T2 = T1 + mm0;
-  double* Q = T2 + mm0;
+  double* Q = T1 + mm0;
   double* lam = Q + mm0;
-  double* rot = lam + 2 * kMaxK;
+  double* rot = lam + 2 * kMaxK;  // 100: pivots' square roots of both views
   double* phig = rot + 100;  // 2 x (2k)^2
   __shared__ int s_ok;
   const int nv = a.kind == kCCA ? 2 : 1;
@@ -1689,13 +1696,14 @@ __global__ void rr_kernel(RRArgs a) {
     __syncthreads();
     const double dxmax = T1[0], dymax = T1[1];
     __syncthreads();
-    bool ok = blk_chol(Gx, m);
-    if (a.kind == kCCA) ok = blk_chol(Gy, m) && ok;
+    // L^{-1} of both views (the pivots L_ii^2 stay on the diagonals of Gx, Gy)
+    bool ok = group_chol_inverse<256>(Gx, Lxi, rot, m, threadIdx.x, 0);
+    if (a.kind == kCCA) ok = group_chol_inverse<256>(Gy, Lyi, rot + 2 * kMaxK, m, threadIdx.x, 0) && ok;
     if (threadIdx.x == 0) {
       bool full = ok;
       for (int i = 0; i < m && full; ++i) {
-        if (Gx[i * m + i] * Gx[i * m + i] < 1e-12 * dxmax) full = false;
-        if (a.kind == kCCA && Gy[i * m + i] * Gy[i * m + i] < 1e-12 * dymax) full = false;
+        if (Gx[i * m + i] < 1e-12 * dxmax) full = false;
+        if (a.kind == kCCA && Gy[i * m + i] < 1e-12 * dymax) full = false;
       }
       s_ok = full ? 1 : (ok ? 2 : 0);  // 1: full rank, 2: factored but near rank deficient
     }
@@ -1713,9 +1721,7 @@ __global__ void rr_kernel(RRArgs a) {
     m = k;  // fall back to the point alone
     __syncthreads();
   }
-  blk_lower_inv(Gx, Lxi, m);
-  if (a.kind == kCCA) blk_lower_inv(Gy, Lyi, m);
-  else
+  if (a.kind != kCCA)
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) Lyi[e] = Lxi[e];
   __syncthreads();
   blk_mm(Lxi, false, C, false, T1, m, m, m, m, m);   // Lx^{-1} C
@@ -1729,7 +1735,7 @@ __global__ void rr_kernel(RRArgs a) {
     }
     __syncthreads();
   }
-  blk_jacobi(T1, Q, lam, m, rot);                    // right singular vectors (CCA) / eigvecs (FDA), descending
+  sym_eig(T1, Q, lam, m, Gx);                        // right singular vectors (CCA) / eigvecs (FDA), descending
   // the leading k: CCA sigma_i = ||C q_i||, left vectors a_i = C q_i / sigma_i
   if (a.kind == kCCA) {
     blk_mm(C, false, Q, false, T2, m, m, k, m, m);   // C Q[:, :k] (columns a_i sigma_i), m x k
@@ -2684,16 +2690,18 @@ __global__ void __launch_bounds__(kApplyRows * 2 * kMaxK) apply_small_kernel(dou
 
 // Rayleigh-Ritz of the power iteration: Bsmall = U^T (C V) (c x c), take the
 // top-k singular pairs: U A_k, V B_k in out (d x k each).
-__global__ void small_svd_kernel(const double* part, int nblk, int c, int k, double* rotU, double* rotV) {
+// (fp64: the plan is FP64, see small_chol64_kernel)
+__global__ void __launch_bounds__(256) small_svd_kernel(const double* part, int nblk, int c, int k, double* rotU, double* rotV, int fp64) {
   extern __shared__ double wsm[];
   double* Bm = wsm;
   double* T = Bm + c * c;
   double* Q = T + c * c;
   double* lam = Q + c * c;
-  double* rot = lam + 2 * kMaxK;
+  double* W = lam + 2 * kMaxK;  // 3 c^2, at least 100
   sum_blocks(part, nblk, c * c, Bm);
   blk_mm(Bm, true, Bm, false, T, c, c, c, c, c);  // B^T B
-  blk_jacobi(T, Q, lam, c, rot);                 // right singular vectors
+  if (fp64) blk_jacobi(T, Q, lam, c, W);         // right singular vectors
+  else sym_eig(T, Q, lam, c, W);
   blk_mm(Bm, false, Q, false, T, c, c, c, c, c);  // B Q = A Sigma
   for (int e = threadIdx.x; e < c * k; e += blockDim.x) {
     int r = e / k, i = e % k;
@@ -2723,14 +2731,15 @@ __global__ void transpose_kernel(const double* A, int r, int c, double* At) {
   At[(int64_t)j * r + i] = A[e];
 }
 
-__global__ void fda_warm_kernel(const double* part, int nblk, int l, int k, double* rot) {
+__global__ void __launch_bounds__(256) fda_warm_kernel(const double* part, int nblk, int l, int k, double* rot, int fp64) {
   extern __shared__ double fsm[];
   double* K = fsm;
   double* Q = K + l * l;
   double* lam = Q + l * l;
-  double* r = lam + kMaxClasses;
+  double* r = lam + kMaxClasses;  // 3 l^2 (l <= 40), else 100
   sum_blocks(part, nblk, l * l, K);
-  blk_jacobi(K, Q, lam, l, r);
+  if (l <= 40 && !fp64) sym_eig(K, Q, lam, l, r);
+  else blk_jacobi(K, Q, lam, l, r);
   for (int e = threadIdx.x; e < l * k; e += blockDim.x) {
     int q = e / k, i = e % k;
     rot[e] = lam[i] > 0 ? Q[q * l + i] / sqrt(lam[i]) : 0.0;
@@ -2879,9 +2888,9 @@ int warm_start(Plan& p, cudaStream_t st) {
       GB_CHECK_LAUNCH();
       double* rotU = small;
       double* rotV = small + c * k;
-      size_t sm2 = sizeof(double) * (3 * c * c + 2 * kMaxK + 100);
+      size_t sm2 = sizeof(double) * (3 * c * c + 2 * kMaxK + std::max(100, 3 * c * c));
       GB_CUDA(cudaFuncSetAttribute(small_svd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2));
-      small_svd_kernel<<<1, 256, sm2, st>>>(part, a.nblk, c, k, rotU, rotV);
+      small_svd_kernel<<<1, 256, sm2, st>>>(part, a.nblk, c, k, rotU, rotV, p.dtype == GBCCA_FP64);
       GB_CHECK_LAUNCH();
       // whitened top-k vectors, then back through R^{-1}
       thin_apply_kernel<<<ceil_div(dx, 128), 128, 0, st>>>(Ub, dx, c, rotU, k, x.wsT);
@@ -2918,9 +2927,9 @@ int warm_start(Plan& p, cudaStream_t st) {
     thin_gram_kernel<<<dim3(a.nblk, 1), 256, smem, st>>>(a);
     GB_CHECK_LAUNCH();
     double* rot = p.phigram;  // l x k
-    size_t sm2 = sizeof(double) * (2 * l * l + kMaxClasses + 100);
+    size_t sm2 = sizeof(double) * (2 * l * l + kMaxClasses + (l <= 40 ? std::max(100, 3 * l * l) : 100));
     GB_CUDA(cudaFuncSetAttribute(fda_warm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2));
-    fda_warm_kernel<<<1, 256, sm2, st>>>(p.crosspart, a.nblk, l, k, rot);
+    fda_warm_kernel<<<1, 256, sm2, st>>>(p.crosspart, a.nblk, l, k, rot, p.dtype == GBCCA_FP64);
     GB_CHECK_LAUNCH();
     double* Wwh = p.ws + 2 * (int64_t)d * l;  // d x k
     thin_apply_kernel<<<ceil_div(d, 128), 128, 0, st>>>(Gt, d, l, rot, k, Wwh);

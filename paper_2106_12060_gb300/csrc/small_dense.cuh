@@ -92,7 +92,7 @@ __device__ bool group_chol_inverse(double* A, double* Li, double* rs, int n, int
 }
 
 // Symmetric eigendecomposition in FP32 by parallel (round-robin ordered)
-// two-sided Jacobi, n <= 20, by all 256 threads of the CTA: on return the
+// two-sided Jacobi, n * n <= 256 kI, by all 256 threads of the CTA: on return the
 // diagonal of *A holds the eigenvalues (unsorted) and the columns of *Q the
 // eigenvectors.  A2 and Q2 are second buffers; the pointers come back swapped
 // as the last round left them.  Every warp forms all rotations of a round in
@@ -118,12 +118,13 @@ __device__ __forceinline__ void jacobi_role(int i, int r, int m, int np, int& pa
   }
 }
 
+template <int kI>
 __device__ __forceinline__ void blk_jacobi_f32(float*& A, float*& A2, float*& Q, float*& Q2, int n) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int m = n + (n & 1), np = m / 2;
-  int ei[2], ej[2];
+  int ei[kI], ej[kI];
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
+  for (int u = 0; u < kI; ++u) {
     const int e = tid + 256 * u;
     ei[u] = e / n;
     ej[u] = e - ei[u] * n;
@@ -152,9 +153,9 @@ __device__ __forceinline__ void blk_jacobi_f32(float*& A, float*& A2, float*& Q,
         }
       }
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < kI; ++u) {
         const bool in = ei[u] < n;
-        if (u == 1 && n * n <= 256) break;  // uniform
+        if (n * n <= 256 * u) break;  // uniform
         const int i = in ? ei[u] : 0, j = in ? ej[u] : 0;
         int pi, qi, pj, qj;
         jacobi_role(i, r, m, np, pi, qi);
@@ -183,6 +184,153 @@ __device__ __forceinline__ void blk_jacobi_f32(float*& A, float*& A2, float*& Q,
     // every warp formed the same rotations: the verdict is uniform
     if (!__any_sync(0xffffffffu, big)) break;
   }
+}
+
+// Eigendecomposition of a symmetric FP64 matrix T (n x n, n <= 40, row-major
+// in shared memory, unchanged) by all 256 threads: eigenvalues descending in
+// lam, eigenvectors in the columns of Q.  W is scratch of 3 n^2 doubles.
+//
+// FP32 Jacobi gives vectors good to ~1e-6, which two steps of the refinement
+// of Ogita and Aishima (Iterative refinement for symmetric eigenvalue
+// decomposition, 2018; quadratically convergent, products of n x n matrices
+// only) bring to FP64: with R = I - Q^T Q, S = Q^T T Q and lam_j = S_jj /
+// (1 - R_jj), Q += Q E, E_ij = (S_ij + lam_j R_ij) / (lam_j - lam_i) for
+// separated pairs and R_ij / 2 for the others.  The result is accepted when
+// Q^T T Q is diagonal to 1e-13 of its diagonal; clusters that the refinement
+// leaves coupled are finished by FP64 Jacobi sweeps on that nearly diagonal
+// matrix.  (FP64 Jacobi from the start is bound by the FP64 rate of one SM,
+// divisions and square roots above all: 390 us for n = 20.)
+template <typename F>
+__device__ void blk_eig(const double* T, double* Q, double* lam, int n, double* W, F jacobi64) {
+  const int tid = threadIdx.x, nn = n * n;
+  double* S = W;
+  double* E = W + nn;
+  double* Y = W + 2 * nn;
+  __shared__ double s_red[2][8];
+  __shared__ double s_lam[40];
+  __shared__ int s_rank[40];
+  {
+    float* A = reinterpret_cast<float*>(W);
+    float *A2 = A + nn, *Qf = A2 + nn, *Q2 = Qf + nn;
+    // scaled by the largest diagonal entry into the FP32 range
+    double mx = 0;
+    for (int i = 0; i < n; ++i) mx = fmax(mx, fabs(T[i * n + i]));
+    const double inv = mx > 0 ? 1.0 / mx : 1.0;
+    for (int e = tid; e < nn; e += 256) A[e] = (float)(T[e] * inv);
+    if (nn <= 512) blk_jacobi_f32<2>(A, A2, Qf, Q2, n);
+    else blk_jacobi_f32<7>(A, A2, Qf, Q2, n);
+    for (int e = tid; e < nn; e += 256) Q[e] = (double)Qf[e];
+  }
+  __syncthreads();
+  auto form = [&]() {  // Y = T Q; S = Q^T Y
+    for (int e = tid; e < nn; e += 256) {
+      const int i = e / n, j = e - i * n;
+      double s = 0;
+#pragma unroll 4
+      for (int q = 0; q < n; ++q) s += T[i * n + q] * Q[q * n + j];
+      Y[e] = s;
+    }
+    __syncthreads();
+    for (int e = tid; e < n * (n + 1) / 2; e += 256) {
+      int j = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+      while ((j + 1) * (j + 2) / 2 <= e) ++j;
+      while (j * (j + 1) / 2 > e) --j;
+      const int i = e - j * (j + 1) / 2;
+      double s = 0;
+#pragma unroll 4
+      for (int q = 0; q < n; ++q) s += Q[q * n + i] * Y[q * n + j];
+      S[i * n + j] = s;
+      S[j * n + i] = s;
+    }
+    __syncthreads();
+  };
+  // sums of squares of S off and on the diagonal
+  auto norms = [&](double& off, double& dg) {
+    double o = 0, d = 0;
+    for (int e = tid; e < nn; e += 256) {
+      const double v = S[e] * S[e];
+      if (e / n == e % n) d += v;
+      else o += v;
+    }
+    o = warp_sum(o);
+    d = warp_sum(d);
+    if ((tid & 31) == 0) {
+      s_red[0][tid >> 5] = o;
+      s_red[1][tid >> 5] = d;
+    }
+    __syncthreads();
+    off = dg = 0;
+    for (int q = 0; q < 8; ++q) {
+      off += s_red[0][q];
+      dg += s_red[1][q];
+    }
+    __syncthreads();
+  };
+  double off = 0, dg = 0;
+  for (int step = 0; step < 2; ++step) {
+    form();
+    norms(off, dg);
+    // R = I - Q^T Q in place of Y
+    for (int e = tid; e < nn; e += 256) {
+      const int i = e / n, j = e - i * n;
+      double s = i == j ? 1.0 : 0.0;
+#pragma unroll 4
+      for (int q = 0; q < n; ++q) s -= Q[q * n + i] * Q[q * n + j];
+      Y[e] = s;
+    }
+    __syncthreads();
+    if (tid < n) s_lam[tid] = S[tid * n + tid] / (1.0 - Y[tid * n + tid]);
+    __syncthreads();
+    // pairs closer than the coupling are left to the orthogonalization
+    const double delta = 2.0 * (sqrt(off) + 1e-15 * sqrt(dg));
+    for (int e = tid; e < nn; e += 256) {
+      const int i = e / n, j = e - i * n;
+      const double gap = s_lam[j] - s_lam[i];
+      E[e] = (i != j && fabs(gap) > delta) ? (S[e] + s_lam[j] * Y[e]) / gap : 0.5 * Y[e];
+    }
+    __syncthreads();
+    for (int e = tid; e < nn; e += 256) {  // Y = Q + Q E
+      const int i = e / n, j = e - i * n;
+      double s = Q[e];
+#pragma unroll 4
+      for (int q = 0; q < n; ++q) s += Q[i * n + q] * E[q * n + j];
+      Y[e] = s;
+    }
+    __syncthreads();
+    for (int e = tid; e < nn; e += 256) Q[e] = Y[e];
+    __syncthreads();
+  }
+  form();
+  norms(off, dg);
+  if (!(off <= 1e-26 * dg)) {
+    // coupled clusters: S = J diag J^T by FP64 Jacobi, Q <- Q J
+    jacobi64(S, E, s_lam, n);  // S destroyed, J in E
+    __syncthreads();
+    for (int e = tid; e < nn; e += 256) {
+      const int i = e / n, j = e - i * n;
+      double s = 0;
+      for (int q = 0; q < n; ++q) s += Q[i * n + q] * E[q * n + j];
+      Y[e] = s;
+    }
+  } else {
+    if (tid < n) s_lam[tid] = S[tid * n + tid];
+    for (int e = tid; e < nn; e += 256) Y[e] = Q[e];
+  }
+  __syncthreads();
+  // descending order (ties keep the lower index first)
+  if (tid < n) {
+    const double l = s_lam[tid];
+    int r = 0;
+    for (int j = 0; j < n; ++j) {
+      const double o = s_lam[j];
+      if (o > l || (o == l && j < tid)) ++r;
+    }
+    s_rank[tid] = r;
+    lam[r] = l;
+  }
+  __syncthreads();
+  for (int e = tid; e < nn; e += 256) Q[(e / n) * n + s_rank[e % n]] = Y[e];
+  __syncthreads();
 }
 
 }  // namespace gbcca
