@@ -109,7 +109,7 @@ int alloc_plan(Plan* p) {
     GB_TRY(dalloc(&p->perm, p->s));
     size_t tsz = p->dtype == GBCCA_FP64 ? sizeof(double) : sizeof(float);
     void* t = nullptr;
-    cudaError_t e = counted_malloc(&t, tsz * (size_t)p->n_pad * dmax);
+    cudaError_t e = counted_malloc(&t, tsz * (size_t)p->n_pad * (size_t)((dmax + 31) / 32 * 32));
     if (e != cudaSuccess) {
       cudaGetLastError();
       set_last_error("SRHT scratch allocation failed");

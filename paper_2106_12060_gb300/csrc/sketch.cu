@@ -312,55 +312,7 @@ int countsketch_apply(Plan& p, int view, bool center, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------- SRHT
-constexpr int kLoadBatch = 8;
-
-// Unnormalized Walsh-Hadamard transform of one column of length N (32 <= N
-// <= 1024, power of two) held in shared memory with row stride `stride`, by
-// one warp: lane l holds rows l + 32 t; butterflies of span < 32 go across
-// lanes (shuffles), larger spans within the lane's registers.
-template <typename T, int NT>
-__device__ __forceinline__ void fwht_warp_col_n(T* col, int stride) {
-  const int lane = threadIdx.x & 31;
-  T v[NT];
-#pragma unroll
-  for (int t = 0; t < NT; ++t) v[t] = col[(lane + 32 * t) * stride];
-#pragma unroll
-  for (int h = 1; h < 32; h <<= 1) {
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const T x = v[t];
-      const T y = __shfl_xor_sync(0xffffffffu, x, h);
-      v[t] = (lane & h) ? (y - x) : (x + y);
-    }
-  }
-#pragma unroll
-  for (int hb = 1; hb < NT; hb <<= 1) {  // span 32 hb rows = hb register slots
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      if ((t & hb) == 0) {
-        const T a = v[t], b = v[t + hb];
-        v[t] = a + b;
-        v[t + hb] = a - b;
-      }
-    }
-  }
-#pragma unroll
-  for (int t = 0; t < NT; ++t) col[(lane + 32 * t) * stride] = v[t];
-}
-
-template <typename T>
-__device__ __forceinline__ void fwht_warp_col(T* col, int stride, int N) {
-  switch (N >> 5) {
-    case 1: fwht_warp_col_n<T, 1>(col, stride); break;
-    case 2: fwht_warp_col_n<T, 2>(col, stride); break;
-    case 4: fwht_warp_col_n<T, 4>(col, stride); break;
-    case 8: fwht_warp_col_n<T, 8>(col, stride); break;
-    case 16: fwht_warp_col_n<T, 16>(col, stride); break;
-    default: fwht_warp_col_n<T, 32>(col, stride); break;
-  }
-}
-
-// Transform of length N < 32 (tiny n): one thread per column
+// Transform of length N < 64 (tiny n): one thread per column
 template <typename T>
 __device__ __forceinline__ void fwht_thread_col(T* col, int stride, int N) {
   for (int h = 1; h < N; h <<= 1)
@@ -372,109 +324,172 @@ __device__ __forceinline__ void fwht_thread_col(T* col, int stride, int N) {
       }
 }
 
-// Stage 1: per block of N1 consecutive rows and CB = 32 columns, D Z
-// (signs, and the class means for LDA) then the N1-point transform along the
-// rows of each column, written to the intermediate buffer.  Tile in shared
-// memory as [N1][33] (padded: column reads are conflict-free); FP32 data is
-// converted on FP32 units.
+// The intermediate between the stages is stored as tiles of 32 columns,
+// [residue a1][column block][row block][32], so that stage 2 reads one
+// contiguous tile and stage 1's 128-byte rows of neighbouring row blocks lie
+// side by side.
+
+// Walsh-Hadamard transform of N = 32 NW rows (NW = 2 .. 32 warps) of 32 columns,
+// lane = column: warp w holds rows 32 w .. 32 w + 31 in registers (spans 1 ..
+// 16), the tile is exchanged once through shared memory, and the same warp
+// then holds the residues w (32 / NW) .. of the row index modulo 32, NW rows
+// each (spans 32 .. N / 2): about nine additions and two shared-memory
+// accesses per element.  (A column per warp with shuffles for the first five
+// levels and two passes over shared memory was bound by its instructions:
+// 437 us a view for 262144 x 512 BF16, 1.8 TB/s.)  buf: N x 32; on return it
+// holds the transform.
+template <typename T, int NW>
+__device__ __forceinline__ void fwht_tile(T (&v)[32], T* buf) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int h = 1; h < 32; h <<= 1) {
+#pragma unroll
+    for (int t = 0; t < 32; ++t)
+      if ((t & h) == 0) {
+        const T a = v[t], b = v[t + h];
+        v[t] = a + b;
+        v[t + h] = a - b;
+      }
+  }
+#pragma unroll
+  for (int t = 0; t < 32; ++t) buf[(32 * w + t) * 32 + lane] = v[t];
+  __syncthreads();
+  constexpr int NJ = 32 / NW;  // residues of this warp: j = w NJ + q, rows j + 32 m
+#pragma unroll
+  for (int q = 0; q < NJ; ++q) {
+    T u[NW];
+#pragma unroll
+    for (int m = 0; m < NW; ++m) u[m] = buf[(w * NJ + q + 32 * m) * 32 + lane];
+#pragma unroll
+    for (int h = 1; h < NW; h <<= 1) {
+#pragma unroll
+      for (int m = 0; m < NW; ++m)
+        if ((m & h) == 0) {
+          const T a = u[m], b = u[m + h];
+          u[m] = a + b;
+          u[m + h] = a - b;
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < NW; ++m) buf[(w * NJ + q + 32 * m) * 32 + lane] = u[m];
+  }
+  __syncthreads();
+}
+
+// One element of D Z (signs, and the class means for LDA) in the working type.
 template <typename Tin, typename T>
-__global__ void __launch_bounds__(512)
-srht_stage1_kernel(const Tin* __restrict__ Z, int64_t ld, int64_t n, int d, int N1, const int8_t* __restrict__ sg,
+__device__ __forceinline__ T signed_value(Tin z, int g, const int32_t* labels, const double* means, int64_t row, int d,
+                                          int col) {
+  if (labels != nullptr) {
+    const double x = to_f64(z) - means[(int64_t)labels[row] * d + col];
+    return (T)(g < 0 ? -x : x);
+  }
+  const T x = to_work<T>(z);
+  return g < 0 ? -x : x;
+}
+
+// Stage 1: per block of N1 = 32 NW consecutive rows and 32 columns, D Z then
+// the N1-point transform along the rows.  All 32 loads of a thread are in
+// flight together.
+template <typename Tin, typename T, int NW>
+__global__ void __launch_bounds__(32 * NW)
+srht_stage1_kernel(const Tin* __restrict__ Z, int64_t ld, int64_t n, int d, const int8_t* __restrict__ sg,
                    const int32_t* __restrict__ labels, const double* __restrict__ means, T* __restrict__ Tmid) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf = reinterpret_cast<T*>(smem_raw);
-  constexpr int CB = 32, LD = 33;
-  const int64_t i2 = blockIdx.y;   // column blocks of one row block run next to each other
-  const int c0 = blockIdx.x * CB;
-  // loads batched (kLoadBatch in flight per thread), then signs and stores
-  for (int base = 0; base < N1 * CB; base += blockDim.x * kLoadBatch) {
-    Tin z[kLoadBatch];
-    int8_t g[kLoadBatch];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t i2 = blockIdx.y, N2 = gridDim.y;
+  const int cb = blockIdx.x, ncb = gridDim.x, col = 32 * cb + lane;
+  const int64_t row0 = i2 * 32 * NW + 32 * w;
+  // the signs of this warp's 32 rows (a zero drops the row)
+  const int g = row0 + lane < n ? (int)sg[row0 + lane] : 0;
+  const unsigned neg = __ballot_sync(0xffffffffu, g < 0), use = __ballot_sync(0xffffffffu, g != 0);
+  Tin z[32];
+  const Tin* src = Z + row0 * ld + col;
 #pragma unroll
-    for (int u = 0; u < kLoadBatch; ++u) {
-      const int e = base + threadIdx.x + blockDim.x * u;
-      const int r = e >> 5, c = e & 31;
-      const int64_t row = i2 * N1 + r;
-      const bool in = e < N1 * CB && row < n && c0 + c < d;
-      z[u] = in ? Z[row * ld + c0 + c] : Tin(0.0f);
-      g[u] = in ? sg[row] : int8_t(0);
-    }
+  for (int t = 0; t < 32; ++t) z[t] = (use >> t & 1) && col < d ? src[(int64_t)t * ld] : Tin(0.0f);
+  T v[32];
 #pragma unroll
-    for (int u = 0; u < kLoadBatch; ++u) {
-      const int e = base + threadIdx.x + blockDim.x * u;
-      if (e >= N1 * CB) continue;
-      const int r = e >> 5, c = e & 31;
-      const int64_t row = i2 * N1 + r;
-      T val = T(0);
-      if (g[u] != 0) {
-        if (labels != nullptr) {
-          const double x = to_f64(z[u]) - means[(int64_t)labels[row] * d + c0 + c];
-          val = (T)(g[u] < 0 ? -x : x);
-        } else {
-          const T x = to_work<T>(z[u]);
-          val = g[u] < 0 ? -x : x;
-        }
-      }
-      buf[r * LD + c] = val;
-    }
+  for (int t = 0; t < 32; ++t)
+    v[t] = (use >> t & 1) && col < d
+               ? signed_value<Tin, T>(z[t], (neg >> t & 1) ? -1 : 1, labels, means, row0 + t, d, col)
+               : T(0);
+  fwht_tile<T, NW>(v, buf);
+  // row r of the block is residue a1 = r
+#pragma unroll
+  for (int t = 0; t < 32; ++t) {
+    const int64_t r = 32 * w + t;
+    Tmid[((r * ncb + cb) * N2 + i2) * 32 + lane] = buf[r * 32 + lane];
   }
-  __syncthreads();
-  if (N1 >= 32) {
-    for (int c = threadIdx.x >> 5; c < CB; c += blockDim.x >> 5) fwht_warp_col<T>(buf + c, LD, N1);
-  } else if (threadIdx.x < CB) {
-    fwht_thread_col<T>(buf + threadIdx.x, LD, N1);
+}
+
+// The same for short blocks (N1 < 64): one thread per column.
+template <typename Tin, typename T>
+__global__ void srht_stage1_small_kernel(const Tin* __restrict__ Z, int64_t ld, int64_t n, int d, int N1,
+                                         const int8_t* __restrict__ sg, const int32_t* __restrict__ labels,
+                                         const double* __restrict__ means, T* __restrict__ Tmid) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* buf = reinterpret_cast<T*>(smem_raw);
+  const int lane = threadIdx.x;
+  const int64_t i2 = blockIdx.y, N2 = gridDim.y;
+  const int cb = blockIdx.x, ncb = gridDim.x, col = 32 * cb + lane;
+  for (int r = 0; r < N1; ++r) {
+    const int64_t row = i2 * N1 + r;
+    const int g = row < n ? (int)sg[row] : 0;
+    buf[r * 32 + lane] =
+        g != 0 && col < d ? signed_value<Tin, T>(Z[row * ld + col], g, labels, means, row, d, col) : T(0);
   }
-  __syncthreads();
-  // intermediate row r * N2 + i2: stage 2 then reads N2 consecutive rows
-  const int64_t N2 = gridDim.y;
-  for (int e = threadIdx.x; e < N1 * CB; e += blockDim.x) {
-    const int r = e >> 5, c = e & 31;
-    if (c0 + c < d) Tmid[((int64_t)r * N2 + i2) * d + c0 + c] = buf[r * LD + c];
+  fwht_thread_col<T>(buf + lane, 32, N1);
+  for (int r = 0; r < N1; ++r) Tmid[(((int64_t)r * ncb + cb) * N2 + i2) * 32 + lane] = buf[r * 32 + lane];
+}
+
+// Sampled rows of the transform of residue a1: SZ[j] = scale * row (rows[j] >> m1).
+template <typename T>
+__device__ __forceinline__ void srht_pick(const T* buf, int d, int cb, int a1, int nsel, int m1, const int32_t* off1,
+                                          const int32_t* list, const int32_t* rows, double scale, double* SZ) {
+  for (int e = threadIdx.x; e < nsel * 32; e += blockDim.x) {
+    const int q = e >> 5, c = 32 * cb + (e & 31);
+    const int j = list[off1[a1] + q];
+    if (c < d) SZ[(int64_t)j * d + c] = scale * (double)buf[(rows[j] >> m1) * 32 + (e & 31)];
   }
 }
 
 // Stage 2: for one residue a1 of the low m1 row bits, the N2-point transform
 // across the row blocks of each column, kept only at the sampled rows and
 // scaled by sqrt(n'/s) / sqrt(n') = 1 / sqrt(s) (App. A).
-template <typename T>
-__global__ void __launch_bounds__(512)
-srht_stage2_kernel(const T* __restrict__ Tmid, int d, int N1, int N2, int m1, const int32_t* __restrict__ off1,
+template <typename T, int NW>
+__global__ void __launch_bounds__(32 * NW)
+srht_stage2_kernel(const T* __restrict__ Tmid, int d, int m1, const int32_t* __restrict__ off1,
                    const int32_t* __restrict__ list, const int32_t* __restrict__ rows, double scale,
                    double* __restrict__ SZ) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf = reinterpret_cast<T*>(smem_raw);
-  constexpr int CB = 32, LD = 33;
-  const int a1 = blockIdx.y;
-  const int c0 = blockIdx.x * CB;
+  const int a1 = blockIdx.y, cb = blockIdx.x, ncb = gridDim.x;
   const int nsel = off1[a1 + 1] - off1[a1];
   if (nsel == 0) return;
-  for (int base = 0; base < N2 * CB; base += blockDim.x * kLoadBatch) {
-    T v[kLoadBatch];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const T* src = Tmid + ((int64_t)a1 * ncb + cb) * (32 * NW) * 32;
+  T v[32];
 #pragma unroll
-    for (int u = 0; u < kLoadBatch; ++u) {
-      const int e = base + threadIdx.x + blockDim.x * u;
-      const int r = e >> 5, c = e & 31;
-      v[u] = (e < N2 * CB && c0 + c < d) ? Tmid[((int64_t)a1 * N2 + r) * d + c0 + c] : T(0);
-    }
-#pragma unroll
-    for (int u = 0; u < kLoadBatch; ++u) {
-      const int e = base + threadIdx.x + blockDim.x * u;
-      if (e < N2 * CB) buf[(e >> 5) * LD + (e & 31)] = v[u];
-    }
-  }
-  __syncthreads();
-  if (N2 >= 32) {
-    for (int c = threadIdx.x >> 5; c < CB; c += blockDim.x >> 5) fwht_warp_col<T>(buf + c, LD, N2);
-  } else if (threadIdx.x < CB) {
-    fwht_thread_col<T>(buf + threadIdx.x, LD, N2);
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < nsel * CB; e += blockDim.x) {
-    const int q = e >> 5, c = e & 31;
-    const int j = list[off1[a1] + q];
-    const int a2 = rows[j] >> m1;
-    if (c0 + c < d) SZ[(int64_t)j * d + c0 + c] = scale * (double)buf[a2 * LD + c];
-  }
+  for (int t = 0; t < 32; ++t) v[t] = src[(32 * w + t) * 32 + lane];
+  fwht_tile<T, NW>(v, buf);
+  srht_pick(buf, d, cb, a1, nsel, m1, off1, list, rows, scale, SZ);
+}
+
+template <typename T>
+__global__ void srht_stage2_small_kernel(const T* __restrict__ Tmid, int d, int N2, int m1,
+                                         const int32_t* __restrict__ off1, const int32_t* __restrict__ list,
+                                         const int32_t* __restrict__ rows, double scale, double* __restrict__ SZ) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* buf = reinterpret_cast<T*>(smem_raw);
+  const int a1 = blockIdx.y, cb = blockIdx.x, ncb = gridDim.x;
+  const int nsel = off1[a1 + 1] - off1[a1];
+  if (nsel == 0) return;
+  const T* src = Tmid + ((int64_t)a1 * ncb + cb) * N2 * 32;
+  for (int r = 0; r < N2; ++r) buf[r * 32 + threadIdx.x] = src[r * 32 + threadIdx.x];
+  fwht_thread_col<T>(buf + threadIdx.x, 32, N2);
+  __syncwarp();
+  srht_pick(buf, d, cb, a1, nsel, m1, off1, list, rows, scale, SZ);
 }
 
 // group the sampled rows by their low m1 bits (order within a group is free:
@@ -517,9 +532,29 @@ __global__ void srht_group_kernel(const int32_t* __restrict__ rows, int64_t s, i
   }
 }
 
+template <typename Tin, typename T, int NW>
+int srht_stage1(const View& v, const Plan& p, int N2, const int32_t* lab, T* Tmid, cudaStream_t st) {
+  const size_t sm = sizeof(T) * 32 * NW * 32;
+  auto k1 = srht_stage1_kernel<Tin, T, NW>;
+  GB_CUDA(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  k1<<<dim3(ceil_div(v.d, 32), N2), 32 * NW, sm, st>>>((const Tin*)v.Z, v.ld, p.n, v.d, p.g, lab, p.means, Tmid);
+  GB_CHECK_LAUNCH();
+  return GBCCA_OK;
+}
+
+template <typename T, int NW>
+int srht_stage2(const View& v, const Plan& p, int N1, int m1, const int32_t* off1, const int32_t* list, const T* Tmid,
+                cudaStream_t st) {
+  const size_t sm = sizeof(T) * 32 * NW * 32;
+  auto k2 = srht_stage2_kernel<T, NW>;
+  GB_CUDA(cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  k2<<<dim3(ceil_div(v.d, 32), N1), 32 * NW, sm, st>>>(Tmid, v.d, m1, off1, list, p.h, 1.0 / sqrt((double)p.s), v.SZ);
+  GB_CHECK_LAUNCH();
+  return GBCCA_OK;
+}
+
 template <typename Tin, typename T>
 int srht_run(Plan& p, View& v, cudaStream_t st) {
-  constexpr int CB = 32;
   int m = 0;
   while ((1ll << m) < p.n_pad) ++m;
   const int m1 = std::min(m, 9), m2 = m - m1;
@@ -530,11 +565,16 @@ int srht_run(Plan& p, View& v, cudaStream_t st) {
   }
   T* Tmid = reinterpret_cast<T*>(p.srht_T);
   const int32_t* lab = p.kind == kLDA ? p.labels : nullptr;
-  size_t sm1 = sizeof(T) * N1 * (CB + 1);
-  auto k1 = srht_stage1_kernel<Tin, T>;
-  GB_CUDA(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
-  k1<<<dim3(ceil_div(v.d, CB), N2), 512, sm1, st>>>((const Tin*)v.Z, v.ld, p.n, v.d, N1, p.g, lab, p.means, Tmid);
-  GB_CHECK_LAUNCH();
+  switch (N1) {
+    case 64: GB_TRY((srht_stage1<Tin, T, 2>(v, p, N2, lab, Tmid, st))); break;
+    case 128: GB_TRY((srht_stage1<Tin, T, 4>(v, p, N2, lab, Tmid, st))); break;
+    case 256: GB_TRY((srht_stage1<Tin, T, 8>(v, p, N2, lab, Tmid, st))); break;
+    case 512: GB_TRY((srht_stage1<Tin, T, 16>(v, p, N2, lab, Tmid, st))); break;
+    default:
+      srht_stage1_small_kernel<Tin, T><<<dim3(ceil_div(v.d, 32), N2), 32, sizeof(T) * 32 * N1, st>>>(
+          (const Tin*)v.Z, v.ld, p.n, v.d, N1, p.g, lab, p.means, Tmid);
+      GB_CHECK_LAUNCH();
+  }
   int32_t* cnt = p.cs_tab;
   int32_t* off1 = p.cs_off;
   int32_t* list = p.perm;
@@ -545,11 +585,15 @@ int srht_run(Plan& p, View& v, cudaStream_t st) {
   GB_CHECK_LAUNCH();
   srht_group_kernel<<<ceil_div(p.s, 256), 256, 0, st>>>(p.h, p.s, N1, cnt, off1, list, 2);
   GB_CHECK_LAUNCH();
-  size_t sm2 = sizeof(T) * N2 * (CB + 1);
-  auto k2 = srht_stage2_kernel<T>;
-  GB_CUDA(cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2));
-  k2<<<dim3(ceil_div(v.d, CB), N1), 512, sm2, st>>>(Tmid, v.d, N1, N2, m1, off1, list, p.h,
-                                                     1.0 / sqrt((double)p.s), v.SZ);
+  switch (N2) {
+    case 64: return srht_stage2<T, 2>(v, p, N1, m1, off1, list, Tmid, st);
+    case 128: return srht_stage2<T, 4>(v, p, N1, m1, off1, list, Tmid, st);
+    case 256: return srht_stage2<T, 8>(v, p, N1, m1, off1, list, Tmid, st);
+    case 512: return srht_stage2<T, 16>(v, p, N1, m1, off1, list, Tmid, st);
+    case 1024: return srht_stage2<T, 32>(v, p, N1, m1, off1, list, Tmid, st);
+  }
+  srht_stage2_small_kernel<T><<<dim3(ceil_div(v.d, 32), N1), 32, sizeof(T) * 32 * N2, st>>>(
+      Tmid, v.d, N2, m1, off1, list, p.h, 1.0 / sqrt((double)p.s), v.SZ);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }

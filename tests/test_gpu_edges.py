@@ -327,3 +327,29 @@ def test_warm_start_blocks_f32(gb, d, k):
     sig = np.diag(C)
     assert np.max(np.abs(C - np.diag(sig))) < 1e-10
     assert np.all(sig > 0) and np.all(np.diff(sig) <= 0)
+
+
+@pytest.mark.parametrize("dt", ["bf16", "f32", "f64"])
+@pytest.mark.parametrize("n,d,s", [(3, 1, 2), (40, 33, 40), (100, 31, 60), (700, 5, 300), (5000, 65, 500),
+                                   (40000, 33, 999), (270000, 3, 2000)])
+def test_srht_sizes(gb, dt, n, d, s):
+    """The SRHT at every class of its two stages' lengths (up to 2^9 and 2^10),
+    ragged columns and padding rows.  A sample is a sum of +-x over the column
+    by log2(n') levels of additions, in FP32 (BF16/FP32 data) or FP64."""
+    import torch
+    from oracle.sketch import srht_apply
+    from synth import srht_draws
+    n_pad = 1 << max(int(n - 1).bit_length(), 0)
+    if dt == "f64" and n_pad > 1 << 18:
+        pytest.skip("more than the FP64 transform takes")
+    tdt = {"bf16": torch.bfloat16, "f32": torch.float32, "f64": torch.float64}[dt]
+    s = min(s, n_pad)
+    X = torch.from_numpy(np.random.default_rng(n).standard_normal((n, d))).to(tdt).double().numpy()
+    D, rows = srht_draws(n_pad, s, seed=3)
+    gamma = (np.log2(n_pad) + 4) * (2.0 ** -53 if dt == "f64" else 2.0 ** -24)
+    ref = np.broadcast_to(np.abs(X).sum(0) / np.sqrt(s), (s, d))
+    for x in _layouts(X, tdt)[:3]:
+        plan = gb.cca_plan(n, d, d, 1, dt, gb.default_options(sketch=gb.SRHT, s=s, warm_start=0))
+        gb.cca_precondition(plan, x, x, 1e3, 1e3, torch.from_numpy(rows).cuda(), torch.from_numpy(D).cuda())
+        got = np64(gb.query(plan, gb.Q_SKETCH_X)).reshape(s, d)
+        assert bound_ratio(got, srht_apply(X, D, rows), ref, gamma) <= 1.0
