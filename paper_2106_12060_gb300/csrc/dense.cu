@@ -10,6 +10,7 @@
 #include <string>
 
 #include "plan.h"
+#include "small_dense.cuh"
 
 namespace gbcca {
 
@@ -632,28 +633,101 @@ __global__ void __launch_bounds__(32 * kTrsmRows) chol_trsm_kernel(double* A, in
   if (lane < nb) A[(int64_t)row * d + o + lane] = x;
 }
 
-// trailing update A[I, J] -= A[I, p] A[J, p]^T for block pairs I >= J > p.
-__global__ void chol_syrk_kernel(double* A, int d, int p) {
-  const int o = p * kNB, nb = min(kNB, d - o);
-  int I = blockIdx.y + p + 1, J = blockIdx.x + p + 1;
-  if (J > I) return;
-  __shared__ double a[kNB][kNB + 1], b[kNB][kNB + 1];
-  const int i0 = I * kNB, j0 = J * kNB;
-  for (int e = threadIdx.x; e < kNB * kNB; e += blockDim.x) {
-    int r = e / kNB, c = e % kNB;
-    a[r][c] = (i0 + r < d && c < nb) ? A[(int64_t)(i0 + r) * d + o + c] : 0.0;
-    b[r][c] = (j0 + r < d && c < nb) ? A[(int64_t)(j0 + r) * d + o + c] : 0.0;
+// Tile t of the trailing matrix's lower triangle in 16 x 16 tiles (row-major
+// order: t = ti (ti + 1) / 2 + tj), A[I, J] -= A[I, p] A[J, p]^T with p the panel
+// of 32 columns at `o`: one entry per thread, its 32 terms in order.  (On 32 x
+// 32 tiles a step had few CTAs with 10 us of FP64 each.)
+constexpr int kUT = 16;
+__device__ __forceinline__ void chol_update_tile(double* A, int d, int o, int t, double (*a)[kNB + 1],
+                                                 double (*b)[kNB + 1]) {
+  int ti = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+  while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+  while (ti * (ti + 1) / 2 > t) --ti;
+  const int tj = t - ti * (ti + 1) / 2;
+  const int i0 = o + kNB + kUT * ti, j0 = o + kNB + kUT * tj;
+  for (int e = threadIdx.x; e < kUT * kNB; e += blockDim.x) {
+    const int r = e / kNB, c = e % kNB;
+    a[r][c] = i0 + r < d ? A[(int64_t)(i0 + r) * d + o + c] : 0.0;
+    b[r][c] = j0 + r < d ? A[(int64_t)(j0 + r) * d + o + c] : 0.0;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < kNB * kNB; e += blockDim.x) {
-    int r = e / kNB, c = e % kNB;
-    int i = i0 + r, j = j0 + c;
-    if (i >= d || j >= d || j > i) continue;
-    double s = 0;
+  const int r = threadIdx.x / kUT, c = threadIdx.x % kUT;
+  const int i = i0 + r, j = j0 + c;
+  if (i >= d || j > i) return;
+  double s = 0;
 #pragma unroll 8
-    for (int q = 0; q < kNB; ++q) s += a[r][q] * b[c][q];
-    A[(int64_t)i * d + j] -= s;
+  for (int q = 0; q < kNB; ++q) s += a[r][q] * b[c][q];
+  A[(int64_t)i * d + j] -= s;
+}
+inline int update_tiles(int rows) {
+  const int T = ceil_div(rows, kUT);
+  return T * (T + 1) / 2;
+}
+
+// trailing update behind panel p (FP64 plans)
+__global__ void __launch_bounds__(256) chol_syrk_kernel(double* A, int d, int p) {
+  __shared__ double a[kUT][kNB + 1], b[kUT][kNB + 1];
+  chol_update_tile(A, d, p * kNB, blockIdx.x, a, b);
+}
+
+// FP32/BF16 plans: the trailing update behind panel p with the next diagonal
+// block factored in the same launch (CTA 0: its own update, then L and
+// L^{-1} by group_chol_inverse, 32 dependent steps; L^{-T} goes to the
+// diagonal block of Rinv).  p = -1: the first diagonal block only.
+__global__ void __launch_bounds__(256) chol_next_kernel(double* A, double* Rinv, int d, int p, int* flag) {
+  __shared__ double sa[kNB][kNB + 1], sb[kNB][kNB + 1], rs[kNB];
+  if (blockIdx.x > 0) {  // tiles 0 .. 2 are the diagonal block
+    chol_update_tile(A, d, p * kNB, (int)blockIdx.x + 2, sa, sb);
+    return;
   }
+  const int o = (p + 1) * kNB, nb = min(kNB, d - o), tid = threadIdx.x;
+  if (p >= 0) {
+    for (int e = tid; e < kNB * kNB; e += 256) {
+      const int r = e / kNB, c = e % kNB;
+      sb[r][c] = r < nb ? A[(int64_t)(o + r) * d + o - kNB + c] : 0.0;
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < nb * (nb + 1) / 2; e += 256) {
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    while ((i + 1) * (i + 2) / 2 <= e) ++i;
+    while (i * (i + 1) / 2 > e) --i;
+    const int c = e - i * (i + 1) / 2;
+    double s = 0;
+    if (p >= 0) {
+#pragma unroll 8
+      for (int q = 0; q < kNB; ++q) s += sb[i][q] * sb[c][q];
+    }
+    sa[i][c] = A[(int64_t)(o + i) * d + o + c] - s;
+  }
+  __syncthreads();
+  const bool ok = group_chol_inverse<256>(&sa[0][0], &sb[0][0], rs, nb, tid, 0, kNB + 1);
+  if (!ok && tid == 0) atomicExch(flag, kFlagNotSpd);
+  for (int e = tid; e < nb * nb; e += 256) {
+    const int r = e / nb, c = e % nb;
+    if (c <= r) {
+      A[(int64_t)(o + r) * d + o + c] = sa[r][c] * rs[c];      // L_cc = L_cc^2 / L_cc on the diagonal
+      Rinv[(int64_t)(o + c) * d + o + r] = sb[r][c];
+    }
+  }
+}
+
+// A[rows below, p] <- A[rows below, p] L_pp^{-T}: a warp per row, lane c the
+// column, the 32 terms of a product with the inverse block (no substitution
+// chain).
+__global__ void __launch_bounds__(256) chol_panel_kernel(double* A, const double* __restrict__ Rinv, int d, int p) {
+  __shared__ double Ls[kNB][kNB];  // L^{-T}: row q, column c >= q
+  const int o = p * kNB, lane = threadIdx.x & 31;
+  for (int e = threadIdx.x; e < kNB * kNB; e += 256)
+    Ls[e / kNB][e % kNB] = Rinv[(int64_t)(o + e / kNB) * d + o + e % kNB];
+  __syncthreads();
+  const int row = o + kNB + blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (row >= d) return;  // uniform over the warp
+  const double v = A[(int64_t)row * d + o + lane];
+  double x = 0.0;
+#pragma unroll 8
+  for (int q = 0; q < kNB; ++q) x += __shfl_sync(0xffffffffu, v, q) * Ls[q][lane];
+  A[(int64_t)row * d + o + lane] = x;
 }
 
 __global__ void lower_to_upper_kernel(double* A, int d) {
@@ -664,6 +738,8 @@ __global__ void lower_to_upper_kernel(double* A, int d) {
   if (j > i) A[(int64_t)j * d + i] = 0.0;
 }
 
+// FP64 plans: their iterations amplify a change of rounding in R, so every
+// entry keeps the order of its sums (pivots by 1 / sqrt, substitution).
 int cholesky_upper(double* A, int d, int* flag, cudaStream_t st) {
   int nbk = ceil_div(d, kNB);
   for (int p = 0; p < nbk; ++p) {
@@ -673,10 +749,29 @@ int cholesky_upper(double* A, int d, int* flag, cudaStream_t st) {
     if (below > 0) {
       chol_trsm_kernel<<<ceil_div(below, kTrsmRows), 32 * kTrsmRows, 0, st>>>(A, d, p);
       GB_CHECK_LAUNCH();
-      int nt = nbk - p - 1;
-      chol_syrk_kernel<<<dim3(nt, nt), 256, 0, st>>>(A, d, p);
+      chol_syrk_kernel<<<update_tiles(below), 256, 0, st>>>(A, d, p);
       GB_CHECK_LAUNCH();
     }
+  }
+  lower_to_upper_kernel<<<dim3(ceil_div(d, 32), ceil_div(d, 32)), dim3(32, 32), 0, st>>>(A, d);
+  GB_CHECK_LAUNCH();
+  return GBCCA_OK;
+}
+
+// FP32/BF16 plans: the same factor, two launches per 32 columns; also writes the
+// diagonal blocks of Rinv = R^{-1} (which must be zero elsewhere in them).  A
+// step took a 32 us factorization of the diagonal block by four warps, an 8 us
+// substitution and a 15 us update (0.9 ms for d = 512), one after another.
+int cholesky_upper_blocks(double* A, double* Rinv, int d, int* flag, cudaStream_t st) {
+  const int nbk = ceil_div(d, kNB);
+  chol_next_kernel<<<1, 256, 0, st>>>(A, Rinv, d, -1, flag);
+  GB_CHECK_LAUNCH();
+  for (int p = 0; p + 1 < nbk; ++p) {
+    const int below = d - (p + 1) * kNB;
+    chol_panel_kernel<<<ceil_div(below, 8), 256, 0, st>>>(A, Rinv, d, p);
+    GB_CHECK_LAUNCH();
+    chol_next_kernel<<<1 + std::max(0, update_tiles(below) - 3), 256, 0, st>>>(A, Rinv, d, p, flag);
+    GB_CHECK_LAUNCH();
   }
   lower_to_upper_kernel<<<dim3(ceil_div(d, 32), ceil_div(d, 32)), dim3(32, 32), 0, st>>>(A, d);
   GB_CHECK_LAUNCH();
@@ -718,30 +813,35 @@ __global__ void tri_diag_inv_kernel(const double* __restrict__ R, double* __rest
 
 // stage 0: T_p = R[A, C] Rinv[C, C]  (h x w, row stride h)
 // stage 1: Rinv[A, C] = -Rinv[A, A] T_p
-// Grid (ceil(h/32), ceil(h/32), pairs); each CTA one 32 x 32 output tile,
-// K in chunks of 32 restricted to where the triangular factor is non-zero.
+// Grid (ceil(h/16), ceil(h/16), pairs); each CTA one 16 x 16 output tile, an
+// entry per thread with its terms in order, K in chunks of 32 restricted to
+// where the triangular factor is non-zero.  Bound by the FP64 rate: 32 x 32
+// tiles left most SMs without work on all levels but the last (41 us a launch
+// on average at d = 512).
+constexpr int kTT = 16;
 template <int kStage>
 __global__ void __launch_bounds__(256) tri_level_kernel(const double* __restrict__ R, double* __restrict__ Rinv,
                                                         double* __restrict__ T, int d, int h) {
-  __shared__ double As[kTB][kTB + 1], Bs[kTB][kTB + 1];
+  __shared__ double As[kTT][kTB + 1], Bs[kTB][kTT + 1];
   const int p = blockIdx.z;
   const int r0 = 2 * p * h, c0 = r0 + h;
   if (c0 >= d) return;
   const int w = min(d, c0 + h) - c0;
-  const int i0 = blockIdx.y * kTB, j0 = blockIdx.x * kTB;
+  const int i0 = blockIdx.y * kTT, j0 = blockIdx.x * kTT;
   if (i0 >= h || j0 >= w) return;
   double* Tp = T + (int64_t)p * h * h;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   // K range: stage 0 runs q in [0, w) with Rinv[C,C][q][j] = 0 for q > j;
   // stage 1 runs q in [0, h) with Rinv[A,A][i][q] = 0 for q < i
   const int klo = kStage == 0 ? 0 : i0;
-  const int khi = kStage == 0 ? min(w, j0 + kTB) : h;
-  double acc[2][2] = {};
+  const int khi = kStage == 0 ? min(w, j0 + kTT) : h;
+  double acc = 0.0;
   for (int k0 = klo; k0 < khi; k0 += kTB) {
-    for (int e = threadIdx.x; e < kTB * kTB; e += 256) {
-      const int r = e / kTB, c = e % kTB;
-      const int ia = i0 + r, qa = k0 + c;  // A tile element (i, q)
-      const int qb = k0 + r, jb = j0 + c;  // B tile element (q, j)
+    for (int e = threadIdx.x; e < kTT * kTB; e += 256) {
+      const int r = e / kTB, c = e % kTB;       // A tile element (i, q)
+      const int ia = i0 + r, qa = k0 + c;
+      const int qr = e / kTT, jc = e % kTT;     // B tile element (q, j)
+      const int qb = k0 + qr, jb = j0 + jc;
       double av = 0.0, bv = 0.0;
       if (kStage == 0) {
         if (ia < h && qa < khi) av = R[(int64_t)(r0 + ia) * d + c0 + qa];
@@ -751,45 +851,37 @@ __global__ void __launch_bounds__(256) tri_level_kernel(const double* __restrict
         if (qb < khi && jb < w) bv = Tp[(int64_t)qb * h + jb];
       }
       As[r][c] = av;
-      Bs[r][c] = bv;
+      Bs[qr][jc] = bv;
     }
     __syncthreads();
+    const int kn = min(kTB, khi - k0);
 #pragma unroll 8
-    for (int q = 0; q < kTB; ++q) {
-      const double a0 = As[ty][q], a1 = As[ty + 16][q];
-      const double b0 = Bs[q][tx], b1 = Bs[q][tx + 16];
-      acc[0][0] += a0 * b0;
-      acc[0][1] += a0 * b1;
-      acc[1][0] += a1 * b0;
-      acc[1][1] += a1 * b1;
-    }
+    for (int q = 0; q < kn; ++q) acc += As[ty][q] * Bs[q][tx];
     __syncthreads();
   }
-#pragma unroll
-  for (int u = 0; u < 2; ++u)
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      const int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
-      if (i < h && j < w) {
-        if (kStage == 0)
-          Tp[(int64_t)i * h + j] = acc[u][v];
-        else
-          Rinv[(int64_t)(r0 + i) * d + c0 + j] = -acc[u][v];
-      }
-    }
+  const int i = i0 + ty, j = j0 + tx;
+  if (i < h && j < w) {
+    if (kStage == 0)
+      Tp[(int64_t)i * h + j] = acc;
+    else
+      Rinv[(int64_t)(r0 + i) * d + c0 + j] = -acc;
+  }
 }
 
-int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t ws_len, cudaStream_t st) {
+// have_diag: the diagonal blocks of Rinv are in place (and it is zero elsewhere)
+int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t ws_len, cudaStream_t st, bool have_diag) {
   if (ws_len < (int64_t)d * d) {
     set_last_error("tri_inverse_upper: workspace too small");
     return GBCCA_ERR_INVALID_ARG;
   }
-  GB_CUDA(cudaMemsetAsync(Rinv, 0, sizeof(double) * d * d, st));
-  tri_diag_inv_kernel<<<ceil_div(d, kTB), kTB, 0, st>>>(R, Rinv, d);
-  GB_CHECK_LAUNCH();
+  if (!have_diag) {
+    GB_CUDA(cudaMemsetAsync(Rinv, 0, sizeof(double) * d * d, st));
+    tri_diag_inv_kernel<<<ceil_div(d, kTB), kTB, 0, st>>>(R, Rinv, d);
+    GB_CHECK_LAUNCH();
+  }
   for (int h = kTB; h < d; h *= 2) {
     const int pairs = ceil_div(d - h, 2 * h);
-    dim3 grid(ceil_div(h, kTB), ceil_div(h, kTB), pairs);
+    dim3 grid(ceil_div(h, kTT), ceil_div(h, kTT), pairs);
     tri_level_kernel<0><<<grid, 256, 0, st>>>(R, Rinv, ws, d, h);
     GB_CHECK_LAUNCH();
     tri_level_kernel<1><<<grid, 256, 0, st>>>(R, Rinv, ws, d, h);

@@ -204,6 +204,7 @@ int gram_df_split(const float* Ah, const float* Al, int64_t lda, const float* Bh
                   int64_t m, int d1, int d2, double* C, double diag_add, double* ws, int64_t ws_len, cudaStream_t st,
                   bool tri = false);
 int cholesky_upper(double* A, int d, int* flag, cudaStream_t st);
+int cholesky_upper_blocks(double* A, double* Rinv, int d, int* flag, cudaStream_t st);
 // C = A^T A + lambda I (A: m x d FP64, row stride lda) with the split-K
 // partials in a static device scratch instead of plan memory; d <= noalloc_max_d().
 int gram_noalloc(const double* A, int64_t lda, int64_t m, int d, double lambda, double* C, cudaStream_t st);
@@ -237,7 +238,8 @@ int split_df(const double* A, int r, int c, bool trans, float* hi, float* lo, cu
 // M^{-1} = R^{-1} R^{-T} as a double-float pair (d x d)
 int minv_df_build(const double* Rinv, int d, float* hi, float* lo, double* ws, int64_t ws_len, cudaStream_t st);
 // Rinv = R^{-1} (upper triangular, d x d); ws holds at least d * d doubles.
-int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t ws_len, cudaStream_t st);
+int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t ws_len, cudaStream_t st,
+                      bool have_diag = false);
 // C (m x c, ldc) = op(A) B (rows of B = columns of op(A), ldb), A ra x ca
 // row-major, for one or two problems in one launch; tri: A upper triangular,
 // its zero half skipped.

@@ -29,7 +29,9 @@ __device__ __forceinline__ void group_sync(int id) {
 // L^{-1} of the Cholesky factor A = L L^T of an n x n symmetric positive
 // definite matrix (row-major, lower triangle read and destroyed) by G threads
 // with barrier `id`; g is the thread's index in the group.  Li (n x n,
-// row-major) receives L^{-1}, its upper triangle zero; rs is scratch of n.
+// row-major) receives L^{-1}, its upper triangle zero; rs is scratch of n and
+// receives 1 / L_ii (column c of A is left as L_ic / rs_c, i > c, and the pivot
+// L_cc^2).  ld: row stride of A and Li (0: n).
 // Returns false, in every thread of the group, if a pivot is not positive
 // (the result is then void).  n <= 20 with G = 128, n <= 40 with G = 256.
 //
@@ -41,7 +43,8 @@ __device__ __forceinline__ void group_sync(int id) {
 // at once.  (A Cholesky by one warp followed by the inverse, a column per
 // lane, was a chain of several hundred FP64 instructions.)
 template <int G>
-__device__ bool group_chol_inverse(double* A, double* Li, double* rs, int n, int g, int id) {
+__device__ bool group_chol_inverse(double* A, double* Li, double* rs, int n, int g, int id, int ld = 0) {
+  if (ld == 0) ld = n;
   constexpr int kItems = G == 128 ? 2 : 4;  // entries (i, c), c <= i, per thread
   int ri[kItems], ci[kItems];
 #pragma unroll
@@ -53,14 +56,14 @@ __device__ bool group_chol_inverse(double* A, double* Li, double* rs, int n, int
     ri[u] = i;
     ci[u] = e - i * (i + 1) / 2;
     if (i < n) {
-      Li[i * n + ci[u]] = i == ci[u] ? 1.0 : 0.0;
-      if (i != ci[u]) Li[ci[u] * n + i] = 0.0;
+      Li[i * ld + ci[u]] = i == ci[u] ? 1.0 : 0.0;
+      if (i != ci[u]) Li[ci[u] * ld + i] = 0.0;
     }
   }
   bool ok = true;
   for (int j = 0; j < n; ++j) {
     group_sync<G>(id);
-    double d = A[j * n + j];
+    double d = A[j * ld + j];
     if (!(d > 0.0)) {
       ok = false;
       d = 1.0;
@@ -71,22 +74,22 @@ __device__ bool group_chol_inverse(double* A, double* Li, double* rs, int n, int
     for (int u = 0; u < kItems; ++u) {
       const int i = ri[u], c = ci[u];
       if (i > j && i < n) {
-        const double a = A[i * n + j];
+        const double a = A[i * ld + j];
         if (c > j)
-          A[i * n + c] -= a * (A[c * n + j] * r);
+          A[i * ld + c] -= a * (A[c * ld + j] * r);
         else
-          Li[i * n + c] -= a * (Li[j * n + c] * r);
+          Li[i * ld + c] -= a * (Li[j * ld + c] * r);
       }
     }
   }
   if (g < n) {
-    const double d = A[g * n + g];
+    const double d = A[g * ld + g];
     rs[g] = d > 0.0 ? rsqrt_nr(d) : 1.0;
   }
   group_sync<G>(id);
 #pragma unroll
   for (int u = 0; u < kItems; ++u)
-    if (ri[u] < n) Li[ri[u] * n + ci[u]] *= rs[ri[u]];
+    if (ri[u] < n) Li[ri[u] * ld + ci[u]] *= rs[ri[u]];
   group_sync<G>(id);
   return ok;
 }

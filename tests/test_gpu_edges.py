@@ -353,3 +353,25 @@ def test_srht_sizes(gb, dt, n, d, s):
         gb.cca_precondition(plan, x, x, 1e3, 1e3, torch.from_numpy(rows).cuda(), torch.from_numpy(D).cuda())
         got = np64(gb.query(plan, gb.Q_SKETCH_X)).reshape(s, d)
         assert bound_ratio(got, srht_apply(X, D, rows), ref, gamma) <= 1.0
+
+
+@pytest.mark.parametrize("d", [1, 15, 16, 17, 31, 32, 33, 48, 64, 65, 81, 260])
+def test_factor_blocks_f32(gb, d):
+    """R of FP32 plans at sizes around the 32-column panels and the 16-row
+    tiles of the trailing update: upper, positive diagonal, R^T R equal to the
+    sketch's Gram.  Gram: s terms of 2^-44 each; factor: chains of d terms in
+    FP64 and one inverse of a 32 x 32 block."""
+    import torch
+    from synth import countsketch_draws
+    n, s, lam = 4 * d + 20, 2 * d + 10, 1e-1
+    X = np.random.default_rng(d).standard_normal((n, d)).astype(np.float32)
+    h, g = countsketch_draws(n, s, seed=5)
+    plan = gb.cca_plan(n, d, d, 1, "f32", gb.default_options(s=s, warm_start=0))
+    x = torch.from_numpy(X).cuda()
+    gb.cca_precondition(plan, x, x, lam, lam, torch.from_numpy(h).cuda(), torch.from_numpy(g).cuda())
+    S = np64(gb.query(plan, gb.Q_SKETCH_X)).reshape(s, d)
+    ref = np.abs(S).T @ np.abs(S) + lam * np.eye(d)
+    for q in (gb.Q_R_X, gb.Q_R_Y):  # the two views are factored side by side
+        R = np64(gb.query(plan, q)).reshape(d, d)
+        assert np.all(np.tril(R, -1) == 0) and np.all(np.diag(R) > 0)
+        assert bound_ratio(R.T @ R, S.T @ S + lam * np.eye(d), ref, (s + 4 * d) * 2.0 ** -44) <= 1.0
