@@ -490,9 +490,9 @@ def batched_workload(gb, count: int = 64, seed: int = 0):
                            "GBps": gbps, "frac_of_hbm": gbps / hbm if gbps else None,
                            "expected_instances": len(served)},
         "prepare_s": prep_s,
-        "note": "two batched launches per iteration serve every instance: 2-CTA clusters for dx, dy <= 512 and "
-                "4-CTA clusters for a wider view (its column pairs split over two CTAs); 2k > 24 in two column "
-                "groups of Phi, which read the data twice; the bytes and time are those of both launches",
+        "note": "a batched launch of 2-CTA clusters serves the instances with dx, dy <= 512 and k <= 12, two "
+                "launches of the two-sweep pass the others (they read the data twice); the bytes, each plan's data "
+                "once, and time are those of all launches",
     }
     batch.close()
     for p in plans:

@@ -297,11 +297,11 @@ int32_t gbcca_sketch_gram_noalloc_max_d(void);
  * (cca_precondition / lda_solve's preconditioning through a previous call)
  * with opt.warm_start on, and stays owned by the caller; its data must stay
  * valid while the batch exists.  Every iteration, the data passes of the
- * plans the tensor-core pass serves (CCA, BF16 or FP32 data; k > 12 in two
- * column groups of Phi) run as ONE persistent launch (two when some plans
- * have a view wider than 512 columns: those run in 4-CTA clusters) over a schedule of (instance,
- * 64-row tile range) segments cut into near-equal work per 2-CTA cluster;
- * the other plans run their own passes.  Each plan's small kernels run on a
+ * plans the tensor-core pass serves (CCA, BF16 or FP32 data) run as ONE
+ * persistent launch (and the two launches of the two-sweep pass when some
+ * plans have k > 12 or a view wider than 512 columns) over a schedule of
+ * (instance, 64-row tile range) segments cut into near-equal work per 2-CTA
+ * cluster; the other plans run their own passes.  Each plan's small kernels run on a
  * graph branch of their own, and each plan stops on its own rule (its
  * options); a finished plan leaves the schedule.  The result of every plan
  * is the one its own cca_solve / lda_solve would give up to the rounding of

@@ -130,10 +130,12 @@ int alloc_plan(Plan* p) {
   int nb = 0;
   for (int v = 0; v < p->nviews; ++v) nb += ceil_div(p->v[v].d, 64);
   p->chunksB = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(2 * p->sm_count, nb), (p->n + 31) / 32));
-  size_t esz = sizeof(double);
   {
+    // W of the CUDA-core passes, or the two-sweep tensor-core pass's image of it
     void* t = nullptr;
-    if (counted_malloc(&t, esz * (size_t)p->n * p->NC) != cudaSuccess) {
+    const int64_t wb = std::max((int64_t)sizeof(double) * p->n * p->NC,
+                                p->dtype != GBCCA_FP64 && p->opt.tensor_cores ? tc_wimg_bytes(*p) : 0);
+    if (counted_malloc(&t, (size_t)wb) != cudaSuccess) {
       cudaGetLastError();
       set_last_error("pass intermediate allocation failed");
       return GBCCA_ERR_OOM;
@@ -179,10 +181,8 @@ int alloc_plan(Plan* p) {
   const bool tc_cca = p->kind == kCCA && (p->dtype == GBCCA_BF16 || p->dtype == GBCCA_FP32);
   const bool tc_fda = p->kind == kLDA && p->dtype == GBCCA_FP32 && dmax <= 1024;
   if ((tc_cca || tc_fda) && p->opt.tensor_cores) {
-    // Phi images per column group (two groups for 2k > 24): CCA both views'
-    // (twice the K-boxes for views wider than 512), FDA the one view's in 16
-    // K-boxes; and the per-cluster partial slabs of every group
-    const int64_t img = (2 * k <= 24 ? 1 : 2) * (tc_cca ? 2 * (dmax > 512 ? 2 : 1) : 2) * 49152;
+    // the views' Phi images, the partial slabs and the row blocks' Grams
+    const int64_t img = tc_img_len(*p);
     GB_TRY(dalloc(&p->tc_img, img));
     GB_CUDA(cudaMemset(p->tc_img, 0, img));
     GB_TRY(dalloc(&p->tc_gpart, tc_gpart_len(*p)));

@@ -24,8 +24,9 @@
 
 namespace gbcca {
 
-// Two batched launches serve the tensor-core plans: table 0 in 2-CTA
-// clusters, table 1 in 4-CTA clusters (plans with a view wider than 512).
+// Two batched passes serve the tensor-core plans: table 0 the one-sweep
+// kernel in 2-CTA clusters, table 1 the two-sweep kernels (plans with k > 12 or
+// a view wider than 512; `clusters` pairs of CTAs).
 struct Batch {
   std::vector<Plan*> plans;
   std::vector<int> tc_table;       // 0 or 1: the table that serves the plan's pass; -1: its own pass
@@ -242,7 +243,7 @@ Batch* batch_make(Plan* const* plans, int count, const gbcca_batch_options* opt,
     b->plans.push_back(p);
     const bool tc = p->kind == kCCA && p->dtype != GBCCA_FP64 && p->opt.tensor_cores && p->tc_img != nullptr &&
                     tc_pass_eligible(*p);
-    const int t = tc ? (tc_quad(*p) ? 1 : 0) : -1;
+    const int t = tc ? (tc_two(*p) ? 1 : 0) : -1;
     b->tc_table.push_back(t);
     b->tc_index.push_back(t >= 0 ? (int)b->tc_plans[t].size() : -1);
     if (t >= 0) b->tc_plans[t].push_back(p);

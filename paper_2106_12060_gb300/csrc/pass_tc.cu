@@ -53,7 +53,7 @@
 #include <cstring>
 #include <vector>
 
-#include "tc_ptx.cuh"
+#include "pass_two.h"
 
 namespace gbcca {
 
@@ -73,7 +73,7 @@ constexpr long long kTimeout = kWaitCycles;       // cycles (~1 s)
 // Shared-memory layout and barriers for GEMM 1 with N = 2 kH1 (Phi columns as
 // bf16 hi rows 0 .. kH1 - 1 and lo rows kH1 .. 2 kH1 - 1; kH1 = 20 serves
 // 2k <= 20 and leaves room for a 10-slot ring, kH1 = 24 a 9-slot ring).
-template <int kH1, bool kQuad = false, bool kSolo = false>
+template <int kH1, bool kSolo = false>
 struct Lay {
   static constexpr int kN1 = 2 * kH1;
   static constexpr int kKBox1 = kN1 * 128;       // one K-box (64 columns) of the Phi image
@@ -96,10 +96,9 @@ struct Lay {
   // every 50 cycles, two streams overlap in the tensor pipe.
   static constexpr int kNAcc = (4 * kTW + kTileSlots * kN2 <= (int)kTmemCols) ? 2 : 1;
   static constexpr int kTG = 2 * kNAcc * kTW;    // first TMEM column of the G accumulators
-  // 4-CTA clusters (views wider than 512 columns, split over two CTAs each)
-  // and one-view clusters (FDA: the view's columns split over the two CTAs):
-  // two FP32 buffers that receive the other half's partial W of a tile
-  static constexpr bool kHalves = kQuad || kSolo;  // a view's pairs over two CTAs
+  // one-view clusters (FDA: the view's columns split over the two CTAs): two
+  // FP32 buffers that receive the other half's partial W of a tile
+  static constexpr bool kHalves = kSolo;  // a view's pairs over two CTAs
   static constexpr int kXC = 24;                 // floats per row of an exchange buffer
   static constexpr int kXBytes = kHalves ? 2 * kRows * kXC * 4 : 0;
   static constexpr int kStages = (kMaxSmem - kPhiBytes - 2 * kWBuf - kXBytes - 512 - 1024) / kSlot;
@@ -116,10 +115,9 @@ struct Lay {
   static constexpr int kPhiFull = kFinal + 3;  // Phi image in shared memory
   static constexpr int kGFree = kPhiFull + 1;   // G drained (128 arrivals)
   static constexpr int kPhiFree = kGFree + 1;  // GEMM 1 done with a segment's Phi
-  static constexpr int kXFull = kPhiFree + 1, kXFree = kXFull + 2;  // [2], [2]: partial-W exchange (quad)
+  static constexpr int kXFull = kPhiFree + 1, kXFree = kXFull + 2;  // [2], [2]: partial-W exchange
   static constexpr int kEpiSyncB = kXFree + 2;  // the second epilogue group's kEpiSync
   static constexpr int kNumBars = kEpiSyncB + 1;
-  static_assert(!(kQuad && kSolo), "one cluster shape");
   static_assert(kStages >= 2 * kTileSlots, "two resident tiles");
   static_assert(kN1 <= kTW && kD1Cols <= kTW, "W buffers in TMEM");
   static_assert(kN2 % 16 == 0 && kTG + kTileSlots * kN2 <= (int)kTmemCols, "G accumulators in TMEM");
@@ -128,12 +126,6 @@ struct Lay {
   static_assert(kNumBars * 8 + 8 <= 512, "barrier area");
   static_assert(kSmemBytes <= kMaxSmem, "shared memory");
 };
-
-// Rows of a view in a partial slab: padded so that a block of kPostRows rows
-// belongs to one view and starts on a 16-byte boundary.  The padding is never
-// written and its sums are never used.
-constexpr int kPostRows = 8;
-__host__ __device__ __forceinline__ int pad_rows(int d) { return (d + kPostRows - 1) / kPostRows * kPostRows; }
 
 // One instance of a batched pass (device memory; the tensor maps are read by
 // the TMA unit from there; CUtensorMap carries its own 128-byte alignment).
@@ -193,13 +185,13 @@ struct SegView {
   float* out;              // partial slab of the segment
   int first, stride, count;
   int d0, d1, npairs, k2, pair_sum;
-  int pb;                  // first 128-column pair of this CTA (4-CTA clusters: half h of the view)
+  int pb;                  // first 128-column pair of this CTA
   bool skip;
 };
 
 // The 128-column pairs of a view of P pairs that CTA half h takes: all of
-// them in a 2-CTA cluster of two views; in a 4-CTA cluster, or a one-view
-// cluster, the first ceil(P / 2) for h = 0 and the rest for h = 1, at least
+// them in a cluster of two views; in a one-view cluster the first ceil(P / 2)
+// for h = 0 and the rest for h = 1, at least
 // one (a pair past the view's last column reads zeros from the tensor map and
 // the image, and drains nothing).
 __device__ __forceinline__ void half_pairs(int P, bool split, int h, int* pb, int* np) {
@@ -257,12 +249,11 @@ __device__ __forceinline__ SegView seg_view(const Args& a, const CUtensorMap* tm
 
 constexpr int kThreads = 384;  // 4 role warps + two epilogue groups of 4 warps
 
-template <int kH1, bool kQuad = false, bool kSolo = false>
+template <int kH1, bool kSolo = false>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmy, Args a) {
-  using L = Lay<kH1, kQuad, kSolo>;
+  using L = Lay<kH1, kSolo>;
   constexpr bool kHalves = L::kHalves;
-  constexpr int kNvs = kSolo ? 1 : 2;  // views per row of a partial slab
   constexpr int kStages = L::kStages;
   constexpr int kFull = L::kFull, kEmpty = L::kEmpty, kD1Full = L::kD1Full, kD1Free = L::kD1Free;
   constexpr int kEpiSync = L::kEpiSync, kWReady = L::kWReady, kWPeer = L::kWPeer, kWFree = L::kWFree;
@@ -281,15 +272,13 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* xbuf = reinterpret_cast<float*>(smem + L::kXOff);  // [buffer][64 rows][kXC]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // rank = 2 half + view: CTAs 2h and 2h + 1 form the pair that shares the
-  // tile's W (views X and Y); in a 4-CTA cluster, CTAs v and v + 2 hold the
-  // two column halves of view v and add their partial W of every tile.  A
-  // one-view cluster (FDA): rank = half, the two CTAs add their partial W.
+  // rank = view: the two CTAs share the tile's W (views X and Y).  A one-view
+  // cluster (FDA): rank = half, the two CTAs add their partial W.
   const uint32_t rank = cluster_ctarank();
   const int view = kSolo ? 0 : (int)(rank & 1u);  // 0: X, 1: Y
-  const int half = kQuad ? (int)(rank >> 1) : (kSolo ? (int)rank : 0);
+  const int half = kSolo ? (int)rank : 0;
   const uint32_t peer = rank ^ 1u;
-  const uint32_t hpeer = kSolo ? rank ^ 1u : rank ^ 2u;
+  const uint32_t hpeer = peer;  // the CTA with the other half
   (void)hpeer;
   (void)xbuf;
   // bound of one pipeline wait: the plan's for a one-view cluster, whose only
@@ -521,7 +510,7 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
           if constexpr (kSolo) {
             mma_commit(bar(kWFree + b));
           } else {
-            mma_commit_mc(bar(kWFree + b), (uint16_t)(0x3u << (2 * half)));
+            mma_commit_mc(bar(kWFree + b), (uint16_t)0x3u);
           }
         }
         if (ok) mma_commit(bar(kGDone));  // this segment's G is complete
@@ -703,7 +692,7 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
       if (!(ok = mbar_wait(bar(kGDone), sp & 1, abort_flag, wl))) break;
       tc_fence_after();
       {
-        // the slab is column-major (D rows, kNvs k2 columns): the 32 lanes
+        // the slab is column-major (D rows, nv k2 columns): the 32 lanes
         // of a warp hold 32 consecutive rows, so every store of a column is
         // one 128-byte line
         // (each view's rows padded to kPostRows)
@@ -750,20 +739,19 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
 }
 
 // Phi image: per view, K-boxes of 64 columns; B rows 0..h-1 hold the bf16 hi
-// parts of the 2k columns [U | eta] (of a column group of them), rows h ..
-// their lo parts (x - hi); 128B-swizzled.  The point the pass evaluates, hi +
+// parts of the 2k columns [U | eta], rows h .. their lo parts (x - hi);
+// 128B-swizzled.  The point the pass evaluates, hi +
 // lo, is written to Phi, so that it is exactly the point the solver holds
-// (src may be Phi itself).  One thread per element of Phi (every view and
-// group in one launch); the padding of the image is zero from its allocation
+// (src may be Phi itself).  One thread per element of Phi (every view in
+// one launch); the padding of the image is zero from its allocation
 // and never written.
 struct ImageArgs {
   const double* src[2];  // d x k2 row-major
   double* Phi[2];
   int d[2];
   int k2;
-  int ng0;               // columns of group 0 (the rest are group 1's)
-  int h[2];              // image rows per half of each group
-  uint8_t* img[2];       // per group
+  int h;                 // image rows per half
+  uint8_t* img;
   int64_t img_view;
   const int* done;
 };
@@ -779,14 +767,12 @@ __global__ void __launch_bounds__(256) phi_image_kernel(const __grid_constant__ 
   const int e = blockIdx.x * blockDim.x + threadIdx.x;  // (data column j, Phi column q)
   if (e >= d * m.k2) return;
   const int j = e / m.k2, q = e - j * m.k2;
-  const int g = q < m.ng0 ? 0 : 1, c = q - (g == 0 ? 0 : m.ng0);
   const double x = (v == 0 ? m.src[0] : m.src[1])[e];
-  const int h1 = g == 0 ? m.h[0] : m.h[1];
   const __nv_bfloat16 hi = __double2bfloat16(x);
   const __nv_bfloat16 lo = __double2bfloat16(x - (double)__bfloat162float(hi));
-  uint8_t* base = (g == 0 ? m.img[0] : m.img[1]) + (int64_t)v * m.img_view + (int64_t)(j >> 6) * (2 * h1 * 128);
-  *reinterpret_cast<__nv_bfloat16*>(base + swz(c, j & 63)) = hi;
-  *reinterpret_cast<__nv_bfloat16*>(base + swz(h1 + c, j & 63)) = lo;
+  uint8_t* base = m.img + (int64_t)v * m.img_view + (int64_t)(j >> 6) * (2 * m.h * 128);
+  *reinterpret_cast<__nv_bfloat16*>(base + swz(q, j & 63)) = hi;
+  *reinterpret_cast<__nv_bfloat16*>(base + swz(m.h + q, j & 63)) = lo;
   (v == 0 ? m.Phi[0] : m.Phi[1])[e] = (double)__bfloat162float(hi) + (double)__bfloat162float(lo);
 }
 
@@ -811,11 +797,12 @@ __global__ void __launch_bounds__(256) phi_image_kernel(const __grid_constant__ 
 constexpr int kPostThreads = 512;
 constexpr int kPostLoads = 8;
 struct PostArgs {
-  const float* part[2];      // per column group
-  int64_t slab[2];
-  const int* nparts_dev[2];  // batched pass: the schedule's slab counts
+  const float* part;
+  int64_t slab;
+  const int* nparts_dev;     // batched pass: the schedule's slab count (by_pair: 16 of them)
   int nparts;
-  int ng0;                   // columns of group 0 (per view)
+  int by_pair;               // slab counts per (view, 128-column pair): np / nparts_dev[8 view + pair]
+  int np[16];
   int d[2], nv, k2;
   const double* Phi[2];
   double* G[2];              // row-major, nv k2 columns
@@ -857,14 +844,10 @@ __global__ void __launch_bounds__(kPostThreads) tc_post_kernel(const __grid_cons
   }
   if (sl < S) {
     const int c = it >> 1;  // column of G: view-x products, then view-y products
-    const int vv = c / m.k2, q = c - vv * m.k2;
-    const int g = q < m.ng0 ? 0 : 1;
-    const int ng = g == 0 ? m.ng0 : m.k2 - m.ng0;
-    const int sc = vv * ng + (g == 0 ? q : q - m.ng0);  // its column in the slab
-    const int* np = g == 0 ? m.nparts_dev[0] : m.nparts_dev[1];
-    const int nparts = np != nullptr ? *np : m.nparts;
-    const int64_t stride = (g == 0 ? m.slab[0] : m.slab[1]) / 4;
-    const float4* src = reinterpret_cast<const float4*>((g == 0 ? m.part[0] : m.part[1]) + (int64_t)sc * D + r0) + (it & 1);
+    const int at = m.by_pair ? 8 * v + (row0 >> 7) : 0;
+    const int nparts = m.nparts_dev != nullptr ? m.nparts_dev[at] : (m.by_pair ? m.np[at] : m.nparts);
+    const int64_t stride = m.slab / 4;
+    const float4* src = reinterpret_cast<const float4*>(m.part + (int64_t)c * D + r0) + (it & 1);
     float s[4] = {0.f, 0.f, 0.f, 0.f}, cp[4] = {0.f, 0.f, 0.f, 0.f};
     for (int b0 = sl; b0 < nparts; b0 += S * kPostLoads) {
       float4 x4[kPostLoads];
@@ -964,13 +947,12 @@ int make_map(CUtensorMap* map, const void* base, int64_t n, int d, int64_t ld) {
 }  // namespace
 
 // The tensor-core pass serves CCA plans with BF16 data (or FP32 data through
-// the interleaved copy), dx, dy <= 1024 (views wider than 512 columns in
-// 4-CTA clusters, each view's column pairs split over two CTAs), 16-byte
-// aligned rows (ld a multiple of 8) and 16-byte aligned bases; Phi columns
-// beyond 24 per view (k > 12, up to the library's k <= 20) are taken in a
-// second column group, which reads the data a second time.  FDA plans with
-// FP32 data and d <= 1024 stream the interleaved copy of their class-centred
-// rows in one-view clusters (the view's column pairs split over two CTAs).
+// the interleaved copy), dx, dy <= 1024, 16-byte aligned rows (ld a multiple
+// of 8) and 16-byte aligned bases, and FDA plans with FP32 data and d <= 1024
+// (the interleaved copy of their class-centred rows, in one-view clusters that
+// split the view's column pairs over the two CTAs).  More than 24 columns of
+// Phi per view, or a CCA view wider than 512 columns, take the two-sweep
+// kernels of pass_two.cu.
 bool tc_pass_eligible(const Plan& p) {
   if (p.kind == kLDA) return p.dtype == GBCCA_FP32 && 2 * p.k <= 2 * tc::kHalfMax && p.v[0].d <= 1024 && p.ts_ready;
   if (p.kind != kCCA || 2 * p.k > 2 * tc::kHalfMax || p.v[0].d > 1024 || p.v[1].d > 1024) return false;
@@ -982,54 +964,52 @@ bool tc_pass_eligible(const Plan& p) {
   return true;
 }
 
-// Column groups of Phi for the tensor-core pass: one group for 2k <= 24,
-// else two of ng0 = k rounded up to even columns (an even group keeps every
-// partial slab a multiple of 4 floats), each at most 24.
-int tc_groups(const Plan& p) { return 2 * p.k <= tc::kHalfMax ? 1 : 2; }
-static void tc_group(const Plan& p, int g, int* col0, int* ng) {
-  const int k2 = 2 * p.k;
-  if (tc_groups(p) == 1) {
-    *col0 = 0;
-    *ng = k2;
-    return;
-  }
-  const int ng0 = (p.k + 1) / 2 * 2;
-  *col0 = g * ng0;
-  *ng = g == 0 ? ng0 : k2 - ng0;
-}
 // one-view plans (FDA): clusters of two CTAs that split the view's column
 // pairs
 static bool tc_solo(const Plan& p) { return p.kind == kLDA; }
-static int tc_group_h1(const Plan& p, int ng) { return ng <= 20 ? 20 : tc::kHalfMax; }
-// views wider than 512 columns: 4-CTA clusters and images of 16 K-boxes
-bool tc_quad(const Plan& p) { return p.kind == kCCA && std::max(p.v[0].d, p.v[1].d) > 512; }
-// bytes between the views' images of a group (one-view plans: 16 K-boxes,
-// the second CTA's pairs starting at K-box 8 at most)
-static int64_t tc_img_view(const Plan& p) { return (tc_quad(p) || tc_solo(p) ? 2 : 1) * (int64_t)tc::kPhiView; }
+// Plans that take two sweeps: the one-sweep kernel's accumulators hold 24
+// columns per view and its CTAs 512 columns of one.  Where both could serve (a
+// view of at most 512 columns, k <= 12) one sweep reads the data once and is
+// faster at every width measured (262144 x (512 + 512), k = 10: 106 against
+// 185 us).
+bool tc_two(const Plan& p) {
+  return 2 * p.k > tc::kHalfMax || (p.kind == kCCA && std::max(p.v[0].d, p.v[1].d) > 512);
+}
+// rows per half of the Phi image
+static int tc_h1(const Plan& p) { return tc_two(p) ? (2 * p.k + 7) / 8 * 8 : (2 * p.k <= 20 ? 20 : tc::kHalfMax); }
 static int tc_nviews(const Plan& p) { return tc_solo(p) ? 1 : 2; }
-static uint8_t* tc_group_img(const Plan& p, int g) { return p.tc_img + (int64_t)g * tc_nviews(p) * tc_img_view(p); }
-// floats of one cluster's partial slab of a group of ng columns: 2 ng columns
-// (one view: ng) of the views' padded rows
+// bytes between the views' images: two sweeps, every 64-column box with up
+// to 40 rows per half; one-view plans, 16 K-boxes (the second CTA's pairs
+// start at K-box 8 at most); else 8 K-boxes
+static int64_t tc_img_view(const Plan& p) {
+  if (tc_two(p)) return (int64_t)ceil_div(std::max(p.v[0].d, tc_nviews(p) > 1 ? p.v[1].d : 0), 64) * 2 * 40 * 128;
+  return (tc_solo(p) ? 2 : 1) * (int64_t)tc::kPhiView;
+}
+int64_t tc_img_len(const Plan& p) { return tc_nviews(p) * tc_img_view(p); }
 static int tc_rows(const Plan& p) { return tc::pad_rows(p.v[0].d) + (tc_nviews(p) > 1 ? tc::pad_rows(p.v[1].d) : 0); }
-static int64_t tc_slab(const Plan& p, int ng) { return (int64_t)tc_rows(p) * tc_nviews(p) * ng; }
-// partial slabs of group g: clusters (at most half the SMs) x one slab each
-static float* tc_group_part(const Plan& p, int g) {
-  int col0 = 0, ng0 = 0;
-  tc_group(p, 0, &col0, &ng0);
-  return p.tc_part + (int64_t)g * (p.sm_count / 2) * tc_slab(p, ng0);
+// floats of one partial slab: 2 x 2k columns (one view: 2k) of the views'
+// padded rows; a slab per cluster (two sweeps: per CTA)
+static int64_t tc_slab(const Plan& p) { return (int64_t)tc_rows(p) * tc_nviews(p) * 2 * p.k; }
+static int tc_max_slabs(const Plan& p) { return tc_two(p) ? p.sm_count : p.sm_count / 2; }
+// operand rows of one part of the W image (two sweeps)
+static int tc_nw(const Plan& p) { return (tc_nviews(p) * 2 * p.k + 7) / 8 * 8; }
+int64_t tc_wimg_bytes(const Plan& p) {
+  if (!tc_two(p)) return 0;
+  const int64_t rows = p.dtype == GBCCA_FP32 ? 2 * p.n : p.n;
+  return (rows + 63) / 64 * (2 * (int64_t)tc_nw(p) * 128);
 }
 
 // Doubles of the partial Grams and floats of the partial slabs that a
-// tensor-core plan needs (all its column groups).
+// tensor-core plan needs.
 int64_t tc_gpart_len(const Plan& p) {
   const int k2 = 2 * p.k;
   return (int64_t)(tc_rows(p) / tc::kPostRows) * k2 * (tc_nviews(p) * k2 + k2);
 }
-int64_t tc_part_len(const Plan& p) { return (int64_t)(p.sm_count / 2) * tc_slab(p, 2 * p.k); }
+int64_t tc_part_len(const Plan& p) { return tc_max_slabs(p) * tc_slab(p); }
 
-// Arguments of the Phi images of a plan (both views, every column group),
-// group g with h1 rows per half (h1 = 0: each group's own); Phi is read from
-// the caller's blocks when `io` is given, else from the plan's own.
+// Arguments of the Phi images of a plan, h1 rows per half (0: the plan's own);
+// Phi is read from the caller's blocks when `io` is given, else from the
+// plan's own.
 static tc::ImageArgs tc_image_args(const Plan& p, int h1, const int* done, const PassIO* io) {
   tc::ImageArgs a{};
   const int nv = tc_nviews(p);
@@ -1039,13 +1019,8 @@ static tc::ImageArgs tc_image_args(const Plan& p, int h1, const int* done, const
     a.d[v] = p.v[v].d;
   }
   a.k2 = 2 * p.k;
-  for (int g = 0; g < tc_groups(p); ++g) {
-    int col0 = 0, ng = 0;
-    tc_group(p, g, &col0, &ng);
-    if (g == 0) a.ng0 = ng;
-    a.h[g] = h1 > 0 ? h1 : tc_group_h1(p, ng);
-    a.img[g] = tc_group_img(p, g);
-  }
+  a.h = h1 > 0 ? h1 : tc_h1(p);
+  a.img = p.tc_img;
   a.img_view = tc_img_view(p);
   a.done = done;
   return a;
@@ -1065,18 +1040,20 @@ int tc_phi_image(Plan& p, int h1, cudaStream_t st, const int* done, const PassIO
   return GBCCA_OK;
 }
 
-static tc::PostArgs tc_post_args(const Plan& p, int nparts, const int* nparts_dev, const int* done, const PassIO* io) {
+static tc::PostArgs tc_post_args(const Plan& p, const int* nparts, const int* nparts_dev, const int* done,
+                                 const PassIO* io) {
   tc::PostArgs a{};
   const int nv = tc_nviews(p), k2 = 2 * p.k;
-  for (int g = 0; g < tc_groups(p); ++g) {
-    int col0 = 0, ng = 0;
-    tc_group(p, g, &col0, &ng);
-    if (g == 0) a.ng0 = ng;
-    a.part[g] = tc_group_part(p, g);
-    a.slab[g] = tc_slab(p, ng);
-    a.nparts_dev[g] = nparts_dev != nullptr ? nparts_dev + g : nullptr;
+  a.part = p.tc_part;
+  a.slab = tc_slab(p);
+  a.nparts_dev = nparts_dev;
+  a.by_pair = tc_two(p) ? 1 : 0;
+  if (nparts != nullptr) {
+    if (a.by_pair)
+      std::memcpy(a.np, nparts, sizeof(a.np));
+    else
+      a.nparts = *nparts;
   }
-  a.nparts = nparts;
   a.nv = nv;
   a.k2 = k2;
   for (int v = 0; v < nv; ++v) {
@@ -1122,6 +1099,28 @@ static void tc_sources(const Plan& p, const void* src[2], int64_t ld[2], int64_t
   }
 }
 
+// A plan's pass in two sweeps (rows: of the streamed matrices).
+static two::Inst tc_two_inst(const Plan& p, int64_t rows, const CUtensorMap& mx, const CUtensorMap& my,
+                             const int* done) {
+  two::Inst I{};
+  I.map[0] = mx;
+  I.map[1] = my;
+  I.phi_img = p.tc_img;
+  I.img_view = tc_img_view(p);
+  I.wimg = static_cast<uint8_t*>(p.Wbuf);
+  I.part = p.tc_part;
+  I.slab = tc_slab(p);
+  I.done = done;
+  I.nv = tc_nviews(p);
+  for (int v = 0; v < I.nv; ++v) I.d[v] = p.v[v].d;
+  I.ncol = 2 * p.k;
+  I.nw = tc_nw(p);
+  I.pair_sum = p.dtype == GBCCA_FP32 ? 1 : 0;
+  I.ntiles = ceil_div(rows, tc::kRows);
+  I.wait = I.nv == 1 && p.opt.wait_cycles > 0 ? p.opt.wait_cycles : tc::kWaitCycles;
+  return I;
+}
+
 int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io) {
   // FP32 data: the row-interleaved hi/lo copy (2n rows) made when the data
   // was bound; BF16 data: the caller's matrices
@@ -1141,42 +1140,39 @@ int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io) {
   GB_TRY(tc_phi_image(p, 0, st, done, io));
   const CUtensorMap* mx = reinterpret_cast<const CUtensorMap*>(p.tc_map[0]);
   const CUtensorMap* my = reinterpret_cast<const CUtensorMap*>(p.tc_map[1]);
-  const int groups = tc_groups(p);
   if (p.kev0 != nullptr) GB_CUDA(record_timing_event(p.kev0, st));
-  int ncl = 1;
-  for (int g = 0; g < groups; ++g) {
-    int col0 = 0, ng = 0;
-    tc_group(p, g, &col0, &ng);
-    const int h1 = tc_group_h1(p, ng);  // Phi image rows per half (GEMM 1 N = 2 h1)
+  int nparts[16] = {};  // slabs written (two sweeps: per view and pair)
+  if (tc_two(p)) {
+    const two::Inst one = tc_two_inst(p, rows, *mx, *my, done);
+    GB_TRY(two::sweep_w(one, tc_h1(p), p.flag, p.sm_count, st));
+    GB_TRY(two::sweep_g(one, p.flag, p.sm_count, tc_max_slabs(p), nparts, st));
+  } else {
+    const int h1 = tc_h1(p);  // Phi image rows per half (GEMM 1 N = 2 h1)
     tc::Args a{};
     a.n = p.n;
     for (int v = 0; v < 2; ++v) {
       a.d[v] = v < nv ? p.v[v].d : 0;
       a.pairs[v] = ceil_div(a.d[v], 128);
     }
-    a.k2 = ng;
-    a.slab = tc_slab(p, ng);
+    a.k2 = 2 * p.k;
+    a.slab = tc_slab(p);
     a.wait_limit = p.opt.wait_cycles > 0 ? p.opt.wait_cycles : tc::kWaitCycles;
     a.ntiles = ceil_div(rows, tc::kRows);
     a.pair_sum = fp32 ? 1 : 0;
-    a.phi_img = tc_group_img(p, g);
+    a.phi_img = p.tc_img;
     a.img_view = tc_img_view(p);
-    a.partG = tc_group_part(p, g);
+    a.partG = p.tc_part;
     a.err = p.flag;
     a.done = done;
-    const bool quad = tc_quad(p);
-    const int csz = quad ? 4 : 2;  // CTAs per cluster
-    auto kern = solo ? (h1 == 20 ? tc::tc_pass_kernel<20, false, true> : tc::tc_pass_kernel<tc::kHalfMax, false, true>)
-                : quad ? (h1 == 20 ? tc::tc_pass_kernel<20, true> : tc::tc_pass_kernel<tc::kHalfMax, true>)
-                       : (h1 == 20 ? tc::tc_pass_kernel<20> : tc::tc_pass_kernel<tc::kHalfMax>);
-    const int smem = solo ? (h1 == 20 ? tc::Lay<20, false, true>::kSmemBytes : tc::Lay<tc::kHalfMax, false, true>::kSmemBytes)
-                     : quad ? (h1 == 20 ? tc::Lay<20, true>::kSmemBytes : tc::Lay<tc::kHalfMax, true>::kSmemBytes)
-                            : (h1 == 20 ? tc::Lay<20>::kSmemBytes : tc::Lay<tc::kHalfMax>::kSmemBytes);
+    auto kern = solo ? (h1 == 20 ? tc::tc_pass_kernel<20, true> : tc::tc_pass_kernel<tc::kHalfMax, true>)
+                     : (h1 == 20 ? tc::tc_pass_kernel<20> : tc::tc_pass_kernel<tc::kHalfMax>);
+    const int smem = solo ? (h1 == 20 ? tc::Lay<20, true>::kSmemBytes : tc::Lay<tc::kHalfMax, true>::kSmemBytes)
+                          : (h1 == 20 ? tc::Lay<20>::kSmemBytes : tc::Lay<tc::kHalfMax>::kSmemBytes);
     GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = csz;
+    attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.blockDim = dim3(tc::kThreads, 1, 1);
@@ -1186,13 +1182,13 @@ int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io) {
     cfg.numAttrs = 1;
     if (p.tc_clusters <= 0) {
       // persistent grid: as many clusters as can be resident at once
-      cfg.gridDim = dim3(csz * (p.sm_count / csz), 1, 1);
+      cfg.gridDim = dim3(2 * (p.sm_count / 2), 1, 1);
       int nc = 0;
       GB_CUDA(cudaOccupancyMaxActiveClusters(&nc, kern, &cfg));
-      p.tc_clusters = std::max(1, std::min(nc, p.sm_count / csz));
+      p.tc_clusters = std::max(1, std::min(nc, p.sm_count / 2));
     }
-    ncl = std::min(p.tc_clusters, a.ntiles);
-    cfg.gridDim = dim3(csz * ncl, 1, 1);
+    nparts[0] = std::min(p.tc_clusters, a.ntiles);
+    cfg.gridDim = dim3(2 * nparts[0], 1, 1);
     GB_CUDA(cudaLaunchKernelEx(&cfg, kern, *mx, *my, a));
     GB_CHECK_LAUNCH();
   }
@@ -1203,7 +1199,7 @@ int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io) {
     p.pass_forked = true;
   }
   tc::Posts<1> m{};
-  m.a[0] = tc_post_args(p, ncl, nullptr, done, io);
+  m.a[0] = tc_post_args(p, nparts, nullptr, done, io);
   Plan* one = &p;
   return tc_post_launch<1>(m, &one, 1, st);
 }
@@ -1215,14 +1211,10 @@ int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io) {
 // counts live in device memory, so a captured graph keeps one launch while
 // the schedule is rewritten between replays (finished plans drop out).
 struct TcBatch {
-  bool quad = false;           // 4-CTA clusters (plans with a view wider than 512)
-  int csz = 2;                 // CTAs per cluster
-  int n = 0;                   // table entries: one per (plan, column group)
-  int nplans = 0;
+  two::Batch* two = nullptr;   // plans that take two sweeps: their tables and schedules
+  int n = 0;                   // plans
   int h1 = tc::kHalfMax;       // Phi image rows per half, common to the batch
-  std::vector<int64_t> rows;   // streamed rows per entry
-  std::vector<int> first;      // per plan: its first entry (entries first .. first + count - 1)
-  std::vector<int> count;
+  std::vector<int64_t> rows;   // streamed rows per plan
   std::vector<int64_t> plan_bytes;  // algorithmic bytes of one pass per plan
   tc::Inst* inst_h = nullptr;  // pinned host copies of the tables
   tc::Seg* seg_h = nullptr;
@@ -1240,6 +1232,7 @@ struct TcBatch {
 
 void tc_batch_destroy(TcBatch* b) {
   if (b == nullptr) return;
+  two::batch_destroy(b->two);
   cudaFreeHost(b->inst_h);
   cudaFreeHost(b->seg_h);
   cudaFreeHost(b->off_h);
@@ -1261,26 +1254,45 @@ TcBatch* tc_batch_create(Plan* const* plans, int n, cudaStream_t st, int* rc) {
     *rc = GBCCA_ERR_OOM;
     return nullptr;
   }
-  b->nplans = n;
-  b->quad = n > 0 && tc_quad(*plans[0]);
-  b->csz = b->quad ? 4 : 2;
-  int entries = 0, h1 = 20, sm = 1;
+  b->n = n;
+  int h1 = 0, sm = 1;
   for (int i = 0; i < n; ++i) {
-    b->first.push_back(entries);
-    b->count.push_back(tc_groups(*plans[i]));
-    for (int g = 0; g < tc_groups(*plans[i]); ++g) {
-      int col0 = 0, ng = 0;
-      tc_group(*plans[i], g, &col0, &ng);
-      h1 = std::max(h1, tc_group_h1(*plans[i], ng));
-    }
-    entries += tc_groups(*plans[i]);
+    h1 = std::max(h1, tc_h1(*plans[i]));
     sm = std::max(sm, plans[i]->sm_count);
   }
-  b->n = entries;
   b->h1 = h1;
-  b->max_clusters = std::max(1, sm / b->csz);
-  b->max_segs = b->max_clusters + entries + 1;  // a contiguous partition has at most clusters + entries pieces
-  const int n1 = std::max(entries, 1);
+  b->max_clusters = std::max(1, sm / 2);
+  b->rows.assign(n, 0);
+  b->plan_bytes.assign(n, 0);
+  if (n > 0 && tc_two(*plans[0])) {
+    if (cudaMalloc(&b->err_d, sizeof(int)) != cudaSuccess || cudaMemsetAsync(b->err_d, 0, sizeof(int), st) != cudaSuccess) {
+      cudaGetLastError();
+      tc_batch_destroy(b);
+      set_last_error("allocation of the batch schedule failed");
+      *rc = GBCCA_ERR_OOM;
+      return nullptr;
+    }
+    std::vector<two::Inst> insts;
+    for (int i = 0; i < n && *rc == GBCCA_OK; ++i) {
+      Plan& p = *plans[i];
+      const void* src[2];
+      int64_t ld[2], rows = 0;
+      tc_sources(p, src, ld, &rows);
+      b->rows[i] = rows;
+      b->plan_bytes[i] = rows * (int64_t)(p.v[0].d + p.v[1].d) * 2;
+      CUtensorMap map[2];
+      for (int v = 0; v < 2 && *rc == GBCCA_OK; ++v) *rc = make_map(&map[v], src[v], rows, p.v[v].d, ld[v]);
+      if (*rc == GBCCA_OK) insts.push_back(tc_two_inst(p, rows, map[0], map[1], &p.st->done));
+    }
+    if (*rc == GBCCA_OK) b->two = two::batch_create(insts, h1, sm, st, rc);
+    if (b->two == nullptr) {
+      tc_batch_destroy(b);
+      return nullptr;
+    }
+    return b;
+  }
+  b->max_segs = b->max_clusters + n + 1;  // a contiguous partition has at most clusters + plans pieces
+  const int n1 = std::max(n, 1);
   bool ok = cudaMallocHost(&b->inst_h, sizeof(tc::Inst) * n1) == cudaSuccess &&
             cudaMallocHost(&b->seg_h, sizeof(tc::Seg) * b->max_segs) == cudaSuccess &&
             cudaMallocHost(&b->off_h, sizeof(int) * (b->max_clusters + 1)) == cudaSuccess &&
@@ -1298,37 +1310,30 @@ TcBatch* tc_batch_create(Plan* const* plans, int n, cudaStream_t st, int* rc) {
     return nullptr;
   }
   std::memset(b->inst_h, 0, sizeof(tc::Inst) * n1);
-  b->rows.assign(entries, 0);
-  b->plan_bytes.assign(n, 0);
   for (int i = 0; i < n; ++i) {
     Plan& p = *plans[i];
     const void* src[2];
     int64_t ld[2], rows = 0;
     tc_sources(p, src, ld, &rows);
     b->plan_bytes[i] = rows * (int64_t)(p.v[0].d + p.v[1].d) * 2;
-    for (int g = 0; g < b->count[i]; ++g) {
-      const int e = b->first[i] + g;
-      tc::Inst& I = b->inst_h[e];
-      b->rows[e] = rows;
-      for (int v = 0; v < 2; ++v) {
-        *rc = make_map(&I.map[v], src[v], rows, p.v[v].d, ld[v]);
-        if (*rc != GBCCA_OK) {
-          tc_batch_destroy(b);
-          return nullptr;
-        }
-        I.d[v] = p.v[v].d;
-        I.pairs[v] = ceil_div(p.v[v].d, 128);
+    b->rows[i] = rows;
+    tc::Inst& I = b->inst_h[i];
+    for (int v = 0; v < 2; ++v) {
+      *rc = make_map(&I.map[v], src[v], rows, p.v[v].d, ld[v]);
+      if (*rc != GBCCA_OK) {
+        tc_batch_destroy(b);
+        return nullptr;
       }
-      int col0 = 0, ng = 0;
-      tc_group(p, g, &col0, &ng);
-      I.phi_img = tc_group_img(p, g);
-      I.img_view = tc_img_view(p);
-      I.partG = tc_group_part(p, g);
-      I.done = &p.st->done;
-      I.k2 = ng;
-      I.pair_sum = p.dtype == GBCCA_FP32 ? 1 : 0;
-      I.slab = tc_slab(p, ng);
+      I.d[v] = p.v[v].d;
+      I.pairs[v] = ceil_div(p.v[v].d, 128);
     }
+    I.phi_img = p.tc_img;
+    I.img_view = tc_img_view(p);
+    I.partG = p.tc_part;
+    I.done = &p.st->done;
+    I.k2 = 2 * p.k;
+    I.pair_sum = p.dtype == GBCCA_FP32 ? 1 : 0;
+    I.slab = tc_slab(p);
   }
   cudaError_t e = cudaMemcpyAsync(b->inst_d, b->inst_h, sizeof(tc::Inst) * n1, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->err_d, 0, sizeof(int), st);
@@ -1347,10 +1352,10 @@ int* tc_batch_err(TcBatch* b) { return b->err_d; }
 int tc_batch_max_clusters(const TcBatch* b) { return b->max_clusters; }
 int tc_batch_clusters(const TcBatch* b) { return b->clusters; }
 // Algorithmic bytes of one batched pass over the active plans (each plan's
-// data once, whatever its column groups).
+// data once, also where two sweeps read it).
 int64_t tc_batch_bytes(const TcBatch* b, const bool* active) {
   int64_t s = 0;
-  for (int i = 0; i < b->nplans; ++i)
+  for (int i = 0; i < b->n; ++i)
     if (active == nullptr || active[i]) s += b->plan_bytes[i];
   return s;
 }
@@ -1364,16 +1369,13 @@ int64_t tc_batch_bytes(const TcBatch* b, const bool* active) {
 // adds that many slabs.  The tables go
 // to the device on `st`; the pinned host copies are rewritten only by the
 // next schedule, after the caller has synchronized `st`.
-int tc_batch_schedule(TcBatch* b, const bool* plan_active, int clusters, cudaStream_t st) {
+int tc_batch_schedule(TcBatch* b, const bool* active, int clusters, cudaStream_t st) {
   clusters = std::max(1, std::min(clusters, b->max_clusters));
-  std::vector<char> active(b->n, 0);  // per entry
-  for (int i = 0; i < b->nplans; ++i)
-    for (int g = 0; g < b->count[i]; ++g) active[b->first[i] + g] = plan_active[i] ? 1 : 0;
-  // pairs of a tile per CTA (4-CTA clusters: each view's pairs over two CTAs)
-  auto cta_pairs = [&](int i) {
-    const int P = std::max(b->inst_h[i].pairs[0], b->inst_h[i].pairs[1]);
-    return b->quad ? (P + 1) / 2 : P;
-  };
+  if (b->two != nullptr) {
+    b->clusters = clusters;
+    return two::batch_schedule(b->two, active, 2 * clusters, st);
+  }
+  auto cta_pairs = [&](int i) { return std::max(b->inst_h[i].pairs[0], b->inst_h[i].pairs[1]); };
   int64_t total = 0;
   for (int i = 0; i < b->n; ++i) {
     b->nparts_h[i] = 0;
@@ -1418,7 +1420,7 @@ int tc_batch_pre(const TcBatch* b, Plan& p, cudaStream_t st) {
 }
 
 // The same for all n plans of the table, a few plans per launch, from the
-// callers' blocks.
+// callers' blocks (two views: only CCA plans are batched).
 int tc_batch_pre_all(const TcBatch* b, Plan* const* plans, int n, const PassIO* io, cudaStream_t st) {
   for (int i0 = 0; i0 < n; i0 += tc::kManyPlans) {
     const int m = std::min(tc::kManyPlans, n - i0);
@@ -1436,20 +1438,24 @@ int tc_batch_pre_all(const TcBatch* b, Plan* const* plans, int n, const PassIO* 
 
 // One launch over every scheduled tile of the batch.
 int tc_batch_launch(TcBatch* b, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1) {
+  if (b->two != nullptr) {
+    if (e0 != nullptr) GB_CUDA(record_timing_event(e0, st));
+    GB_TRY(two::batch_launch(b->two, b->err_d, st));
+    if (e1 != nullptr) GB_CUDA(record_timing_event(e1, st));
+    return GBCCA_OK;
+  }
   tc::Args a{};
   a.err = b->err_d;
   a.insts = b->inst_d;
   a.segs = b->seg_d;
   a.seg_off = b->off_d;
-  auto kern = b->quad ? (b->h1 == 20 ? tc::tc_pass_kernel<20, true> : tc::tc_pass_kernel<tc::kHalfMax, true>)
-                      : (b->h1 == 20 ? tc::tc_pass_kernel<20> : tc::tc_pass_kernel<tc::kHalfMax>);
-  const int smem = b->quad ? (b->h1 == 20 ? tc::Lay<20, true>::kSmemBytes : tc::Lay<tc::kHalfMax, true>::kSmemBytes)
-                           : (b->h1 == 20 ? tc::Lay<20>::kSmemBytes : tc::Lay<tc::kHalfMax>::kSmemBytes);
+  auto kern = b->h1 == 20 ? tc::tc_pass_kernel<20> : tc::tc_pass_kernel<tc::kHalfMax>;
+  const int smem = b->h1 == 20 ? tc::Lay<20>::kSmemBytes : tc::Lay<tc::kHalfMax>::kSmemBytes;
   GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = b->csz;
+  attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.blockDim = dim3(tc::kThreads, 1, 1);
@@ -1457,7 +1463,7 @@ int tc_batch_launch(TcBatch* b, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1)
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cfg.gridDim = dim3(b->csz * std::max(1, b->clusters), 1, 1);
+  cfg.gridDim = dim3(2 * std::max(1, b->clusters), 1, 1);
   // the tensor-map parameters are unused in batch mode; any valid map will do
   const CUtensorMap* m0 = &b->inst_h[0].map[0];
   const CUtensorMap* m1 = &b->inst_h[0].map[1];
@@ -1468,10 +1474,15 @@ int tc_batch_launch(TcBatch* b, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1)
   return GBCCA_OK;
 }
 
-// Sum of plan i's slabs (every column group) into its G, then its Grams.
+// Slab counts of plan i in the device tables (two sweeps: 16, per view and pair).
+static const int* tc_batch_nparts(const TcBatch* b, int i) {
+  return b->two != nullptr ? b->two->np_d + 16 * i : b->nparts_d + i;
+}
+
+// Sum of plan i's slabs into its G, then its Grams.
 int tc_batch_post(const TcBatch* b, int i, Plan& p, cudaStream_t st, const int* done) {
   tc::Posts<1> m{};
-  m.a[0] = tc_post_args(p, 1, b->nparts_d + b->first[i], done, nullptr);
+  m.a[0] = tc_post_args(p, nullptr, tc_batch_nparts(b, i), done, nullptr);
   Plan* one = &p;
   return tc_post_launch<1>(m, &one, 1, st);
 }
@@ -1483,7 +1494,7 @@ int tc_batch_post_all(const TcBatch* b, Plan* const* plans, int n, const PassIO*
     const int c = std::min(tc::kManyPlans, n - i0);
     tc::Posts<tc::kManyPlans> m{};
     for (int i = 0; i < c; ++i)
-      m.a[i] = tc_post_args(*plans[i0 + i], 1, b->nparts_d + b->first[i0 + i], nullptr, &io[i0 + i]);
+      m.a[i] = tc_post_args(*plans[i0 + i], nullptr, tc_batch_nparts(b, i0 + i), nullptr, &io[i0 + i]);
     GB_TRY(tc_post_launch<tc::kManyPlans>(m, plans + i0, c, st));
   }
   return GBCCA_OK;

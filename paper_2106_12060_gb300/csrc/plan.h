@@ -270,8 +270,9 @@ int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io);
 int tc_phi_image(Plan& p, int h1, cudaStream_t st, const int* done, const PassIO* io);
 int64_t tc_gpart_len(const Plan& p);
 int64_t tc_part_len(const Plan& p);
-int tc_groups(const Plan& p);
-bool tc_quad(const Plan& p);
+bool tc_two(const Plan& p);
+int64_t tc_img_len(const Plan& p);
+int64_t tc_wimg_bytes(const Plan& p);
 // batched tensor-core pass over several eligible plans (one persistent launch)
 struct TcBatch;
 TcBatch* tc_batch_create(Plan* const* plans, int n, cudaStream_t st, int* rc);

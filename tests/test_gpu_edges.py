@@ -375,3 +375,72 @@ def test_factor_blocks_f32(gb, d):
         R = np64(gb.query(plan, q)).reshape(d, d)
         assert np.all(np.tril(R, -1) == 0) and np.all(np.diag(R) > 0)
         assert bound_ratio(R.T @ R, S.T @ S + lam * np.eye(d), ref, (s + 4 * d) * 2.0 ** -44) <= 1.0
+
+
+@pytest.mark.parametrize("dt", ["bf16", "f32"])
+@pytest.mark.parametrize("n,dx,dy,k", [(14, 13, 13, 13), (66, 64, 65, 14), (520, 513, 1, 1), (650, 385, 640, 16),
+                                       (1025, 1024, 1024, 2), (30011, 128, 24, 20)])
+def test_two_sweep_pass(gb, dt, n, dx, dy, k):
+    """The two-sweep pass where the one-sweep kernel cannot hold the columns
+    or the views: tiles and boxes of one row or column, every number of blocks
+    per view, alone and in a batch with a second plan (other slab counts),
+    within the bound of test_tc_pass_sums."""
+    import torch
+    tdt = {"bf16": torch.bfloat16, "f32": torch.float32}[dt]
+    plans, Phis, refs = [], [], []
+    for i, (m, a, b, kk) in enumerate(((n, dx, dy, k), (n + 70, dy, dx, k))):
+        rng = np.random.default_rng(n + k + i)
+        data = []
+        for d in (a, b):
+            t = torch.zeros(m, (d + 7) // 8 * 8, dtype=tdt, device="cuda")[:, :d]
+            t.copy_(torch.from_numpy(rng.standard_normal((m, d))))
+            data.append(t)
+        P = [rng.standard_normal((d, 2 * kk)) for d in (a, b)]
+        plan = gb.cca_plan(m, a, b, kk, dt, gb.default_options())
+        gb.cca_precondition(plan, *data, 1.0, 1.0)
+        Z = [np64(t) for t in data]
+        W = np.hstack([z @ p for z, p in zip(Z, P)])
+        aW = np.hstack([np.abs(z) @ np.abs(p) for z, p in zip(Z, P)])
+        plans.append((plan, data))
+        Phis.append([torch.from_numpy(p).cuda() for p in P])
+        refs.append((np.vstack([z.T @ W for z in Z]), np.vstack([np.abs(z).T @ aW for z in Z]), W.T @ W,
+                     np.vstack([np.abs(p).T @ (np.abs(z).T @ aW) for p, z in zip(P, Z)]),
+                     6 * 2.0 ** -16 + 2 * (m + a + b + 8) * 2.0 ** -23))
+    batch = gb.Batch([p for p, _ in plans])
+    Gb, Mb = gb.batch_fused_pass(batch, [f[0] for f in Phis], [f[1] for f in Phis])
+    for i, (plan, _) in enumerate(plans):
+        Gx, Gy, Gram = gb.fused_pass(plan, *Phis[i])
+        G, aG, M, aM, gamma = refs[i]
+        for got, gram in ((np.vstack([np64(Gx), np64(Gy)]), Gram), (np64(Gb[i]), Mb[i])):
+            assert bound_ratio(got, G, aG, gamma) <= 1.0
+            assert bound_ratio(np64(gram), M, aM, gamma) <= 1.0
+    batch.close()
+
+
+@pytest.mark.parametrize("n,d,k", [(80, 40, 13), (777, 385, 14), (5000, 1024, 20)])
+def test_two_sweep_pass_fda(gb, n, d, k):
+    """One view and more columns than one sweep holds; with a wait bound of
+    one cycle (where a wait is long enough to run out) the pass gives up,
+    drains what it has in flight and the solve reports it, and the next plan
+    solves as before."""
+    import torch
+    l = k + 2
+    P = lda_problem(n, d, l, dtype="f32", seed=d)
+    x, y = to_dev(P["X"], "f32"), torch.from_numpy(P["y"]).cuda()
+    if n == 5000:
+        plan = gb.lda_plan(n, d, l, k, "f32", gb.default_options(wait_cycles=1, max_iter=3))
+        with pytest.raises(gb.GbccaError) as e:
+            gb.lda_solve(plan, x, y, 1e-1)
+        assert e.value.code == gb.ERR_TIMEOUT
+        plan.close()
+    plan = gb.lda_plan(n, d, l, k, "f32", gb.default_options(max_iter=1))
+    gb.lda_solve(plan, x, y, 1e-1)
+    Phi = np.random.default_rng(d + 1).standard_normal((d, 2 * k))
+    G, _, Gram = gb.fused_pass(plan, torch.from_numpy(Phi).cuda())
+    X = P["X64"]
+    M = np.stack([X[P["y"] == c].mean(0) for c in range(l)])
+    Xc = X - M[P["y"]]
+    W, aW = Xc @ Phi, np.abs(Xc) @ np.abs(Phi)
+    gamma = 6 * 2.0 ** -16 + 2 * (n + d + 8) * 2.0 ** -23
+    assert bound_ratio(np64(G), Xc.T @ W, np.abs(Xc).T @ aW, gamma) <= 1.0
+    assert bound_ratio(np64(Gram), W.T @ W, np.abs(Phi).T @ (np.abs(Xc).T @ aW), gamma) <= 1.0
