@@ -9,13 +9,14 @@
 
 namespace gbcca {
 
-// 1 / x in FP64: the FP32 reciprocal corrected by one third-order step,
-// y (1 + e + e^2) with e = 1 - x y, |e| < 2^-22: three dependent
-// multiply-adds instead of a division.  Outside the float range: 1 / x.
+// 1 / x in FP64: the hardware's approximation (about 20 bits) corrected by one
+// third-order step, y (1 + e + e^2) with e = 1 - x y: three dependent
+// multiply-adds instead of a division, and no conversion (which would run at
+// the FP64 rate).  Near the ends of the exponent range: 1 / x.
 __device__ __forceinline__ double rcp_nr(double x) {
-  const float xf = (float)x;
-  if (!(fabsf(xf) > 1e-37f && fabsf(xf) < 1e37f)) return 1.0 / x;
-  const double y = (double)__frcp_rn(xf);
+  if (((uint32_t)__double2hiint(x) & 0x7fffffffu) - 0x00200000u >= 0x7fa00000u) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
@@ -37,19 +38,28 @@ __device__ __forceinline__ void group_sync(int id) {
 //
 // LDL^T with the inverse carried along: at step j the entry (i, c) of row
 // i > j, c in 0 .. i, is the trailing matrix for c > j and the unit inverse
-// for c <= j, and both are updated by -a_ij (row j entry) / d_j, so a step is
-// one reciprocal, one multiply and one multiply-add per entry behind a single
-// barrier, over all entries at once; the square roots follow at the end, all
-// at once.  (A Cholesky by one warp followed by the inverse, a column per
-// lane, was a chain of several hundred FP64 instructions.)
+// for c <= j, and both are updated by -a_ij y_c with y_c = (entry c of row j
+// of L^T or L^{-1}) / d_j; the square roots follow at the end, all at once.
+// The group's first warp runs one step ahead: it updates column j + 1 of the
+// matrix and row j + 1 of the inverse (a lane per entry), and so has the next
+// pivot, its reciprocal and the next y while the other warps update the rest,
+// one multiply-add per entry.  A step is that warp's chain (a multiply-add,
+// the reciprocal, a multiplication) and one barrier.  With the reciprocal and
+// the products a_ij / d_j formed by every thread a 32 x 32 block took 36 us of
+// FP64 issue; a Cholesky by one warp followed by the inverse, a column per
+// lane, was a chain of several hundred FP64 instructions.
 template <int G>
 __device__ bool group_chol_inverse(double* A, double* Li, double* rs, int n, int g, int id, int ld = 0) {
   if (ld == 0) ld = n;
-  constexpr int kItems = G == 128 ? 2 : 4;  // entries (i, c), c <= i, per thread
+  __shared__ double s_y[3][2][40];  // one per barrier id (0, or 1 and 2)
+  double(*ys)[40] = s_y[id];
+  constexpr int kItems = G == 128 ? 3 : 4;       // entries (i, c), c <= i, per thread of the other warps
+  constexpr int kT = G - 32;
+  static_assert(kItems * (G - 32) >= (G == 128 ? 210 : 820), "entries per thread");
   int ri[kItems], ci[kItems];
 #pragma unroll
   for (int u = 0; u < kItems; ++u) {
-    const int e = g + G * u;
+    const int e = g < 32 ? 900 : g - 32 + kT * u;
     int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
     while ((i + 1) * (i + 2) / 2 <= e) ++i;
     while (i * (i + 1) / 2 > e) --i;
@@ -60,33 +70,64 @@ __device__ bool group_chol_inverse(double* A, double* Li, double* rs, int n, int
       if (i != ci[u]) Li[ci[u] * ld + i] = 0.0;
     }
   }
+  group_sync<G>(id);
   bool ok = true;
-  for (int j = 0; j < n; ++j) {
-    group_sync<G>(id);
-    double d = A[j * ld + j];
-    if (!(d > 0.0)) {
-      ok = false;
-      d = 1.0;
-    }
-    if (j == n - 1) break;
-    const double r = rcp_nr(d);
+  for (int j = -1; j < n - 1; ++j) {
+    if (g < 32) {
+      const int p = j + 1;  // the next pivot
+      double val[2];
 #pragma unroll
-    for (int u = 0; u < kItems; ++u) {
-      const int i = ri[u], c = ci[u];
-      if (i > j && i < n) {
-        const double a = A[i * ld + j];
-        if (c > j)
-          A[i * ld + c] -= a * (A[c * ld + j] * r);
-        else
-          Li[i * ld + c] -= a * (Li[j * ld + c] * r);
+      for (int h = 0; h < 2; ++h) {
+        const int c = g + 32 * h;
+        val[h] = 0.0;
+        if (c < n && h * 32 < n) {
+          double* at = c >= p ? A + c * ld + p : Li + p * ld + c;
+          val[h] = *at;
+          if (j >= 0) {
+            const double f = c >= p ? A[c * ld + j] : A[p * ld + j];
+            val[h] -= f * ys[j & 1][c >= p ? p : c];
+            *at = val[h];
+          }
+        }
+      }
+      double d = __shfl_sync(0xffffffffu, p < 32 ? val[0] : val[1], p & 31);
+      if (!(d > 0.0)) {
+        ok = false;
+        d = 1.0;
+      }
+      const double r = rcp_nr(d);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = g + 32 * h;
+        if (c < n && h * 32 < n) ys[p & 1][c] = c == p ? r : val[h] * r;
+      }
+    } else if (j >= 0) {
+      const double* y = ys[j & 1];
+#pragma unroll
+      for (int u = 0; u < kItems; ++u) {
+        const int i = ri[u], c = ci[u];
+        if (i > j + 1 && i < n && c != j + 1) {
+          double* at = (c > j ? A : Li) + i * ld + c;
+          *at -= A[i * ld + j] * y[c];
+        }
       }
     }
+    group_sync<G>(id);
   }
-  if (g < n) {
-    const double d = A[g * ld + g];
-    rs[g] = d > 0.0 ? rsqrt_nr(d) : 1.0;
+  if (g < 32) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = g + 32 * h;
+      if (c < n) {
+        const double d = A[c * ld + c];
+        rs[c] = d > 0.0 ? rsqrt_nr(d) : 1.0;
+      }
+    }
+    __syncwarp();
+    if (!ok && g == 0) rs[0] = -1.0;  // the verdict, for every thread
   }
   group_sync<G>(id);
+  ok = __double2hiint(rs[0]) > 0;
 #pragma unroll
   for (int u = 0; u < kItems; ++u)
     if (ri[u] < n) Li[ri[u] * ld + ci[u]] *= rs[ri[u]];
