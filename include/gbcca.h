@@ -105,8 +105,9 @@ typedef struct {
   int32_t tensor_cores;  /* 1 (default): the data pass runs on the tensor-core
                             kernels where the plan is eligible (CCA: BF16 or
                             FP32 data, any shape, BF16 rows 16-byte aligned;
-                            FDA: FP32 data, d <= 1024); 0:
-                            the CUDA-core kernels only (for comparisons)     */
+                            FDA: FP32 data, d <= 1024), and so do the Grams
+                            of the sketches of FP32/BF16 plans; 0: the
+                            CUDA-core kernels only (for comparisons)         */
   int32_t warm_iters;    /* block power iterations of the CCA warm start (the
                             exact CCA of the sketched pair, Alg. 1 step 4);
                             0 = the default 12, which reaches the exact

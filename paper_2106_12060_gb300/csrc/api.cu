@@ -42,7 +42,7 @@ void free_plan(Plan* p) {
   if (p == nullptr) return;
   for (int v = 0; v < 2; ++v) {
     View& w = p->v[v];
-    for (void* q : {(void*)w.SZ, (void*)w.R, (void*)w.Rinv, (void*)w.Minv_hi, (void*)w.Minv_lo, (void*)w.SZh, (void*)w.SZl, (void*)w.RRh, (void*)w.RRl, (void*)w.Phi, (void*)w.Phi32,
+    for (void* q : {(void*)w.SZ, (void*)w.R, (void*)w.Rinv, (void*)w.Minv_hi, (void*)w.Minv_lo, (void*)w.SZh, (void*)w.SZl, (void*)w.SZs, (void*)w.SZe, (void*)w.RRh, (void*)w.RRl, (void*)w.Phi, (void*)w.Phi32,
                     (void*)w.Meta, (void*)w.gold, (void*)w.Mgold, (void*)w.LL, (void*)w.RR, (void*)w.tmp,
                     (void*)w.warm, (void*)w.wsU, (void*)w.wsT})
       dfree(q);
@@ -85,8 +85,13 @@ int alloc_plan(Plan* p) {
       GB_TRY(dalloc(&w.Minv_lo, (int64_t)d * d));
       GB_TRY(dalloc(&w.RRh, (int64_t)d * k2));
       GB_TRY(dalloc(&w.RRl, (int64_t)d * k2));
-      GB_TRY(dalloc(&w.SZh, p->s * d));
-      GB_TRY(dalloc(&w.SZl, p->s * d));
+      if (p->opt.tensor_cores) {
+        GB_TRY(dalloc(&w.SZs, gram_slices_len(p->s, d)));
+        GB_TRY(dalloc(&w.SZe, d));
+      } else {
+        GB_TRY(dalloc(&w.SZh, p->s * d));
+        GB_TRY(dalloc(&w.SZl, p->s * d));
+      }
     }
     GB_TRY(dalloc(&w.Phi, (int64_t)d * k2));
     GB_TRY(dalloc(&w.Phi32, (int64_t)d * k2));
@@ -327,9 +332,13 @@ int precondition_common(Plan& p, const int32_t* sh, const int8_t* sg, cudaStream
   }
   for (int v = 0; v < p.nviews; ++v) {
     View& w = p.v[v];
-    if (w.SZh != nullptr) {
-      // FP32/BF16 data: the Gram only shapes the preconditioner; double-float
-      // arithmetic (~2^-44 relative per product) at FP32 instruction rates
+    // FP32/BF16 data: the Gram only shapes the preconditioner; exact sums of
+    // 55-bit digits on the tensor cores, or double-float arithmetic (~2^-44
+    // relative per product) at FP32 instruction rates
+    if (w.SZs != nullptr) {
+      GB_TRY(gram_slice(w.SZ, p.s, w.d, w.SZe, w.SZs, st));
+      GB_TRY(gram_sliced(w.SZs, w.SZe, w.d, w.SZs, w.SZe, w.d, p.s, w.R, w.lam, p.ws, p.ws_len, p.sm_count, p.flag, st));
+    } else if (w.SZh != nullptr) {
       GB_TRY(split_rows(w.SZ, (int)p.s, w.d, w.d, w.SZh, w.SZl, st));
       GB_TRY(gram_df_split(w.SZh, w.SZl, w.d, w.SZh, w.SZl, w.d, p.s, w.d, w.d, w.R, w.lam, p.ws, p.ws_len, st));
     } else {

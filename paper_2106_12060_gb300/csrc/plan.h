@@ -51,7 +51,11 @@ struct View {
   double lam = 0;
   int ocol = 0;             // first column of this view's block in the pass W
   double* SZ = nullptr;     // sketch S Z (s x d)
-  float* SZh = nullptr;     // S Z as a float pair (FP32/BF16 plans)
+  // S Z for its Grams (FP32/BF16 plans): digit slices and column exponents
+  // with tensor cores, else a float pair
+  __nv_bfloat16* SZs = nullptr;
+  int* SZe = nullptr;
+  float* SZh = nullptr;
   float* SZl = nullptr;
   double* R = nullptr;      // d x d upper triangular, R^T R = M
   double* Rinv = nullptr;   // d x d, R^{-1}
@@ -203,6 +207,10 @@ int gram_tn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t 
 int gram_df_split(const float* Ah, const float* Al, int64_t lda, const float* Bh, const float* Bl, int64_t ldb,
                   int64_t m, int d1, int d2, double* C, double diag_add, double* ws, int64_t ws_len, cudaStream_t st,
                   bool tri = false);
+int64_t gram_slices_len(int64_t s, int d);
+int gram_slice(const double* A, int64_t s, int d, int* ex, __nv_bfloat16* S, cudaStream_t st);
+int gram_sliced(const __nv_bfloat16* A, const int* ea, int d1, const __nv_bfloat16* B, const int* eb, int d2, int64_t s,
+                double* C, double diag_add, double* ws, int64_t ws_len, int sm_count, int* err, cudaStream_t st);
 int cholesky_upper(double* A, int d, int* flag, cudaStream_t st);
 int cholesky_upper_blocks(double* A, double* Rinv, int d, int* flag, cudaStream_t st);
 // C = A^T A + lambda I (A: m x d FP64, row stride lda) with the split-K

@@ -2785,7 +2785,10 @@ int warm_start(Plan& p, cudaStream_t st) {
     const int c = std::min(2 * k, std::min(dx, dy));
     // Cxy = X_S^T Y_S (dx x dy), kept in ws after the Gram partials
     double* Cxy = p.ws + (p.ws_len - (int64_t)dx * dy);
-    if (x.SZh != nullptr)
+    if (x.SZs != nullptr)
+      GB_TRY(gram_sliced(x.SZs, x.SZe, dx, y.SZs, y.SZe, dy, p.s, Cxy, 0.0, p.ws, p.ws_len - (int64_t)dx * dy,
+                         p.sm_count, p.flag, st));
+    else if (x.SZh != nullptr)
       GB_TRY(gram_df_split(x.SZh, x.SZl, dx, y.SZh, y.SZl, dy, p.s, dx, dy, Cxy, 0.0, p.ws,
                            p.ws_len - (int64_t)dx * dy, st));
     else

@@ -444,3 +444,47 @@ def test_two_sweep_pass_fda(gb, n, d, k):
     gamma = 6 * 2.0 ** -16 + 2 * (n + d + 8) * 2.0 ** -23
     assert bound_ratio(np64(G), Xc.T @ W, np.abs(Xc).T @ aW, gamma) <= 1.0
     assert bound_ratio(np64(Gram), W.T @ W, np.abs(Phi).T @ (np.abs(Xc).T @ aW), gamma) <= 1.0
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("n,dx,dy,s", [(20, 1, 2, 7), (600, 63, 9, 66), (400, 129, 64, 300), (900, 200, 321, 897),
+                                       (12000, 40, 33, 9000)])
+def test_sketch_grams(gb, dt, n, dx, dy, s):
+    """Grams of the sketches: tiles and row windows with remainders, one and
+    several ranges of rows, columns over many orders of magnitude with a zero
+    and an outlier row.  R^T R against the sketch's own Gram: entries are
+    scaled to their columns, so the bound is 2^-46 of the columns' norms plus
+    the factorization's chain of d terms."""
+    import torch
+    from synth import countsketch_draws
+    rng = np.random.default_rng(dx)
+    tdt = {"f32": torch.float32, "bf16": torch.bfloat16}[dt]
+    lam = 1e-30
+    data = []
+    for d in (dx, dy):
+        Z = rng.standard_normal((n, d)) * 10.0 ** rng.integers(-9, 9, d)
+        Z[3] *= 1e4
+        Z[5] = 0.0
+        data.append(torch.from_numpy(Z).to(tdt).cuda())
+    h, g = countsketch_draws(n, s, seed=5)
+    plan = gb.cca_plan(n, dx, dy, 1, dt, gb.default_options(s=s, warm_start=0))
+    gb.cca_precondition(plan, *data, lam, lam, torch.from_numpy(h).cuda(), torch.from_numpy(g).cuda())
+    for qs, qr, d in ((gb.Q_SKETCH_X, gb.Q_R_X, dx), (gb.Q_SKETCH_Y, gb.Q_R_Y, dy)):
+        S = np64(gb.query(plan, qs)).reshape(s, d)
+        R = np64(gb.query(plan, qr)).reshape(d, d)
+        nrm = np.linalg.norm(S, axis=0)
+        # NumPy's own sum of s terms is in FP64
+        assert bound_ratio(R.T @ R, S.T @ S, np.outer(nrm, nrm), 2.0 ** -46 + (s + 4 * d) * 2.0 ** -53) <= 1.0
+
+
+def test_sketch_gram_rejects_overflow(gb):
+    """A sketch beyond the FP32 range, or not finite, is reported as before."""
+    import torch
+    n, d = 64, 5
+    for bad in (float("inf"), float("nan")):
+        X = np.random.default_rng(0).standard_normal((n, d)).astype(np.float32)
+        X[7, 2] = bad
+        x = torch.from_numpy(X).cuda()
+        plan = gb.cca_plan(n, d, d, 1, "f32", gb.default_options(warm_start=0))
+        with pytest.raises(gb.GbccaError):
+            gb.cca_precondition(plan, x, x, 1e-1, 1e-1)
