@@ -782,15 +782,17 @@ __global__ void __launch_bounds__(256) phi_image_kernel(const __grid_constant__ 
 //
 // The slabs (12.5 MB for 1024 x 40 columns and 76 clusters) sit in L2 when
 // the data kernel ends, so this is a matter of loads in flight and of FP64
-// rate (about two multiply-adds per clock and SM: 1.2M of them for the two
-// Grams, 2 us over 128 SMs), and of launches: one pass over the slabs, with
-// the Grams formed from the block's rows while they are in shared memory,
-// replaces a reduction, a Gram kernel that read G back (27 us together for
-// 1024 x 40, 19 now, cold) and the Gram of Phi (two launches).  A slab is column-major with the views' rows
-// padded to kPostRows; a CTA reads kPostRows rows of every column as two
-// float4 per (column, slab), the slabs strided over the S threads that share
-// an item (S = kPostThreads / items, so narrow plans split their slabs wider),
-// kPostLoads loads in flight each.  Sums are Neumaier-compensated FP32 per
+// rate (about two multiply-adds per clock and SM), and of launches: one pass
+// over the slabs, with the Grams formed from the block's rows while they are
+// in shared memory, replaces a reduction, a Gram kernel that read G back (27
+// us together for 1024 x 40) and the Gram of Phi (two launches).  The FP64 work
+// of a block, not the slabs, sets the time, so the blocks are as small as one
+// float4 of rows: with 8 rows and all of Phi^T Phi a launch took 23 us for 128 x
+// 80 columns (16 blocks) and 36 for 2048 x 80.  A slab is column-major with
+// the views' rows padded to kPostRows; a CTA reads kPostRows rows of every
+// column as one float4 per (column, slab), the slabs strided over the S
+// threads that share an item (S = kPostThreads / items, so narrow plans split
+// their slabs wider), kPostLoads loads in flight each.  Sums are Neumaier-compensated FP32 per
 // thread, then the S pairs are added in double-float, in fixed order: the
 // error is ~2^-45 of the largest partial, far below the partials' own
 // rounding, and does not depend on scheduling.
@@ -832,22 +834,22 @@ __global__ void __launch_bounds__(kPostThreads) tc_post_kernel(const __grid_cons
   const int v = r0 < d0p ? 0 : 1;
   const int row0 = v == 0 ? r0 : r0 - d0p;                              // row within the view
   const int nr = min(kPostRows, (v == 0 ? m.d[0] : m.d[1]) - row0);
-  const int NC = m.nv * m.k2, items = 2 * NC;
+  const int NC = m.nv * m.k2, items = NC;  // (column: one float4 of a slab)
+  static_assert(kPostRows == 4, "a float4 holds a block's rows");
   __shared__ float4 red_s[kPostThreads], red_c[kPostThreads];
   __shared__ double Gs[kPostRows][4 * kMaxK], Ps[kPostRows][2 * kMaxK];
   const int t = threadIdx.x;
-  const int S = kPostThreads / items;  // items <= 160
+  const int S = kPostThreads / items;  // items <= 80
   const int it = t % items, sl = t / items;
   for (int e = t; e < kPostRows * m.k2; e += kPostThreads) {
     const int r = e / m.k2, c = e - r * m.k2;
     Ps[r][c] = r < nr ? (v == 0 ? m.Phi[0] : m.Phi[1])[(int64_t)(row0 + r) * m.k2 + c] : 0.0;
   }
   if (sl < S) {
-    const int c = it >> 1;  // column of G: view-x products, then view-y products
     const int at = m.by_pair ? 8 * v + (row0 >> 7) : 0;
     const int nparts = m.nparts_dev != nullptr ? m.nparts_dev[at] : (m.by_pair ? m.np[at] : m.nparts);
     const int64_t stride = m.slab / 4;
-    const float4* src = reinterpret_cast<const float4*>(m.part + (int64_t)c * D + r0) + (it & 1);
+    const float4* src = reinterpret_cast<const float4*>(m.part + (int64_t)it * D + r0);
     float s[4] = {0.f, 0.f, 0.f, 0.f}, cp[4] = {0.f, 0.f, 0.f, 0.f};
     for (int b0 = sl; b0 < nparts; b0 += S * kPostLoads) {
       float4 x4[kPostLoads];
@@ -874,25 +876,32 @@ __global__ void __launch_bounds__(kPostThreads) tc_post_kernel(const __grid_cons
   const float* rc = reinterpret_cast<const float*>(red_c);
   for (int e = t; e < kPostRows * NC; e += kPostThreads) {
     const int r = e / NC, c = e - r * NC;
-    const int o = 4 * (2 * c + (r >> 2)) + (r & 3);
+    const int o = 4 * c + r;
     float sum = 0.f, comp = 0.f;
     for (int q = 0; q < S; ++q) df_pair_add(sum, comp, rs[4 * q * items + o], rc[4 * q * items + o]);
-    const double gv = (double)sum + (double)comp;
+    const double gv = widen(sum) + widen(comp);
     Gs[r][c] = gv;
     if (r < nr) G[(int64_t)(row0 + r) * NC + c] = gv;
   }
   __syncthreads();
   const int W = NC + m.k2;
   double* out = m.gpart + (int64_t)blockIdx.x * m.k2 * W;
-  for (int e = t; e < m.k2 * W; e += kPostThreads) {
-    const int i = e / W, b = e - i * W;
+  for (int e = t; e < m.k2 * NC; e += kPostThreads) {
+    const int i = e / NC, b = e - i * NC;
     double sum = 0.0;
-    if (b < NC) {
-      for (int r = 0; r < nr; ++r) sum += Ps[r][i] * Gs[r][b];
-    } else {
-      for (int r = 0; r < nr; ++r) sum += Ps[r][i] * Ps[r][b - NC];
-    }
-    out[e] = sum;
+    for (int r = 0; r < nr; ++r) sum += Ps[r][i] * Gs[r][b];
+    out[i * W + b] = sum;
+  }
+  // Phi^T Phi: one triangle, mirrored (products commute)
+  for (int e = t; e < m.k2 * (m.k2 + 1) / 2; e += kPostThreads) {
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    while ((i + 1) * (i + 2) / 2 <= e) ++i;
+    while (i * (i + 1) / 2 > e) --i;
+    const int b = e - i * (i + 1) / 2;
+    double sum = 0.0;
+    for (int r = 0; r < nr; ++r) sum += Ps[r][i] * Ps[r][b];
+    out[i * W + NC + b] = sum;
+    out[b * W + NC + i] = sum;
   }
 }
 

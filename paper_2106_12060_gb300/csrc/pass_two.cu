@@ -557,9 +557,11 @@ int batch_schedule(Batch* b, const bool* active, int ctas, cudaStream_t st) {
       if (!active[i]) continue;
       const Inst& I = b->inst_h[i];
       if (k == 0) {
-        int boxes = 1;
+        // a tile costs its boxes, but at least its epilogue (about a box per 8
+        // columns of Phi and view)
+        int boxes = 0;
         for (int v = 0; v < I.nv; ++v) boxes += (I.d[v] + 63) / 64;
-        items.push_back(Item{i, 0, I.ntiles, boxes});
+        items.push_back(Item{i, 0, I.ntiles, std::max(boxes, I.nv * I.ncol / 8) + 1});
       } else {
         for (int c = 0; c < block_count(I.d, I.nv); ++c)
           items.push_back(Item{i, c, I.ntiles, block_weight(I, c)});

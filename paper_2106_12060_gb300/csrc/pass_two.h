@@ -10,7 +10,7 @@ namespace tc {
 // Rows of a view in a partial slab: padded so that a block of kPostRows rows
 // belongs to one view and starts on a 16-byte boundary.  The padding is never
 // written and its sums are never used.
-constexpr int kPostRows = 8;
+constexpr int kPostRows = 4;
 __host__ __device__ __forceinline__ int pad_rows(int d) { return (d + kPostRows - 1) / kPostRows * kPostRows; }
 }  // namespace tc
 
