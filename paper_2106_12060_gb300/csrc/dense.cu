@@ -929,17 +929,27 @@ __global__ void __launch_bounds__(256) mat_thin_kernel(ThinMul p0, ThinMul p1, i
     if (i < m) {
       const double* Ai = transA ? A + i : A + (int64_t)i * ca;
       const int64_t sa = transA ? ca : 1;
-      for (int l = lo; l < hi; l += 8) {
-        double x[8], y[8];
+      // eight terms at a time, the next eight in flight under the arithmetic
+      double x0[8], y0[8], x1[8], y1[8];
+      auto load = [&](int l, double(&x)[8], double(&y)[8]) {
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int q = min(l + u, hi - 1);
           x[u] = Ai[q * sa];
           y[u] = B[q * ldb + col];
         }
+      };
+      auto add = [&](int l, const double(&x)[8], const double(&y)[8]) {
 #pragma unroll
         for (int u = 0; u < 8; ++u)
           if (l + u < hi) s += x[u] * y[u];
+      };
+      if (lo < hi) load(lo, x0, y0);
+      for (int l = lo; l < hi; l += 16) {
+        load(l + 8, x1, y1);
+        add(l, x0, y0);
+        load(l + 16, x0, y0);
+        add(l + 8, x1, y1);
       }
     }
     red[f] = s;

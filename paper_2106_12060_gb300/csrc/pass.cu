@@ -345,17 +345,25 @@ pass_g_async_kernel(PassViews pv, int64_t n, int NC, int D, const float* __restr
   }
 }
 
-// Sums of the partials, in order, sixteen loads in flight per thread (one at a
-// time it was a chain of loads: 12 us for 1800 + 400 entries of 63 and 32
-// partials).
+// Sums of the partials, in order, sixteen loads in flight per thread under the
+// additions of the sixteen before.
 __device__ __forceinline__ double sum_strided(const double* __restrict__ src, int64_t stride, int n) {
-  double s = 0.0;
-  for (int b0 = 0; b0 < n; b0 += 16) {
-    double x[16];
+  double s = 0.0, x[16], y[16];
+  auto load = [&](int b0, double(&v)[16]) {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) x[u] = b0 + u < n ? src[(int64_t)(b0 + u) * stride] : 0.0;
+    for (int u = 0; u < 16; ++u) v[u] = b0 + u < n ? src[(int64_t)(b0 + u) * stride] : 0.0;
+  };
+  auto add = [&](int b0, const double(&v)[16]) {  // (no additions past the end: each takes 64 cycles)
 #pragma unroll
-    for (int u = 0; u < 16; ++u) s += x[u];
+    for (int u = 0; u < 16; ++u)
+      if (b0 + u < n) s += v[u];
+  };
+  load(0, x);
+  for (int b0 = 0; b0 < n; b0 += 32) {
+    load(b0 + 16, y);
+    add(b0, x);
+    load(b0 + 32, x);
+    add(b0 + 16, y);
   }
   return s;
 }
@@ -401,8 +409,9 @@ __global__ void phi_convert_kernel(const double* __restrict__ a, Tacc* __restric
 // flight, a fixed shuffle tree.  Latency bound (r c is a few hundred, d at
 // most 1024): one thread per entry walking all d terms is a chain of d
 // dependent FP64 adds behind d loads (l = 10, d = 784, 18 columns: 184 us a
-// launch, once per iteration); with a warp per entry 25 terms per lane remain.
-__global__ void __launch_bounds__(256) table_phi_kernel(const double* __restrict__ T, const double* __restrict__ Phi,
+// launch, once per iteration); with a warp per entry 25 terms per lane remain,
+// and two warps per CTA put them on all SMs (eight on 23 of them: 17 us).
+__global__ void __launch_bounds__(64) table_phi_kernel(const double* __restrict__ T, const double* __restrict__ Phi,
                                                         int r, int d, int c, int stride, double* __restrict__ out,
                                                         const int* done) {
   if (done != nullptr && *done) return;
@@ -412,6 +421,7 @@ __global__ void __launch_bounds__(256) table_phi_kernel(const double* __restrict
   const double* t = T + (int64_t)row * d;
   double s[4] = {0.0, 0.0, 0.0, 0.0};
   int j = lane;
+#pragma unroll 2
   for (; j + 96 < d; j += 128) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) s[u] += t[j + 32 * u] * Phi[(int64_t)(j + 32 * u) * stride + q];
@@ -610,7 +620,7 @@ int run_pass64(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int
 
 int table_phi(const double* T, const double* Phi, int r, int d, int c, int stride, double* out, cudaStream_t st,
               const int* done) {
-  table_phi_kernel<<<ceil_div(r * c, 8), 256, 0, st>>>(T, Phi, r, d, c, stride, out, done);
+  table_phi_kernel<<<ceil_div(r * c, 2), 64, 0, st>>>(T, Phi, r, d, c, stride, out, done);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }
