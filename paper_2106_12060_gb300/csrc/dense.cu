@@ -263,9 +263,8 @@ __device__ __forceinline__ void df_add(float& S, float& Cc, float s2, float c2) 
   Cc += err + c2;
 }
 
-constexpr int kMvRows = 8;             // output rows per CTA
 constexpr int kMvThreads = 256;
-constexpr int kMvStageBytes = 118784;  // shared memory of one staged K chunk (A rows + X rows)
+constexpr int kMvStageBytes = 212992;  // shared memory of one staged K chunk (A rows + X rows) at most
 
 // n floats (4, 2 or 1) from global to shared memory, asynchronously
 __device__ __forceinline__ void cp_async_f(float* smem, const float* gmem, int n) {
@@ -284,7 +283,9 @@ __host__ __device__ __forceinline__ int mv_cols(int c) { return (c + 3) / 4 * 4;
 
 // Y_b (m x c) = A_b X_b for problem b = blockIdx.y, A_b (m x K, row-major)
 // and X_b (K x c, row stride ldx) as double-float pairs hi + lo; optionally
-// Y_b as a pair too (Yh, Yl, row stride c).  A CTA owns kMvRows rows of Y.  The
+// Y_b as a pair too (Yh, Yl, row stride c).  A CTA owns kMvRows rows of Y, as
+// few (2, 4, 6 or 8) as put one CTA on every SM: a CTA stages all of X, so more
+// CTAs than SMs only stage it again.  The
 // K range is walked in chunks staged in shared memory by the widest
 // asynchronous copies the alignment allows, in two halves, so that the first
 // is worked on while the second arrives.  A thread owns 2 rows x 4 columns of
@@ -295,6 +296,7 @@ __host__ __device__ __forceinline__ int mv_cols(int c) { return (c + 3) / 4 * 4;
 // scheduling.  Bound by FP32 issue (512 x 512 x 20, two views: 3 us of
 // arithmetic); one output per thread behind 4-byte copies of all of X per
 // four rows took 13 to 19 us a launch.
+template <int kMvRows>
 __global__ void __launch_bounds__(kMvThreads) dfmv_kernel(DfmvArgs a) {
   if (a.done != nullptr && *a.done) return;
   // the problem's fields by selection (a dynamic index into the parameter
@@ -319,7 +321,7 @@ __global__ void __launch_bounds__(kMvThreads) dfmv_kernel(DfmvArgs a) {
   float* Xh = Al + kMvRows * lda;  // [Kc][cp]
   float* Xl = Xh + Kc * cp;
   const int t = threadIdx.x;
-  const int CG = cp / 4, per = 4 * CG;  // threads of a slice: 4 row pairs x CG column groups
+  const int CG = cp / 4, per = kMvRows / 2 * CG;  // threads of a slice: row pairs x CG column groups
   const int KS = kMvThreads / per;
   const int ks = t / per, w = t - ks * per, rg = w / CG, cg = w - rg * CG;
   const bool active = ks < KS;
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(kMvThreads) dfmv_kernel(DfmvArgs a) {
   }
 }
 
-int dfmv(const DfmvArgs& a, int nprob, cudaStream_t st) {
+int dfmv(const DfmvArgs& a, int nprob, int sm_count, cudaStream_t st) {
   if (a.c < 1 || a.c > 64 || nprob < 1 || nprob > 2) {
     set_last_error("dfmv: unsupported column count");
     return GBCCA_ERR_INVALID_ARG;
@@ -424,12 +426,16 @@ int dfmv(const DfmvArgs& a, int nprob, cudaStream_t st) {
     g.p[b].wa = copy_width(a.p[b].hi, a.p[b].lo, a.p[b].K, 0);
     g.p[b].wx = copy_width(a.p[b].Xh, a.p[b].Xl, a.c, a.p[b].ldx);
   }
-  const int per_q = 8 * (kMvRows + mv_cols(a.c));
+  int64_t rows_all = 0;
+  for (int b = 0; b < nprob; ++b) rows_all += a.p[b].m;
+  const int rows = 2 * (int)std::max<int64_t>(1, std::min<int64_t>(4, ceil_div(rows_all, 2 * sm_count)));
+  const int per_q = 8 * (rows + mv_cols(a.c));
   const int chunks = ceil_div((int64_t)kmax * per_q, kMvStageBytes);
   g.kc = (ceil_div(kmax, chunks) + 31) / 32 * 32;
-  const size_t smem = std::max<size_t>((size_t)per_q * g.kc + 8 * kMvRows * 4, 8 * 8 * (size_t)kMvThreads);
-  GB_CUDA(cudaFuncSetAttribute(dfmv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dfmv_kernel<<<dim3(ceil_div(mmax, kMvRows), nprob), kMvThreads, smem, st>>>(g);
+  const size_t smem = std::max<size_t>((size_t)per_q * g.kc + 8 * rows * 4, 8 * 8 * (size_t)kMvThreads);
+  auto kern = rows == 2 ? dfmv_kernel<2> : rows == 4 ? dfmv_kernel<4> : rows == 6 ? dfmv_kernel<6> : dfmv_kernel<8>;
+  GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<dim3(ceil_div(mmax, rows), nprob), kMvThreads, smem, st>>>(g);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }

@@ -238,7 +238,7 @@ struct DfmvArgs {
   const int* done;
   int kc;            // K chunk staged in shared memory (set by dfmv)
 };
-int dfmv(const DfmvArgs& a, int nprob, cudaStream_t st);
+int dfmv(const DfmvArgs& a, int nprob, int sm_count, cudaStream_t st);
 // hi/lo split of the first c columns of X (rows x ldx) into rows x c floats
 int split_rows(const double* X, int rows, int c, int ldx, float* hi, float* lo, cudaStream_t st);
 // hi/lo split of A (r x c, row-major) or of its transpose (c x r)

@@ -2243,7 +2243,7 @@ int iteration_post(Plan& p, bool low, cudaStream_t st) {
                            0,              0};
     m.c = 2 * k;
     m.done = done;
-    GB_TRY(dfmv(m, p.nviews, st));
+    GB_TRY(dfmv(m, p.nviews, p.sm_count, st));
   } else {
     GB_TRY(minv(p, st, done));
   }
@@ -2830,7 +2830,7 @@ int warm_start(Plan& p, cudaStream_t st) {
       g.p[0] = DfmvProblem{A[0], A[1], B[0], B[1], Y, m, K, c, c, Yp != nullptr ? Yp[0] : nullptr,
                            Yp != nullptr ? Yp[1] : nullptr, 0, 0};
       g.c = c;
-      return dfmv(g, 1, st);
+      return dfmv(g, 1, p.sm_count, st);
     };
     auto rx = [&](bool tr, const double* B, double* C, int cc) {
       const ThinMul t{x.Rinv, dx, dx, B, cc, C, cc};
