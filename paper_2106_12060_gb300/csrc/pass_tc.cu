@@ -754,6 +754,7 @@ struct ImageArgs {
   uint8_t* img;
   int64_t img_view;
   const int* done;
+  int* restart;          // a convergence flag to clear (the plan takes part again), or null
 };
 constexpr int kManyPlans = 16;  // plans of one launch of the per-plan kernels
 template <int N> struct Images { ImageArgs a[N]; };
@@ -763,6 +764,7 @@ __global__ void __launch_bounds__(256) phi_image_kernel(const __grid_constant__ 
   const ImageArgs& m = many.a[blockIdx.z];
   if (m.done != nullptr && *m.done) return;
   const int v = blockIdx.y;
+  if (m.restart != nullptr && v == 0 && blockIdx.x == 0 && threadIdx.x == 0) *m.restart = 0;
   const int d = v == 0 ? m.d[0] : m.d[1];
   const int e = blockIdx.x * blockDim.x + threadIdx.x;  // (data column j, Phi column q)
   if (e >= d * m.k2) return;
@@ -1234,6 +1236,7 @@ struct TcBatch {
   int* off_d = nullptr;
   int* nparts_d = nullptr;
   int* err_d = nullptr;
+  std::vector<char> sched;     // active set of the tables in device memory (empty: none yet)
   int max_clusters = 0;        // clusters the tables have room for
   int clusters = 0;            // clusters of the current schedule
   int max_segs = 0;
@@ -1380,9 +1383,15 @@ int64_t tc_batch_bytes(const TcBatch* b, const bool* active) {
 // next schedule, after the caller has synchronized `st`.
 int tc_batch_schedule(TcBatch* b, const bool* active, int clusters, cudaStream_t st) {
   clusters = std::max(1, std::min(clusters, b->max_clusters));
+  // the same set over as many CTAs: the tables in device memory stand
+  const std::vector<char> want(active, active + b->n);
+  if (clusters == b->clusters && want == b->sched) return GBCCA_OK;
+  b->sched.clear();
   if (b->two != nullptr) {
+    GB_TRY(two::batch_schedule(b->two, active, 2 * clusters, st));
     b->clusters = clusters;
-    return two::batch_schedule(b->two, active, 2 * clusters, st);
+    b->sched = want;
+    return GBCCA_OK;
   }
   auto cta_pairs = [&](int i) { return std::max(b->inst_h[i].pairs[0], b->inst_h[i].pairs[1]); };
   int64_t total = 0;
@@ -1419,6 +1428,7 @@ int tc_batch_schedule(TcBatch* b, const bool* active, int clusters, cudaStream_t
   GB_CUDA(cudaMemcpyAsync(b->seg_d, b->seg_h, sizeof(tc::Seg) * std::max(nseg, 1), cudaMemcpyHostToDevice, st));
   GB_CUDA(cudaMemcpyAsync(b->off_d, b->off_h, sizeof(int) * (clusters + 1), cudaMemcpyHostToDevice, st));
   GB_CUDA(cudaMemcpyAsync(b->nparts_d, b->nparts_h, sizeof(int) * std::max(b->n, 1), cudaMemcpyHostToDevice, st));
+  b->sched = want;
   return GBCCA_OK;
 }
 
@@ -1429,7 +1439,8 @@ int tc_batch_pre(const TcBatch* b, Plan& p, cudaStream_t st) {
 }
 
 // The same for all n plans of the table, a few plans per launch, from the
-// callers' blocks (two views: only CCA plans are batched).
+// callers' blocks (two views: only CCA plans are batched); the plans' flags are
+// cleared, so that the pass serves all of them.
 int tc_batch_pre_all(const TcBatch* b, Plan* const* plans, int n, const PassIO* io, cudaStream_t st) {
   for (int i0 = 0; i0 < n; i0 += tc::kManyPlans) {
     const int m = std::min(tc::kManyPlans, n - i0);
@@ -1437,6 +1448,7 @@ int tc_batch_pre_all(const TcBatch* b, Plan* const* plans, int n, const PassIO* 
     int blocks = 1;
     for (int i = 0; i < m; ++i) {
       a.a[i] = tc_image_args(*plans[i0 + i], b->h1, nullptr, &io[i0 + i]);
+      a.a[i].restart = &plans[i0 + i]->st->done;
       blocks = std::max(blocks, tc_image_blocks(*plans[i0 + i]));
     }
     tc::phi_image_kernel<tc::kManyPlans><<<dim3(blocks, 2, m), 256, 0, st>>>(a);
