@@ -60,6 +60,44 @@ gram_tn_kernel(const double* __restrict__ A, int64_t lda, const double* __restri
     }
 }
 
+// The same partials on 16 x 16 tiles, one entry per thread (the same chain of
+// terms), for matrices whose 64 x 64 tiles would leave SMs idle: a tile's 64 rows
+// are 70 us of FP64 issue on one SM, three times in a solve with 50 columns.
+__global__ void __launch_bounds__(256)
+gram_tn_small_kernel(const double* __restrict__ A, int64_t lda, const double* __restrict__ B, int64_t ldb,
+                     int64_t m, int d1, int d2, int64_t kchunk, double* __restrict__ part) {
+  constexpr int kR = 64;  // rows per step
+  __shared__ double As[kR][17], Bs[kR][17];
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int i0 = blockIdx.y * 16, j0 = blockIdx.x * 16;
+  const int64_t k0 = blockIdx.z * kchunk, k1 = min(m, k0 + kchunk);
+  double acc = 0.0;
+  for (int64_t kk = k0; kk < k1; kk += kR) {
+#pragma unroll
+    for (int u = 0; u < kR / 16; ++u) {
+      const int r = ty + 16 * u;
+      const int64_t row = kk + r;
+      As[r][tx] = row < k1 && i0 + tx < d1 ? A[row * lda + i0 + tx] : 0.0;
+      Bs[r][tx] = row < k1 && j0 + tx < d2 ? B[row * ldb + j0 + tx] : 0.0;
+    }
+    __syncthreads();
+    const int nr = (int)min((int64_t)kR, k1 - kk);
+#pragma unroll 8
+    for (int r = 0; r < nr; ++r) acc += As[r][ty] * Bs[r][tx];
+    __syncthreads();
+  }
+  if (i0 + ty < d1 && j0 + tx < d2) part[((int64_t)blockIdx.z * d1 + i0 + ty) * d2 + j0 + tx] = acc;
+}
+
+static void launch_gram_tn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t m, int d1, int d2, int ks,
+                           int64_t kchunk, double* part, cudaStream_t st) {
+  if (ceil_div(d1, kGT) * ceil_div(d2, kGT) * ks < 152)
+    gram_tn_small_kernel<<<dim3(ceil_div(d2, 16), ceil_div(d1, 16), ks), 256, 0, st>>>(A, lda, B, ldb, m, d1, d2, kchunk,
+                                                                                     part);
+  else
+    gram_tn_kernel<<<dim3(ceil_div(d2, kGT), ceil_div(d1, kGT), ks), 256, 0, st>>>(A, lda, B, ldb, m, d1, d2, kchunk, part);
+}
+
 // C (d x d) from the split-K partials of a symmetric Gram whose tiles were
 // formed on and below the diagonal only: the upper tiles mirror the lower.
 __global__ void sum_parts_sym_kernel(const double* __restrict__ part, int nparts, int d, double diag_add,
@@ -212,8 +250,7 @@ int gram_tn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t 
     return GBCCA_ERR_INVALID_ARG;
   }
   int64_t kchunk = (m + ks - 1) / ks;
-  dim3 grid(ceil_div(d2, kGT), ceil_div(d1, kGT), ks);
-  gram_tn_kernel<<<grid, 256, 0, st>>>(A, lda, B, ldb, m, d1, d2, kchunk, ws);
+  launch_gram_tn(A, lda, B, ldb, m, d1, d2, ks, kchunk, ws, st);
   GB_CHECK_LAUNCH();
   sum_parts_kernel<<<ceil_div(len, 256), 256, 0, st>>>(ws, ks, len, d1, d2, diag_add, C);
   GB_CHECK_LAUNCH();
@@ -547,8 +584,7 @@ int gram_noalloc(const double* A, int64_t lda, int64_t m, int d, double lambda, 
   int ks = std::max(1, std::min<int>(ceil_div(304, tiles), ceil_div(m, 64)));
   while (ks > 1 && (int64_t)ks * len > kNoAllocScratch) --ks;
   const int64_t kchunk = (m + ks - 1) / ks;
-  dim3 grid(ceil_div(d, kGT), ceil_div(d, kGT), ks);
-  gram_tn_kernel<<<grid, 256, 0, st>>>(A, lda, A, lda, m, d, d, kchunk, ws);
+  launch_gram_tn(A, lda, A, lda, m, d, d, ks, kchunk, ws, st);
   GB_CHECK_LAUNCH();
   sum_parts_kernel<<<ceil_div(len, 256), 256, 0, st>>>(ws, ks, len, d, d, lambda, C);
   GB_CHECK_LAUNCH();
@@ -909,14 +945,20 @@ int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t 
 // 40 columns whatever the shape took 23 + 3 us per product of a 50 x 50 factor
 // with 10 columns, eight of them an iteration for two views.
 constexpr int kSlice = 64;
+constexpr size_t kThinStageBytes = 65536;  // staged operands (beyond it every CTA copying B costs more than it saves)
 
 // (rows per CTA: as many as its 256 threads hold outputs x slices of, at most 8)
 static int thin_rows(int c, int K) { return std::max(1, std::min(8, 256 / (c * ceil_div(K, kSlice)))); }
 
+// kStage (operands that fit shared memory): the CTA's rows of op(A) and all of
+// B are copied there at once, so that a product waits for memory once, not once
+// per eight terms (50 x 50 times 5 columns: 6.6 us a launch with the loads in
+// registers).
+template <bool kStage>
 __global__ void __launch_bounds__(256) mat_thin_kernel(ThinMul p0, ThinMul p1, int rows0, int rows1, int transA, int tri,
                                                        int c, int c0, const int* done) {
-  if (done != nullptr && *done) return;
-  extern __shared__ double red[];  // [slice][rows x c]
+  extern __shared__ double red[];  // [slice][rows x c], then with kStage [rows][K + 1] of op(A) and [K][c] of B
+  if (!kStage && done != nullptr && *done) return;
   const bool b1 = blockIdx.y != 0;
   const double* A = b1 ? p1.A : p0.A;
   const double* B = (b1 ? p1.B : p0.B) + c0;
@@ -926,13 +968,35 @@ __global__ void __launch_bounds__(256) mat_thin_kernel(ThinMul p0, ThinMul p1, i
   const int i0 = blockIdx.x * rows;
   if (i0 >= m) return;  // uniform over the CTA
   const int nout = rows * c, ns = (K + kSlice - 1) / kSlice;
+  double* As = red + nout * ns;
+  double* Bs = As + rows * (K + 1);
+  if constexpr (kStage) {
+    auto copy = [](double* dst, const double* src) {
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                   : "memory");
+    };
+    const int nr = min(rows, m - i0);
+    for (int f = threadIdx.x; f < rows * K; f += 256) {
+      const int r = transA ? f % rows : f / K, l = transA ? f / rows : f - r * K;
+      if (r < nr) copy(As + r * (K + 1) + l, transA ? A + (int64_t)l * ca + i0 + r : A + (int64_t)(i0 + r) * ca + l);
+    }
+    for (int f = threadIdx.x; f < K * c; f += 256) copy(Bs + f, B + (f / c) * ldb + f % c);
+    const bool skip = done != nullptr && *done;  // read behind the copies' issue
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (skip) return;
+  }
   for (int f = threadIdx.x; f < nout * ns; f += 256) {
     const int sl = f / nout, e = f - sl * nout, r = e / c, col = e - r * c, i = i0 + r;
     // op(A)[i][l] is non-zero for l >= i (A upper) or l <= i (its transpose)
     const int lo = max(sl * kSlice, tri && !transA ? i : 0);
     const int hi = min(min(K, (sl + 1) * kSlice), tri && transA ? i + 1 : K);
     double s = 0.0;
-    if (i < m) {
+    if (kStage && i < m) {
+      const double *Ar = As + r * (K + 1), *Bc = Bs + col;
+#pragma unroll 8
+      for (int l = lo; l < hi; ++l) s += Ar[l] * Bc[l * c];
+    } else if (i < m) {
       const double* Ai = transA ? A + i : A + (int64_t)i * ca;
       const int64_t sa = transA ? ca : 1;
       // eight terms at a time, the next eight in flight under the arithmetic
@@ -974,15 +1038,21 @@ int mat_thin(const ThinMul* p, int nprob, bool transA, bool tri, int c, cudaStre
   for (int c0 = 0; c0 < c; c0 += 64) {
     const int cw = std::min(64, c - c0);
     int blocks = 1, rows[2] = {1, 1};
-    size_t smem = 0;
+    size_t smem = 0, stage = 0;
     for (int b = 0; b < nprob; ++b) {
       const int m = transA ? p[b].ca : p[b].ra, K = transA ? p[b].ra : p[b].ca;
       rows[b] = thin_rows(cw, K);
       blocks = std::max(blocks, ceil_div(m, rows[b]));
-      smem = std::max(smem, sizeof(double) * rows[b] * cw * ceil_div(K, kSlice));
+      const size_t red = sizeof(double) * rows[b] * cw * ceil_div(K, kSlice);
+      smem = std::max(smem, red);
+      stage = std::max(stage, red + sizeof(double) * ((size_t)rows[b] * (K + 1) + (size_t)K * cw));
     }
-    mat_thin_kernel<<<dim3(blocks, nprob), 256, smem, st>>>(p[0], p[nprob > 1 ? 1 : 0], rows[0], rows[1],
-                                                            transA ? 1 : 0, tri ? 1 : 0, cw, c0, done);
+    const bool staged = stage <= kThinStageBytes;
+    if (staged) smem = stage;
+    auto kern = staged ? mat_thin_kernel<true> : mat_thin_kernel<false>;
+    GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<dim3(blocks, nprob), 256, smem, st>>>(p[0], p[nprob > 1 ? 1 : 0], rows[0], rows[1], transA ? 1 : 0, tri ? 1 : 0,
+                                                 cw, c0, done);
     GB_CHECK_LAUNCH();
   }
   return GBCCA_OK;

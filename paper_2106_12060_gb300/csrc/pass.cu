@@ -368,15 +368,41 @@ __device__ __forceinline__ double sum_strided(const double* __restrict__ src, in
   return s;
 }
 
-__global__ void __launch_bounds__(64) pass_reduce_kernel(const double* __restrict__ partG, int chunks, int64_t nG,
-                                                         const double* __restrict__ partGram, int ctas, int64_t nGram,
-                                                         double* __restrict__ G0, double* __restrict__ G1, int64_t n0,
-                                                         double* __restrict__ Gram, const int* done) {
-  if (done != nullptr && *done) return;
-  const int64_t e = blockIdx.x * (int64_t)64 + threadIdx.x;
-  if (e < n0 && e < nG) G0[e] = sum_strided(partG + e, nG, chunks);  // view 0's rows, then view 1's
-  else if (e < nG) G1[e - n0] = sum_strided(partG + e, nG, chunks);
-  else if (e < nG + nGram) Gram[e - nG] = sum_strided(partGram + (e - nG), nGram, ctas);
+// G and the Gram: a CTA takes 64 entries; its 256 threads bring 64 partials of
+// each into shared memory at once, then a thread per entry adds them in order
+// (bound by that chain, 67 cycles an addition; with sixteen loads in flight per
+// thread 1800 + 400 entries of 63 and 32 partials took 9.6 us, 4.4 now).
+__global__ void __launch_bounds__(256) pass_reduce_kernel(const double* __restrict__ partG, int chunks, int64_t nG,
+                                                          const double* __restrict__ partGram, int ctas, int64_t nGram,
+                                                          double* __restrict__ G0, double* __restrict__ G1, int64_t n0,
+                                                          double* __restrict__ Gram, const int* done) {
+  __shared__ double sm[64][65];
+  const int t = threadIdx.x & 63, w = threadIdx.x >> 6;
+  const int64_t e = blockIdx.x * (int64_t)64 + t;
+  const bool g = e < nG;
+  const double* src = g ? partG + e : partGram + (e - nG);
+  const int64_t stride = g ? nG : nGram;
+  const int n = e < nG + nGram ? (g ? chunks : ctas) : 0, most = max(nG > 0 ? chunks : 0, ctas);
+  double s = 0.0;
+  for (int b0 = 0; b0 < most; b0 += 64) {
+    double x[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) x[u] = b0 + w + 4 * u < n ? src[(int64_t)(b0 + w + 4 * u) * stride] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) sm[w + 4 * u][t] = x[u];
+    if (done != nullptr && *done) return;  // (uniform; read behind the loads)
+    __syncthreads();
+    if (w == 0) {
+      const int nb = min(64, n - b0);
+#pragma unroll 8
+      for (int q = 0; q < nb; ++q) s += sm[q][t];
+    }
+    __syncthreads();
+  }
+  if (w != 0 || n == 0) return;
+  if (e < n0 && g) G0[e] = s;  // view 0's rows, then view 1's
+  else if (g) G1[e - n0] = s;
+  else Gram[e - nG] = s;
 }
 
 // FDA: Xhat^T P = X^T P - sum_k m_k (sum_{i in k} P_i)^T.
@@ -405,32 +431,43 @@ __global__ void phi_convert_kernel(const double* __restrict__ a, Tacc* __restric
 
 // out (r x c) = T (r x d) Phi[:, 0:c], Phi row-major with row stride `stride`:
 // a class table (FDA: the class means, or Yhat) times the current Phi.  One
-// warp per entry, the lanes over the inner index with four partial sums in
-// flight, a fixed shuffle tree.  Latency bound (r c is a few hundred, d at
+// warp per entry, the lanes over the inner index with four partial sums, a
+// fixed shuffle tree.  A CTA takes one column and kTableRows rows of T, both
+// copied to shared memory at once.  Latency bound (r c is a few hundred, d at
 // most 1024): one thread per entry walking all d terms is a chain of d
 // dependent FP64 adds behind d loads (l = 10, d = 784, 18 columns: 184 us a
-// launch, once per iteration); with a warp per entry 25 terms per lane remain,
-// and two warps per CTA put them on all SMs (eight on 23 of them: 17 us).
-__global__ void __launch_bounds__(64) table_phi_kernel(const double* __restrict__ T, const double* __restrict__ Phi,
+// launch, once per iteration); a warp per entry whose lanes read the column
+// from memory, four terms at a time, took 12 us in the solve.
+constexpr int kTableRows = 8;
+__global__ void __launch_bounds__(256) table_phi_kernel(const double* __restrict__ T, const double* __restrict__ Phi,
                                                         int r, int d, int c, int stride, double* __restrict__ out,
                                                         const int* done) {
-  if (done != nullptr && *done) return;
-  const int e = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (e >= r * c) return;
-  const int row = e / c, q = e - row * c;
-  const double* t = T + (int64_t)row * d;
+  extern __shared__ double tab[];  // [kTableRows][d] of T, then the column
+  const int q = blockIdx.x, r0 = blockIdx.y * kTableRows, nr = min(kTableRows, r - r0);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double* col = tab + kTableRows * d;
+  auto copy = [](double* dst, const double* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+  };
+  for (int e = threadIdx.x; e < d; e += 256) copy(col + e, Phi + (int64_t)e * stride + q);
+  for (int e = threadIdx.x; e < nr * d; e += 256) copy(tab + e, T + (int64_t)r0 * d + e);
+  const bool skip = done != nullptr && *done;  // read behind the copies' issue
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  if (skip || w >= nr) return;
+  const double* t = tab + w * d;
   double s[4] = {0.0, 0.0, 0.0, 0.0};
   int j = lane;
-#pragma unroll 2
   for (; j + 96 < d; j += 128) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) s[u] += t[j + 32 * u] * Phi[(int64_t)(j + 32 * u) * stride + q];
+    for (int u = 0; u < 4; ++u) s[u] += t[j + 32 * u] * col[j + 32 * u];
   }
 #pragma unroll
   for (int u = 0; u < 3; ++u)
-    if (j + 32 * u < d) s[u] += t[j + 32 * u] * Phi[(int64_t)(j + 32 * u) * stride + q];
+    if (j + 32 * u < d) s[u] += t[j + 32 * u] * col[j + 32 * u];
   const double v = warp_sum((s[0] + s[1]) + (s[2] + s[3]));
-  if (lane == 0) out[e] = v;
+  if (lane == 0) out[(r0 + w) * c + q] = v;
 }
 
 template <typename Tacc>
@@ -537,7 +574,7 @@ int reduce_parts(Plan& p, const double* partG, int NC, int ctas, cudaStream_t st
   const int64_t n0 = (int64_t)p.v[0].d * NC;
   double* G0 = io != nullptr ? io->G[0] : p.G;
   double* G1 = io != nullptr ? io->G[1] : p.G + n0;
-  pass_reduce_kernel<<<ceil_div(nG + nGram, 64), 64, 0, st>>>(partG, p.chunksB, nG,
+  pass_reduce_kernel<<<ceil_div(nG + nGram, 64), 256, 0, st>>>(partG, p.chunksB, nG,
                                                                reinterpret_cast<const double*>(p.partGram), ctas, nGram,
                                                                G0, G1, n0, io != nullptr ? io->Gram : p.Gram, done);
   GB_CHECK_LAUNCH();
@@ -620,7 +657,9 @@ int run_pass64(Plan& p, bool gram_only, cudaStream_t st, int phi_cols, const int
 
 int table_phi(const double* T, const double* Phi, int r, int d, int c, int stride, double* out, cudaStream_t st,
               const int* done) {
-  table_phi_kernel<<<ceil_div(r * c, 2), 64, 0, st>>>(T, Phi, r, d, c, stride, out, done);
+  const size_t smem = sizeof(double) * (kTableRows + 1) * (size_t)d;
+  GB_CUDA(cudaFuncSetAttribute(table_phi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  table_phi_kernel<<<dim3(c, ceil_div(r, kTableRows)), 256, smem, st>>>(T, Phi, r, d, c, stride, out, done);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }

@@ -23,7 +23,6 @@ namespace {
 
 constexpr int kJ = 64;      // columns of Z per step of the W kernel
 constexpr int kGRows = 64;  // rows of a Gram tile (one chain of its sums)
-constexpr int kCols = 32;   // columns of Z of a CTA of the G kernel
 constexpr int kRows = 32;   // rows per step of the G kernel
 constexpr int kFlush = 4;   // G kernel: steps per partial chain
 constexpr int kGE = 13;     // Gram entries per thread (80 * 81 / 2 of them at most)
@@ -108,14 +107,17 @@ __global__ void __launch_bounds__(R == 16 ? 640 : 1024) pass_w64_kernel(Pass64 a
 // CTAs [0, gctas): W^T W (and the FDA class sums) over tiles of kGRows rows
 // (tile b, b + gctas, ...), entries a <= b only (products commute, so the
 // mirrored entry is the same number).  The other CTAs: Z^T W of (row chunk,
-// kCols columns of Z): lane = column, warp w the columns w, w + 8, ... of W,
-// one chain over the chunk's rows per entry, restarted every kFlush steps.
-template <int KQ>
+// kCols columns of Z), a thread per entry (column of Z, column of W) and KQ of
+// them, one chain over the chunk's rows per entry, restarted every kFlush
+// steps.  kCols = 8 where 32 would leave the SMs with one or two CTAs each (2000
+// x 90, 10 columns per view: 16 us of a pass, one SM's two CTAs of 32 columns
+// setting the time), 32 otherwise (a CTA copies all of its rows of W).
+template <int KQ, int kCols>
 __global__ void __launch_bounds__(256) pass_g64_kernel(Pass64 a, int gctas, int chunks, int64_t rows_per_chunk, int nb0,
                                                        int D, double* __restrict__ partG) {
   if (a.done != nullptr && *a.done) return;
   extern __shared__ __align__(16) double sm64[];
-  const int NC = a.NC, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int NC = a.NC, tid = threadIdx.x;
   if ((int)blockIdx.x < gctas) {
     double* Wt = sm64;  // [kGRows][NC]
     int* ys = reinterpret_cast<int*>(Wt + kGRows * NC);
@@ -189,6 +191,14 @@ __global__ void __launch_bounds__(256) pass_g64_kernel(Pass64 a, int gctas, int 
   }
   double* Zs = sm64;                          // [2][kRows][kCols + 1]
   double* Ws = Zs + 2 * kRows * (kCols + 1);  // [2][kRows][NC]
+  int zc[KQ], wc[KQ];  // this thread's entries: column of Z, column of W
+#pragma unroll
+  for (int q = 0; q < KQ; ++q) {
+    const int e = tid + 256 * q;
+    // (lanes along the columns of Z at 32, so that W is broadcast)
+    zc[q] = kCols == 32 ? e % kCols : e / NC;
+    wc[q] = kCols == 32 ? e / kCols : e - zc[q] * NC;
+  }
   const int b = (int)blockIdx.x - gctas, chunk = b % chunks, block = b / chunks;
   const int v = block < nb0 ? 0 : 1;
   const int c0 = kCols * (block - (v == 0 ? 0 : nb0));
@@ -201,10 +211,11 @@ __global__ void __launch_bounds__(256) pass_g64_kernel(Pass64 a, int gctas, int 
     const int64_t i0 = r0 + (int64_t)s * kRows;
     double* zb = Zs + (s & 1) * kRows * (kCols + 1);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int64_t r = i0 + w + 8 * i;
-      const bool ok = r < r1 && c0 + lane < d;
-      cp_async8(zb + (w + 8 * i) * (kCols + 1) + lane, ok ? Z + r * ld + c0 + lane : Z, ok);
+    for (int i = 0; i < kRows * kCols / 256; ++i) {
+      const int e = tid + 256 * i, rr = e / kCols, cc = e % kCols;
+      const int64_t r = i0 + rr;
+      const bool ok = r < r1 && c0 + cc < d;
+      cp_async8(zb + rr * (kCols + 1) + cc, ok ? Z + r * ld + c0 + cc : Z, ok);
     }
     double* wb = Ws + (s & 1) * kRows * NC;
     const int nw = (int)min((int64_t)kRows, r1 - i0) * NC;
@@ -222,25 +233,22 @@ __global__ void __launch_bounds__(256) pass_g64_kernel(Pass64 a, int gctas, int 
 #pragma unroll
       for (int q = 0; q < KQ; ++q) acc64[q] += acc[q], acc[q] = 0.0;
     }
-    const double* zb = Zs + (s & 1) * kRows * (kCols + 1) + lane;
-    const double* wb = Ws + (s & 1) * kRows * NC + w;
+    const double* zb = Zs + (s & 1) * kRows * (kCols + 1);
+    const double* wb = Ws + (s & 1) * kRows * NC;
     const int nr = (int)min((int64_t)kRows, r1 - r0 - (int64_t)s * kRows);
 #pragma unroll 2
     for (int r = 0; r < nr; ++r) {
-      const double z = zb[r * (kCols + 1)];
 #pragma unroll
       for (int q = 0; q < KQ; ++q)
-        if (w + 8 * q < NC) acc[q] += z * wb[r * NC + 8 * q];
+        if (tid + 256 * q < kCols * NC) acc[q] += zb[r * (kCols + 1) + zc[q]] * wb[r * NC + wc[q]];
     }
     cp_async_wait();
     __syncthreads();
   }
-  const int col = c0 + lane;
-  if (col >= d) return;
-  double* out = partG + ((int64_t)chunk * D + (v == 0 ? 0 : a.d[0]) + col) * NC;
+  double* out = partG + ((int64_t)chunk * D + (v == 0 ? 0 : a.d[0])) * NC;
 #pragma unroll
   for (int q = 0; q < KQ; ++q)
-    if (w + 8 * q < NC) out[w + 8 * q] = acc64[q] + acc[q];
+    if (tid + 256 * q < kCols * NC && c0 + zc[q] < d) out[(int64_t)(c0 + zc[q]) * NC + wc[q]] = acc64[q] + acc[q];
 }
 
 template <typename Tin, int R>
@@ -259,13 +267,13 @@ int w64(const Pass64& a, cudaStream_t st) {
   return a.NC <= 40 ? launch_w64<Tin, 16>(a, st) : launch_w64<Tin, 8>(a, st);
 }
 
-template <int KQ>
+template <int KQ, int kCols>
 int launch_g64(const Pass64& a, int gctas, int chunks, int D, double* partG, cudaStream_t st) {
   const size_t gram = sizeof(double) * kGRows * a.NC + sizeof(int) * kGRows;
   const size_t stage = sizeof(double) * (2 * kRows * (kCols + 1) + 2 * (size_t)kRows * a.NC);
   const size_t smem = std::max(gram, stage);
   const int nb0 = ceil_div(a.d[0], kCols), nb = nb0 + (a.nviews > 1 ? ceil_div(a.d[1], kCols) : 0);
-  auto kern = pass_g64_kernel<KQ>;
+  auto kern = pass_g64_kernel<KQ, kCols>;
   GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int blocks = partG == nullptr ? 0 : chunks * nb;
   kern<<<gctas + blocks, 256, smem, st>>>(a, gctas, std::max(1, chunks), (a.n + chunks - 1) / chunks, nb0, D, partG);
@@ -281,17 +289,25 @@ int pass64(const Pass64& a, int dtype, int gctas, int chunks, int D, double* par
     case GBCCA_FP32: GB_TRY(w64<float>(a, st)); break;
     default: GB_TRY(w64<__nv_bfloat16>(a, st));
   }
+  const int blocks32 = chunks * (ceil_div(a.d[0], 32) + (a.nviews > 1 ? ceil_div(a.d[1], 32) : 0));
+  if (partG != nullptr && blocks32 < 4 * 152) {
+    switch (ceil_div(a.NC, 32)) {
+      case 1: return launch_g64<1, 8>(a, gctas, chunks, D, partG, st);
+      case 2: return launch_g64<2, 8>(a, gctas, chunks, D, partG, st);
+      default: return launch_g64<3, 8>(a, gctas, chunks, D, partG, st);
+    }
+  }
   switch (ceil_div(a.NC, 8)) {
-    case 1: return launch_g64<1>(a, gctas, chunks, D, partG, st);
-    case 2: return launch_g64<2>(a, gctas, chunks, D, partG, st);
-    case 3: return launch_g64<3>(a, gctas, chunks, D, partG, st);
-    case 4: return launch_g64<4>(a, gctas, chunks, D, partG, st);
-    case 5: return launch_g64<5>(a, gctas, chunks, D, partG, st);
-    case 6: return launch_g64<6>(a, gctas, chunks, D, partG, st);
-    case 7: return launch_g64<7>(a, gctas, chunks, D, partG, st);
-    case 8: return launch_g64<8>(a, gctas, chunks, D, partG, st);
-    case 9: return launch_g64<9>(a, gctas, chunks, D, partG, st);
-    default: return launch_g64<10>(a, gctas, chunks, D, partG, st);
+    case 1: return launch_g64<1, 32>(a, gctas, chunks, D, partG, st);
+    case 2: return launch_g64<2, 32>(a, gctas, chunks, D, partG, st);
+    case 3: return launch_g64<3, 32>(a, gctas, chunks, D, partG, st);
+    case 4: return launch_g64<4, 32>(a, gctas, chunks, D, partG, st);
+    case 5: return launch_g64<5, 32>(a, gctas, chunks, D, partG, st);
+    case 6: return launch_g64<6, 32>(a, gctas, chunks, D, partG, st);
+    case 7: return launch_g64<7, 32>(a, gctas, chunks, D, partG, st);
+    case 8: return launch_g64<8, 32>(a, gctas, chunks, D, partG, st);
+    case 9: return launch_g64<9, 32>(a, gctas, chunks, D, partG, st);
+    default: return launch_g64<10, 32>(a, gctas, chunks, D, partG, st);
   }
 }
 

@@ -488,3 +488,12 @@ def test_sketch_gram_rejects_overflow(gb):
         plan = gb.cca_plan(n, d, d, 1, "f32", gb.default_options(warm_start=0))
         with pytest.raises(gb.GbccaError):
             gb.cca_precondition(plan, x, x, 1e-1, 1e-1)
+
+
+@pytest.mark.parametrize("d", [400, 640])
+def test_wide_f64_dispatch(gb, d):
+    """FP64 plans beyond the lines of their dispatch rules: thin products
+    whose operands do not fit shared memory, and a pass with so many blocks of
+    columns that a CTA takes 32 of them."""
+    test_thin_products_f64(gb, d, 20)
+    test_pass_f64_edges(gb, 3000, d + 60, 300, 3)
