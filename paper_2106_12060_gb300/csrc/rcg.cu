@@ -2587,26 +2587,53 @@ __global__ void rand_block_kernel(double* B, int d, int c, uint64_t seed) {
   B[e] = (double)(r >> 11) * (1.0 / 9007199254740992.0) - 0.5;
 }
 
-// small Gram G (c x c, c <= 40) of a d x c block: the lower triangle of the
-// partials' sum, a ridge for safety, and R^{-1} = L^{-T} of G = L L^T in out.
-__global__ void __launch_bounds__(256) small_chol_kernel(const double* part, int nblk, int c, double* out, int* flag) {
+// B (d x c, c <= 40) <- B R^{-1} with R^T R = B^T B (+ a ridge for safety), from
+// the Gram's partials; optionally the result as a float pair (Bh, Bl) as well.
+// A CTA owns kApplyRows rows of B and factors the Gram for itself (L L^T = G,
+// R^{-1} = L^{-T}): the same latency as once on one CTA and a second launch of
+// 5 us for the product.
+constexpr int kApplyRows = 8;
+inline size_t orth_smem(int c) { return sizeof(double) * (2 * (size_t)c * c + c + kApplyRows * c); }
+
+__device__ __forceinline__ void orth_apply(double* B, int d, int c, const double* rows, const double* Li, float* Bh,
+                                           float* Bl) {
+  const int j0 = blockIdx.x * kApplyRows, nr = min(kApplyRows, d - j0);
+  for (int e = threadIdx.x; e < nr * c; e += blockDim.x) {
+    const int r = e / c, q = e - r * c;
+    double s = 0;
+    for (int t = 0; t <= q; ++t) s += rows[r * c + t] * Li[q * c + t];
+    const int64_t o = (int64_t)j0 * c + e;
+    B[o] = s;
+    if (Bh != nullptr) {
+      const float h = (float)s;
+      Bh[o] = h;
+      Bl[o] = (float)(s - (double)h);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) orth_kernel(const double* part, int nblk, int c, double* B, int d, float* Bh,
+                                                   float* Bl, int* flag) {
   extern __shared__ double ssm[];
   double* G = ssm;
   double* Li = G + c * c;
   double* rs = Li + c * c;
+  double* rows = rs + c;
   __shared__ double s_tr;
+  const int j0 = blockIdx.x * kApplyRows, nr = min(kApplyRows, d - j0);
+  for (int e = threadIdx.x; e < nr * c; e += blockDim.x) rows[e] = B[(int64_t)j0 * c + e];
   for (int e = threadIdx.x; e < c * (c + 1) / 2; e += blockDim.x) {
     int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
     while ((i + 1) * (i + 2) / 2 <= e) ++i;
     while (i * (i + 1) / 2 > e) --i;
     const int f = i * c + (e - i * (i + 1) / 2);
     double s = 0;
-    for (int b0 = 0; b0 < nblk; b0 += 8) {
-      double x[8];
+    for (int b0 = 0; b0 < nblk; b0 += 16) {
+      double x[16];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] = b0 + u < nblk ? part[(int64_t)(b0 + u) * c * c + f] : 0.0;
+      for (int u = 0; u < 16; ++u) x[u] = b0 + u < nblk ? part[(int64_t)(b0 + u) * c * c + f] : 0.0;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) s += x[u];
+      for (int u = 0; u < 16; ++u) s += x[u];
     }
     G[f] = s;
   }
@@ -2621,19 +2648,20 @@ __global__ void __launch_bounds__(256) small_chol_kernel(const double* part, int
   if (threadIdx.x < c) G[threadIdx.x * c + threadIdx.x] += 1e-14 * s_tr / c;
   const bool ok = group_chol_inverse<256>(G, Li, rs, c, threadIdx.x, 0);
   if (!ok && threadIdx.x == 0) atomicExch(flag, kFlagNotSpd);
-  for (int e = threadIdx.x; e < c * c; e += blockDim.x) {
-    const int i = e / c, j = e - i * c;
-    out[e] = Li[j * c + i];
-  }
+  orth_apply(B, d, c, rows, Li, Bh, Bl);
 }
 
 // The same for FP64 plans, whose iterations amplify a change of rounding in
-// their starting point: reduce partials, Cholesky (ridge for
-// safety) -> upper R in out (R^T R = G), and its inverse in out + c*c.
-__global__ void small_chol64_kernel(const double* part, int nblk, int c, double* out, int* flag) {
+// their starting point: one warp factors G (c <= 32), pivots used through
+// their reciprocals.
+__global__ void __launch_bounds__(256) orth64_kernel(const double* part, int nblk, int c, double* B, int d, float* Bh,
+                                                     float* Bl, int* flag) {
   extern __shared__ double ssm[];
   double* G = ssm;
   double* Li = G + c * c;
+  double* rows = Li + c * c + c;
+  const int j0 = blockIdx.x * kApplyRows, nr = min(kApplyRows, d - j0);
+  for (int e = threadIdx.x; e < nr * c; e += blockDim.x) rows[e] = B[(int64_t)j0 * c + e];
   sum_blocks(part, nblk, c * c, G);
   double tr = 0;
   for (int i = 0; i < c; ++i) tr += G[i * c + i];
@@ -2641,7 +2669,6 @@ __global__ void small_chol64_kernel(const double* part, int nblk, int c, double*
   if (threadIdx.x < c) G[threadIdx.x * c + threadIdx.x] += 1e-14 * tr / c;
   __syncthreads();
   if (c <= 32) {
-    // c <= 32: one warp factors G, pivots used through their reciprocals
     if (threadIdx.x < 32) {
       double* invd = Li + c * c;
       const bool ok = warp_chol(G, c, invd);
@@ -2655,42 +2682,12 @@ __global__ void small_chol64_kernel(const double* part, int nblk, int c, double*
     }
     blk_lower_inv(G, Li, c);
   }
-  // R^{-1} = (L^{-1})^T
-  for (int e = threadIdx.x; e < c * c; e += blockDim.x) {
-    int i = e / c, j = e % c;
-    out[e] = Li[j * c + i];
-  }
-}
-
-// B (d x c) <- B Rinv (c x c upper): a CTA stages kApplyRows rows of B in
-// shared memory and each thread forms one entry (at most c multiply-adds),
-// so the FP64 work spreads over many SMs instead of one chain per row.
-// Optionally the result as a float pair (Bh, Bl) as well.
-constexpr int kApplyRows = 8;
-__global__ void __launch_bounds__(kApplyRows * 2 * kMaxK) apply_small_kernel(double* B, int d, int c,
-                                                                            const double* Rinv, float* Bh, float* Bl) {
-  __shared__ double rows[kApplyRows * 2 * kMaxK];
-  const int j0 = blockIdx.x * kApplyRows;
-  const int nr = min(kApplyRows, d - j0);
-  for (int e = threadIdx.x; e < nr * c; e += blockDim.x) rows[e] = B[(int64_t)j0 * c + e];
-  __syncthreads();
-  const int e = threadIdx.x;
-  if (e >= nr * c) return;
-  const int r = e / c, q = e - r * c;
-  double s = 0;
-  for (int t = 0; t <= q; ++t) s += rows[r * c + t] * Rinv[t * c + q];
-  const int64_t o = (int64_t)(j0 + r) * c + q;
-  B[o] = s;
-  if (Bh != nullptr) {
-    const float h = (float)s;
-    Bh[o] = h;
-    Bl[o] = (float)(s - (double)h);
-  }
+  orth_apply(B, d, c, rows, Li, Bh, Bl);
 }
 
 // Rayleigh-Ritz of the power iteration: Bsmall = U^T (C V) (c x c), take the
 // top-k singular pairs: U A_k, V B_k in out (d x k each).
-// (fp64: the plan is FP64, see small_chol64_kernel)
+// (fp64: the plan is FP64, see orth64_kernel)
 __global__ void __launch_bounds__(256) small_svd_kernel(const double* part, int nblk, int c, int k, double* rotU, double* rotV, int fp64) {
   extern __shared__ double wsm[];
   double* Bm = wsm;
@@ -2748,8 +2745,7 @@ __global__ void __launch_bounds__(256) fda_warm_kernel(const double* part, int n
 
 namespace {
 
-int orth(Plan& p, double* B, int d, int c, double* part, double* small, cudaStream_t st, float* Bh = nullptr,
-         float* Bl = nullptr) {
+int orth(Plan& p, double* B, int d, int c, double* part, cudaStream_t st, float* Bh = nullptr, float* Bl = nullptr) {
   // Gram of B (d x c) via a one-view thin Gram
   ThinArgs a{};
   a.A[0] = B;
@@ -2766,10 +2762,8 @@ int orth(Plan& p, double* B, int d, int c, double* part, double* small, cudaStre
   GB_CUDA(cudaFuncSetAttribute(thin_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   thin_gram_kernel<<<dim3(a.nblk, 1), 256, smem, st>>>(a);
   GB_CHECK_LAUNCH();
-  auto chol = p.dtype == GBCCA_FP64 ? small_chol64_kernel : small_chol_kernel;
-  chol<<<1, 256, sizeof(double) * (2 * c * c + c), st>>>(part, a.nblk, c, small, p.flag);
-  GB_CHECK_LAUNCH();
-  apply_small_kernel<<<ceil_div(d, kApplyRows), kApplyRows * 2 * kMaxK, 0, st>>>(B, d, c, small, Bh, Bl);
+  auto kern = p.dtype == GBCCA_FP64 ? orth64_kernel : orth_kernel;
+  kern<<<ceil_div(d, kApplyRows), 256, orth_smem(c), st>>>(part, a.nblk, c, B, d, Bh, Bl, p.flag);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }
@@ -2846,7 +2840,7 @@ int warm_start(Plan& p, cudaStream_t st) {
     };
     rand_block_kernel<<<ceil_div(dy * c, 256), 256, 0, st>>>(Vb, dy, c, p.opt.seed);
     GB_CHECK_LAUNCH();
-    GB_TRY(orth(p, Vb, dy, c, part, small, st, low ? Vp[0] : nullptr, low ? Vp[1] : nullptr));
+    GB_TRY(orth(p, Vb, dy, c, part, st, low ? Vp[0] : nullptr, low ? Vp[1] : nullptr));
     const int iters = p.opt.warm_iters > 0 ? p.opt.warm_iters : 12;
     for (int it = 0; it <= iters; ++it) {
       // U = C V
@@ -2869,11 +2863,11 @@ int warm_start(Plan& p, cudaStream_t st) {
         GB_TRY(cxy(true, x.wsT, y.wsT));
         GB_TRY(ry(true, y.wsT, Vb, c));
       }
-      GB_TRY(orth(p, Vb, dy, c, part, small, st, low ? Vp[0] : nullptr, low ? Vp[1] : nullptr));
+      GB_TRY(orth(p, Vb, dy, c, part, st, low ? Vp[0] : nullptr, low ? Vp[1] : nullptr));
     }
     // Ub = C V: take U0 = orth(Ub) and Bm = U0^T (C V)
     GB_CUDA(cudaMemcpyAsync(x.wsT, Ub, sizeof(double) * dx * c, cudaMemcpyDeviceToDevice, st));
-    GB_TRY(orth(p, Ub, dx, c, part, small, st));
+    GB_TRY(orth(p, Ub, dx, c, part, st));
     {
       ThinArgs a{};
       a.A[0] = Ub;
