@@ -160,6 +160,21 @@ __device__ void blk_jacobi(R* A, R* Q, R* lam, int n, double* rot) {
   __syncthreads();
 }
 
+// apq^2 > 1e-34 |app aqq|, decided on the exponents where they are clear of the
+// threshold and of under- and overflow (else false: the caller compares).  An
+// FP64 instruction takes a warp 64 cycles, an integer one a few.
+__device__ __forceinline__ bool clearly_coupled(double apq, double app, double aqq) {
+  const int ea = (__double2hiint(apq) >> 20) & 0x7ff, ep = (__double2hiint(app) >> 20) & 0x7ff,
+            eq = (__double2hiint(aqq) >> 20) & 0x7ff;
+  auto mid = [](int e) { return (unsigned)(e - 600) < 800u; };
+  return mid(ea) && mid(ep) && mid(eq) && 2 * ea + 110 >= ep + eq;
+}
+__device__ __forceinline__ bool clearly_coupled(float, float, float) { return false; }
+__device__ __forceinline__ bool not_negative(double x) {  // x >= 0 (x not NaN)
+  return __double2hiint(x) >= 0 || (__double_as_longlong(x) << 1) == 0;
+}
+__device__ __forceinline__ bool not_negative(float x) { return x >= 0; }
+
 // The same parallel Jacobi sweeps for n <= 40 by one warp: rotation pairs
 // on lanes, warp-level barriers only (the block version spends most of its
 // time in block-wide barriers for matrices this small).  Called by all 32
@@ -206,9 +221,10 @@ __device__ void warp_jacobi(R* A, R* Q, R* lam, int n, int max_sweeps = 20, R to
         if (q < n) {
           const R apq = A[p * n + q];
           const R eps = R(sizeof(R) == 8 ? 1e-17 : 1e-8);
-          if (apq * apq > eps * eps * fabs(A[p * n + p] * A[q * n + q])) {
-            const R tau = (A[q * n + q] - A[p * n + p]) / (R(2) * apq);
-            const R t = (tau >= 0 ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
+          const R app = A[p * n + p], aqq = A[q * n + q];
+          if (clearly_coupled(apq, app, aqq) || apq * apq > eps * eps * fabs(app * aqq)) {
+            const R tau = (aqq - app) / (R(2) * apq);
+            const R t = (not_negative(tau) ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
             c = R(1) / sqrt(R(1) + t * t);
             sv = t * c;
           }
@@ -228,16 +244,16 @@ __device__ void warp_jacobi(R* A, R* Q, R* lam, int n, int max_sweeps = 20, R to
         A[q * n + j] = w_sn[i] * ap + w_cs[i] * aq;
       }
       __syncwarp();
-      for (int e = lane; e < (m / 2) * n; e += 32) {  // columns: A <- A J, Q <- Q J
-        const int i = e / n, j = e % n;
+      // columns: A <- A J and Q <- Q J, side by side on the lanes
+      for (int e = lane; e < 2 * (m / 2) * n; e += 32) {
+        const bool second = e >= (m / 2) * n;
+        const int f = second ? e - (m / 2) * n : e, i = f / n, j = f % n;
         if (w_q[i] < 0) continue;
+        R* M = (second ? Q : A) + j * n;
         const int p = w_p[i], q = w_q[i];
-        const R ap = A[j * n + p], aq = A[j * n + q];
-        A[j * n + p] = w_cs[i] * ap - w_sn[i] * aq;
-        A[j * n + q] = w_sn[i] * ap + w_cs[i] * aq;
-        const R qp = Q[j * n + p], qv = Q[j * n + q];
-        Q[j * n + p] = w_cs[i] * qp - w_sn[i] * qv;
-        Q[j * n + q] = w_sn[i] * qp + w_cs[i] * qv;
+        const R ap = M[p], aq = M[q];
+        M[p] = w_cs[i] * ap - w_sn[i] * aq;
+        M[q] = w_sn[i] * ap + w_cs[i] * aq;
       }
       __syncwarp();
     }
