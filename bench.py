@@ -53,8 +53,8 @@ LDA_CHECK_EVERY = 8
 # from an ncu capture of 131072 rows of this workload (reads scaled by rows
 # to 262144, partial writes as measured).  Valid only for the kernel source
 # it was taken on (SHA-256 below); any other source reports null.
-PASS_TRAFFIC_BYTES = 268.594432e6 * 2 + 10.445568e6
-PASS_TRAFFIC_SRC_SHA256 = "9d24d54d17e5ed4796e5193140eca44aa1fbb4484d9ebf552ee99eb935eed408"
+PASS_TRAFFIC_BYTES = 268.592384e6 * 2 + 9.835264e6
+PASS_TRAFFIC_SRC_SHA256 = "0af0f2d42128f3999a0aa51479853ae4cae07e2f79bab88ff8e27163d83a9b98"
 
 
 def pass_traffic():
