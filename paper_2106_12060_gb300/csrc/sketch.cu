@@ -336,10 +336,10 @@ __device__ __forceinline__ void fwht_thread_col(T* col, int stride, int N) {
 // each (spans 32 .. N / 2): about nine additions and two shared-memory
 // accesses per element.  (A column per warp with shuffles for the first five
 // levels and two passes over shared memory was bound by its instructions:
-// 437 us a view for 262144 x 512 BF16, 1.8 TB/s.)  buf: N x 32; on return it
-// holds the transform.
-template <typename T, int NW>
-__device__ __forceinline__ void fwht_tile(T (&v)[32], T* buf) {
+// 437 us a view for 262144 x 512 BF16, 1.8 TB/s.)  buf: N x 32, scratch; out(r,
+// x) receives row r of the lane's column (each warp its own rows).
+template <typename T, int NW, typename F>
+__device__ __forceinline__ void fwht_tile(T (&v)[32], T* buf, F out) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int h = 1; h < 32; h <<= 1) {
@@ -371,9 +371,8 @@ __device__ __forceinline__ void fwht_tile(T (&v)[32], T* buf) {
         }
     }
 #pragma unroll
-    for (int m = 0; m < NW; ++m) buf[(w * NJ + q + 32 * m) * 32 + lane] = u[m];
+    for (int m = 0; m < NW; ++m) out(w * NJ + q + 32 * m, u[m]);
   }
-  __syncthreads();
 }
 
 // One element of D Z (signs, and the class means for LDA) in the working type.
@@ -416,13 +415,9 @@ srht_stage1_kernel(const Tin* __restrict__ Z, int64_t ld, int64_t n, int d, cons
     v[t] = (use >> t & 1) && col < d
                ? signed_value<Tin, T>(z[t], (neg >> t & 1) ? -1 : 1, labels, means, row0 + t, d, col)
                : T(0);
-  fwht_tile<T, NW>(v, buf);
-  // row r of the block is residue a1 = r
-#pragma unroll
-  for (int t = 0; t < 32; ++t) {
-    const int64_t r = 32 * w + t;
-    Tmid[((r * ncb + cb) * N2 + i2) * 32 + lane] = buf[r * 32 + lane];
-  }
+  // row r of the block is residue a1 = r: straight from registers, 128 bytes a
+  // warp (back through shared memory first: 267 us a view, 255 now)
+  fwht_tile<T, NW>(v, buf, [&](int r, T x) { Tmid[(((int64_t)r * ncb + cb) * N2 + i2) * 32 + lane] = x; });
 }
 
 // The same for short blocks (N1 < 64): one thread per column.
@@ -474,7 +469,8 @@ srht_stage2_kernel(const T* __restrict__ Tmid, int d, int m1, const int32_t* __r
   T v[32];
 #pragma unroll
   for (int t = 0; t < 32; ++t) v[t] = src[(32 * w + t) * 32 + lane];
-  fwht_tile<T, NW>(v, buf);
+  fwht_tile<T, NW>(v, buf, [&](int r, T x) { buf[r * 32 + lane] = x; });
+  __syncthreads();
   srht_pick(buf, d, cb, a1, nsel, m1, off1, list, rows, scale, SZ);
 }
 
