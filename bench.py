@@ -53,8 +53,8 @@ LDA_CHECK_EVERY = 8
 # from an ncu capture of 131072 rows of this workload (reads scaled by rows
 # to 262144, partial writes as measured).  Valid only for the kernel source
 # it was taken on (SHA-256 below); any other source reports null.
-PASS_TRAFFIC_BYTES = 268.592384e6 * 2 + 9.835264e6
-PASS_TRAFFIC_SRC_SHA256 = "0af0f2d42128f3999a0aa51479853ae4cae07e2f79bab88ff8e27163d83a9b98"
+PASS_TRAFFIC_BYTES = 268.589056e6 * 2 + 9.728256e6
+PASS_TRAFFIC_SRC_SHA256 = "2b775a423f024040bf6b29a32e978e8699ee1967f517693e817ffaacaa99c993"
 
 
 def pass_traffic():
