@@ -336,7 +336,7 @@ int precondition_common(Plan& p, const int32_t* sh, const int8_t* sg, cudaStream
     // 55-bit digits on the tensor cores, or double-float arithmetic (~2^-44
     // relative per product) at FP32 instruction rates
     if (w.SZs != nullptr) {
-      GB_TRY(gram_slice(w.SZ, p.s, w.d, w.SZe, w.SZs, st));
+      GB_TRY(gram_slice(w.SZ, p.s, w.d, w.SZe, w.SZs, p.ws_len, st));
       GB_TRY(gram_sliced(w.SZs, w.SZe, w.d, w.SZs, w.SZe, w.d, p.s, w.R, w.lam, p.ws, p.ws_len, p.sm_count, p.flag, st));
     } else if (w.SZh != nullptr) {
       GB_TRY(split_rows(w.SZ, (int)p.s, w.d, w.d, w.SZh, w.SZl, st));

@@ -212,6 +212,18 @@ gram_dfs_kernel(const float* __restrict__ Ahg, const float* __restrict__ Alg, in
     }
 }
 
+// Ranges of rows over which a Gram of `tiles` tiles and `len` entries is summed
+// in FP32, as many as fill the GPU and the workspace holds.
+static int df_splits(int tiles, int64_t len, int64_t m, bool tri, int64_t ws_len) {
+  int ks = std::max(1, std::min<int>(ceil_div(tri ? 2 * 304 : 304, tiles), ceil_div(m, 64)));
+  while (ks > 1 && (int64_t)ks * len > ws_len) --ks;
+  return ks;
+}
+int64_t gram_df_chunk(int64_t m, int d, int64_t ws_len) {
+  const int td = ceil_div(d, kGT), ks = df_splits(td * (td + 1) / 2, (int64_t)d * d, m, false, ws_len);
+  return (m + ks - 1) / ks;
+}
+
 int gram_df_split(const float* Ah, const float* Al, int64_t lda, const float* Bh, const float* Bl, int64_t ldb,
                   int64_t m, int d1, int d2, double* C, double diag_add, double* ws, int64_t ws_len, cudaStream_t st,
                   bool tri) {
@@ -220,9 +232,8 @@ int gram_df_split(const float* Ah, const float* Al, int64_t lda, const float* Bh
   const bool sym = Ah == Bh && Al == Bl && lda == ldb && d1 == d2;
   const int td = ceil_div(d1, kGT);
   const int tiles = sym ? td * (td + 1) / 2 : ceil_div(d1, kGT) * ceil_div(d2, kGT);
-  int ks = std::max(1, std::min<int>(ceil_div(tri ? 2 * 304 : 304, tiles), ceil_div(m, 64)));
   const int64_t len = (int64_t)d1 * d2;
-  while (ks > 1 && (int64_t)ks * len > ws_len) --ks;
+  const int ks = df_splits(tiles, len, m, tri, ws_len);
   if ((int64_t)ks * len > ws_len) {
     set_last_error("gram_df_split: workspace too small");
     return GBCCA_ERR_INVALID_ARG;

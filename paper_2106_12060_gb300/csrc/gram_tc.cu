@@ -46,20 +46,45 @@ static_assert(kSlices * kWindow * (1 << 14) < (1 << 24), "exact FP32 sums of a l
 static_assert(kSlices * kN <= (int)kTmemCols, "accumulators");
 static_assert(kStages * kStage + 1280 <= 232448, "shared memory");
 
-// Largest biased exponent of every column (zeroed before).
-__global__ void __launch_bounds__(256) col_exp_kernel(const double* __restrict__ A, int64_t s, int d,
-                                                      int* __restrict__ ex) {
-  const int col = blockIdx.x * 32 + (threadIdx.x & 31);
-  __shared__ int red[8][32];
+// Exponents (biased) at which the FP32 range ends for the entries of a column:
+// beyond kMaxExp not finite; below kMinExp every square rounds to zero.
+constexpr int kMaxExp = 1150, kMinExp = 948;
+
+// Largest biased exponent of every column (zeroed before); 2047, as for a
+// column that is not finite, where the column's squares sum to more than FP32
+// holds over one of the row ranges of the double-float form.  The rest of a
+// plan (M^{-1} as float pairs above all) has no more range than that, so both
+// forms refuse the same sketches.  blockIdx.y: a range of `chunk` rows.
+__global__ void __launch_bounds__(1024) col_exp_kernel(const double* __restrict__ A, int64_t s, int d, int64_t chunk,
+                                                       int* __restrict__ ex) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, col = blockIdx.x * 32 + lane;
+  __shared__ int red_m[32][32];
+  __shared__ float red_q[32][32];
+  const int64_t r1 = min(s, (int64_t)(blockIdx.y + 1) * chunk);
   int m = 0;
-  if (col < d)
-    for (int64_t r = blockIdx.y * 8 + (threadIdx.x >> 5); r < s; r += 8 * (int64_t)gridDim.y)
-      m = max(m, (__double2hiint(A[r * d + col]) >> 20) & 0x7ff);
-  red[threadIdx.x >> 5][threadIdx.x & 31] = m;
+  float q = 0.f;
+  if (col < d) {
+#pragma unroll 4
+    for (int64_t r = blockIdx.y * chunk + w; r < r1; r += 32) {
+      const double x = A[r * d + col];
+      const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+      const int e = (int)(hi >> 20 & 0x7ff);
+      m = max(m, e);
+      // |x| to 24 bits, by moving the bits (a conversion runs at the FP64 rate)
+      const float a = e > kMaxExp ? INFINITY
+                                  : (e < 897 ? 0.f : __uint_as_float((uint32_t)(e - 896) << 23 | (hi & 0xfffff) << 3 | lo >> 29));
+      q = fmaf(a, a, q);
+    }
+  }
+  red_m[w][lane] = m;
+  red_q[w][lane] = q;
   __syncthreads();
-  if (threadIdx.x >= 32 || col >= d) return;
-  for (int q = 1; q < 8; ++q) m = max(m, red[q][threadIdx.x]);
-  atomicMax(&ex[col], m);
+  if (w != 0 || col >= d) return;
+  for (int u = 1; u < 32; ++u) {
+    m = max(m, red_m[u][lane]);
+    q += red_q[u][lane];
+  }
+  atomicMax(&ex[col], q <= 3.402823466e38f ? m : 2047);
 }
 
 // Digits of every entry: slice t at S + t sp dp, rows s .. sp - 1 zero.  Two
@@ -267,7 +292,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
 
 // C = the splits' integers summed (exactly, as high and low words) and scaled
 // back, + diag_add on the diagonal.  A column beyond the FP32 range (or not
-// finite) makes its entries NaN, which the factorization reports.
+// finite) makes its entries NaN, and one whose squares vanish in FP32 has no
+// square here either, which the factorization reports (with diag_add = 0).
 __global__ void __launch_bounds__(256) gram_scale_kernel(const long long* __restrict__ part, int ks, int d1, int d2,
                                                          const int* __restrict__ ea, const int* __restrict__ eb,
                                                          int sym, int drop, double diag_add, double* __restrict__ C) {
@@ -285,7 +311,8 @@ __global__ void __launch_bounds__(256) gram_scale_kernel(const long long* __rest
   lo &= 0xffffffffll;
   const int Ei = max(ea[i], 1), Ej = max(eb[j], 1);
   double x = scalbn(fma((double)hi, 4294967296.0, (double)lo), Ei + Ej - 2 * 1022 - 50 + drop);
-  if (Ei > 1150 || Ej > 1150) x = __longlong_as_double(0x7ff8000000000000ll);
+  if (Ei > kMaxExp || Ej > kMaxExp) x = __longlong_as_double(0x7ff8000000000000ll);
+  if (sym && i == j && Ei < kMinExp) x = 0.0;
   C[e] = x + (i == j ? diag_add : 0.0);
 }
 
@@ -294,11 +321,11 @@ __global__ void __launch_bounds__(256) gram_scale_kernel(const long long* __rest
 int64_t gram_slice_rows(int64_t s) { return (s + gram::kStageRows - 1) / gram::kStageRows * gram::kStageRows; }
 int64_t gram_slices_len(int64_t s, int d) { return gram::kSlices * gram_slice_rows(s) * ((d + 7) / 8 * 8); }
 
-int gram_slice(const double* A, int64_t s, int d, int* ex, __nv_bfloat16* S, cudaStream_t st) {
+int gram_slice(const double* A, int64_t s, int d, int* ex, __nv_bfloat16* S, int64_t ws_len, cudaStream_t st) {
   const int dp = (d + 7) / 8 * 8;
-  const int64_t sp = gram_slice_rows(s);
+  const int64_t sp = gram_slice_rows(s), chunk = gram_df_chunk(s, d, ws_len);
   GB_CUDA(cudaMemsetAsync(ex, 0, sizeof(int) * d, st));
-  gram::col_exp_kernel<<<dim3(ceil_div(d, 32), (unsigned)std::min<int64_t>(64, (s + 63) / 64)), 256, 0, st>>>(A, s, d, ex);
+  gram::col_exp_kernel<<<dim3(ceil_div(d, 32), ceil_div(s, chunk)), 1024, 0, st>>>(A, s, d, chunk, ex);
   GB_CHECK_LAUNCH();
   gram::slice_kernel<<<ceil_div(sp * (dp / 2), 256), 256, 0, st>>>(A, s, sp, d, dp, ex, reinterpret_cast<uint32_t*>(S));
   GB_CHECK_LAUNCH();

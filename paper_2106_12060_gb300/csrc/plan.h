@@ -207,8 +207,10 @@ int gram_tn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t 
 int gram_df_split(const float* Ah, const float* Al, int64_t lda, const float* Bh, const float* Bl, int64_t ldb,
                   int64_t m, int d1, int d2, double* C, double diag_add, double* ws, int64_t ws_len, cudaStream_t st,
                   bool tri = false);
+// rows of one range of its sums for a symmetric Gram of d columns
+int64_t gram_df_chunk(int64_t m, int d, int64_t ws_len);
 int64_t gram_slices_len(int64_t s, int d);
-int gram_slice(const double* A, int64_t s, int d, int* ex, __nv_bfloat16* S, cudaStream_t st);
+int gram_slice(const double* A, int64_t s, int d, int* ex, __nv_bfloat16* S, int64_t ws_len, cudaStream_t st);
 int gram_sliced(const __nv_bfloat16* A, const int* ea, int d1, const __nv_bfloat16* B, const int* eb, int d2, int64_t s,
                 double* C, double diag_add, double* ws, int64_t ws_len, int sm_count, int* err, cudaStream_t st);
 int cholesky_upper(double* A, int d, int* flag, cudaStream_t st);

@@ -497,3 +497,63 @@ def test_wide_f64_dispatch(gb, d):
     columns that a CTA takes 32 of them."""
     test_thin_products_f64(gb, d, 20)
     test_pass_f64_edges(gb, 3000, d + 60, 300, 3)
+
+
+def _refused(call):
+    """Status of a call: True if it reported a factor that is not SPD, False
+    if it went through; anything else is an error."""
+    import paper_2106_12060_gb300 as gb
+    try:
+        call()
+    except gb.GbccaError as e:
+        assert e.code == gb.ERR_NOT_SPD
+        return True
+    return False
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("n,d,s", [(64, 5, 40), (900, 65, 700)])
+def test_sketch_gram_range(gb, dt, n, d, s):
+    """Sketches whose products leave the FP32 range, which the rest of a plan
+    shares: one column of 1e21 beside columns of order one, everything of that
+    size, and squares that vanish without a ridge are refused by both forms of
+    the Gram; and over columns of 2^58 to 2^68 both refuse the same ones."""
+    import torch
+    tdt = {"f32": torch.float32, "bf16": torch.bfloat16}[dt]
+    X = np.random.default_rng(d).standard_normal((n, d))
+
+    def cca(Z, lam, tc):
+        x = torch.from_numpy(Z).to(tdt).cuda()
+        plan = gb.cca_plan(n, d, d, 1, dt, gb.default_options(s=s, tensor_cores=tc, warm_start=0))
+        return _refused(lambda: gb.cca_precondition(plan, x, x, lam, lam))
+
+    for tc in (1, 0):
+        assert not cca(X, 1e-1, tc)
+        assert not cca(X * 1e15, 1e-1, tc)
+        big = X.copy()
+        big[:, 2] *= 1e21
+        assert cca(big, 1e-1, tc)
+        assert cca(X * 1e22, 1e-1, tc)
+        assert cca(X * 1e-26, 0.0, tc)
+        assert not cca(X * 1e-26, 1e-1, tc)
+    verdicts = []
+    for e in np.arange(58, 68, 0.25):
+        col = X.copy()
+        col[:, 3] *= 2.0 ** e
+        verdicts.append(cca(col, 1e-1, 1))
+        assert verdicts[-1] == cca(col, 1e-1, 0)
+    assert not verdicts[0] and verdicts[-1]
+
+
+def test_fda_sketch_range(gb):
+    """The same for FDA: data of 1e22 are refused, data of 1e15 are not, by
+    both forms of the Gram."""
+    import torch
+    n, d, l = 300, 9, 3
+    P = lda_problem(n, d, l, dtype="f32", seed=1)
+    y = torch.from_numpy(P["y"]).cuda()
+    for tc in (1, 0):
+        for scale, refused in ((1.0, False), (1e15, False), (1e22, True)):
+            x = torch.from_numpy((P["X64"] * scale).astype(np.float32)).cuda()
+            plan = gb.lda_plan(n, d, l, 2, "f32", gb.default_options(max_iter=1, tensor_cores=tc))
+            assert _refused(lambda: gb.lda_solve(plan, x, y, 1e-1)) == refused
