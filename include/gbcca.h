@@ -91,8 +91,9 @@ typedef struct {
   int32_t graphs;        /* 1: each batch of check_every iterations is replayed
                             from a CUDA graph that the plan captures on its own
                             stream at the first solve (re-captured when the
-                            data pointers change; with time_passes the timing
-                            events are recorded by the graph); 0: the kernels
+                            data pointers or row strides change; with
+                            time_passes the timing events are recorded by the
+                            graph); 0: the kernels
                             are launched one by one.  Both run the same
                             kernels in the same order.                          */
   double rtol;           /* stop when the Rayleigh-Ritz values of the subspace

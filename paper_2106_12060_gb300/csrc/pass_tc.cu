@@ -1144,11 +1144,12 @@ int tc_pass(Plan& p, cudaStream_t st, const int* done, const PassIO* io) {
   tc_sources(p, src, ld, &rows);
   const bool solo = tc_solo(p);
   const int nv = tc_nviews(p);
-  if (p.tc_map_for[0] != src[0] || p.tc_map_for[1] != src[1]) {
-    for (int v = 0; v < 2; ++v)
-      GB_TRY(make_map(reinterpret_cast<CUtensorMap*>(p.tc_map[v]), src[v], rows, p.v[v < nv ? v : 0].d, ld[v]));
-    p.tc_map_for[0] = src[0];
-    p.tc_map_for[1] = src[1];
+  for (int v = 0; v < 2; ++v) {
+    if (p.tc_map_for[v] == src[v] && p.tc_map_ld[v] == ld[v]) continue;
+    p.tc_map_for[v] = nullptr;
+    GB_TRY(make_map(reinterpret_cast<CUtensorMap*>(p.tc_map[v]), src[v], rows, p.v[v < nv ? v : 0].d, ld[v]));
+    p.tc_map_for[v] = src[v];
+    p.tc_map_ld[v] = ld[v];
   }
   GB_TRY(tc_phi_image(p, 0, st, done, io));
   const CUtensorMap* mx = reinterpret_cast<const CUtensorMap*>(p.tc_map[0]);

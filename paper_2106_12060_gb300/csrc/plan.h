@@ -144,10 +144,11 @@ struct Plan {
   int nev = 0;
 
   // tensor-core pass (BF16 CCA): TMA descriptors of X and Y (CUtensorMap,
-  // 128 bytes each, rebuilt when the data pointers change), the swizzled Phi
+  // 128 bytes each, rebuilt when a data pointer or row stride changes), the swizzled Phi
   // image and the per-CTA FP32 partials of G
   alignas(64) unsigned char tc_map[2][128];
   const void* tc_map_for[2] = {nullptr, nullptr};
+  int64_t tc_map_ld[2] = {0, 0};
   uint8_t* tc_img = nullptr;
   float* tc_part = nullptr;
   int tc_clusters = 0;
@@ -168,6 +169,7 @@ struct Plan {
   bool phired_ready = false;  // the pass has also formed the Grams of Phi (tensor-core pass)
   cudaGraphExec_t batch_exec = nullptr;
   const void* batch_key_ptr[3] = {nullptr, nullptr, nullptr};
+  int64_t batch_key_ld[2] = {0, 0};
   int batch_key_n = 0;
   bool batch_key_timed = false;
   long long batch_launches = 0;  // kernels in one replay (for the launch counter)

@@ -2332,9 +2332,9 @@ int run_batch_direct(Plan& p, bool low, int nb, bool timed, cudaStream_t st) {
 }
 
 // The same batch replayed from a CUDA graph.  The graph is captured on the
-// plan's own stream and holds plan-owned pointers, the data pointers (X, Y,
-// labels; the TMA descriptors are captured by value) and the batch shape; it
-// is captured again when any of those differ.  Every kernel reads its
+// plan's own stream and holds plan-owned pointers, the data pointers and row
+// strides (X, Y, labels; the TMA descriptors are captured by value) and the
+// batch shape; it is captured again when any of those differ.  Every kernel reads its
 // per-iteration state (step, direction, convergence flag) from device memory,
 // so one capture serves every batch of every solve.  With pass timing the
 // events around the data kernels are captured as external event-record nodes,
@@ -2342,7 +2342,8 @@ int run_batch_direct(Plan& p, bool low, int nb, bool timed, cudaStream_t st) {
 int run_batch_graph(Plan& p, bool low, int nb, bool timed, cudaStream_t st) {
   const void* key[3] = {p.v[0].Z, p.nviews > 1 ? (const void*)p.v[1].Z : nullptr, (const void*)p.labels};
   const bool same = p.batch_exec != nullptr && p.batch_key_n == nb && p.batch_key_timed == timed &&
-                    key[0] == p.batch_key_ptr[0] && key[1] == p.batch_key_ptr[1] && key[2] == p.batch_key_ptr[2];
+                    key[0] == p.batch_key_ptr[0] && key[1] == p.batch_key_ptr[1] && key[2] == p.batch_key_ptr[2] &&
+                    p.batch_key_ld[0] == p.v[0].ld && p.batch_key_ld[1] == p.v[1].ld;
   if (!same) {
     if (p.batch_exec != nullptr) {
       GB_CUDA(cudaGraphExecDestroy(p.batch_exec));
@@ -2376,6 +2377,7 @@ int run_batch_graph(Plan& p, bool low, int nb, bool timed, cudaStream_t st) {
     p.batch_key_n = nb;
     p.batch_key_timed = timed;
     for (int i = 0; i < 3; ++i) p.batch_key_ptr[i] = key[i];
+    for (int v = 0; v < 2; ++v) p.batch_key_ld[v] = p.v[v].ld;
   }
   GB_CUDA(cudaGraphLaunch(p.batch_exec, st));
   g_launches.fetch_add(p.batch_launches);

@@ -557,3 +557,30 @@ def test_fda_sketch_range(gb):
             x = torch.from_numpy((P["X64"] * scale).astype(np.float32)).cuda()
             plan = gb.lda_plan(n, d, l, 2, "f32", gb.default_options(max_iter=1, tensor_cores=tc))
             assert _refused(lambda: gb.lda_solve(plan, x, y, 1e-1)) == refused
+
+
+@pytest.mark.parametrize("dt", ["bf16", "f32", "f64"])
+@pytest.mark.parametrize("k", [2, 14])
+def test_rebind_row_stride(gb, dt, k):
+    """One plan bound to the same addresses with another row stride: the pass
+    (one and two sweeps) and a solve replayed from a captured graph read the
+    data as bound, so they give what a new plan gives, bitwise."""
+    import torch
+    n, dx, dy = 900, 40, 32
+    tdt = {"bf16": torch.bfloat16, "f32": torch.float32, "f64": torch.float64}[dt]
+    rng = np.random.default_rng(k)
+    buf = [torch.from_numpy(rng.standard_normal(n * 64)).to(tdt).cuda() for _ in range(2)]
+    Phi = [torch.from_numpy(rng.standard_normal((d, 2 * k))).cuda() for d in (dx, dy)]
+
+    def make():
+        return gb.cca_plan(n, dx, dy, k, dt, gb.default_options(max_iter=8, gtol=0.0, check_every=4))
+
+    def results(plan, lds):
+        X, Y = (b.as_strided((n, d), (ld, 1)) for b, d, ld in zip(buf, (dx, dy), lds))
+        gb.cca_precondition(plan, X, Y, 1e-1, 1e-1)
+        return [np64(t) for t in (*gb.fused_pass(plan, *Phi), *gb.cca_solve(plan)[:3])]
+
+    kept = make()
+    for lds in ((64, 64), (48, 64), (48, 40), (45, 40)):
+        for got, exp in zip(results(kept, lds), results(make(), lds)):
+            assert np.array_equal(got, exp)
