@@ -34,6 +34,7 @@ struct Status {
   do {                                                                                    \
     cudaError_t e_ = (call);                                                              \
     if (e_ != cudaSuccess) {                                                              \
+      cudaGetLastError(); /* reported here, not by the next launch check */               \
       ::gbcca::set_last_error(std::string(#call) + ": " + cudaGetErrorString(e_));        \
       return GBCCA_ERR_CUDA;                                                              \
     }                                                                                     \

@@ -9,8 +9,8 @@
 // SRHT (App. A, Def. A.1, scale sqrt(n/s) so that E[S^T S] = I): the
 // Walsh-Hadamard transform of length n_pad = 2^m factors as
 // H_{2^m} = H_{N2} (x) H_{N1}; stage 1 transforms each block of N1 consecutive
-// rows in shared memory, stage 2 transforms the strided columns of the
-// intermediate and writes only the s sampled rows.
+// rows in registers, stage 2 transforms the strided columns of the intermediate
+// and writes only the s sampled rows.
 #include "plan.h"
 
 namespace gbcca {
@@ -336,11 +336,12 @@ __device__ __forceinline__ void fwht_thread_col(T* col, int stride, int N) {
 // each (spans 32 .. N / 2): about nine additions and two shared-memory
 // accesses per element.  (A column per warp with shuffles for the first five
 // levels and two passes over shared memory was bound by its instructions:
-// 437 us a view for 262144 x 512 BF16, 1.8 TB/s.)  buf: N x 32, scratch; out(r,
-// x) receives row r of the lane's column (each warp its own rows).
-template <typename T, int NW, typename F>
+// 437 us a view for 262144 x 512 BF16, 1.8 TB/s.)  buf: N x kC, scratch; out(r,
+// x) receives row r of the lane's column (each warp its own rows).  kC: columns
+// of the tile; with 16 a half-warp takes the part of a warp.
+template <typename T, int NW, int kC = 32, typename F>
 __device__ __forceinline__ void fwht_tile(T (&v)[32], T* buf, F out) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x % kC, w = threadIdx.x / kC;
 #pragma unroll
   for (int h = 1; h < 32; h <<= 1) {
 #pragma unroll
@@ -352,14 +353,14 @@ __device__ __forceinline__ void fwht_tile(T (&v)[32], T* buf, F out) {
       }
   }
 #pragma unroll
-  for (int t = 0; t < 32; ++t) buf[(32 * w + t) * 32 + lane] = v[t];
+  for (int t = 0; t < 32; ++t) buf[(32 * w + t) * kC + lane] = v[t];
   __syncthreads();
   constexpr int NJ = 32 / NW;  // residues of this warp: j = w NJ + q, rows j + 32 m
 #pragma unroll
   for (int q = 0; q < NJ; ++q) {
     T u[NW];
 #pragma unroll
-    for (int m = 0; m < NW; ++m) u[m] = buf[(w * NJ + q + 32 * m) * 32 + lane];
+    for (int m = 0; m < NW; ++m) u[m] = buf[(w * NJ + q + 32 * m) * kC + lane];
 #pragma unroll
     for (int h = 1; h < NW; h <<= 1) {
 #pragma unroll
@@ -440,38 +441,45 @@ __global__ void srht_stage1_small_kernel(const Tin* __restrict__ Z, int64_t ld, 
   for (int r = 0; r < N1; ++r) Tmid[(((int64_t)r * ncb + cb) * N2 + i2) * 32 + lane] = buf[r * 32 + lane];
 }
 
-// Sampled rows of the transform of residue a1: SZ[j] = scale * row (rows[j] >> m1).
-template <typename T>
-__device__ __forceinline__ void srht_pick(const T* buf, int d, int cb, int a1, int nsel, int m1, const int32_t* off1,
+// Sampled rows of the transform of residue a1, columns c0 .. c0 + kC - 1: SZ[j] =
+// scale * row (rows[j] >> m1).
+template <typename T, int kC = 32>
+__device__ __forceinline__ void srht_pick(const T* buf, int d, int c0, int a1, int nsel, int m1, const int32_t* off1,
                                           const int32_t* list, const int32_t* rows, double scale, double* SZ) {
-  for (int e = threadIdx.x; e < nsel * 32; e += blockDim.x) {
-    const int q = e >> 5, c = 32 * cb + (e & 31);
+  for (int e = threadIdx.x; e < nsel * kC; e += blockDim.x) {
+    const int q = e / kC, c = c0 + e % kC;
     const int j = list[off1[a1] + q];
-    if (c < d) SZ[(int64_t)j * d + c] = scale * (double)buf[(rows[j] >> m1) * 32 + (e & 31)];
+    if (c < d) SZ[(int64_t)j * d + c] = scale * (double)buf[(rows[j] >> m1) * kC + e % kC];
   }
 }
+
+// Columns of a CTA of stage 2: a whole tile of the intermediate, or half of one
+// where 32 columns do not fit shared memory (FP64 of 1024 rows: 262144 bytes of
+// the 232448).
+template <typename T, int NW> constexpr int kStage2Cols = sizeof(T) * 32 * NW * 32 > 232448 ? 16 : 32;
 
 // Stage 2: for one residue a1 of the low m1 row bits, the N2-point transform
 // across the row blocks of each column, kept only at the sampled rows and
 // scaled by sqrt(n'/s) / sqrt(n') = 1 / sqrt(s) (App. A).
 template <typename T, int NW>
-__global__ void __launch_bounds__(32 * NW)
+__global__ void __launch_bounds__(kStage2Cols<T, NW> * NW)
 srht_stage2_kernel(const T* __restrict__ Tmid, int d, int m1, const int32_t* __restrict__ off1,
                    const int32_t* __restrict__ list, const int32_t* __restrict__ rows, double scale,
                    double* __restrict__ SZ) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf = reinterpret_cast<T*>(smem_raw);
-  const int a1 = blockIdx.y, cb = blockIdx.x, ncb = gridDim.x;
+  constexpr int kC = kStage2Cols<T, NW>, kPer = 32 / kC;  // CTAs of a tile
+  const int a1 = blockIdx.y, cb = blockIdx.x / kPer, ncb = gridDim.x / kPer, first = kC * (blockIdx.x % kPer);
   const int nsel = off1[a1 + 1] - off1[a1];
   if (nsel == 0) return;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const T* src = Tmid + ((int64_t)a1 * ncb + cb) * (32 * NW) * 32;
+  const int lane = threadIdx.x % kC, w = threadIdx.x / kC;
+  const T* src = Tmid + ((int64_t)a1 * ncb + cb) * (32 * NW) * 32 + first;
   T v[32];
 #pragma unroll
   for (int t = 0; t < 32; ++t) v[t] = src[(32 * w + t) * 32 + lane];
-  fwht_tile<T, NW>(v, buf, [&](int r, T x) { buf[r * 32 + lane] = x; });
+  fwht_tile<T, NW, kC>(v, buf, [&](int r, T x) { buf[r * kC + lane] = x; });
   __syncthreads();
-  srht_pick(buf, d, cb, a1, nsel, m1, off1, list, rows, scale, SZ);
+  srht_pick<T, kC>(buf, d, 32 * cb + first, a1, nsel, m1, off1, list, rows, scale, SZ);
 }
 
 template <typename T>
@@ -487,7 +495,7 @@ __global__ void srht_stage2_small_kernel(const T* __restrict__ Tmid, int d, int 
   for (int r = 0; r < N2; ++r) buf[r * 32 + threadIdx.x] = src[r * 32 + threadIdx.x];
   fwht_thread_col<T>(buf + threadIdx.x, 32, N2);
   __syncwarp();
-  srht_pick(buf, d, cb, a1, nsel, m1, off1, list, rows, scale, SZ);
+  srht_pick(buf, d, 32 * cb, a1, nsel, m1, off1, list, rows, scale, SZ);
 }
 
 // group the sampled rows by their low m1 bits (order within a group is free:
@@ -543,10 +551,11 @@ int srht_stage1(const View& v, const Plan& p, int N2, const int32_t* lab, T* Tmi
 template <typename T, int NW>
 int srht_stage2(const View& v, const Plan& p, int N1, int m1, const int32_t* off1, const int32_t* list, const T* Tmid,
                 cudaStream_t st) {
-  const size_t sm = sizeof(T) * 32 * NW * 32;
+  constexpr int kC = kStage2Cols<T, NW>;
+  const size_t sm = sizeof(T) * 32 * NW * kC;
   auto k2 = srht_stage2_kernel<T, NW>;
   GB_CUDA(cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k2<<<dim3(ceil_div(v.d, 32), N1), 32 * NW, sm, st>>>(Tmid, v.d, m1, off1, list, p.h, 1.0 / sqrt((double)p.s), v.SZ);
+  k2<<<dim3(32 / kC * ceil_div(v.d, 32), N1), kC * NW, sm, st>>>(Tmid, v.d, m1, off1, list, p.h, 1.0 / sqrt((double)p.s), v.SZ);
   GB_CHECK_LAUNCH();
   return GBCCA_OK;
 }

@@ -584,3 +584,23 @@ def test_rebind_row_stride(gb, dt, k):
     for lds in ((64, 64), (48, 64), (48, 40), (45, 40)):
         for got, exp in zip(results(kept, lds), results(make(), lds)):
             assert np.array_equal(got, exp)
+
+
+def test_srht_f64_longest(gb):
+    """FP64 data of more than 2^18 rows, whose second stage takes 16 columns a
+    CTA (a ragged last tile, tiles with one and with two halves): within the
+    bound of test_srht_sizes."""
+    import torch
+    from oracle.sketch import srht_apply
+    from synth import srht_draws
+    n, s = 262145, 700
+    n_pad = 1 << 19
+    D, rows = srht_draws(n_pad, s, seed=3)
+    for d in (3, 16, 50):
+        X = np.random.default_rng(d).standard_normal((n, d))
+        x = torch.from_numpy(X).cuda()
+        plan = gb.cca_plan(n, d, d, 1, "f64", gb.default_options(sketch=gb.SRHT, s=s, warm_start=0))
+        gb.cca_precondition(plan, x, x, 1e3, 1e3, torch.from_numpy(rows).cuda(), torch.from_numpy(D).cuda())
+        ref = np.broadcast_to(np.abs(X).sum(0) / np.sqrt(s), (s, d))
+        got = np64(gb.query(plan, gb.Q_SKETCH_X)).reshape(s, d)
+        assert bound_ratio(got, srht_apply(X, D, rows), ref, (19 + 4) * 2.0 ** -53) <= 1.0
