@@ -77,6 +77,11 @@ constexpr int kFlagBucket = 3;    // CountSketch bucket index out of [0, s)
 constexpr int kFlagTimeout = 4;   // a bounded device wait ran out (kernel aborted)
 constexpr int kFlagLabel = 5;     // an FDA label outside [0, n_classes)
 
+// Records `code` unless an error stands already: the first one is the cause,
+// and what follows it (a factor of data that a sketch or a kernel which gave
+// up left void) is not.
+__device__ __forceinline__ void raise_flag(int* flag, int code) { atomicCAS(flag, 0, code); }
+
 // Status and message for a flag value read back from the device.
 inline int flag_status(int f) {
   switch (f) {

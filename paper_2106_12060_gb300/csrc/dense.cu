@@ -650,7 +650,7 @@ __global__ void __launch_bounds__(128) chol_diag_kernel(double* A, int d, int p,
     }
     __syncthreads();
   }
-  if (tid == 0 && s_bad) atomicExch(flag, kFlagNotSpd);
+  if (tid == 0 && s_bad) raise_flag(flag, kFlagNotSpd);
   for (int e = tid; e < nb * nb; e += blockDim.x) {
     const int r = e / nb, c = e % nb;
     if (c <= r) A[(int64_t)(o + r) * d + o + c] = L[r][c];
@@ -755,7 +755,7 @@ __global__ void __launch_bounds__(256) chol_next_kernel(double* A, double* Rinv,
   }
   __syncthreads();
   const bool ok = group_chol_inverse<256>(&sa[0][0], &sb[0][0], rs, nb, tid, 0, kNB + 1);
-  if (!ok && tid == 0) atomicExch(flag, kFlagNotSpd);
+  if (!ok && tid == 0) raise_flag(flag, kFlagNotSpd);
   for (int e = tid; e < nb * nb; e += 256) {
     const int r = e / nb, c = e % nb;
     if (c <= r) {

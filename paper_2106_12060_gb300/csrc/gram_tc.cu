@@ -283,7 +283,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0 && B->abort_flag) atomicExch(a.err, kFlagTimeout);
+  if (threadIdx.x == 0 && B->abort_flag) raise_flag(a.err, kFlagTimeout);
   if (warp == 2) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");

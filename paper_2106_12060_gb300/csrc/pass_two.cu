@@ -120,7 +120,7 @@ __device__ __forceinline__ uint32_t prologue(Bars* B, int stages, int acc_free_c
 }
 __device__ __forceinline__ void epilogue(Bars* B, uint32_t tmem, int* err) {
   __syncthreads();
-  if (threadIdx.x == 0 && B->abort_flag) atomicExch(err, kFlagTimeout);
+  if (threadIdx.x == 0 && B->abort_flag) raise_flag(err, kFlagTimeout);
   if ((threadIdx.x >> 5) == 2) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");

@@ -2665,7 +2665,7 @@ __global__ void __launch_bounds__(256) orth_kernel(const double* part, int nblk,
   __syncthreads();
   if (threadIdx.x < c) G[threadIdx.x * c + threadIdx.x] += 1e-14 * s_tr / c;
   const bool ok = group_chol_inverse<256>(G, Li, rs, c, threadIdx.x, 0);
-  if (!ok && threadIdx.x == 0) atomicExch(flag, kFlagNotSpd);
+  if (!ok && threadIdx.x == 0) raise_flag(flag, kFlagNotSpd);
   orth_apply(B, d, c, rows, Li, Bh, Bl);
 }
 
@@ -2690,13 +2690,13 @@ __global__ void __launch_bounds__(256) orth64_kernel(const double* part, int nbl
     if (threadIdx.x < 32) {
       double* invd = Li + c * c;
       const bool ok = warp_chol(G, c, invd);
-      if (!ok && threadIdx.x == 0) atomicExch(flag, kFlagNotSpd);
+      if (!ok && threadIdx.x == 0) raise_flag(flag, kFlagNotSpd);
       warp_lower_inv(G, invd, Li, c);
     }
     __syncthreads();
   } else {
     if (!blk_chol(G, c)) {
-      if (threadIdx.x == 0) atomicExch(flag, kFlagNotSpd);
+      if (threadIdx.x == 0) raise_flag(flag, kFlagNotSpd);
     }
     blk_lower_inv(G, Li, c);
   }

@@ -604,3 +604,21 @@ def test_srht_f64_longest(gb):
         ref = np.broadcast_to(np.abs(X).sum(0) / np.sqrt(s), (s, d))
         got = np64(gb.query(plan, gb.Q_SKETCH_X)).reshape(s, d)
         assert bound_ratio(got, srht_apply(X, D, rows), ref, (19 + 4) * 2.0 ** -53) <= 1.0
+
+
+@pytest.mark.parametrize("dt", ["bf16", "f32", "f64"])
+def test_first_error_is_reported(gb, dt):
+    """Buckets outside the sketch leave it empty, so that without a ridge the
+    factorization fails too: the call reports the buckets."""
+    import torch
+    n, d, s = 200, 4, 60
+    tdt = {"bf16": torch.bfloat16, "f32": torch.float32, "f64": torch.float64}[dt]
+    x = torch.from_numpy(np.random.default_rng(0).standard_normal((n, d))).to(tdt).cuda()
+    h = torch.full((n,), s, dtype=torch.int32, device="cuda")
+    g = torch.ones(n, dtype=torch.int8, device="cuda")
+    plan = gb.cca_plan(n, d, d, 1, dt, gb.default_options(s=s))
+    for lam in (1.0, 0.0):
+        with pytest.raises(gb.GbccaError) as e:
+            gb.cca_precondition(plan, x, x, lam, lam, h, g)
+        assert e.value.code == gb.ERR_INVALID_ARG
+    gb.cca_precondition(plan, x, x, 1.0, 1.0)  # the flag does not outlive the call
