@@ -9,16 +9,27 @@
 
 namespace gbcca {
 
-// 1 / x in FP64: the hardware's approximation (about 20 bits) corrected by one
-// third-order step, y (1 + e + e^2) with e = 1 - x y: three dependent
-// multiply-adds instead of a division, and no conversion (which would run at
-// the FP64 rate).  Near the ends of the exponent range: 1 / x.
+// 1 / x in FP64 by the Newton-Raphson iteration for 1 / y - x, y <- y + y (1 - x y),
+// which doubles the correct bits: a single-precision quotient (about 22 bits),
+// one step in FP32 with the mantissa of x split into a float and the rest, one
+// step in FP64.  Only that last step is FP64 work (two dependent multiply-adds):
+// the mantissa comes out of, and the reciprocal goes back into, a double as
+// integers, since conversions run at the FP64 rate.  At most one unit in the
+// last place from the quotient; 1 / x where x or the result is not normal.
 __device__ __forceinline__ double rcp_nr(double x) {
-  if (((uint32_t)__double2hiint(x) & 0x7fffffffu) - 0x00200000u >= 0x7fa00000u) return 1.0 / x;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int ex = (int)(hi >> 20 & 0x7ff);
+  if ((unsigned)(ex - 2) > 2041u) return 1.0 / x;
+  const float m = __uint_as_float(0x3f800000u | (hi & 0xfffffu) << 3 | lo >> 29);  // |x| = 2^(ex - 1023) (m + rest)
+  const float rest = (float)(lo & 0x1fffffffu) * 2.220446049250313e-16f;          // 2^-52 a bit
+  const float r = __fdividef(1.f, m);
+  const float c = r * (fmaf(-m, r, 1.f) - rest * r);
+  // r + c in units of 2^-52: r is a multiple of 2^-25, and 2^51 (one half)
+  // starts the mantissa of exponent field 1022
+  const long long y52 = ((long long)__float2int_rn(r * 33554432.f) << 27) + __float2int_rn(c * 4503599627370496.f);
+  const long long bits = ((long long)(2045 - ex) << 52) + ((y52 - (1ll << 51)) << 1);
+  const double y = __longlong_as_double(bits | (long long)(hi & 0x80000000u) << 32);
+  return fma(y, fma(-x, y, 1.0), y);
 }
 
 // Barrier over the G threads of a group (id 0: the whole CTA).
