@@ -743,12 +743,16 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
 // 128B-swizzled.  The point the pass evaluates, hi +
 // lo, is written to Phi, so that it is exactly the point the solver holds
 // (src may be Phi itself).  One thread per element of Phi (every view in
-// one launch); the padding of the image is zero from its allocation
-// and never written.
+// one launch), and per element of the columns that fill up the boxes the pass
+// reads, which are zero: a batch lays the image out with its own number of
+// rows, so what was padding of one layout held entries of another (an infinity
+// or NaN there would reach every product).  Rows beyond the 2k of a half are left
+// as they are; the columns of W that they form are never used.
 struct ImageArgs {
   const double* src[2];  // d x k2 row-major
   double* Phi[2];
   int d[2];
+  int pad[2];            // columns of the boxes that the pass reads
   int k2;
   int h;                 // image rows per half
   uint8_t* img;
@@ -765,17 +769,17 @@ __global__ void __launch_bounds__(256) phi_image_kernel(const __grid_constant__ 
   if (m.done != nullptr && *m.done) return;
   const int v = blockIdx.y;
   if (m.restart != nullptr && v == 0 && blockIdx.x == 0 && threadIdx.x == 0) *m.restart = 0;
-  const int d = v == 0 ? m.d[0] : m.d[1];
   const int e = blockIdx.x * blockDim.x + threadIdx.x;  // (data column j, Phi column q)
-  if (e >= d * m.k2) return;
+  if (e >= (v == 0 ? m.pad[0] : m.pad[1]) * m.k2) return;
   const int j = e / m.k2, q = e - j * m.k2;
-  const double x = (v == 0 ? m.src[0] : m.src[1])[e];
+  const bool in = j < (v == 0 ? m.d[0] : m.d[1]);
+  const double x = in ? (v == 0 ? m.src[0] : m.src[1])[e] : 0.0;
   const __nv_bfloat16 hi = __double2bfloat16(x);
   const __nv_bfloat16 lo = __double2bfloat16(x - (double)__bfloat162float(hi));
   uint8_t* base = m.img + (int64_t)v * m.img_view + (int64_t)(j >> 6) * (2 * m.h * 128);
   *reinterpret_cast<__nv_bfloat16*>(base + swz(q, j & 63)) = hi;
   *reinterpret_cast<__nv_bfloat16*>(base + swz(m.h + q, j & 63)) = lo;
-  (v == 0 ? m.Phi[0] : m.Phi[1])[e] = (double)__bfloat162float(hi) + (double)__bfloat162float(lo);
+  if (in) (v == 0 ? m.Phi[0] : m.Phi[1])[e] = (double)__bfloat162float(hi) + (double)__bfloat162float(lo);
 }
 
 // After the data kernel: G = the sum of the clusters' partial slabs, and the
@@ -1020,6 +1024,13 @@ int64_t tc_gpart_len(const Plan& p) {
 }
 int64_t tc_part_len(const Plan& p) { return tc_max_slabs(p) * tc_slab(p); }
 
+// Columns of a view's image: whole boxes of 64, which the one-sweep pass over two
+// views reads in pairs.
+static int tc_image_cols(const Plan& p, int v) {
+  const int unit = tc_two(p) || tc_solo(p) ? 64 : 128;
+  return ceil_div(p.v[v].d, unit) * unit;
+}
+
 // Arguments of the Phi images of a plan, h1 rows per half (0: the plan's own);
 // Phi is read from the caller's blocks when `io` is given, else from the
 // plan's own.
@@ -1030,6 +1041,7 @@ static tc::ImageArgs tc_image_args(const Plan& p, int h1, const int* done, const
     a.src[v] = io != nullptr ? io->Phi[v] : p.v[v].Phi;
     a.Phi[v] = p.v[v].Phi;
     a.d[v] = p.v[v].d;
+    a.pad[v] = tc_image_cols(p, v);
   }
   a.k2 = 2 * p.k;
   a.h = h1 > 0 ? h1 : tc_h1(p);
@@ -1039,8 +1051,8 @@ static tc::ImageArgs tc_image_args(const Plan& p, int h1, const int* done, const
   return a;
 }
 static int tc_image_blocks(const Plan& p) {
-  const int dmax = std::max(p.v[0].d, tc_nviews(p) > 1 ? p.v[1].d : 0);
-  return ceil_div(dmax * 2 * p.k, 256);
+  const int cols = std::max(tc_image_cols(p, 0), tc_nviews(p) > 1 ? tc_image_cols(p, 1) : 0);
+  return ceil_div(cols * 2 * p.k, 256);
 }
 
 // The Phi images of a plan; also rounds Phi to the bf16 hi + lo point the

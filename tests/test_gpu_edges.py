@@ -622,3 +622,38 @@ def test_first_error_is_reported(gb, dt):
             gb.cca_precondition(plan, x, x, lam, lam, h, g)
         assert e.value.code == gb.ERR_INVALID_ARG
     gb.cca_precondition(plan, x, x, 1.0, 1.0)  # the flag does not outlive the call
+
+
+@pytest.mark.parametrize("shapes", [((500, 40, 9), (600, 40, 12)), ((500, 200, 3), (600, 129, 11)),
+                                    ((700, 600, 4), (800, 530, 17))])
+def test_phi_image_after_nan(gb, shapes):
+    """A batch of plans with different k lays their Phi images out alike; NaN
+    in one call leaves nothing in the next, alone or in the batch: both give
+    what they gave before, bitwise."""
+    import torch
+    rng = np.random.default_rng(0)
+    plans, data, Phi = [], [], []
+    for n, d, k in shapes:
+        data.append([torch.zeros(n, (d + 7) // 8 * 8, dtype=torch.bfloat16, device="cuda")[:, :d] for _ in range(2)])
+        for t in data[-1]:
+            t.copy_(torch.from_numpy(rng.standard_normal((n, d))))
+        plans.append(gb.cca_plan(n, d, d, k, "bf16", gb.default_options()))
+        gb.cca_precondition(plans[-1], *data[-1], 1.0, 1.0)
+        Phi.append([torch.from_numpy(rng.standard_normal((d, 2 * k))).cuda() for _ in range(2)])
+    alone = [[np64(t) for t in gb.fused_pass(p, *f)] for p, f in zip(plans, Phi)]
+    batch = gb.Batch(plans)
+
+    def together(f):
+        G, Gram = gb.batch_fused_pass(batch, [a for a, _ in f], [b for _, b in f])
+        return [np64(t) for t in (*G, *Gram)]
+
+    first = together(Phi)
+    nan = [[torch.full_like(a, float("nan")) for a in f] for f in Phi]
+    for _ in range(2):
+        together(nan)
+        for p, f, exp in zip(plans, Phi, alone):
+            assert all(np.array_equal(np64(g), e) for g, e in zip(gb.fused_pass(p, *f), exp))
+        for p, f in zip(plans, nan):
+            gb.fused_pass(p, *f)
+        assert all(np.array_equal(g, e) for g, e in zip(together(Phi), first))
+    batch.close()
