@@ -252,6 +252,8 @@ int minv_df_build(const double* Rinv, int d, float* hi, float* lo, double* ws, i
 // Rinv = R^{-1} (upper triangular, d x d); ws holds at least d * d doubles.
 int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t ws_len, cudaStream_t st,
                       bool have_diag = false);
+// C (m x n) = T^T B, or B T with `right`; T upper triangular
+int tri_mul(bool right, const double* T, const double* B, int m, int n, double* C, cudaStream_t st);
 // C (m x c, ldc) = op(A) B (rows of B = columns of op(A), ldb), A ra x ca
 // row-major, for one or two problems in one launch; tri: A upper triangular,
 // its zero half skipped.

@@ -2811,29 +2811,20 @@ int warm_start(Plan& p, cudaStream_t st) {
     double* small = p.phigram;
     // Products of the power iteration with C = R_x^{-T} Cxy R_y^{-1}.  FP64
     // plans: FP64 triangular / dense products one after another.  FP32/BF16
-    // plans: C is formed once in double-float (~2^-44 relative, at FP32
-    // instruction rates), in place of three products per half step; FP32
-    // copies of R^{-1} (kappa ~ 1e4) give a visibly worse start point and
-    // more solver iterations.
+    // plans: C is formed once, in FP64 (its factors amplify a rounding by the
+    // condition of R_x and R_y), and applied to the blocks in double-float
+    // (2^-44, nothing amplified: C has no entry beyond 1), in place of three
+    // products per half step.
     const bool low = p.dtype != GBCCA_FP64;
-    const int64_t N = (std::max((int64_t)dx * dx, std::max((int64_t)dy * dy, (int64_t)dx * dy)) + 1) / 2 * 2;
-    float* w0 = reinterpret_cast<float*>(p.ws);          // pairs of at most N entries each
-    float* w1 = reinterpret_cast<float*>(p.ws + N);
-    const int64_t nx = (int64_t)dx * dx, ny = (int64_t)dy * dy, nc = (int64_t)dx * dy;
-    float* Cf[2] = {w0, w0 + nc};
-    float* CfT[2] = {w1, w1 + nc};
+    const int64_t nc = (int64_t)dx * dy;
+    float* Cf[2] = {reinterpret_cast<float*>(p.ws), reinterpret_cast<float*>(p.ws) + nc};
+    float* CfT[2] = {Cf[0] + 2 * nc, Cf[0] + 3 * nc};
     float* Vp[2] = {p.dfx, p.dfx + (int64_t)dy * c};
     float* Up[2] = {p.dfx + 2 * (int64_t)dy * c, p.dfx + 2 * (int64_t)dy * c + (int64_t)dx * c};
     if (low) {
-      double* P = p.ws + 2 * N;
-      double* part64 = p.ws + 3 * N;
-      const int64_t plen = p.ws_len - nc - 3 * N;
-      GB_TRY(split_df(x.Rinv, dx, dx, false, w0, w0 + nx, st));
-      GB_TRY(split_df(Cxy, dx, dy, false, w1, w1 + nc, st));
-      GB_TRY(gram_df_split(w0, w0 + nx, dx, w1, w1 + nc, dy, dx, dx, dy, P, 0.0, part64, plen, st));   // R_x^{-T} Cxy
-      GB_TRY(split_df(P, dx, dy, true, w0, w0 + nc, st));
-      GB_TRY(split_df(y.Rinv, dy, dy, false, w1, w1 + ny, st));
-      GB_TRY(gram_df_split(w0, w0 + nc, dx, w1, w1 + ny, dy, dy, dx, dy, Cxy, 0.0, part64, plen, st));  // ... R_y^{-1}
+      double* P = p.ws + 2 * nc;
+      GB_TRY(tri_mul(false, x.Rinv, Cxy, dx, dy, P, st));
+      GB_TRY(tri_mul(true, y.Rinv, P, dx, dy, Cxy, st));
       GB_TRY(split_df(Cxy, dx, dy, false, Cf[0], Cf[1], st));
       GB_TRY(split_df(Cxy, dx, dy, true, CfT[0], CfT[1], st));
     }

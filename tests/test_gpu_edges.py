@@ -657,3 +657,47 @@ def test_phi_image_after_nan(gb, shapes):
             gb.fused_pass(p, *f)
         assert all(np.array_equal(g, e) for g, e in zip(together(Phi), first))
     batch.close()
+
+
+@pytest.mark.parametrize("dx,dy,k", [(40, 30, 5), (101, 37, 3), (5, 40, 3), (3, 3, 2)])
+def test_warm_start_rounding_f32(gb, dx, dy, k):
+    """The whitened cross matrix C of an FP32 plan's warm start, for views of
+    condition about 1e4 and power iterations to their end: the pairs are
+    singular pairs of C, up to sixteen times what the rounding of NumPy's FP64
+    products of the same factors does to such a residual (their sums run in
+    another order).  Products in double-float pairs are 2^9 times coarser."""
+    import torch
+    from synth import countsketch_draws
+    big, lam, kap = np.longdouble, 1e-8, 1e4
+    s = 4 * (dx + dy)
+    n = 4 * s
+    rng = np.random.default_rng(dx)
+    m = min(dx, dy)
+    z = rng.standard_normal((n, m)) * np.concatenate([np.linspace(3, 1, k), np.full(m - k, 0.1)])
+    data = []
+    for d in (dx, dy):
+        A = 0.5 * rng.standard_normal((n, d))
+        A[:, :m] += z
+        A = (A * np.logspace(0, -np.log10(kap), d)) @ np.linalg.qr(rng.standard_normal((d, d)))[0]
+        data.append(torch.from_numpy(A.astype(np.float32)).cuda())
+    h, g = countsketch_draws(n, s, seed=3)
+    plan = gb.cca_plan(n, dx, dy, k, "f32", gb.default_options(s=s, warm_iters=400))
+    gb.cca_precondition(plan, *data, lam, lam, torch.from_numpy(h).cuda(), torch.from_numpy(g).cuda())
+    S = [np64(gb.query(plan, q)).reshape(s, d) for q, d in ((gb.Q_SKETCH_X, dx), (gb.Q_SKETCH_Y, dy))]
+    R = [np64(gb.query(plan, q)).reshape(d, d) for q, d in ((gb.Q_R_X, dx), (gb.Q_R_Y, dy))]
+    A, B = (r.astype(big) @ np64(gb.query(plan, q)).reshape(-1, k).astype(big)
+            for r, q in zip(R, (gb.Q_WARM_U, gb.Q_WARM_V)))
+
+    def solve(r, M):  # r^{-T} M by forward substitution
+        X = M.copy()
+        for i in range(len(r)):
+            X[i] = (X[i] - r[:i, i] @ X[:i]) / r[i, i]
+        return X
+
+    C = solve(R[0].astype(big), S[0].astype(big).T @ S[1].astype(big))
+    C = solve(R[1].astype(big), C.T.copy()).T
+    Ri = [np.linalg.inv(r) for r in R]
+    E = Ri[0].T @ (S[0].T @ S[1]) @ Ri[1] - C
+    sig = np.sum(A * (C @ B), axis=0)
+    got = max(np.max(np.abs(C @ B - A * sig)), np.max(np.abs(C.T @ A - B * sig)))
+    assert got <= 16 * max(np.max(np.abs(E @ B)), np.max(np.abs(E.T @ A)))
