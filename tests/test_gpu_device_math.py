@@ -19,6 +19,14 @@ __global__ void rcp_k(const double* x, double* y, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = gbcca::rcp_nr(x[i]);
 }
+__global__ void widen_k(const float* x, double* y, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = gbcca::widen(x[i]);
+}
+extern "C" int widen(const float* x, double* y, int n) {
+  widen_k<<<(n + 255) / 256, 256>>>(x, y, n);
+  return (int)cudaDeviceSynchronize();
+}
 extern "C" int rcp(const double* x, double* y, int n) {
   rcp_k<<<(n + 255) / 256, 256>>>(x, y, n);
   return (int)cudaDeviceSynchronize();
@@ -63,3 +71,19 @@ def test_reciprocal(lib):
     assert np.array_equal(np.signbit(got[plain & ~np.isnan(x)]), np.signbit(exp[plain & ~np.isnan(x)]))
     ulp = np.abs(got[~plain].view(np.int64) - exp[~plain].view(np.int64))
     assert ulp.max() <= 1
+
+
+def test_widen(lib):
+    """FP32 to FP64 by moving the bits: every exponent field (subnormals and
+    infinities among them) with mantissas at the ends of their range, single
+    bits and random ones, both signs: the same bits as a conversion; NaN stays
+    NaN."""
+    rng = np.random.default_rng(0)
+    ends = np.concatenate([1 << np.arange(23), (1 << 23) - 1 - (1 << np.arange(23)), [0, (1 << 23) - 1]])
+    man = np.concatenate([np.broadcast_to(ends, (256, len(ends))), rng.integers(0, 1 << 23, (256, 2000))], 1)
+    bits = ((np.arange(256, dtype=np.uint32)[:, None] << np.uint32(23)) | man.astype(np.uint32)).ravel()
+    x = np.concatenate([bits, bits | np.uint32(1 << 31)]).view(np.float32)
+    got = _call(lib.widen, x, np.float64)
+    nan = np.isnan(x)
+    assert np.all(np.isnan(got[nan]))
+    assert np.array_equal(got[~nan].view(np.int64), x[~nan].astype(np.float64).view(np.int64))

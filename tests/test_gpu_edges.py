@@ -701,3 +701,37 @@ def test_warm_start_rounding_f32(gb, dx, dy, k):
     sig = np.sum(A * (C @ B), axis=0)
     got = max(np.max(np.abs(C @ B - A * sig)), np.max(np.abs(C.T @ A - B * sig)))
     assert got <= 16 * max(np.max(np.abs(E @ B)), np.max(np.abs(E.T @ A)))
+
+
+@pytest.mark.parametrize("dt", ["bf16", "f32"])
+def test_two_sweep_long_ranges(gb, dt):
+    """So many rows beside so few columns that a CTA's range of tiles is summed
+    in several accumulations (alone and in a batch beside a short plan):
+    entries of -1, 0 and 1 and a Phi that picks columns make every sum an
+    integer below 2^24, so the products are exact."""
+    import torch
+    n, dx, dy, k = 350003, 32, 24, 20
+    tdt = {"bf16": torch.bfloat16, "f32": torch.float32}[dt]
+    g = torch.Generator(device="cuda").manual_seed(1)
+    plans, data, Phi, exact = [], [], [], []
+    for m in (n, 700):
+        Z = [torch.randint(-1, 2, (m, d), generator=g, device="cuda").to(tdt) for d in (dx, dy)]
+        P = [torch.zeros(d, 2 * k, dtype=torch.float64, device="cuda") for d in (dx, dy)]
+        for p, step in zip(P, (7, 5)):
+            c = torch.arange(2 * k, device="cuda")
+            p[(c * step) % p.shape[0], c] = 1.0
+        plan = gb.cca_plan(m, dx, dy, k, dt, gb.default_options())
+        gb.cca_precondition(plan, *Z, 1.0, 1.0)
+        W = torch.cat([z.double() @ p for z, p in zip(Z, P)], 1)
+        plans.append(plan)
+        data.append(Z)
+        Phi.append(P)
+        exact.append(([z.double().T @ W for z in Z], W.T @ W))
+    batch = gb.Batch(plans)
+    Gb, Mb = gb.batch_fused_pass(batch, [p[0] for p in Phi], [p[1] for p in Phi])
+    for i, plan in enumerate(plans):
+        (Ex, Ey), Em = exact[i]
+        Gx, Gy, Gram = gb.fused_pass(plan, *Phi[i])
+        assert torch.equal(Gx, Ex) and torch.equal(Gy, Ey) and torch.equal(Gram, Em)
+        assert torch.equal(Gb[i], torch.cat([Ex, Ey])) and torch.equal(Mb[i], Em)
+    batch.close()
