@@ -949,9 +949,9 @@ int tri_inverse_upper(const double* R, double* Rinv, int d, double* ws, int64_t 
 // R_x^{-T} C_xy R_y^{-1}.  Each CTA one 16 x 16 tile, an entry per thread with its
 // terms in order, the inner range cut to where T is non-zero, the longest
 // ranges first.  Bound by the FP64 rate: with 512 columns in both views a
-// preconditioner takes 160 us longer than with double-float products (3.12 to
-// 3.29 ms), whose rounding, amplified by the factors, left singular pairs 17
-// to 30 times further off than FP64 products do.
+// preconditioner takes 130 us longer than with double-float products (3.16 to
+// 3.29 ms), whose rounding, amplified by the factors, left singular pairs 9
+// to 29 times further off than FP64 products do (condition 1e4).
 template <bool kRight>
 __global__ void __launch_bounds__(256) tri_mul_kernel(const double* __restrict__ T, const double* __restrict__ B, int m,
                                                       int n, double* __restrict__ C) {

@@ -1,5 +1,5 @@
-// Grams of sketched views on the tensor cores (tcgen05 + TMA, sm_103a), exact
-// to far below FP64's needs here: C = A^T B for the FP64 sketches A (s x d1)
+// Grams of sketched views on the tensor cores (tcgen05 + TMA, sm_103a), with
+// about the error of FP64 sums: C = A^T B for the FP64 sketches A (s x d1)
 // and B (s x d2) of FP32/BF16 plans (Alg. 1 steps 2-4, Alg. 2 step 3).
 //
 // Method (error-free splitting for matrix products: Ozaki, Ogita, Oishi, Rump,
@@ -10,10 +10,17 @@
 // rows, stay below 2^24, so the FP32 accumulators of the 28 MMAs per K step
 // (levels 0 .. 6) hold exact integers.  After every window the epilogue adds
 // them, shifted by their levels, into one 64-bit integer per entry in units of
-// 2^-50 (rounding below 2^-51 of the columns' largest products), which is
-// exact up to kMaxRows rows per CTA (coarser units serve longer ranges).
-// Against the double-float sums before (2^-44 of each term) the error is
-// smaller.
+// 2^-50, up to kMaxRows rows per CTA (coarser units serve longer ranges).
+//
+// Error of an entry, in units of the product of its columns' largest entries:
+// at most 2^-55 a row from the digits' rounding, 6 x 2^-56 a row from the levels
+// left out (t + u >= 7), 2^-51 a window from the units (2^(drop - 51) with coarser
+// ones): s 2^-53 and a thirty-second of it.  So it is bounded by the columns'
+// norms, as an FP64 sum's is, not by the sum of an entry's own |terms|: where
+// outlier rows dwarf the rest of a column, entries among the rest keep fewer
+// bits than the double-float sums before gave them (2^-44 of each term).  For the
+// factorization, whose error is relative to the columns' norms too, that does
+// not matter.
 //
 // Bound by MMA issue (one thread issues an MMA about every 50 cycles; 56 per
 // 32 rows) and the windows' epilogue, which the single set of 7 x 64
@@ -21,7 +28,7 @@
 // FP32 issue (12 instructions a term): 690 us for 4096 x (512 + 512) and 370 us
 // for each symmetric 512 x 512; 84 and 57 us now, and 26 us for the digits and
 // the scaling of each.  Error of R^T R against FP64 over 24 to 1000 columns and
-// both sketches: 2.5e-15 of the columns' norms before, 5e-17 now.
+// both sketches, measured: 2.5e-15 of the columns' norms before, 5e-17 now.
 #include "tc_ptx.cuh"
 
 namespace gbcca {

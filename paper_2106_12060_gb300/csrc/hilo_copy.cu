@@ -46,7 +46,10 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // Uncentred data need no FP64 at all: z - bf16(z) is exact in FP32.  The
 // class means are float pairs (mh + ml = the FP64 mean to 2^-48), z - mh is
 // taken with its rounding error, and both roundings to bf16 use the
-// remainder on ties, so the values are those of FP64 arithmetic to 2^-48.
+// remainder on ties.  The centred value is within 2^-48 |m|, and never further
+// than 2^-24 of itself, from FP64's; rounded to the copy's 17 bits, none of 4e6
+// pairs differed from FP64 centring for means of up to ten deviations, one in
+// 35000 at 1e4 and one in 700 at 1e6.
 // A CTA takes `rows` whole rows as 4-column chunks, kChunks chunks of a thread
 // in flight; kVec: 16-byte loads (row starts and stride 16-byte aligned), a
 // ragged last chunk by element (nothing past a row's d columns is read).

@@ -12,7 +12,7 @@
 // outputs only, and small inputs are spread over all SMs: the products of
 // 2000 x 90 data with 10 columns per view run on 125 CTAs of 16 rows, where
 // 64-row tiles with columns padded to a multiple of 8 took 55 us on 32 SMs
-// (98 us for the whole call; 45 us now).  One refinement pass over 100000
+// (98 us for the whole call; 31 us now).  One refinement pass over 100000
 // x 784 FP32 with 9 columns is most of what took an LDA solve from 15.2 to
 // 14.0 ms.
 #include "pass64.h"

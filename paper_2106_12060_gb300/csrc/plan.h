@@ -151,7 +151,7 @@ struct Plan {
   int64_t tc_map_ld[2] = {0, 0};
   uint8_t* tc_img = nullptr;
   float* tc_part = nullptr;
-  int tc_clusters = 0;
+  int tc_clusters = 0;  // resident 2-CTA clusters of the tensor-core pass (0: not yet queried)
   // one batch of RCG iterations as a CUDA graph: captured on the plan's own
   // stream (the caller's may be the legacy default stream, which cannot be
   // captured), replayed on the solve's stream; the key records what the
@@ -161,9 +161,10 @@ struct Plan {
   cudaStream_t side_stream = nullptr;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   cudaEvent_t ritz_fork = nullptr, ritz_join = nullptr;  // the Ritz-check branch of an iteration
-  // an iteration's Phi Gram on a branch beside the pass reduction: the
-  // solver asks for it (fork_after_pass), the tensor-core pass records
-  // pass_fork after its data kernels (pass_forked)
+  // FDA: an iteration's Yhat Phi (and the Grams of Phi where the pass does not
+  // form them) on a branch beside the pass reduction: the solver asks for it
+  // (fork_after_pass), the tensor-core pass records pass_fork after its data
+  // kernels (pass_forked)
   cudaEvent_t pass_fork = nullptr, pass_join = nullptr;
   bool fork_after_pass = false, pass_forked = false;
   bool phired_ready = false;  // the pass has also formed the Grams of Phi (tensor-core pass)
@@ -181,7 +182,7 @@ struct Plan {
   bool ts_ready = false;
   float* means_df = nullptr;  // FDA: the class means as float pairs (l x d padded to 4: hi, then lo)
   cudaEvent_t kev0 = nullptr;  // when set: recorded around the data kernel of the next pass
-  cudaEvent_t kev1 = nullptr;  // resident 2-CTA clusters of the tensor-core pass (0: not yet queried)
+  cudaEvent_t kev1 = nullptr;
 };
 
 // Blocks of a stand-alone pass: Phi read from, and G (per view) and the Gram
