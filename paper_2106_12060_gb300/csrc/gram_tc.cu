@@ -299,8 +299,9 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
 
 // C = the splits' integers summed (exactly, as high and low words) and scaled
 // back, + diag_add on the diagonal.  A column beyond the FP32 range (or not
-// finite) makes its entries NaN, and one whose squares vanish in FP32 has no
-// square here either, which the factorization reports (with diag_add = 0).
+// finite) makes its entries NaN, and columns whose products vanish in FP32 have
+// none here either: the factorization reports both (the second with diag_add =
+// 0), and the warm start a cross matrix of zeros.
 __global__ void __launch_bounds__(256) gram_scale_kernel(const long long* __restrict__ part, int ks, int d1, int d2,
                                                          const int* __restrict__ ea, const int* __restrict__ eb,
                                                          int sym, int drop, double diag_add, double* __restrict__ C) {
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(256) gram_scale_kernel(const long long* __rest
   const int Ei = max(ea[i], 1), Ej = max(eb[j], 1);
   double x = scalbn(fma((double)hi, 4294967296.0, (double)lo), Ei + Ej - 2 * 1022 - 50 + drop);
   if (Ei > kMaxExp || Ej > kMaxExp) x = __longlong_as_double(0x7ff8000000000000ll);
-  if (sym && i == j && Ei < kMinExp) x = 0.0;
+  if (Ei + Ej < 2 * kMinExp) x = 0.0;
   C[e] = x + (i == j ? diag_add : 0.0);
 }
 

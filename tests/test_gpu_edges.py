@@ -735,3 +735,22 @@ def test_two_sweep_long_ranges(gb, dt):
         assert torch.equal(Gx, Ex) and torch.equal(Gy, Ey) and torch.equal(Gram, Em)
         assert torch.equal(Gb[i], torch.cat([Ex, Ey])) and torch.equal(Mb[i], Em)
     batch.close()
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+def test_warm_start_range(gb, dt):
+    """Cross products of the sketches that vanish in FP32 leave the warm start
+    nothing to start from, whatever the ridge: both forms of the Gram report
+    it, and neither does where the products are there."""
+    import torch
+    n, d = 300, 9
+    tdt = {"f32": torch.float32, "bf16": torch.bfloat16}[dt]
+    rng = np.random.default_rng(0)
+    X = rng.standard_normal((n, d))
+    Y = 0.5 * X + rng.standard_normal((n, d))
+    for tc in (1, 0):
+        for scale, lam, refused in ((1e-26, 1e-30, True), (1e-24, 1e-30, True), (1e-26, 1e-1, True),
+                                    (1e-18, 1e-30, False), (1e-10, 1e-1, False), (1.0, 1e-1, False)):
+            x, y = (torch.from_numpy(a * scale).to(tdt).cuda() for a in (X, Y))
+            plan = gb.cca_plan(n, d, d, 2, dt, gb.default_options(tensor_cores=tc))
+            assert _refused(lambda: gb.cca_precondition(plan, x, y, lam, lam)) == refused
