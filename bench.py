@@ -53,8 +53,8 @@ LDA_CHECK_EVERY = 8
 # from an ncu capture of 131072 rows of this workload (reads scaled by rows
 # to 262144, partial writes as measured).  Valid only for the kernel source
 # it was taken on (SHA-256 below); any other source reports null.
-PASS_TRAFFIC_BYTES = 268.589056e6 * 2 + 9.728256e6
-PASS_TRAFFIC_SRC_SHA256 = "2b775a423f024040bf6b29a32e978e8699ee1967f517693e817ffaacaa99c993"
+PASS_TRAFFIC_BYTES = 268.59008e6 * 2 + 9.76896e6
+PASS_TRAFFIC_SRC_SHA256 = "15e3b8025cecca3cfe255afe45f453f04384e2b2294c55e31c554799c79abf92"
 
 
 def pass_traffic():
